@@ -17,6 +17,9 @@ size_t edge_checks_workspace(uint64_t);
 cudaError_t launch_edge_screen(const pcl_params &, const pcl_clipset &, pcl_pair *, uint64_t,
                                unsigned long long *, unsigned long long *, cudaStream_t, uint32_t, uint32_t, void *,
                                size_t, int);
+size_t edge_join_workspace(uint32_t);
+cudaError_t launch_edge_join(const pcl_params &, const pcl_clipset &, void *, size_t, pcl_pair *, uint64_t,
+                             unsigned long long *, unsigned long long *, int, cudaStream_t);
 cudaError_t launch_edge_screen_cross(const pcl_params &, const pcl_clipset &, const pcl_clipset &, pcl_pair *,
                                      uint64_t, unsigned long long *, unsigned long long *, cudaStream_t, void *,
                                      size_t, int);
@@ -303,6 +306,11 @@ pcl_status pcl_candidates_shard(pcl_ctx *ctx, const pcl_params *P, uint32_t mode
         e = launch_band_join(*P, *cs, ctx->ws, ctx->ws_bytes, d_out, cap, cnt, gates, ctx->num_sms, st, shard,
                              n_shards);
         return e == cudaSuccess ? PCL_OK : cuda_fail(ctx, e, "band join");
+    }
+    if (mode == PCL_MODE_EDGE && n_shards == 1 && !topo) {
+        if ((s = ensure_ws(ctx, edge_join_workspace(cs->n_clips)))) return s;
+        e = launch_edge_join(*P, *cs, ctx->ws, ctx->ws_bytes, d_out, cap, cnt, gates, ctx->num_sms, st);
+        return e == cudaSuccess ? PCL_OK : cuda_fail(ctx, e, "edge join");
     }
     if (mode == PCL_MODE_EDGE) {
         const uint64_t n = cs->n_clips;

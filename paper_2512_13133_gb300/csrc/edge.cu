@@ -1,12 +1,14 @@
 // a2 (edge gates) and a7: edge-displacement mode (Sec. 2.2.2) with the
 // geometric Min-Max closed form of Sec. 3.2.2 (Eq. 6), integer dbu throughout.
 //
-// edge_screen_kernel: the self-join screen of all pairs i < j through E2 and
-// E1 (tiles of 32 row clips x 256 column clips; the cheap occupancy-grid
-// tests of E1 run one pair per lane; the few survivors go to a list whose
-// exact correspondence edge_check_kernel checks afterwards, one pair per
-// warp).  edge_match_kernel: the Min-Max record of each listed pair, one pair
-// per warp (lanes hold the polygons).
+// edge_screen_kernel: the screen of pairs through E2 and E1 one by one, for a
+// shard of the self-join, two clip sets and the topological pre-screen (the
+// whole self-join takes the bit tables of edge_join.cu: 10.2 against 78.6 ms at
+// 100,000 clips); tiles of 32 row clips x 256 column clips; the cheap
+// occupancy-grid tests of E1 run one pair per lane; the few survivors go to a
+// list whose exact correspondence edge_check_kernel checks afterwards, one pair
+// per warp.  edge_match_kernel: the Min-Max record of each listed pair, one
+// pair per warp (lanes hold the polygons).
 #include "edge_dev.cuh"
 
 namespace pcl {
@@ -21,21 +23,6 @@ struct EdgeChecks {
     uint64_t cap;
     unsigned long long *count;
 };
-
-__device__ __forceinline__ void emit_pair(pcl_pair *out, uint64_t cap, unsigned long long *count,
-                                          bool keep, uint32_t a, uint32_t b) {
-    const unsigned mask = __ballot_sync(0xffffffffu, keep);
-    if (!mask) return;
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(mask) - 1;
-    unsigned long long base = 0;
-    if (lane == leader) base = atomicAdd(count, (unsigned long long)__popc(mask));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (keep) {
-        const unsigned long long idx = base + __popc(mask & ((1u << lane) - 1u));
-        if (idx < cap) out[idx] = pcl_pair{a, b};
-    }
-}
 
 // cell_of with the cell side known to be a power of two (P2) or not
 template <bool P2>
@@ -60,82 +47,6 @@ __device__ __forceinline__ bool grid_hit_any(const uint64_t *occ, int x0, int y0
 constexpr int kColsB = 256;  // column clips per block (32 row clips: one per lane)
 constexpr int kQueue = 64;   // per-warp queue capacity (grid tests, full checks)
 constexpr int kGS = 65;      // stride of a staged grid in shared memory (u64, padded against bank conflicts)
-
-// Warp-cooperative correspondence (Sec. 2.2.2 condition 1) of small list rs
-// against large list rl at shift t: every small polygon has exactly one
-// partner and no large polygon overlaps two small polygons.  Lanes take the
-// large polygons; the result is warp-uniform and equals correspond().
-// The small polygons are visited smallest first (ro: the small clip's area
-// order); the result does not depend on the order.
-__device__ __forceinline__ bool warp_correspond(const int4 *__restrict__ rs, const uint16_t *__restrict__ ro,
-                                                int ns, const int4 *__restrict__ rl, int nl, bool small_is_a,
-                                                int tx, int ty, int lane) {
-    if (ns <= 64 && nl <= 64) {
-        // both lists in registers, two polygons per lane at most; the large
-        // list is moved by the shift once: A's polygon first and B's moved by
-        // t is (s, l + t) with the small clip on side A, else (l, s + t), and
-        // both overlap tests equal the plain test of s against l + t or l - t
-        const bool v0 = lane < nl, v1 = lane + 32 < nl;
-        const int ux = small_is_a ? tx : -tx, uy = small_is_a ? ty : -ty;
-        int4 l0 = v0 ? __ldg(rl + lane) : make_int4(0, 0, 0, 0);
-        int4 l1 = v1 ? __ldg(rl + lane + 32) : make_int4(0, 0, 0, 0);
-        l0 = make_int4(l0.x + ux, l0.y + uy, l0.z + ux, l0.w + uy);
-        l1 = make_int4(l1.x + ux, l1.y + uy, l1.z + ux, l1.w + uy);
-        // small polygons in ascending area, where a missing partner is most likely
-        const int4 sv0 = lane < ns ? __ldg(rs + __ldg(ro + lane)) : make_int4(0, 0, 0, 0);
-        const int4 sv1 = lane + 32 < ns ? __ldg(rs + __ldg(ro + lane + 32)) : make_int4(0, 0, 0, 0);
-        int c0 = 0, c1 = 0;
-        if (nl <= 32) {
-            for (int k = 0; k < ns; ++k) {
-                const int4 sk = k < 32 ? sv0 : sv1;
-                const int src = k & 31;
-                const int sx0 = __shfl_sync(0xffffffffu, sk.x, src), sy0 = __shfl_sync(0xffffffffu, sk.y, src);
-                const int sx1 = __shfl_sync(0xffffffffu, sk.z, src), sy1 = __shfl_sync(0xffffffffu, sk.w, src);
-                const bool h0 = v0 && sx0 < l0.z && l0.x < sx1 && sy0 < l0.w && l0.y < sy1;
-                const unsigned b0 = __ballot_sync(0xffffffffu, h0);
-                if (b0 == 0u || (b0 & (b0 - 1u))) return false;  // not exactly one partner
-                c0 += h0 ? 1 : 0;
-            }
-        } else {
-            for (int k = 0; k < ns; ++k) {
-                const int4 sk = k < 32 ? sv0 : sv1;
-                const int src = k & 31;
-                const int sx0 = __shfl_sync(0xffffffffu, sk.x, src), sy0 = __shfl_sync(0xffffffffu, sk.y, src);
-                const int sx1 = __shfl_sync(0xffffffffu, sk.z, src), sy1 = __shfl_sync(0xffffffffu, sk.w, src);
-                const bool h0 = v0 && sx0 < l0.z && l0.x < sx1 && sy0 < l0.w && l0.y < sy1;
-                const bool h1 = v1 && sx0 < l1.z && l1.x < sx1 && sy0 < l1.w && l1.y < sy1;
-                const unsigned b0 = __ballot_sync(0xffffffffu, h0), b1 = __ballot_sync(0xffffffffu, h1);
-                if (__popc(b0) + __popc(b1) != 1) return false;
-                c0 += h0 ? 1 : 0;
-                c1 += h1 ? 1 : 0;
-            }
-        }
-        return !__any_sync(0xffffffffu, c0 > 1 || c1 > 1);
-    }
-    for (int k = 0; k < ns; ++k) {
-        const int4 s = __ldg(rs + k);
-        int cnt = 0;
-        for (int m0 = 0; m0 < nl && cnt < 2; m0 += 32) {
-            const int m = m0 + lane;
-            const bool h = m < nl && (small_is_a ? ovl(s, __ldg(rl + m), tx, ty) : ovl(__ldg(rl + m), s, tx, ty));
-            cnt += __popc(__ballot_sync(0xffffffffu, h));
-        }
-        if (cnt != 1) return false;
-    }
-    for (int m0 = 0; m0 < nl; m0 += 32) {
-        const int m = m0 + lane;
-        int c = 0;
-        if (m < nl) {
-            const int4 l = __ldg(rl + m);
-            for (int k = 0; k < ns && c < 2; ++k) {
-                const int4 s = __ldg(rs + k);
-                c += (small_is_a ? ovl(s, l, tx, ty) : ovl(l, s, tx, ty)) ? 1 : 0;
-            }
-        }
-        if (__any_sync(0xffffffffu, c > 1)) return false;
-    }
-    return true;
-}
 
 // Tiles (bx, by) of 32 row clips x kColsB column clips with any pair i < j,
 // column block by holding the row tiles bx < min(8 by + 8, nbx) (kColsB = 256
