@@ -237,22 +237,26 @@ pcl_status pcl_spectra(pcl_ctx *ctx, const pcl_params *P, pcl_clipset *cs, const
      against a library, say); a and b are clip sets of the same parameters P.
    COSINE: area-sorted band join (exactly the G1 survivors: a contiguous band
    of the other set's area order), then G3 density and G2 profile bounds.
-   EDGE: every pair, E2 bbox then E1 correspondence at the pre-alignment
-   (each polygon of the smaller clip, smallest first, is first checked
-   against the other clip's occupancy grid: no occupied cell under it means
-   no overlap, so E1 fails without scanning rectangles); tiles of 32 clips
-   of a x 256 clips of b (or of a, for the self-join).  Pairs are written to
+   EDGE: every pair, E2 bbox then E1 correspondence at the pre-alignment.
+   Each polygon of the smaller clip must meet an occupied cell of the other
+   clip's occupancy grid: the self-join tests that for 32 clips at a time from
+   bit tables, two sets (and shards) pair by pair, smallest polygon first, in
+   tiles of 32 clips of a x 256 clips of b; the pairs left are checked for the
+   exact correspondence.  Pairs are written to
    d_out[0 .. min(count, cap)) in unspecified order; *d_count (u64, device)
    receives the survivor count, which may exceed cap (then re-run with a
    larger buffer).  d_gate_counts (u64[16], device, may be NULL) is
    incremented: [0] survivors, [g] pairs rejected by gate g (their sum is
-   the number of pairs screened).  COSINE uses the context workspace (two
-   sets: about 16 (N^2 + 2) + 16 |a| + 8 |b| bytes for the area orders of
-   both sets and the bands of a's clips).  EDGE uses it for the list of pairs
-   whose polygons all meet occupied cells, which a second kernel checks for
-   the exact correspondence: 16 bytes per entry, one entry per 256 pairs
-   screened, at least 65,536 and at most 2^24 entries (pairs past the list
-   are checked inside the screen).  Calls that use the context workspace run
+   the number of pairs screened).  COSINE uses the context workspace
+   (about 8 (N^2 + 2) + 8 |a| bytes for the area order; the self-join at
+   256x256 and 512x512 px from 2,048 clips 2 KB per clip more for the vectors of
+   G3 as a matrix product, done without where they do not fit; two sets: about
+   16 (N^2 + 2) + 16 |a| + 8 |b| bytes).  EDGE uses it for the list of pairs
+   left for the exact check (pairs past the list are checked inside the
+   screen): the self-join 8 bytes per entry, 2^19 to 2^23 entries, beside 2 MB
+   of tables per 256 clips (at most 134 MB) and 172 bytes per clip; two sets
+   16 bytes per entry, one entry per 256 pairs screened, at least 65,536 and
+   at most 2^24 entries.  Calls that use the context workspace run
    in stream order on one stream at a time.
    With P->flags & PCL_P_TOPO_HASH (self-join only) a lossy topological
    pre-screen runs first (Sec. 3.1 stage 1 filters with topological hashing

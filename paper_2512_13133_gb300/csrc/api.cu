@@ -12,7 +12,9 @@ namespace pcl {
 cudaError_t launch_raster(const pcl_params &, const pcl_clipset &, cudaStream_t);
 size_t band_join_workspace(const Geo &, uint32_t, bool);
 cudaError_t launch_band_join(const pcl_params &, const pcl_clipset &, void *, size_t, pcl_pair *, uint64_t,
-                             unsigned long long *, unsigned long long *, int, cudaStream_t, uint32_t, uint32_t);
+                             unsigned long long *, unsigned long long *, int, cudaStream_t, uint32_t, uint32_t, int *,
+                             unsigned long long);
+size_t band_mma_workspace(const Geo &, uint32_t);
 size_t edge_checks_workspace(uint64_t);
 cudaError_t launch_edge_screen(const pcl_params &, const pcl_clipset &, pcl_pair *, uint64_t,
                                unsigned long long *, unsigned long long *, cudaStream_t, uint32_t, uint32_t, void *,
@@ -302,9 +304,12 @@ pcl_status pcl_candidates_shard(pcl_ctx *ctx, const pcl_params *P, uint32_t mode
         const Geo g = make_geo(*P);
         if (g.S > g.N / 16) return fail(ctx, PCL_ERR_UNSUPPORTED, "cosine gates need S <= N/16%s%lld");
         const size_t need = band_join_workspace(g, cs->n_clips, topo);
-        if ((s = ensure_ws(ctx, need))) return s;
+        const size_t more = topo || n_shards != 1 ? 0 : band_mma_workspace(g, cs->n_clips);
+        // without memory for the matrix product's vectors the band join alone does it
+        if ((!more || ensure_ws(ctx, need + 256 + more)) && (s = ensure_ws(ctx, need))) return s;
+        ctx->err.clear();
         e = launch_band_join(*P, *cs, ctx->ws, ctx->ws_bytes, d_out, cap, cnt, gates, ctx->num_sms, st, shard,
-                             n_shards);
+                             n_shards, ctx->d_err, ctx->wait_ns);
         return e == cudaSuccess ? PCL_OK : cuda_fail(ctx, e, "band join");
     }
     if (mode == PCL_MODE_EDGE && n_shards == 1 && !topo) {

@@ -1,0 +1,658 @@
+// a2, cosine gates at 256x256 and 512x512 px: the band join's density gate (G3)
+// as a matrix product on the 5th-generation tensor cores.
+//
+// G3 bounds the overlap by sum_k min(cnt_A(k), nbr_B(k)) over the 16x16 blocks
+// (gates.cu).  With thresholds t_0 = 0 < t_1 < .. < t_L (t_L = 256, a block's
+// pixels) and B's sums rounded up to the next threshold,
+//   min(cnt_A, nbr_B) <= sum_l f_l(cnt_A) [nbr_B > t_l],
+//   f_l(a) = min(a, t_{l+1}) - min(a, t_l)  (a's share of the l-th segment),
+// a product of one vector per representative with one 0/1 vector per member:
+// a GEMM over all pairs of the band in E4M3 (f rounded up to its 4 significant
+// bits) with FP32 accumulators, K = 16x16 blocks x L.  A pair whose product is at
+// or below the largest overlap that fails Eq. 2 fails G3 as well; at 256x256 px
+// and L = 4 that decides 99.4 % of the band (the exact sums of this direction
+// would decide 99.7 %), and only the rest take the exact G3 and G2.
+//
+// band_feature_kernel writes both vectors per clip in area order, laid out as
+// the MMA reads them (no-swizzle K-major core matrices, 8 rows x 16 bytes;
+// panels of 128 representatives, blocks of 256 members), so that operands
+// come by plain bulk copies.  band_mma_kernel, one CTA per SM: an item is a
+// panel and up to kSeg member blocks of its band; the panel's vectors stay in
+// shared memory, the blocks stream through a ring; one thread copies, one
+// issues tcgen05.mma (128 x 256 x 32), four warps compare the accumulators
+// (double buffered in tensor memory) with T sqrt(|A| |B|), a 32-column word of
+// decisions per lane, and list the pairs left.  band_list_kernel decides those
+// exactly, a warp per pair.  Should the list be too short (nearly identical
+// clips), it is dropped and the band join of gates.cu runs instead, as it does
+// for smaller rasters, shards, the topological pre-screen and callers without
+// workspace.
+//
+// 100,000 clips of 256x256 px (5.9e8 band pairs), one GB300: 1.5 ms a call - the
+// products 0.68 ms (4.8 GB of operands from L2, 7.2 TB/s, which bounds them:
+// the MMAs alone would take 0.27 ms), the exact check of 3.2 M pairs 0.68 ms,
+// the vectors (205 MB) 0.07 ms, the sort 0.03 ms - against 21.5 ms for the band
+// join's G3 on the CUDA cores.
+#include <type_traits>
+
+#include "gates.cuh"
+#include "tc_dev.cuh"
+
+namespace pcl {
+
+namespace {
+using namespace tc_dev;
+
+constexpr int kPanel = 128, kBlock = 256;  // representatives (M) and members (N) of one MMA tile
+constexpr int kStage = 32768;              // bytes of one ring stage: 256 members x 128 bytes of K
+constexpr int kSeg = 16;                   // member blocks per item at most
+constexpr int kMmaThreads = 256;
+constexpr uint32_t kTmem = 512;
+constexpr float kSlack = 1.0f - 1.0f / 1024.0f;  // on T sqrt(|A| |B|): float rounding, with room to spare
+
+// K bytes per clip: L thresholds of nb2 blocks, at most 1,024
+__host__ __device__ inline int levels_of(int nb2) { return nb2 >= 1024 ? 1 : 4; }
+__host__ __device__ inline int kbytes_of(int nb2) { return nb2 * levels_of(nb2); }
+__host__ __device__ inline int threshold(int levels, int l) {  // t_l
+    return l == 0 ? 0 : l >= levels ? 256 : 32 << (l - 1);     // 0, 32, 64, 128, 256
+}
+
+struct BandWs {
+    unsigned long long *seen;   // band pairs
+    unsigned long long *n_list; // listed pairs
+    unsigned int *overflow;     // 1: the list was too short
+    uint32_t *item_off;         // [panels + 1]
+    uint32_t *end;              // [n] end of each representative's band (area order)
+    float2 *thr;                // [blocks * 256] {T sqrt(area) with the slack, sqrt(area)}
+    unsigned char *P, *Q;       // vectors: panels x K x 128, blocks x K x 256 bytes
+    uint2 *list;                // positions (p, q)
+    uint32_t list_cap, n, panels, blocks;
+    int kb;
+};
+
+size_t up(size_t v) { return (v + 255) & ~(size_t)255; }
+
+size_t band_layout(const Geo &g, uint32_t n, char *ws, BandWs &w) {
+    w.n = n;
+    w.panels = (n + kPanel - 1) / kPanel;
+    w.blocks = (n + kBlock - 1) / kBlock;
+    w.kb = kbytes_of(g.nb * g.nb);
+    const uint64_t c = (uint64_t)n * n / 512;
+    w.list_cap = c < (1u << 16) ? (1u << 16) : c > (1u << 23) ? (1u << 23) : (uint32_t)c;
+    size_t o = 0;
+    auto part = [&](auto *&p, size_t bytes) {
+        p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(ws + o);
+        o += up(bytes);
+    };
+    part(w.seen, 8);
+    part(w.n_list, 8);
+    part(w.overflow, 4);  // the parts so far start as zeros
+    part(w.item_off, 4 * ((size_t)w.panels + 1));
+    part(w.end, 4 * (size_t)n);
+    part(w.thr, 8 * (size_t)kBlock * w.blocks);
+    part(w.list, 8 * (size_t)w.list_cap);
+    part(w.P, (size_t)w.panels * kPanel * w.kb);
+    part(w.Q, (size_t)w.blocks * kBlock * w.kb);
+    return o;
+}
+
+// integer 0..256 as E4M3, rounded up to 4 significant bits
+__device__ __forceinline__ uint32_t e4m3_up(int x) {
+    if (x == 0) return 0u;
+    int e = 31 - __clz(x);
+    int m = e <= 3 ? x << (3 - e) : (x + (1 << (e - 3)) - 1) >> (e - 3);  // 8 .. 16
+    if (m == 16) {
+        ++e;
+        m = 8;
+    }
+    return (uint32_t)(((e + 7) << 3) | (m & 7));
+}
+
+// Both vectors of 64 clips per CTA: a thread takes 16 blocks of one clip, looks
+// their E4M3 codes up for all levels and writes 16 bytes per level and vector;
+// 16 consecutive threads take consecutive clips, whose 16-byte rows of a core
+// matrix are adjacent.  Positions past n are zeros (their products exceed no
+// threshold).  (Converting every value for every level took 185 us at 100,000
+// clips, the table 72 us.)
+constexpr int kFeatureClips = 64;
+
+template <int LV>
+__global__ void __launch_bounds__(256) band_feature_kernel(pcl_params prm, pcl_clipset cs, BandWs w,
+                                                           const uint32_t *order, const uint32_t *spop,
+                                                           const uint32_t *cum) {
+    const Geo g = make_geo(prm);
+    const int nb2 = g.nb * g.nb;
+    // per block count 0..256: byte l is the code of its share of level l
+    __shared__ uint32_t code[257];
+    for (int a = threadIdx.x; a < 257; a += 256) {
+        uint32_t c = 0u;
+#pragma unroll
+        for (int l = 0; l < LV; ++l)
+            c |= e4m3_up(min(a, threshold(LV, l + 1)) - min(a, threshold(LV, l))) << (8 * l);
+        code[a] = c;
+    }
+    __syncthreads();
+    const int r = threadIdx.x & 15;
+    for (int c0 = 0; c0 < kFeatureClips; c0 += 16) {
+        const uint32_t p = blockIdx.x * kFeatureClips + c0 + r;
+        const bool live = p < w.n;
+        const uint32_t *cw = reinterpret_cast<const uint32_t *>(cs.blk + (size_t)(live ? order[p] : 0) * 2 * nb2);
+        unsigned char *P = w.P + (size_t)(p / kPanel) * kPanel * w.kb + (p % kPanel) * 16;
+        unsigned char *Q = w.Q + (size_t)(p / kBlock) * kBlock * w.kb + (p % kBlock) * 16;
+        for (int j = threadIdx.x >> 4; j < nb2 / 16; j += 16) {
+            uint32_t f[LV][4], q[LV][4];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                uint32_t c[4], d[4];  // codes of four counts, and their neighbourhood sums
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const uint32_t x = live ? __ldg(cw + 8 * j + 2 * h + s) : 0u;
+                    const uint32_t y = live ? __ldg(cw + nb2 / 2 + 8 * j + 2 * h + s) : 0u;
+                    c[2 * s] = code[min(x & 0xffffu, 256u)];
+                    c[2 * s + 1] = code[min(x >> 16, 256u)];
+                    d[2 * s] = y & 0xffffu;
+                    d[2 * s + 1] = y >> 16;
+                }
+#pragma unroll
+                for (int l = 0; l < LV; ++l) {
+                    const uint32_t t0 = (uint32_t)threshold(LV, l);
+                    f[l][h] = q[l][h] = 0u;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        f[l][h] |= (c[e] >> (8 * l) & 0xffu) << (8 * e);
+                        q[l][h] |= (d[e] > t0 ? 0x38u : 0u) << (8 * e);  // 1.0
+                    }
+                }
+            }
+#pragma unroll
+            for (int l = 0; l < LV; ++l) {
+                const size_t k = (size_t)(l * nb2 / 16 + j);  // 16-byte column of K
+                if (p < w.panels * kPanel)
+                    *reinterpret_cast<uint4 *>(P + k * (16 * kPanel)) = make_uint4(f[l][0], f[l][1], f[l][2], f[l][3]);
+                if (p < w.blocks * kBlock)
+                    *reinterpret_cast<uint4 *>(Q + k * (16 * kBlock)) = make_uint4(q[l][0], q[l][1], q[l][2], q[l][3]);
+            }
+        }
+    }
+    const uint32_t p = blockIdx.x * kFeatureClips + threadIdx.x;
+    if (threadIdx.x < kFeatureClips && p < w.blocks * kBlock) {
+        unsigned long long band = 0;
+        float s = 0.0f;
+        if (p < w.n) {
+            const uint64_t num2 = (uint64_t)prm.cos_num * prm.cos_num, den2 = (uint64_t)prm.cos_den * prm.cos_den;
+            const uint64_t pa = spop[p], all = (uint64_t)g.N * g.N;
+            uint64_t vmax = pa == 0 ? 0 : (den2 * pa - 1) / num2;
+            if (vmax > all) vmax = all;
+            const uint32_t e = cum[vmax + 1];
+            w.end[p] = e;
+            band = e - p - 1;
+            s = sqrtf((float)pa);
+        }
+        w.thr[p] = make_float2(s * ((float)prm.cos_num / (float)prm.cos_den) * kSlack, s);
+        for (int o = 16; o; o >>= 1) band += __shfl_xor_sync(0xffffffffu, band, o);
+        if ((threadIdx.x & 31) == 0 && band) atomicAdd(w.seen, band);
+    }
+}
+
+// first member block of a panel's band, and how many blocks it meets
+__device__ __forceinline__ void panel_blocks(const BandWs &w, uint32_t panel, uint32_t &first, uint32_t &count) {
+    const uint32_t p0 = panel * kPanel, last = min(w.n, p0 + kPanel) - 1;
+    const uint32_t e = w.end[last];  // ends do not decrease along the area order
+    first = (p0 + 1) / kBlock;
+    count = e > p0 + 1 ? (e + kBlock - 1) / kBlock - first : 0u;
+}
+
+// items of the panels before each panel (one CTA)
+__global__ void __launch_bounds__(1024) band_items_kernel(BandWs w) {
+    __shared__ uint32_t wsum[32];
+    const uint32_t per = (w.panels + 1023) / 1024;
+    const uint32_t lo = min(w.panels, threadIdx.x * per), hi = min(w.panels, lo + per);
+    auto items = [&](uint32_t i) {
+        uint32_t f, c;
+        panel_blocks(w, i, f, c);
+        return (c + kSeg - 1) / kSeg;
+    };
+    uint32_t s = 0;
+    for (uint32_t i = lo; i < hi; ++i) s += items(i);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t x = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        uint32_t t = wsum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        wsum[lane] = t;
+    }
+    __syncthreads();
+    uint32_t run = x - s + (wid ? wsum[wid - 1] : 0u);
+    for (uint32_t i = lo; i < hi; ++i) {
+        w.item_off[i] = run;
+        run += items(i);
+    }
+    if (threadIdx.x == 1023) w.item_off[w.panels] = run;
+}
+
+struct BandItem {
+    uint32_t panel, first, count;  // member blocks [first, first + count)
+};
+__device__ __forceinline__ BandItem band_item(const BandWs &w, uint32_t it) {
+    uint32_t lo = 0, hi = w.panels;  // the last panel with item_off <= it
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) / 2;
+        if (w.item_off[mid] <= it) lo = mid;
+        else hi = mid;
+    }
+    BandItem b;
+    uint32_t f, c;
+    panel_blocks(w, lo, f, c);
+    const uint32_t s = (it - w.item_off[lo]) * kSeg;
+    b.panel = lo;
+    b.first = f + s;
+    b.count = min(c - s, (uint32_t)kSeg);
+    return b;
+}
+
+// barriers: panel full / empty, accumulators full[2] / empty[2], end, ring full[ST] / empty[ST]
+enum { kPFull = 0, kPEmpty = 1, kAcc = 2, kAccFree = 4, kEnd = 6, kRing = 7 };
+
+template <int KB>
+struct BandSmem {
+    static constexpr uint32_t panel = KB * kPanel;
+    static constexpr int stages = (int)((232448u - panel - 4096u) / kStage) > 4 ? 4 : (int)((232448u - panel - 4096u) / kStage);
+    static constexpr uint32_t ring = panel;
+    static constexpr uint32_t queue = ring + stages * kStage;  // [4 warps][64] uint2
+    static constexpr uint32_t bars = queue + 4 * 64 * 8;
+    static constexpr uint32_t bytes = bars + (kRing + 2 * stages) * 8 + 16;
+};
+
+template <int KB>
+__global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(BandWs w, int *err, unsigned long long wait_ns) {
+    using SM = BandSmem<KB>;
+    constexpr int ST = SM::stages, CH = KB / 128;  // ring stages, K chunks per member block
+    extern __shared__ __align__(1024) unsigned char sm[];
+    volatile uint32_t *misc = reinterpret_cast<volatile uint32_t *>(sm + SM::bars + (kRing + 2 * ST) * 8);
+    const volatile uint32_t *abortf = misc + 1;
+    const uint32_t sbase = smem_u32(sm), bar0 = sbase + SM::bars;
+    auto bar = [&](int k) { return bar0 + 8u * (uint32_t)k; };
+    auto raise_abort = [&]() {
+        misc[1] = 1u;
+        atomicExch(err, 1);
+    };
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        mbar_init(bar(kPFull), 1);
+        mbar_init(bar(kPEmpty), 1);
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(bar(kAcc + k), 1);
+            mbar_init(bar(kAccFree + k), 128);
+        }
+        mbar_init(bar(kEnd), 1);
+        for (int k = 0; k < ST; ++k) {
+            mbar_init(bar(kRing + k), 1);
+            mbar_init(bar(kRing + ST + k), 1);
+        }
+        misc[1] = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32((const void *)misc)),
+                     "r"(kTmem));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = misc[0];
+    const uint32_t n_items = w.item_off[w.panels];
+
+    if (warp == 0) {
+        // ---------------------------------------------------------------- copies
+        if (lane == 0) {
+            bool ok = true;
+            uint32_t li = 0, e = 0, panels = 0;  // items, stages and panels so far
+            for (uint32_t it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++li) {
+                const BandItem item = band_item(w, it);
+                if (li && !(ok = wait_phase(bar(kPEmpty), (li - 1) & 1, abortf, wait_ns))) break;
+                mbar_expect(bar(kPFull), SM::panel);
+                const unsigned char *P = w.P + (size_t)item.panel * SM::panel;
+                for (uint32_t o = 0; o < SM::panel; o += 16384) bulk_copy(sbase + o, P + o, 16384, bar(kPFull));
+                ++panels;
+                const unsigned char *Q = w.Q + (size_t)item.first * KB * kBlock;
+                for (uint32_t s = 0; s < item.count * CH; ++s, ++e) {
+                    const uint32_t k = e % ST;
+                    if (e >= ST && !(ok = wait_phase(bar(kRing + ST + k), (e / ST - 1) & 1, abortf, wait_ns))) break;
+                    mbar_expect(bar(kRing + k), kStage);
+                    bulk_copy(sbase + SM::ring + k * kStage, Q + (size_t)s * kStage, kStage, bar(kRing + k));
+                }
+            }
+            if (!ok) raise_abort();
+            // every copy issued has landed before the shared memory is given up
+            for (uint32_t k = 0; k < (uint32_t)ST && k < e; ++k) {
+                const uint32_t last = (e - 1 - k) / ST * ST + k;  // the last use of stage k
+                if (!wait_phase(bar(kRing + k), (last / ST) & 1, nullptr, kWaitNs)) raise_abort();
+            }
+            if (panels && !wait_phase(bar(kPFull), (panels - 1) & 1, nullptr, kWaitNs)) raise_abort();
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ---------------------------------------------------------------- MMA issue
+        if (lane == 0) {
+            constexpr uint32_t idesc = idesc_of(kPanel, kBlock, kOpE4M3);
+            bool ok = true;
+            uint32_t li = 0, e = 0, t = 0;  // items, stages, tiles so far
+            for (uint32_t it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++li) {
+                const BandItem item = band_item(w, it);
+                if (!(ok = wait_phase(bar(kPFull), li & 1, abortf, wait_ns))) break;
+                for (uint32_t b = 0; b < item.count && ok; ++b, ++t) {
+                    const uint32_t buf = t & 1;
+                    if (t >= 2 && !(ok = wait_phase(bar(kAccFree + buf), ((t >> 1) - 1) & 1, abortf, wait_ns))) break;
+                    fence_after();
+                    for (int c = 0; c < CH; ++c, ++e) {
+                        const uint32_t k = e % ST;
+                        if (!(ok = wait_phase(bar(kRing + k), (e / ST) & 1, abortf, wait_ns))) break;
+                        fence_after();
+#pragma unroll
+                        for (int s = 0; s < 4; ++s) {  // K = 32: two core matrices
+                            const uint64_t ad = smem_desc(sbase + (uint32_t)(8 * c + 2 * s) * (16 * kPanel), 16 * kPanel, 128);
+                            const uint64_t bd = smem_desc(sbase + SM::ring + k * kStage + (uint32_t)(2 * s) * (16 * kBlock),
+                                                          16 * kBlock, 128);
+                            mma<true>(tmem + buf * kBlock, ad, bd, idesc, (c | s) != 0 ? 1u : 0u);
+                        }
+                        mma_commit(bar(kRing + ST + k));
+                    }
+                    if (ok) mma_commit(bar(kAcc + buf));
+                }
+                if (ok) mma_commit(bar(kPEmpty));
+            }
+            if (!ok) raise_abort();
+            // every MMA issued so far has completed before the tensor memory is released
+            mma_commit(bar(kEnd));
+            if (!wait_phase(bar(kEnd), 0, nullptr, kWaitNs)) raise_abort();
+        }
+        __syncwarp();
+    } else if (warp >= 4) {
+        // ---------------------------------------------------------------- decisions
+        const int quarter = warp & 3;
+        uint2 *queue = reinterpret_cast<uint2 *>(sm + SM::queue) + quarter * 64;
+        const unsigned lt = (1u << lane) - 1u;
+        uint32_t qn = 0, t = 0;
+        bool ok = true;
+        auto flush = [&](uint32_t m) {
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(w.n_list, (unsigned long long)m);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if ((uint32_t)lane < m && at + lane < w.list_cap) w.list[at + lane] = queue[lane];
+            if (lane == 0 && at + m > w.list_cap) *w.overflow = 1u;
+        };
+        for (uint32_t it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
+            const BandItem item = band_item(w, it);
+            const uint32_t p = item.panel * kPanel + 32 * quarter + lane;
+            const uint32_t end = p < w.n ? w.end[p] : 0u;
+            const float ra = w.thr[min(p, w.n - 1)].x;
+            for (uint32_t b = 0; b < item.count; ++b, ++t) {
+                const uint32_t buf = t & 1;
+                ok = wait_phase(bar(kAcc + buf), (t >> 1) & 1, abortf, wait_ns);
+                if (__any_sync(0xffffffffu, !ok)) {
+                    ok = false;
+                    break;
+                }
+                fence_after();
+                const uint32_t q0 = (item.first + b) * kBlock;
+                const uint32_t src = tmem + ((uint32_t)(32 * quarter) << 16) + buf * kBlock;
+                for (int c = 0; c < kBlock; c += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(src + c, v);
+                    const float4 *th = reinterpret_cast<const float4 *>(w.thr + q0 + c);
+                    tmem_wait_ld();
+                    uint32_t hit = 0u;  // bit 31 - j: v[j] above its threshold
+#pragma unroll
+                    for (int j = 0; j < 32; j += 2) {
+                        const float4 s = __ldg(th + j / 2);  // {.., sqrt, .., sqrt} of two members
+                        hit = __funnelshift_l(__float_as_uint(fmaf(ra, s.y, -__uint_as_float(v[j]))), hit, 1);
+                        hit = __funnelshift_l(__float_as_uint(fmaf(ra, s.w, -__uint_as_float(v[j + 1]))), hit, 1);
+                    }
+                    hit = __brev(hit);
+                    // members p < q < end
+                    const int lo = (int)p + 1 - (int)(q0 + c), hi = (int)end - (int)(q0 + c);
+                    uint32_t in = hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
+                    in &= lo <= 0 ? 0xffffffffu : lo >= 32 ? 0u : 0xffffffffu << lo;
+                    hit &= in;
+                    while (__any_sync(0xffffffffu, hit != 0u)) {
+                        const bool have = hit != 0u;
+                        const unsigned hb = __ballot_sync(0xffffffffu, have);
+                        if (have) {
+                            queue[qn + __popc(hb & lt)] = make_uint2(p, q0 + c + __ffs(hit) - 1);
+                            hit &= hit - 1u;
+                        }
+                        qn += (uint32_t)__popc(hb);
+                        __syncwarp();
+                        if (qn >= 32) {
+                            flush(32);
+                            __syncwarp();
+                            uint2 r = make_uint2(0u, 0u);
+                            if ((uint32_t)lane + 32 < qn) r = queue[lane + 32];
+                            __syncwarp();
+                            if ((uint32_t)lane + 32 < qn) queue[lane] = r;
+                            qn -= 32;
+                            __syncwarp();
+                        }
+                    }
+                }
+                fence_before();
+                mbar_arrive(bar(kAccFree + buf));
+            }
+        }
+        if (qn) flush(qn);
+        if (!ok && lane == 0) raise_abort();
+        __syncwarp();
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmem));
+}
+
+// G2 as a decision (warp_g2_rejects) with the shifts in groups of nine: a
+// group is bounded by the sum against B's profile dilated by 4,
+//   sum_y min(r_A(y), r_B(y - c - e)) <= sum_y min(r_A(y), max_|e|<=4 r_B(y - c - e)),
+// and only a group whose bound is above um has its shifts summed: at 256x256 px
+// 4 group sums and 2.5 shifts instead of 33.  scratch: 2 (N + 2 S + 32) u16 per warp.
+template <int NPL>
+__device__ __forceinline__ bool warp_g2_rejects_groups(const uint16_t *__restrict__ pa,
+                                                       const uint16_t *__restrict__ pb, int S, int64_t um, int lane,
+                                                       uint16_t *scratch) {
+    constexpr int N = 32 * NPL;
+    const int pad = S + 16, len = N + 2 * pad;  // index y + pad, -pad <= y < N + pad
+    uint16_t *B = scratch, *D = scratch + len;
+#pragma unroll 1
+    for (int ax = 0; ax < 2; ++ax) {
+        uint32_t av[NPL];
+#pragma unroll
+        for (int u = 0; u < NPL; ++u) av[u] = __ldg(pa + ax * N + lane + 32 * u);
+        __syncwarp();  // earlier reads of the scratch are done
+        for (int k = lane; k < len; k += 32) {
+            const int y = k - pad;
+            B[k] = y >= 0 && y < N ? __ldg(pb + ax * N + y) : (uint16_t)0;
+        }
+        __syncwarp();
+        for (int k = lane; k < len; k += 32) {  // max over k - 4 .. k + 4
+            uint32_t m = 0;
+#pragma unroll
+            for (int e = -4; e <= 4; ++e) m = max(m, (uint32_t)B[min(max(k + e, 0), len - 1)]);
+            D[k] = (uint16_t)m;
+        }
+        __syncwarp();
+        auto sum = [&](const uint16_t *V, int d) {
+            uint32_t t = 0;
+#pragma unroll
+            for (int u = 0; u < NPL; ++u) t += min(av[u], (uint32_t)V[lane + 32 * u - d + pad]);
+            return (int64_t)__reduce_add_sync(0xffffffffu, t);
+        };
+        bool above = false;
+        for (int c = 4 - S; c - 4 <= S && !above; c += 9) {
+            if (sum(D, c) <= um) continue;
+            for (int d = c - 4; d <= c + 4 && d <= S && !above; ++d) above = sum(B, d) > um;
+        }
+        if (!above) return true;
+    }
+    return false;
+}
+
+// The listed pairs: exact G3, then G2, a warp per pair; and the pairs of empty
+// clips.  A warp takes 32 pairs at a time: lane q reads pair q's clips and
+// finds its threshold, then the pairs go one by one, the next pair's first 64
+// blocks loading while one is tested (1.10 -> 0.68 ms at 100,000 clips).
+template <int NPL>
+__global__ void __launch_bounds__(256) band_list_kernel(pcl_params prm, pcl_clipset cs, BandWs w,
+                                                        const uint32_t *order, const uint32_t *spop,
+                                                        const uint32_t *cum, pcl_pair *out, uint64_t cap,
+                                                        unsigned long long *count, unsigned long long *local) {
+    if (*w.overflow) return;
+    extern __shared__ uint16_t g2_scratch[];
+    const unsigned full = 0xffffffffu;
+    const Geo g = make_geo(prm);
+    const int lane = threadIdx.x & 31, nb2 = g.nb * g.nb, words = nb2 / 2;
+    uint16_t *scratch = g2_scratch + (threadIdx.x >> 5) * 2 * (g.N + 2 * g.S + 32);
+    const uint32_t n = (uint32_t)*w.n_list;
+    const uint32_t w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t *blk = reinterpret_cast<const uint32_t *>(cs.blk);
+    unsigned long long kept = 0, g2 = 0;
+    for (uint32_t t0 = w0 * 32; t0 < n; t0 += nw * 32) {  // warp-uniform
+        const int m = (int)min(n - t0, 32u);
+        uint32_t a = 0, b = 0;
+        int um = 0, pa = 0, pb = 0;  // areas are at most 512^2
+        if (lane < m) {
+            const uint2 e = w.list[t0 + lane];
+            a = order[e.x];
+            b = order[e.y];
+            pa = (int)spop[e.x];
+            pb = (int)spop[e.y];
+            um = (int)cos_umax((uint64_t)pa, (uint64_t)pb, prm.cos_num, prm.cos_den);
+        }
+        uint32_t ca = 0, da = 0, cb = 0, db = 0;  // the next pair's first chunk: counts and neighbourhood sums
+        auto fetch = [&](int q) {
+            const uint32_t *x = blk + (size_t)__shfl_sync(full, a, q) * nb2, *y = blk + (size_t)__shfl_sync(full, b, q) * nb2;
+            ca = __ldg(x + lane);
+            da = __ldg(x + words + lane);
+            cb = __ldg(y + lane);
+            db = __ldg(y + words + lane);
+        };
+        fetch(0);
+        for (int q = 0; q < m; ++q) {
+            const uint32_t qa = __shfl_sync(full, a, q), qb = __shfl_sync(full, b, q);
+            const int u = __shfl_sync(full, um, q);
+            const int tA = __shfl_sync(full, pa, q) - u, tB = __shfl_sync(full, pb, q) - u;
+            // G3: the deficits as warp_g3_rejects sums them, 64 blocks at a time
+            uint32_t sa = __reduce_add_sync(full, ca - __vminu2(ca, db)), sb = __reduce_add_sync(full, cb - __vminu2(cb, da));
+            if (q + 1 < m) fetch(q + 1);
+            int DA = (int)((sa & 0xffffu) + (sa >> 16)), DB = (int)((sb & 0xffffu) + (sb >> 16));
+            bool rej = DA >= tA || DB >= tB;
+            const uint32_t *x = blk + (size_t)qa * nb2, *y = blk + (size_t)qb * nb2;
+            for (int k = 32 + lane; !rej && k < words; k += 32) {  // words is a multiple of 32
+                const uint32_t c0 = __ldg(x + k), d0 = __ldg(x + words + k), c1 = __ldg(y + k), d1 = __ldg(y + words + k);
+                sa = __reduce_add_sync(full, c0 - __vminu2(c0, d1));
+                sb = __reduce_add_sync(full, c1 - __vminu2(c1, d0));
+                DA += (int)((sa & 0xffffu) + (sa >> 16));
+                DB += (int)((sb & 0xffffu) + (sb >> 16));
+                rej = DA >= tA || DB >= tB;
+            }
+            if (rej) continue;
+            if (warp_g2_rejects_groups<NPL>(cs.prof + (size_t)qa * 2 * g.N, cs.prof + (size_t)qb * 2 * g.N, g.S,
+                                            (int64_t)u, lane, scratch)) {
+                ++g2;
+                continue;
+            }
+            ++kept;
+            if (lane == 0) {
+                const unsigned long long at = atomicAdd(count, 1ull);
+                if (at < cap) out[at] = pcl_pair{min(qa, qb), max(qa, qb)};
+            }
+        }
+    }
+    const uint32_t e = cum[1];  // empty clips: similar by definition
+    for (uint32_t p = blockIdx.x; p + 1 < e; p += gridDim.x) {
+        const uint32_t a = order[p];
+        for (uint32_t q0 = p + 1; q0 < e; q0 += blockDim.x) {
+            const uint32_t q = q0 + threadIdx.x;
+            const uint32_t b = q < e ? order[q] : 0u;
+            const unsigned m = __ballot_sync(0xffffffffu, q < e);
+            unsigned long long base = 0;
+            if (lane == 0 && m) base = atomicAdd(count, (unsigned long long)__popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (q < e && base + lane < cap) out[base + lane] = pcl_pair{min(a, b), max(a, b)};
+            kept += (unsigned long long)__popc(m);
+        }
+    }
+    if (lane == 0) {
+        if (kept) atomicAdd(local + 0, kept);
+        if (g2) atomicAdd(local + PCL_GATE_G2_PROFILE, g2);
+    }
+}
+
+// G3's rejections: the band's pairs that neither survived nor failed G2
+__global__ void band_count_kernel(BandWs w, unsigned long long *local) {
+    if (!*w.overflow) local[PCL_GATE_G3_DENSITY] = *w.seen - local[0] - local[PCL_GATE_G2_PROFILE];
+}
+
+template <int KB, int NPL>
+cudaError_t launch_t(const pcl_params &prm, const Geo &g, const pcl_clipset &cs, const BandWs &w,
+                     const uint32_t *order, const uint32_t *spop, const uint32_t *cum, pcl_pair *out, uint64_t cap,
+                     unsigned long long *count, unsigned long long *local, int num_sms, int *d_err,
+                     unsigned long long wait_ns, cudaStream_t st) {
+    const uint32_t bytes = BandSmem<KB>::bytes;
+    cudaError_t e = cudaFuncSetAttribute(band_mma_kernel<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return e;
+    band_mma_kernel<KB><<<num_sms, kMmaThreads, bytes, st>>>(w, d_err, wait_ns ? wait_ns : kWaitNs);
+    const size_t scratch = 8 * 2 * 2 * (size_t)(g.N + 2 * g.S + 32);
+    band_list_kernel<NPL><<<num_sms * 8, 256, scratch, st>>>(prm, cs, w, order, spop, cum, out, cap, count, local);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// 256x256 and 512x512 px (at smaller sizes G3 decides few pairs); from 2,048
+// clips on, below which the band join takes less than the extra launches
+bool band_mma_covers(const Geo &g, uint32_t n) { return (g.N == 256 || g.N == 512) && n >= 2048; }
+
+size_t band_mma_workspace(const Geo &g, uint32_t n) {
+    if (!band_mma_covers(g, n)) return 0;
+    BandWs w;
+    return band_layout(g, n, nullptr, w);
+}
+
+// Decides the whole band into out / count / local unless *overflow (device)
+// ends up 1; the caller then runs the band join.  order, spop, cum: the area
+// sort.  ws: band_mma_workspace bytes, 256-byte aligned.
+cudaError_t launch_band_mma(const pcl_params &prm, const pcl_clipset &cs, const uint32_t *order, const uint32_t *spop,
+                            const uint32_t *cum, void *ws, pcl_pair *out, uint64_t cap, unsigned long long *count,
+                            unsigned long long *local, const unsigned int **overflow, int num_sms, int *d_err,
+                            unsigned long long wait_ns, cudaStream_t st) {
+    const Geo g = make_geo(prm);
+    BandWs w;
+    band_layout(g, cs.n_clips, static_cast<char *>(ws), w);
+    *overflow = w.overflow;
+    cudaError_t e = cudaMemsetAsync(ws, 0, (size_t)(reinterpret_cast<char *>(w.item_off) - static_cast<char *>(ws)), st);
+    if (e != cudaSuccess) return e;
+    const unsigned grid = w.blocks * (kBlock / kFeatureClips);
+    if (g.N == 256) band_feature_kernel<4><<<grid, 256, 0, st>>>(prm, cs, w, order, spop, cum);
+    else band_feature_kernel<1><<<grid, 256, 0, st>>>(prm, cs, w, order, spop, cum);
+    band_items_kernel<<<1, 1024, 0, st>>>(w);
+    if (g.N == 256)
+        e = launch_t<1024, 8>(prm, g, cs, w, order, spop, cum, out, cap, count, local, num_sms, d_err, wait_ns, st);
+    else
+        e = launch_t<1024, 16>(prm, g, cs, w, order, spop, cum, out, cap, count, local, num_sms, d_err, wait_ns, st);
+    if (e != cudaSuccess) return e;
+    band_count_kernel<<<1, 1, 0, st>>>(w, local);
+    return cudaGetLastError();
+}
+
+}  // namespace pcl

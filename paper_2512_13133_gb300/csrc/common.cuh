@@ -346,4 +346,49 @@ __device__ __forceinline__ uint32_t popc_sum(const uint32_t (&x)[n]) {
     return s1 + 2u * s2;
 }
 
+// Exclusive scan of in[0..m) into out (in == out allowed) by one CTA of 1024
+// threads; every thread gets the total.  A warp takes 256 consecutive values as
+// eight rows of 32, so reads and writes are coalesced whatever the alignment
+// (65,538 values: 18 us; a contiguous run per thread took 50 us).
+__device__ __forceinline__ uint32_t cta_scan(const uint32_t *in, uint32_t *out, uint32_t m) {
+    constexpr int R = 8;
+    __shared__ uint32_t wsum[2][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t carry = 0;
+    int h = 0;
+    for (uint32_t base = 0; base < m; base += 1024 * R, h ^= 1) {
+        const uint32_t i0 = base + wid * 32 * R + lane;
+        uint32_t x[R], run = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = i0 + 32 * r < m ? in[i0 + 32 * r] : 0u;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {  // x[r]: sum of the warp's values before this one
+            const uint32_t v = x[r];
+            uint32_t s = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
+                if (lane >= o) s += y;
+            }
+            x[r] = run + s - v;
+            run += __shfl_sync(0xffffffffu, s, 31);
+        }
+        if (lane == 0) wsum[h][wid] = run;
+        __syncthreads();
+        uint32_t t = wsum[h][lane];  // every warp scans the 32 warp sums itself
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        const uint32_t before = carry + (wid ? __shfl_sync(0xffffffffu, t, wid - 1) : 0u);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (i0 + 32 * r < m) out[i0 + 32 * r] = before + x[r];
+        carry += __shfl_sync(0xffffffffu, t, 31);
+    }
+    __syncthreads();
+    return carry;
+}
+
 }  // namespace pcl

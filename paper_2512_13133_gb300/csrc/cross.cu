@@ -75,36 +75,8 @@ __global__ void cross_chunks_kernel(const uint32_t *beg, const uint32_t *end, ui
 
 // exclusive scan of v[0..m) into out[0..m], out[m] = total (single CTA)
 __global__ void __launch_bounds__(1024) scan_items_kernel(const uint32_t *v, uint32_t m, uint32_t *out) {
-    __shared__ uint32_t wsum[32];
-    const uint32_t per = (m + 1023) / 1024;
-    const uint32_t lo = threadIdx.x * per, hi = min(m, lo + per);
-    uint32_t s = 0;
-    for (uint32_t i = lo; i < hi; ++i) s += v[i];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t x = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        uint32_t w = wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        wsum[lane] = w;
-    }
-    __syncthreads();
-    uint32_t run = x - s + (wid ? wsum[wid - 1] : 0u);
-    for (uint32_t i = lo; i < hi; ++i) {
-        out[i] = run;
-        run += v[i];
-    }
-    if (threadIdx.x == 1023) out[m] = run;
+    const uint32_t total = cta_scan(v, out, m);
+    if (threadIdx.x == 0) out[m] = total;
 }
 
 // WPL: u32 words of block counts per lane (the query's are held in registers).

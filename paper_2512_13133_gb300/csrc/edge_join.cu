@@ -163,51 +163,16 @@ __device__ __forceinline__ void place_clip(const pcl_clipset &cs, const JoinWs &
         w.erec[atomicAdd(w.he + min(lo.x, kBins - 1), 1u)] = make_int4(lo.x, lo.w - lo.z, hi.z - hi.y, 0);
 }
 
-// exclusive scan of v[0..m) by one CTA of 1024 threads
-__device__ __forceinline__ void cta_scan(uint32_t *v, uint32_t m) {
-    __shared__ uint32_t wsum[32];
-    const uint32_t per = (m + 1023) / 1024;
-    const uint32_t lo = min(m, threadIdx.x * per), hi = min(m, lo + per);
-    uint32_t s = 0;
-    for (uint32_t i = lo; i < hi; ++i) s += v[i];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t x = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        uint32_t t = wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
-            if (lane >= o) t += y;
-        }
-        wsum[lane] = t;
-    }
-    __syncthreads();
-    uint32_t run = x - s + (wid ? wsum[wid - 1] : 0u);
-    for (uint32_t i = lo; i < hi; ++i) {
-        const uint32_t t = v[i];
-        v[i] = run;
-        run += t;
-    }
-    __syncthreads();
-}
-
 __global__ void __launch_bounds__(256) join_prep_kernel(pcl_clipset cs, JoinWs w, int W) {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < w.n; i += gridDim.x * blockDim.x)
         prep_clip(cs, w, i, W);
 }
 __global__ void __launch_bounds__(1024) join_scan_kernel(JoinWs w, int second) {
     if (second) {
-        cta_scan(w.h2, w.strips * kBins);
+        cta_scan(w.h2, w.h2, w.strips * kBins);
     } else {
-        cta_scan(w.hx, kBins);
-        cta_scan(w.he, kBins);
+        cta_scan(w.hx, w.hx, kBins);
+        cta_scan(w.he, w.he, kBins);
     }
 }
 __global__ void __launch_bounds__(256) join_strip_kernel(JoinWs w, int W) {
@@ -222,11 +187,11 @@ __global__ void __launch_bounds__(256) join_place_kernel(pcl_clipset cs, JoinWs 
 __global__ void __launch_bounds__(1024) join_sort_small_kernel(pcl_clipset cs, JoinWs w, int W) {
     for (uint32_t i = threadIdx.x; i < w.n; i += 1024) prep_clip(cs, w, i, W);
     __syncthreads();
-    cta_scan(w.hx, kBins);
-    cta_scan(w.he, kBins);
+    cta_scan(w.hx, w.hx, kBins);
+    cta_scan(w.he, w.he, kBins);
     for (uint32_t i = threadIdx.x; i < w.n; i += 1024) atomicAdd(w.h2 + strip_bin(w, i, W), 1u);
     __syncthreads();
-    cta_scan(w.h2, w.strips * kBins);
+    cta_scan(w.h2, w.h2, w.strips * kBins);
     for (uint32_t i = threadIdx.x; i < w.n; i += 1024) place_clip(cs, w, i, W);
 }
 

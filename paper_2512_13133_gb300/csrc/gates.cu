@@ -17,8 +17,9 @@
 // den^2/num^2 times the smaller one, so after a counting sort of the clips by
 // area every G1 survivor (i, j) lies in the band of positions
 // (p, end_p) with end_p = #{clips with area <= floor((den^2 a_p - 1)/num^2)}.
-// Warps take positions p from a global counter and test G3 and G2 on every
-// band member with the whole warp.  A shard s of S (several GPUs sharing one
+// The whole self-join at 256x256 and 512x512 px takes G3 as a matrix product
+// (band_mma.cu); otherwise warps take positions p from a global counter and test
+// G3 and G2 on every band member.  A shard s of S (several GPUs sharing one
 // self-join) keeps the pairs a < b with a mod S = s: its warps take the
 // representatives a = s, s + S, ... and walk their two-sided band (the clips
 // whose areas pass G1 with a's, found from the counting sort's bucket
@@ -30,6 +31,12 @@
 #include "gates.cuh"
 
 namespace pcl {
+
+bool band_mma_covers(const Geo &, uint32_t);
+size_t band_mma_workspace(const Geo &, uint32_t);
+cudaError_t launch_band_mma(const pcl_params &, const pcl_clipset &, const uint32_t *, const uint32_t *,
+                            const uint32_t *, void *, pcl_pair *, uint64_t, unsigned long long *,
+                            unsigned long long *, const unsigned int **, int, int *, unsigned long long, cudaStream_t);
 
 namespace {
 
@@ -61,39 +68,7 @@ __global__ void hist_kernel(const uint32_t *pop, uint32_t n, uint32_t *hist) {
 }
 
 // exclusive scan of v[0..m) into v (single CTA of 1024 threads)
-__global__ void __launch_bounds__(1024) scan_kernel(uint32_t *v, uint32_t m) {
-    __shared__ uint32_t wsum[32];
-    const uint32_t per = (m + 1023) / 1024;
-    const uint32_t lo = threadIdx.x * per, hi = min(m, lo + per);
-    uint32_t s = 0;
-    for (uint32_t i = lo; i < hi; ++i) s += v[i];
-    // block exclusive scan of s
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t x = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        uint32_t w = wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        wsum[lane] = w;
-    }
-    __syncthreads();
-    uint32_t run = x - s + (wid ? wsum[wid - 1] : 0u);
-    for (uint32_t i = lo; i < hi; ++i) {
-        const uint32_t t = v[i];
-        v[i] = run;
-        run += t;
-    }
-}
+__global__ void __launch_bounds__(1024) scan_kernel(uint32_t *v, uint32_t m) { cta_scan(v, v, m); }
 
 __global__ void scatter_kernel(const uint32_t *pop, uint32_t n, const uint32_t *cum, uint32_t *fill,
                                uint32_t *order, uint32_t *spop) {
@@ -116,7 +91,8 @@ __global__ void __launch_bounds__(256, LP ? 6 : 8) band_join_kernel(pcl_params p
                                                         unsigned long long *count,
                                                         unsigned long long *local_gates,
                                                         unsigned int *next_pos, uint32_t shard,
-                                                        uint32_t n_shards) {
+                                                        uint32_t n_shards, const unsigned int *only_if) {
+    if (only_if && !*only_if) return;  // decided already
     const Geo g = make_geo(prm);
     const int lane = threadIdx.x & 31;
     const uint32_t n = cs.n_clips;
@@ -382,7 +358,7 @@ uint64_t shard_pairs(uint64_t n, uint32_t s, uint32_t S) {
 cudaError_t launch_band_join(const pcl_params &prm, const pcl_clipset &cs, void *ws, size_t ws_bytes,
                              pcl_pair *out, uint64_t cap, unsigned long long *count,
                              unsigned long long *gates, int num_sms, cudaStream_t st, uint32_t shard,
-                             uint32_t n_shards) {
+                             uint32_t n_shards, int *d_err, unsigned long long wait_ns) {
     if (n_shards == 0 || shard >= n_shards) return cudaErrorInvalidValue;
     const Geo g = make_geo(prm);
     const uint32_t n = cs.n_clips;
@@ -414,22 +390,31 @@ cudaError_t launch_band_join(const pcl_params &prm, const pcl_clipset &cs, void 
     scan_kernel<<<1, 1024, 0, st>>>(cum, Vt);
     scatter_kernel<<<num_sms * 4, 256, 0, st>>>(k, n, cum, fill, order, spop);
     const uint32_t vall = (uint32_t)g.N * g.N;
+    // the whole self-join with the workspace for it takes G3 as a matrix
+    // product; the band join then runs only if that gave up
+    const unsigned int *only_if = nullptr;
+    const size_t own = (band_join_workspace(g, n, topo) + 255) & ~(size_t)255;
+    if (!topo && n_shards == 1 && band_mma_covers(g, n) && d_err && ws_bytes >= own + band_mma_workspace(g, n)) {
+        e = launch_band_mma(prm, cs, order, spop, cum, w + own, out, cap, count, local, &only_if, num_sms, d_err,
+                            wait_ns, st);
+        if (e != cudaSuccess) return e;
+    }
     // the lane-per-member first chunk at 256² (4 words per lane; at 512² the
     // first 64 of 1,024 blocks decide too few pairs to pay for the staging)
     const bool lp = (reinterpret_cast<uintptr_t>(cs.blk) & 15u) == 0;  // 16-byte copies of block rows
     switch ((g.nb * g.nb / 2 + 31) / 32) {  // u32 words of block counts per lane
         case 1: band_join_kernel<1><<<num_sms * 8, 256, band_g2_smem(g.N, g.S), st>>>(prm, cs, order, spop, cum, V,
                                                                                        vall, out, cap, count,
-                                                                 local, next_pos, shard, n_shards); break;
+                                                                 local, next_pos, shard, n_shards, only_if); break;
         case 4:
             if (lp) band_join_kernel<4, true><<<num_sms * 6, 256, band_lp_smem(), st>>>(prm, cs, order, spop, cum, V,
                                                                                      vall, out, cap, count, local,
-                                                                                     next_pos, shard, n_shards);
+                                                                                     next_pos, shard, n_shards, only_if);
             else band_join_kernel<4><<<num_sms * 8, 256, 0, st>>>(prm, cs, order, spop, cum, V, vall, out, cap, count,
-                                                                  local, next_pos, shard, n_shards);
+                                                                  local, next_pos, shard, n_shards, only_if);
             break;
         case 16: band_join_kernel<16><<<num_sms * 8, 256, 0, st>>>(prm, cs, order, spop, cum, V, vall, out, cap,
-                                                                   count, local, next_pos, shard, n_shards); break;
+                                                                   count, local, next_pos, shard, n_shards, only_if); break;
         default: return cudaErrorInvalidValue;
     }
     const unsigned long long total = shard_pairs(n, shard, n_shards);

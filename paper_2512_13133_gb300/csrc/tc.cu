@@ -55,10 +55,12 @@
 #include <climits>
 
 #include "gates.cuh"
+#include "tc_dev.cuh"
 
 namespace pcl {
 
 namespace {
+using namespace tc_dev;
 
 constexpr int kWarps = 12;
 constexpr int kThreads = 32 * kWarps;
@@ -72,13 +74,9 @@ constexpr int kCopies = 16;              // shifted copies of the representative
 constexpr int kMaxCols = 256;            // N of one MMA / one accumulator buffer
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSmemMax = 227 * 1024;
-constexpr unsigned long long kWaitNs = 1000000000ull;
 enum { kBarB = 1, kBarEpi = 2 };
 // mbarrier indices: a_full[2], a_empty[2], acc_full[2], acc_empty[2], fin, b_full[R], b_empty[R]
 enum { kAFull = 0, kAEmpty = 2, kAccFull = 4, kAccEmpty = 6, kFin = 8, kBFull = 9 };
-
-// operand types (both MMA operands always have the same one)
-enum { kOpF16 = 0, kOpBF16 = 1, kOpE4M3 = 2 };
 
 template <int S, int NW, int OP>
 struct Tc {
@@ -132,43 +130,6 @@ struct Tc {
     static_assert(PD >= 2 && BYTES <= kSmemMax, "shared memory plan");
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-// canonical K-major, no-swizzle shared-memory descriptor (tcgen05 format):
-// start >> 4 [0,14), leading (K) core-matrix stride >> 4 [16,30), stride
-// between 8-row groups >> 4 [32,46), version 1 at bit 46, layout 0 (none)
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
-
-// instruction descriptor: D = F32 (bit 4), A and B formats in bits 7-9 and
-// 10-12 (kind::f16: 0 = F16, 1 = BF16; kind::f8f6f4: 0 = E4M3), both K-major,
-// N >> 3 at bit 17, M >> 4 at bit 24
-__host__ __device__ constexpr uint32_t idesc_of(int M, int N, int op) {
-    const uint32_t ab = op == kOpBF16 ? 1u : 0u;  // the same format for A and B
-    return (1u << 4) | (ab << 7) | (ab << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-template <bool FP8>
-__device__ __forceinline__ void mma(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    if constexpr (FP8) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-            "l"(a), "l"(b), "r"(idesc), "r"(acc));
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-            "l"(a), "l"(b), "r"(idesc), "r"(acc));
-    }
-}
-
 // the low CH pixels (bits) of b as one 16-byte core-matrix row of 0 / 1.0
 template <int OP>
 __device__ __forceinline__ uint4 expand(uint32_t b) {
@@ -189,54 +150,6 @@ __device__ __forceinline__ void sts16(uint32_t a, uint4 v) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-                 : "memory");
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar), "r"(count));
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t mbar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(mbar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-__device__ __forceinline__ uint64_t gtimer() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// bounded wait for the phase of the given parity; false after limit_ns or
-// when another role has aborted (abort_flag may be null: wait regardless)
-__device__ __forceinline__ bool wait_phase_slow(uint32_t mbar, uint32_t parity, const volatile uint32_t *abort_flag,
-                                                unsigned long long limit_ns) {
-    const uint64_t t0 = gtimer();
-    for (;;) {
-        for (int i = 0; i < 16; ++i)
-            if (mbar_try_wait(mbar, parity)) return true;
-        if (abort_flag && *abort_flag) return false;
-        if (gtimer() - t0 > limit_ns) return false;
-    }
-}
-__device__ __forceinline__ bool wait_phase(uint32_t mbar, uint32_t parity, const volatile uint32_t *abort_flag,
-                                           unsigned long long limit_ns) {
-    return mbar_try_wait(mbar, parity) || wait_phase_slow(mbar, parity, abort_flag, limit_ns);
-}
-
 // barrier over `count` threads of one role that also ORs a flag
 __device__ __forceinline__ bool bar_any(int id, int count, bool v) {
     uint32_t r;
@@ -254,19 +167,6 @@ __device__ __forceinline__ bool bar_any(int id, int count, bool v) {
 __device__ __forceinline__ void bar_sync(int id, int count) {
     asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
-
-__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // 64 bits of a bit row starting at pixel `base` (zeros outside the row)
 template <int NW>
@@ -853,36 +753,8 @@ __global__ void tc_gate_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B, con
 
 // exclusive scan of v[0..m) into out[0..m] (out[m] = total), single CTA
 __global__ void __launch_bounds__(1024) tc_scan_kernel(const uint32_t *v, uint32_t m, uint32_t *out) {
-    __shared__ uint32_t wsum[32];
-    const uint32_t per = (m + 1023) / 1024;
-    const uint32_t lo = threadIdx.x * per, hi = min(m, lo + per);
-    uint32_t s = 0;
-    for (uint32_t i = lo; i < hi; ++i) s += v[i];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t x = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        uint32_t w = wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        wsum[lane] = w;
-    }
-    __syncthreads();
-    uint32_t run = x - s + (wid ? wsum[wid - 1] : 0u);
-    for (uint32_t i = lo; i < hi; ++i) {
-        out[i] = run;
-        run += v[i];
-    }
-    if (threadIdx.x == 1023) out[m] = run;
+    const uint32_t total = cta_scan(v, out, m);
+    if (threadIdx.x == 0) out[m] = total;
 }
 
 // survivors in list order; item starts where the representative changes or a
