@@ -251,7 +251,8 @@ pcl_status pcl_spectra(pcl_ctx *ctx, const pcl_params *P, pcl_clipset *cs, const
    (about 8 (N^2 + 2) + 8 |a| bytes for the area order; the self-join at
    256x256 and 512x512 px from 2,048 clips 2 KB per clip more for the vectors of
    G3 as a matrix product, done without where they do not fit; two sets: about
-   16 (N^2 + 2) + 16 |a| + 8 |b| bytes).  EDGE uses it for the list of pairs
+   16 (N^2 + 2) + 16 |a| + 8 |b| bytes, with 2,048 or more clips in b at those
+   sizes 1 KB per clip more and |b| / 96 + 512 bytes per clip of a).  EDGE uses it for the list of pairs
    left for the exact check (pairs past the list are checked inside the
    screen): the self-join 8 bytes per entry, 2^19 to 2^23 entries, beside 2 MB
    of tables per 256 clips (at most 134 MB) and 172 bytes per clip; two sets
@@ -369,9 +370,11 @@ pcl_status pcl_match_pairs(pcl_ctx *ctx, const pcl_params *P, uint32_t mode, pcl
                            pcl_record *d_out, pcl_stream stream);
 
 /* Limit of each bounded device-side wait of the kernels launched through ctx
-   from now on, in nanoseconds (0 = the default of one second).  Only the
-   tensor-core engine waits on the device (its warps hand buffers over
-   through shared-memory barriers); a wait that runs out makes the kernel
+   from now on, in nanoseconds (0 = the default of one second).  The
+   tensor-core engine and the cosine candidates' density gate wait on the
+   device (their warps hand buffers over through shared-memory barriers).
+   The gate then leaves its pairs to the band join (same results).  In the
+   engine a wait that runs out makes the kernel
    give up its work, wait (always up to one second) for the tensor-core
    operations it has in flight, release its tensor memory and return, and
    is reported by pcl_device_error (pcl_match_pairs) or as a completion
@@ -488,7 +491,9 @@ pcl_status pcl_match_mixed(pcl_ctx *ctx, const pcl_params *params, pcl_clipset *
    EDGE: the Min-Max procedure).  pcl_server_create_classes takes n_classes
    (1..16) parameter blocks and libraries (class c: params[c], libraries[c]);
    pcl_server_create is the one-class form.  For COSINE each library must be
-   rasterised (bits, pop, prof, blk) and is sorted by area at creation; with
+   rasterised (bits, pop, prof, blk) and is sorted by area at creation (from
+   2,048 clips of 256x256 or 512x512 px the vectors of the density gate are kept
+   as well, 1 KB per clip, where memory allows); with
    the FFT engine its spectra are computed too (spec/spec_state required),
    while the tensor-core engine and the exact scan read the rasters only
    (spec may be NULL: ~10.6 KB per 256^2 clip instead of ~350 KB, so

@@ -12,7 +12,7 @@ namespace pcl {
 cudaError_t launch_raster(const pcl_params &, const pcl_clipset &, cudaStream_t);
 size_t band_join_workspace(const Geo &, uint32_t, bool);
 cudaError_t launch_band_join(const pcl_params &, const pcl_clipset &, void *, size_t, pcl_pair *, uint64_t,
-                             unsigned long long *, unsigned long long *, int, cudaStream_t, uint32_t, uint32_t, int *,
+                             unsigned long long *, unsigned long long *, int, cudaStream_t, uint32_t, uint32_t,
                              unsigned long long);
 size_t band_mma_workspace(const Geo &, uint32_t);
 size_t edge_checks_workspace(uint64_t);
@@ -30,7 +30,12 @@ cudaError_t launch_area_sort(const uint32_t *, uint32_t, uint32_t, uint32_t *, u
 size_t cross_join_workspace(const Geo &, uint32_t, uint32_t);
 cudaError_t launch_cross_join(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const uint32_t *,
                               const uint32_t *, const uint32_t *, void *, size_t, pcl_pair *, uint64_t,
-                              unsigned long long *, unsigned long long *, int, cudaStream_t);
+                              unsigned long long *, unsigned long long *, int, cudaStream_t, void *,
+                              unsigned long long);
+size_t band_lib_bytes(const Geo &, uint32_t);
+size_t band_cross_workspace(const Geo &, uint32_t, uint32_t);
+cudaError_t launch_band_lib(const pcl_params &, const pcl_clipset &, const uint32_t *, const uint32_t *, void *,
+                            cudaStream_t);
 cudaError_t launch_edge_match(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const pcl_pair *, uint64_t,
                               const unsigned long long *, pcl_record *, int, cudaStream_t);
 cudaError_t launch_spectra(const pcl_params &, const pcl_clipset &, const uint32_t *, uint32_t, bool,
@@ -270,16 +275,24 @@ pcl_status pcl_candidates(pcl_ctx *ctx, const pcl_params *P, uint32_t mode, cons
     const Geo g = make_geo(*P);
     if (g.S > g.N / 16) return fail(ctx, PCL_ERR_UNSUPPORTED, "cosine gates need S <= N/16%s%lld");
     // workspace: B's area histogram, fill counters, area order and sorted
-    // areas, then the cross join's own part (16-byte aligned)
+    // areas, B's vectors for G3 as a matrix product (where they fit), then the
+    // cross join's own part
     const uint32_t V = (uint32_t)g.N * g.N + 2, nb = b->n_clips;
-    const size_t sort_bytes = ((4 * (2 * (size_t)V + 2 * (size_t)nb)) + 15) & ~(size_t)15;
-    const size_t join_bytes = cross_join_workspace(g, a->n_clips, nb);
-    if ((s = ensure_ws(ctx, sort_bytes + join_bytes))) return s;
+    const size_t sort_bytes = ((4 * (2 * (size_t)V + 2 * (size_t)nb)) + 255) & ~(size_t)255;
+    const size_t join_bytes = cross_join_workspace(g, a->n_clips, nb) + 256;
+    size_t lib_bytes = a->n_clips ? band_lib_bytes(g, nb) : 0;
+    const size_t more = lib_bytes ? band_cross_workspace(g, a->n_clips, nb) : 0;
+    if (lib_bytes && ensure_ws(ctx, sort_bytes + lib_bytes + join_bytes + more)) lib_bytes = 0;
+    if (!lib_bytes && (s = ensure_ws(ctx, sort_bytes + join_bytes))) return s;
+    ctx->err.clear();
     uint32_t *cum = static_cast<uint32_t *>(ctx->ws), *fill = cum + V, *order = fill + V, *spop = order + nb;
+    char *lib = lib_bytes ? static_cast<char *>(ctx->ws) + sort_bytes : nullptr;
     e = launch_area_sort(b->pop, nb, V, cum, fill, order, spop, ctx->num_sms, st);
+    if (e == cudaSuccess && lib) e = launch_band_lib(*P, *b, order, spop, lib, st);
+    const size_t at = sort_bytes + lib_bytes;
     if (e == cudaSuccess)
-        e = launch_cross_join(*P, *a, *b, order, spop, cum, static_cast<char *>(ctx->ws) + sort_bytes,
-                              ctx->ws_bytes - sort_bytes, d_out, cap, cnt, gates, ctx->num_sms, st);
+        e = launch_cross_join(*P, *a, *b, order, spop, cum, static_cast<char *>(ctx->ws) + at, ctx->ws_bytes - at,
+                              d_out, cap, cnt, gates, ctx->num_sms, st, lib, ctx->wait_ns);
     return e == cudaSuccess ? PCL_OK : cuda_fail(ctx, e, "band join (two sets)");
 }
 
@@ -309,7 +322,7 @@ pcl_status pcl_candidates_shard(pcl_ctx *ctx, const pcl_params *P, uint32_t mode
         if ((!more || ensure_ws(ctx, need + 256 + more)) && (s = ensure_ws(ctx, need))) return s;
         ctx->err.clear();
         e = launch_band_join(*P, *cs, ctx->ws, ctx->ws_bytes, d_out, cap, cnt, gates, ctx->num_sms, st, shard,
-                             n_shards, ctx->d_err, ctx->wait_ns);
+                             n_shards, ctx->wait_ns);
         return e == cudaSuccess ? PCL_OK : cuda_fail(ctx, e, "band join");
     }
     if (mode == PCL_MODE_EDGE && n_shards == 1 && !topo) {

@@ -23,9 +23,9 @@
 // (double buffered in tensor memory) with T sqrt(|A| |B|), a 32-column word of
 // decisions per lane, and list the pairs left.  band_list_kernel decides those
 // exactly, a warp per pair.  Should the list be too short (nearly identical
-// clips), it is dropped and the band join of gates.cu runs instead, as it does
-// for smaller rasters, shards, the topological pre-screen and callers without
-// workspace.
+// clips) or a bounded wait run out, it is dropped and the band join (gates.cu,
+// cross.cu) runs instead, as it does for smaller rasters, shards, the
+// topological pre-screen and callers without workspace.
 //
 // 100,000 clips of 256x256 px (5.9e8 band pairs), one GB300: 1.5 ms a call - the
 // products 0.68 ms (4.8 GB of operands from L2, 7.2 TB/s, which bounds them:
@@ -60,24 +60,30 @@ struct BandWs {
     unsigned long long *seen;   // band pairs
     unsigned long long *n_list; // listed pairs
     unsigned int *overflow;     // 1: the list was too short
+    uint32_t *seg;              // member blocks per item
     uint32_t *item_off;         // [panels + 1]
-    uint32_t *end;              // [n] end of each representative's band (area order)
-    float2 *thr;                // [blocks * 256] {T sqrt(area) with the slack, sqrt(area)}
-    unsigned char *P, *Q;       // vectors: panels x K x 128, blocks x K x 256 bytes
-    uint2 *list;                // positions (p, q)
-    uint32_t list_cap, n, panels, blocks;
+    uint32_t *beg, *end;        // [rows] band of each representative, positions in the members' area order
+    float *ra;                  // [rows] T sqrt(area) with the slack
+    float *cb;                  // [blocks * 256] sqrt(area) of the members
+    unsigned char *P, *Q;       // vectors: panels x K x 128 bytes, blocks x K x 256 bytes
+    uint2 *list;                // positions (representative, member)
+    const uint32_t *row_order, *row_pop, *col_order, *col_pop;  // the area orders
+    uint32_t list_cap, rows, cols, panels, blocks;
     int kb;
 };
 
 size_t up(size_t v) { return (v + 255) & ~(size_t)255; }
 
-size_t band_layout(const Geo &g, uint32_t n, char *ws, BandWs &w) {
-    w.n = n;
-    w.panels = (n + kPanel - 1) / kPanel;
-    w.blocks = (n + kBlock - 1) / kBlock;
+// the parts of the workspace; with_cols: the members' vectors are part of it
+// (and the bands of a self-join), otherwise Q, cb, beg and end are the caller's
+size_t band_layout(const Geo &g, uint32_t rows, uint32_t cols, uint64_t list_cap, bool self, bool with_cols, char *ws,
+                   BandWs &w) {
+    w.rows = rows;
+    w.cols = cols;
+    w.panels = (rows + kPanel - 1) / kPanel;
+    w.blocks = (cols + kBlock - 1) / kBlock;
     w.kb = kbytes_of(g.nb * g.nb);
-    const uint64_t c = (uint64_t)n * n / 512;
-    w.list_cap = c < (1u << 16) ? (1u << 16) : c > (1u << 23) ? (1u << 23) : (uint32_t)c;
+    w.list_cap = list_cap < (1u << 12) ? (1u << 12) : list_cap > (1u << 23) ? (1u << 23) : (uint32_t)list_cap;
     size_t o = 0;
     auto part = [&](auto *&p, size_t bytes) {
         p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(ws + o);
@@ -86,13 +92,27 @@ size_t band_layout(const Geo &g, uint32_t n, char *ws, BandWs &w) {
     part(w.seen, 8);
     part(w.n_list, 8);
     part(w.overflow, 4);  // the parts so far start as zeros
+    part(w.seg, 4);
     part(w.item_off, 4 * ((size_t)w.panels + 1));
-    part(w.end, 4 * (size_t)n);
-    part(w.thr, 8 * (size_t)kBlock * w.blocks);
+    if (self) {
+        part(w.beg, 4 * (size_t)rows);
+        part(w.end, 4 * (size_t)rows);
+    }
+    part(w.ra, 4 * (size_t)rows);
     part(w.list, 8 * (size_t)w.list_cap);
     part(w.P, (size_t)w.panels * kPanel * w.kb);
-    part(w.Q, (size_t)w.blocks * kBlock * w.kb);
+    if (with_cols) {
+        part(w.cb, 4 * (size_t)kBlock * w.blocks);
+        part(w.Q, (size_t)w.blocks * kBlock * w.kb);
+    }
     return o;
+}
+
+// listed pairs there is room for: the bound leaves 0.55 % of a band of about
+// an eighth of the members; nearly identical clips leave more, and overflow
+uint64_t list_room(uint64_t rows, uint64_t cols, bool self) {
+    const uint64_t c = self ? rows * cols / 512 : rows * (cols / 768 + 64);
+    return self && c < (1u << 16) ? 1u << 16 : c;
 }
 
 // integer 0..256 as E4M3, rounded up to 4 significant bits
@@ -115,9 +135,11 @@ __device__ __forceinline__ uint32_t e4m3_up(int x) {
 // clips, the table 72 us.)
 constexpr int kFeatureClips = 64;
 
-template <int LV>
+// ROWS: the representatives' vectors, thresholds and (BANDS, the self-join)
+// bands; COLS: the members' vectors.  order, spop: the set's area order; n clips.
+template <int LV, bool ROWS, bool COLS, bool BANDS>
 __global__ void __launch_bounds__(256) band_feature_kernel(pcl_params prm, pcl_clipset cs, BandWs w,
-                                                           const uint32_t *order, const uint32_t *spop,
+                                                           const uint32_t *order, const uint32_t *spop, uint32_t n,
                                                            const uint32_t *cum) {
     const Geo g = make_geo(prm);
     const int nb2 = g.nb * g.nb;
@@ -134,7 +156,7 @@ __global__ void __launch_bounds__(256) band_feature_kernel(pcl_params prm, pcl_c
     const int r = threadIdx.x & 15;
     for (int c0 = 0; c0 < kFeatureClips; c0 += 16) {
         const uint32_t p = blockIdx.x * kFeatureClips + c0 + r;
-        const bool live = p < w.n;
+        const bool live = p < n;
         const uint32_t *cw = reinterpret_cast<const uint32_t *>(cs.blk + (size_t)(live ? order[p] : 0) * 2 * nb2);
         unsigned char *P = w.P + (size_t)(p / kPanel) * kPanel * w.kb + (p % kPanel) * 16;
         unsigned char *Q = w.Q + (size_t)(p / kBlock) * kBlock * w.kb + (p % kBlock) * 16;
@@ -166,78 +188,69 @@ __global__ void __launch_bounds__(256) band_feature_kernel(pcl_params prm, pcl_c
 #pragma unroll
             for (int l = 0; l < LV; ++l) {
                 const size_t k = (size_t)(l * nb2 / 16 + j);  // 16-byte column of K
-                if (p < w.panels * kPanel)
+                if (ROWS && p < w.panels * kPanel)
                     *reinterpret_cast<uint4 *>(P + k * (16 * kPanel)) = make_uint4(f[l][0], f[l][1], f[l][2], f[l][3]);
-                if (p < w.blocks * kBlock)
+                if (COLS && p < w.blocks * kBlock)
                     *reinterpret_cast<uint4 *>(Q + k * (16 * kBlock)) = make_uint4(q[l][0], q[l][1], q[l][2], q[l][3]);
             }
         }
     }
+    if (threadIdx.x >= kFeatureClips) return;
     const uint32_t p = blockIdx.x * kFeatureClips + threadIdx.x;
-    if (threadIdx.x < kFeatureClips && p < w.blocks * kBlock) {
+    const float s = p < n ? sqrtf((float)spop[p]) : 0.0f;
+    if (COLS && p < w.blocks * kBlock) w.cb[p] = s;
+    if (ROWS) {
         unsigned long long band = 0;
-        float s = 0.0f;
-        if (p < w.n) {
-            const uint64_t num2 = (uint64_t)prm.cos_num * prm.cos_num, den2 = (uint64_t)prm.cos_den * prm.cos_den;
-            const uint64_t pa = spop[p], all = (uint64_t)g.N * g.N;
-            uint64_t vmax = pa == 0 ? 0 : (den2 * pa - 1) / num2;
-            if (vmax > all) vmax = all;
-            const uint32_t e = cum[vmax + 1];
-            w.end[p] = e;
-            band = e - p - 1;
-            s = sqrtf((float)pa);
+        if (p < n) {
+            w.ra[p] = s * ((float)prm.cos_num / (float)prm.cos_den) * kSlack;
+            if (BANDS) {
+                const uint64_t num2 = (uint64_t)prm.cos_num * prm.cos_num, den2 = (uint64_t)prm.cos_den * prm.cos_den;
+                const uint64_t pa = spop[p], all = (uint64_t)g.N * g.N;
+                uint64_t vmax = pa == 0 ? 0 : (den2 * pa - 1) / num2;
+                if (vmax > all) vmax = all;
+                w.beg[p] = p + 1;
+                w.end[p] = cum[vmax + 1];
+            }
+            band = w.end[p] - w.beg[p];
         }
-        w.thr[p] = make_float2(s * ((float)prm.cos_num / (float)prm.cos_den) * kSlack, s);
         for (int o = 16; o; o >>= 1) band += __shfl_xor_sync(0xffffffffu, band, o);
         if ((threadIdx.x & 31) == 0 && band) atomicAdd(w.seen, band);
     }
 }
 
-// first member block of a panel's band, and how many blocks it meets
+// first member block of a panel's band, and how many blocks it meets (begins
+// and ends do not decrease along the area order)
 __device__ __forceinline__ void panel_blocks(const BandWs &w, uint32_t panel, uint32_t &first, uint32_t &count) {
-    const uint32_t p0 = panel * kPanel, last = min(w.n, p0 + kPanel) - 1;
-    const uint32_t e = w.end[last];  // ends do not decrease along the area order
-    first = (p0 + 1) / kBlock;
-    count = e > p0 + 1 ? (e + kBlock - 1) / kBlock - first : 0u;
+    const uint32_t p0 = panel * kPanel, last = min(w.rows, p0 + kPanel) - 1;
+    const uint32_t b = w.beg[p0], e = w.end[last];
+    first = b / kBlock;
+    count = e > b ? (e + kBlock - 1) / kBlock - first : 0u;
 }
 
-// items of the panels before each panel (one CTA)
-__global__ void __launch_bounds__(1024) band_items_kernel(BandWs w) {
-    __shared__ uint32_t wsum[32];
-    const uint32_t per = (w.panels + 1023) / 1024;
-    const uint32_t lo = min(w.panels, threadIdx.x * per), hi = min(w.panels, lo + per);
-    auto items = [&](uint32_t i) {
+// Items of the panels before each panel (one CTA): an item takes up to kSeg
+// member blocks, fewer when that would leave SMs without an item.
+__global__ void __launch_bounds__(1024) band_items_kernel(BandWs w, uint32_t num_sms) {
+    __shared__ unsigned int tiles;
+    if (threadIdx.x == 0) tiles = 0u;
+    __syncthreads();
+    unsigned int t = 0;
+    for (uint32_t i = threadIdx.x; i < w.panels; i += 1024) {
         uint32_t f, c;
         panel_blocks(w, i, f, c);
-        return (c + kSeg - 1) / kSeg;
-    };
-    uint32_t s = 0;
-    for (uint32_t i = lo; i < hi; ++i) s += items(i);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t x = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+        w.item_off[i] = c;
+        t += c;
     }
-    if (lane == 31) wsum[wid] = x;
+    t = __reduce_add_sync(0xffffffffu, t);
+    if ((threadIdx.x & 31) == 0 && t) atomicAdd(&tiles, t);
     __syncthreads();
-    if (wid == 0) {
-        uint32_t t = wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
-            if (lane >= o) t += y;
-        }
-        wsum[lane] = t;
-    }
+    const uint32_t seg = min(max(tiles / (2 * num_sms), 1u), (uint32_t)kSeg);
+    for (uint32_t i = threadIdx.x; i < w.panels; i += 1024) w.item_off[i] = (w.item_off[i] + seg - 1) / seg;
     __syncthreads();
-    uint32_t run = x - s + (wid ? wsum[wid - 1] : 0u);
-    for (uint32_t i = lo; i < hi; ++i) {
-        w.item_off[i] = run;
-        run += items(i);
+    const uint32_t total = cta_scan(w.item_off, w.item_off, w.panels);
+    if (threadIdx.x == 0) {
+        w.item_off[w.panels] = total;
+        *w.seg = seg;
     }
-    if (threadIdx.x == 1023) w.item_off[w.panels] = run;
 }
 
 struct BandItem {
@@ -253,10 +266,10 @@ __device__ __forceinline__ BandItem band_item(const BandWs &w, uint32_t it) {
     BandItem b;
     uint32_t f, c;
     panel_blocks(w, lo, f, c);
-    const uint32_t s = (it - w.item_off[lo]) * kSeg;
+    const uint32_t seg = *w.seg, s = (it - w.item_off[lo]) * seg;
     b.panel = lo;
     b.first = f + s;
-    b.count = min(c - s, (uint32_t)kSeg);
+    b.count = min(c - s, seg);
     return b;
 }
 
@@ -274,7 +287,7 @@ struct BandSmem {
 };
 
 template <int KB>
-__global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(BandWs w, int *err, unsigned long long wait_ns) {
+__global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(BandWs w, unsigned long long wait_ns) {
     using SM = BandSmem<KB>;
     constexpr int ST = SM::stages, CH = KB / 128;  // ring stages, K chunks per member block
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -282,9 +295,10 @@ __global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(BandWs w, int 
     const volatile uint32_t *abortf = misc + 1;
     const uint32_t sbase = smem_u32(sm), bar0 = sbase + SM::bars;
     auto bar = [&](int k) { return bar0 + 8u * (uint32_t)k; };
+    // a wait that ran out gives the product up: the band join decides instead
     auto raise_abort = [&]() {
         misc[1] = 1u;
-        atomicExch(err, 1);
+        *w.overflow = 1u;
     };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
@@ -396,8 +410,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(BandWs w, int 
         for (uint32_t it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
             const BandItem item = band_item(w, it);
             const uint32_t p = item.panel * kPanel + 32 * quarter + lane;
-            const uint32_t end = p < w.n ? w.end[p] : 0u;
-            const float ra = w.thr[min(p, w.n - 1)].x;
+            const uint32_t beg = p < w.rows ? w.beg[p] : 0u, end = p < w.rows ? w.end[p] : 0u;
+            const float ra = w.ra[min(p, w.rows - 1)];
             for (uint32_t b = 0; b < item.count; ++b, ++t) {
                 const uint32_t buf = t & 1;
                 ok = wait_phase(bar(kAcc + buf), (t >> 1) & 1, abortf, wait_ns);
@@ -411,18 +425,20 @@ __global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(BandWs w, int 
                 for (int c = 0; c < kBlock; c += 32) {
                     uint32_t v[32];
                     tmem_ld32(src + c, v);
-                    const float4 *th = reinterpret_cast<const float4 *>(w.thr + q0 + c);
+                    const float4 *th = reinterpret_cast<const float4 *>(w.cb + q0 + c);
                     tmem_wait_ld();
                     uint32_t hit = 0u;  // bit 31 - j: v[j] above its threshold
 #pragma unroll
-                    for (int j = 0; j < 32; j += 2) {
-                        const float4 s = __ldg(th + j / 2);  // {.., sqrt, .., sqrt} of two members
-                        hit = __funnelshift_l(__float_as_uint(fmaf(ra, s.y, -__uint_as_float(v[j]))), hit, 1);
-                        hit = __funnelshift_l(__float_as_uint(fmaf(ra, s.w, -__uint_as_float(v[j + 1]))), hit, 1);
+                    for (int j = 0; j < 32; j += 4) {
+                        const float4 s = __ldg(th + j / 4);
+                        hit = __funnelshift_l(__float_as_uint(fmaf(ra, s.x, -__uint_as_float(v[j]))), hit, 1);
+                        hit = __funnelshift_l(__float_as_uint(fmaf(ra, s.y, -__uint_as_float(v[j + 1]))), hit, 1);
+                        hit = __funnelshift_l(__float_as_uint(fmaf(ra, s.z, -__uint_as_float(v[j + 2]))), hit, 1);
+                        hit = __funnelshift_l(__float_as_uint(fmaf(ra, s.w, -__uint_as_float(v[j + 3]))), hit, 1);
                     }
                     hit = __brev(hit);
-                    // members p < q < end
-                    const int lo = (int)p + 1 - (int)(q0 + c), hi = (int)end - (int)(q0 + c);
+                    // members of the band
+                    const int lo = (int)beg - (int)(q0 + c), hi = (int)end - (int)(q0 + c);
                     uint32_t in = hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
                     in &= lo <= 0 ? 0xffffffffu : lo >= 32 ? 0u : 0xffffffffu << lo;
                     hit &= in;
@@ -508,14 +524,14 @@ __device__ __forceinline__ bool warp_g2_rejects_groups(const uint16_t *__restric
 }
 
 // The listed pairs: exact G3, then G2, a warp per pair; and the pairs of empty
-// clips.  A warp takes 32 pairs at a time: lane q reads pair q's clips and
+// clips.  A warp takes up to 32 pairs at a time: lane q reads pair q's clips and
 // finds its threshold, then the pairs go one by one, the next pair's first 64
 // blocks loading while one is tested (1.10 -> 0.68 ms at 100,000 clips).
-template <int NPL>
-__global__ void __launch_bounds__(256) band_list_kernel(pcl_params prm, pcl_clipset cs, BandWs w,
-                                                        const uint32_t *order, const uint32_t *spop,
-                                                        const uint32_t *cum, pcl_pair *out, uint64_t cap,
-                                                        unsigned long long *count, unsigned long long *local) {
+// CROSS: representatives of set A (rows), members of set B; otherwise one set.
+template <int NPL, bool CROSS>
+__global__ void __launch_bounds__(256) band_list_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B, BandWs w,
+                                                        pcl_pair *out, uint64_t cap, unsigned long long *count,
+                                                        unsigned long long *local) {
     if (*w.overflow) return;
     extern __shared__ uint16_t g2_scratch[];
     const unsigned full = 0xffffffffu;
@@ -524,23 +540,26 @@ __global__ void __launch_bounds__(256) band_list_kernel(pcl_params prm, pcl_clip
     uint16_t *scratch = g2_scratch + (threadIdx.x >> 5) * 2 * (g.N + 2 * g.S + 32);
     const uint32_t n = (uint32_t)*w.n_list;
     const uint32_t w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-    const uint32_t *blk = reinterpret_cast<const uint32_t *>(cs.blk);
+    const uint32_t *blk_a = reinterpret_cast<const uint32_t *>(A.blk), *blk_b = reinterpret_cast<const uint32_t *>(B.blk);
+    auto pair_of = [](uint32_t a, uint32_t b) { return CROSS ? pcl_pair{a, b} : pcl_pair{min(a, b), max(a, b)}; };
     unsigned long long kept = 0, g2 = 0;
-    for (uint32_t t0 = w0 * 32; t0 < n; t0 += nw * 32) {  // warp-uniform
-        const int m = (int)min(n - t0, 32u);
+    const uint32_t per = min(32u, (n + nw - 1) / nw);  // a short list (a request's) is spread over all warps
+    for (uint32_t t0 = w0 * per; t0 < n; t0 += nw * per) {  // warp-uniform
+        const int m = (int)min(n - t0, per);
         uint32_t a = 0, b = 0;
         int um = 0, pa = 0, pb = 0;  // areas are at most 512^2
         if (lane < m) {
             const uint2 e = w.list[t0 + lane];
-            a = order[e.x];
-            b = order[e.y];
-            pa = (int)spop[e.x];
-            pb = (int)spop[e.y];
+            a = w.row_order[e.x];
+            b = w.col_order[e.y];
+            pa = (int)w.row_pop[e.x];
+            pb = (int)w.col_pop[e.y];
             um = (int)cos_umax((uint64_t)pa, (uint64_t)pb, prm.cos_num, prm.cos_den);
         }
         uint32_t ca = 0, da = 0, cb = 0, db = 0;  // the next pair's first chunk: counts and neighbourhood sums
         auto fetch = [&](int q) {
-            const uint32_t *x = blk + (size_t)__shfl_sync(full, a, q) * nb2, *y = blk + (size_t)__shfl_sync(full, b, q) * nb2;
+            const uint32_t *x = blk_a + (size_t)__shfl_sync(full, a, q) * nb2;
+            const uint32_t *y = blk_b + (size_t)__shfl_sync(full, b, q) * nb2;
             ca = __ldg(x + lane);
             da = __ldg(x + words + lane);
             cb = __ldg(y + lane);
@@ -556,7 +575,7 @@ __global__ void __launch_bounds__(256) band_list_kernel(pcl_params prm, pcl_clip
             if (q + 1 < m) fetch(q + 1);
             int DA = (int)((sa & 0xffffu) + (sa >> 16)), DB = (int)((sb & 0xffffu) + (sb >> 16));
             bool rej = DA >= tA || DB >= tB;
-            const uint32_t *x = blk + (size_t)qa * nb2, *y = blk + (size_t)qb * nb2;
+            const uint32_t *x = blk_a + (size_t)qa * nb2, *y = blk_b + (size_t)qb * nb2;
             for (int k = 32 + lane; !rej && k < words; k += 32) {  // words is a multiple of 32
                 const uint32_t c0 = __ldg(x + k), d0 = __ldg(x + words + k), c1 = __ldg(y + k), d1 = __ldg(y + words + k);
                 sa = __reduce_add_sync(full, c0 - __vminu2(c0, d1));
@@ -566,7 +585,7 @@ __global__ void __launch_bounds__(256) band_list_kernel(pcl_params prm, pcl_clip
                 rej = DA >= tA || DB >= tB;
             }
             if (rej) continue;
-            if (warp_g2_rejects_groups<NPL>(cs.prof + (size_t)qa * 2 * g.N, cs.prof + (size_t)qb * 2 * g.N, g.S,
+            if (warp_g2_rejects_groups<NPL>(A.prof + (size_t)qa * 2 * g.N, B.prof + (size_t)qb * 2 * g.N, g.S,
                                             (int64_t)u, lane, scratch)) {
                 ++g2;
                 continue;
@@ -574,21 +593,22 @@ __global__ void __launch_bounds__(256) band_list_kernel(pcl_params prm, pcl_clip
             ++kept;
             if (lane == 0) {
                 const unsigned long long at = atomicAdd(count, 1ull);
-                if (at < cap) out[at] = pcl_pair{min(qa, qb), max(qa, qb)};
+                if (at < cap) out[at] = pair_of(qa, qb);
             }
         }
     }
-    const uint32_t e = cum[1];  // empty clips: similar by definition
-    for (uint32_t p = blockIdx.x; p + 1 < e; p += gridDim.x) {
-        const uint32_t a = order[p];
-        for (uint32_t q0 = p + 1; q0 < e; q0 += blockDim.x) {
+    // empty representatives (the first ones): their band holds the empty
+    // members only, similar by definition
+    for (uint32_t p = blockIdx.x; p < w.rows && w.row_pop[p] == 0; p += gridDim.x) {
+        const uint32_t a = w.row_order[p], e = w.end[p];
+        for (uint32_t q0 = w.beg[p]; q0 < e; q0 += blockDim.x) {
             const uint32_t q = q0 + threadIdx.x;
-            const uint32_t b = q < e ? order[q] : 0u;
-            const unsigned m = __ballot_sync(0xffffffffu, q < e);
+            const uint32_t b = q < e ? w.col_order[q] : 0u;
+            const unsigned m = __ballot_sync(full, q < e);
             unsigned long long base = 0;
             if (lane == 0 && m) base = atomicAdd(count, (unsigned long long)__popc(m));
-            base = __shfl_sync(0xffffffffu, base, 0);
-            if (q < e && base + lane < cap) out[base + lane] = pcl_pair{min(a, b), max(a, b)};
+            base = __shfl_sync(full, base, 0);
+            if (q < e && base + lane < cap) out[base + lane] = pair_of(a, b);
             kept += (unsigned long long)__popc(m);
         }
     }
@@ -603,30 +623,48 @@ __global__ void band_count_kernel(BandWs w, unsigned long long *local) {
     if (!*w.overflow) local[PCL_GATE_G3_DENSITY] = *w.seen - local[0] - local[PCL_GATE_G2_PROFILE];
 }
 
-template <int KB, int NPL>
-cudaError_t launch_t(const pcl_params &prm, const Geo &g, const pcl_clipset &cs, const BandWs &w,
-                     const uint32_t *order, const uint32_t *spop, const uint32_t *cum, pcl_pair *out, uint64_t cap,
-                     unsigned long long *count, unsigned long long *local, int num_sms, int *d_err,
+template <int KB, int NPL, bool CROSS>
+cudaError_t launch_t(const pcl_params &prm, const Geo &g, const pcl_clipset &A, const pcl_clipset &B, const BandWs &w,
+                     pcl_pair *out, uint64_t cap, unsigned long long *count, unsigned long long *local, int num_sms,
                      unsigned long long wait_ns, cudaStream_t st) {
+    band_items_kernel<<<1, 1024, 0, st>>>(w, (uint32_t)num_sms);
     const uint32_t bytes = BandSmem<KB>::bytes;
     cudaError_t e = cudaFuncSetAttribute(band_mma_kernel<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    band_mma_kernel<KB><<<num_sms, kMmaThreads, bytes, st>>>(w, d_err, wait_ns ? wait_ns : kWaitNs);
+    band_mma_kernel<KB><<<num_sms, kMmaThreads, bytes, st>>>(w, wait_ns ? wait_ns : kWaitNs);
     const size_t scratch = 8 * 2 * 2 * (size_t)(g.N + 2 * g.S + 32);
-    band_list_kernel<NPL><<<num_sms * 8, 256, scratch, st>>>(prm, cs, w, order, spop, cum, out, cap, count, local);
+    band_list_kernel<NPL, CROSS><<<num_sms * 8, 256, scratch, st>>>(prm, A, B, w, out, cap, count, local);
+    band_count_kernel<<<1, 1, 0, st>>>(w, local);
     return cudaGetLastError();
+}
+
+template <bool ROWS, bool COLS, bool BANDS>
+void features(const pcl_params &prm, const Geo &g, const pcl_clipset &cs, const BandWs &w, const uint32_t *order,
+              const uint32_t *spop, uint32_t n, const uint32_t *cum, cudaStream_t st) {
+    const uint32_t reach = COLS ? w.blocks * kBlock : w.panels * kPanel;  // COLS reaches at least as far as ROWS of one set
+    const unsigned grid = (reach + kFeatureClips - 1) / kFeatureClips;
+    if (grid == 0) return;
+    if (g.N == 256) band_feature_kernel<4, ROWS, COLS, BANDS><<<grid, 256, 0, st>>>(prm, cs, w, order, spop, n, cum);
+    else band_feature_kernel<1, ROWS, COLS, BANDS><<<grid, 256, 0, st>>>(prm, cs, w, order, spop, n, cum);
+}
+
+cudaError_t clear_counters(const BandWs &w, cudaStream_t st) {
+    return cudaMemsetAsync(w.seen, 0, (size_t)(reinterpret_cast<char *>(w.seg) - reinterpret_cast<char *>(w.seen)), st);
 }
 
 }  // namespace
 
-// 256x256 and 512x512 px (at smaller sizes G3 decides few pairs); from 2,048
-// clips on, below which the band join takes less than the extra launches
-bool band_mma_covers(const Geo &g, uint32_t n) { return (g.N == 256 || g.N == 512) && n >= 2048; }
+// 256x256 and 512x512 px (at smaller sizes G3 decides few pairs)
+static bool size_covered(const Geo &g) { return g.N == 256 || g.N == 512; }
+
+// the self-join: from 2,048 clips on, below which the band join takes less
+// than the extra launches
+bool band_mma_covers(const Geo &g, uint32_t n) { return size_covered(g) && n >= 2048; }
 
 size_t band_mma_workspace(const Geo &g, uint32_t n) {
     if (!band_mma_covers(g, n)) return 0;
     BandWs w;
-    return band_layout(g, n, nullptr, w);
+    return band_layout(g, n, n, list_room(n, n, true), true, true, nullptr, w);
 }
 
 // Decides the whole band into out / count / local unless *overflow (device)
@@ -634,25 +672,72 @@ size_t band_mma_workspace(const Geo &g, uint32_t n) {
 // sort.  ws: band_mma_workspace bytes, 256-byte aligned.
 cudaError_t launch_band_mma(const pcl_params &prm, const pcl_clipset &cs, const uint32_t *order, const uint32_t *spop,
                             const uint32_t *cum, void *ws, pcl_pair *out, uint64_t cap, unsigned long long *count,
-                            unsigned long long *local, const unsigned int **overflow, int num_sms, int *d_err,
+                            unsigned long long *local, const unsigned int **overflow, int num_sms,
                             unsigned long long wait_ns, cudaStream_t st) {
     const Geo g = make_geo(prm);
+    const uint32_t n = cs.n_clips;
     BandWs w;
-    band_layout(g, cs.n_clips, static_cast<char *>(ws), w);
+    band_layout(g, n, n, list_room(n, n, true), true, true, static_cast<char *>(ws), w);
+    w.row_order = w.col_order = order;
+    w.row_pop = w.col_pop = spop;
     *overflow = w.overflow;
-    cudaError_t e = cudaMemsetAsync(ws, 0, (size_t)(reinterpret_cast<char *>(w.item_off) - static_cast<char *>(ws)), st);
+    const cudaError_t e = clear_counters(w, st);
     if (e != cudaSuccess) return e;
-    const unsigned grid = w.blocks * (kBlock / kFeatureClips);
-    if (g.N == 256) band_feature_kernel<4><<<grid, 256, 0, st>>>(prm, cs, w, order, spop, cum);
-    else band_feature_kernel<1><<<grid, 256, 0, st>>>(prm, cs, w, order, spop, cum);
-    band_items_kernel<<<1, 1024, 0, st>>>(w);
+    features<true, true, true>(prm, g, cs, w, order, spop, n, cum, st);
     if (g.N == 256)
-        e = launch_t<1024, 8>(prm, g, cs, w, order, spop, cum, out, cap, count, local, num_sms, d_err, wait_ns, st);
-    else
-        e = launch_t<1024, 16>(prm, g, cs, w, order, spop, cum, out, cap, count, local, num_sms, d_err, wait_ns, st);
-    if (e != cudaSuccess) return e;
-    band_count_kernel<<<1, 1, 0, st>>>(w, local);
+        return launch_t<1024, 8, false>(prm, g, cs, cs, w, out, cap, count, local, num_sms, wait_ns, st);
+    return launch_t<1024, 16, false>(prm, g, cs, cs, w, out, cap, count, local, num_sms, wait_ns, st);
+}
+
+// ---- two sets: the members' vectors apart (a served library keeps them), 256-byte aligned
+size_t band_lib_bytes(const Geo &g, uint32_t n_lib) {
+    if (!size_covered(g) || n_lib < 2048) return 0;
+    const size_t blocks = (n_lib + kBlock - 1) / kBlock;
+    return up(4 * kBlock * blocks) + blocks * kBlock * (size_t)kbytes_of(g.nb * g.nb);
+}
+static void lib_parts(void *lib, uint32_t n_lib, BandWs &w) {
+    w.cb = static_cast<float *>(lib);
+    w.Q = static_cast<unsigned char *>(lib) + up(4 * kBlock * (size_t)((n_lib + kBlock - 1) / kBlock));
+}
+cudaError_t launch_band_lib(const pcl_params &prm, const pcl_clipset &L, const uint32_t *order, const uint32_t *spop,
+                            void *lib, cudaStream_t st) {
+    const Geo g = make_geo(prm);
+    BandWs w;
+    band_layout(g, 0, L.n_clips, 0, false, false, nullptr, w);
+    lib_parts(lib, L.n_clips, w);
+    features<false, true, false>(prm, g, L, w, order, spop, L.n_clips, nullptr, st);
     return cudaGetLastError();
+}
+
+size_t band_cross_workspace(const Geo &g, uint32_t nq, uint32_t n_lib) {
+    BandWs w;
+    return band_layout(g, nq, n_lib, list_room(nq, n_lib, false), false, false, nullptr, w);
+}
+
+// as launch_band_mma for the queries Q (area order qorder, qspop; bands beg,
+// end in the library's area order) against the library with its vectors lib
+cudaError_t launch_band_cross(const pcl_params &prm, const pcl_clipset &Q, const pcl_clipset &L,
+                              const uint32_t *lib_order, const uint32_t *lib_spop, void *lib, const uint32_t *qorder,
+                              const uint32_t *qspop, uint32_t *beg, uint32_t *end, void *ws, pcl_pair *out,
+                              uint64_t cap, unsigned long long *count, unsigned long long *local,
+                              const unsigned int **overflow, int num_sms, unsigned long long wait_ns, cudaStream_t st) {
+    const Geo g = make_geo(prm);
+    BandWs w;
+    band_layout(g, Q.n_clips, L.n_clips, list_room(Q.n_clips, L.n_clips, false), false, false, static_cast<char *>(ws), w);
+    lib_parts(lib, L.n_clips, w);
+    w.beg = beg;
+    w.end = end;
+    w.row_order = qorder;
+    w.row_pop = qspop;
+    w.col_order = lib_order;
+    w.col_pop = lib_spop;
+    *overflow = w.overflow;
+    const cudaError_t e = clear_counters(w, st);
+    if (e != cudaSuccess) return e;
+    features<true, false, false>(prm, g, Q, w, qorder, qspop, Q.n_clips, nullptr, st);
+    if (g.N == 256)
+        return launch_t<1024, 8, true>(prm, g, Q, L, w, out, cap, count, local, num_sms, wait_ns, st);
+    return launch_t<1024, 16, true>(prm, g, Q, L, w, out, cap, count, local, num_sms, wait_ns, st);
 }
 
 }  // namespace pcl

@@ -13,12 +13,21 @@
 // re-read from L2 by the other queries (a band of a large library is larger
 // than L2, and query-major order re-fetched it from DRAM for every query).
 // Each warp tests G3 and G2 on every member of its item, as in the self-join.
+// At 256x256 and 512x512 px against 2,048 or more library clips G3 is a matrix
+// product (band_mma.cu; a pass of 24 requests of up to 4,096 queries against
+// 32,768 clips: 23.7 -> 1.6 ms of kernel time) and the join of the chunks runs
+// only if that gave up.
 #include "gates.cuh"
 
 namespace pcl {
 
 cudaError_t launch_area_sort(const uint32_t *, uint32_t, uint32_t, uint32_t *, uint32_t *, uint32_t *, uint32_t *,
                              int, cudaStream_t);
+size_t band_cross_workspace(const Geo &, uint32_t, uint32_t);
+cudaError_t launch_band_cross(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const uint32_t *,
+                              const uint32_t *, void *, const uint32_t *, const uint32_t *, uint32_t *, uint32_t *,
+                              void *, pcl_pair *, uint64_t, unsigned long long *, unsigned long long *,
+                              const unsigned int **, int, unsigned long long, cudaStream_t);
 
 namespace {
 
@@ -92,7 +101,8 @@ __global__ void __launch_bounds__(256, LP ? 6 : 0) cross_join_kernel(pcl_params 
                                                          const uint32_t *qlo, const uint32_t *item_off,
                                                          uint32_t n_ch, pcl_pair *out, uint64_t cap,
                                                          unsigned long long *count, unsigned long long *local,
-                                                         unsigned int *next_item) {
+                                                         unsigned int *next_item, const unsigned int *only_if) {
+    if (only_if && !*only_if) return;  // decided already
     const Geo g = make_geo(prm);
     const int lane = threadIdx.x & 31;
     const uint32_t total = item_off[n_ch];
@@ -275,7 +285,8 @@ size_t cross_join_workspace(const Geo &g, uint32_t nq, uint32_t n_lib) {
 cudaError_t launch_cross_join(const pcl_params &prm, const pcl_clipset &Q, const pcl_clipset &L,
                               const uint32_t *lib_order, const uint32_t *lib_spop, const uint32_t *lib_cum,
                               void *ws, size_t ws_bytes, pcl_pair *out, uint64_t cap, unsigned long long *count,
-                              unsigned long long *gates, int num_sms, cudaStream_t st) {
+                              unsigned long long *gates, int num_sms, cudaStream_t st, void *lib_vectors,
+                              unsigned long long wait_ns) {
     const Geo g = make_geo(prm);
     const uint32_t nq = Q.n_clips, n_ch = lib_chunks(L.n_clips);
     if (ws_bytes < cross_join_workspace(g, nq, L.n_clips)) return cudaErrorInvalidValue;
@@ -294,6 +305,15 @@ cudaError_t launch_cross_join(const pcl_params &prm, const pcl_clipset &Q, const
         if (e != cudaSuccess) return e;
         cross_prep_kernel<<<(nq + 255) / 256, 256, 0, st>>>(qspop, nq, lib_cum, (uint32_t)g.N * g.N, prm.cos_num,
                                                              prm.cos_den, beg, endp);
+        // with the library's vectors and workspace G3 is a matrix product, and
+        // the join of the chunks runs only if that gave up
+        const unsigned int *only_if = nullptr;
+        const size_t own = (cross_join_workspace(g, nq, L.n_clips) + 255) & ~(size_t)255;
+        if (lib_vectors && ws_bytes >= own + band_cross_workspace(g, nq, L.n_clips)) {
+            e = launch_band_cross(prm, Q, L, lib_order, lib_spop, lib_vectors, qorder, qspop, beg, endp, w + own, out,
+                                  cap, count, local, &only_if, num_sms, wait_ns, st);
+            if (e != cudaSuccess) return e;
+        }
         cross_chunks_kernel<<<(n_ch + 255) / 256, 256, 0, st>>>(beg, endp, nq, n_ch, qlo, cnt);
         scan_items_kernel<<<1, 1024, 0, st>>>(cnt, n_ch, item_off);
         // the lane-per-member first chunk at 256² only, as in the self-join
@@ -302,18 +322,18 @@ cudaError_t launch_cross_join(const pcl_params &prm, const pcl_clipset &Q, const
             case 1: cross_join_kernel<1><<<num_sms * 8, 256, band_g2_smem(g.N, g.S), st>>>(prm, Q, L, lib_order,
                                                                       lib_spop, qorder, qspop,
                                                                       beg, endp, qlo, item_off, n_ch, out, cap,
-                                                                      count, local, next_item); break;
+                                                                      count, local, next_item, only_if); break;
             case 4:
                 if (lp) cross_join_kernel<4, true><<<num_sms * 6, 256, band_lp_smem(), st>>>(
                     prm, Q, L, lib_order, lib_spop, qorder, qspop, beg, endp, qlo, item_off, n_ch, out, cap, count,
-                    local, next_item);
+                    local, next_item, only_if);
                 else cross_join_kernel<4><<<num_sms * 8, 256, 0, st>>>(prm, Q, L, lib_order, lib_spop, qorder, qspop,
                                                                        beg, endp, qlo, item_off, n_ch, out, cap,
-                                                                       count, local, next_item);
+                                                                       count, local, next_item, only_if);
                 break;
             case 16: cross_join_kernel<16><<<num_sms * 8, 256, 0, st>>>(prm, Q, L, lib_order, lib_spop, qorder,
                                                                         qspop, beg, endp, qlo, item_off, n_ch, out,
-                                                                        cap, count, local, next_item); break;
+                                                                        cap, count, local, next_item, only_if); break;
             default: return cudaErrorInvalidValue;
         }
     }

@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(256, 6) join_screen_kernel(pcl_params prm, pcl
     if (lane == 0 && kept) atomicAdd(w.local, (unsigned long long)kept);
 }
 
-// The listed pairs, 32 per warp at a time: lane q reads the signatures of pair
+// The listed pairs, up to 32 per warp at a time: lane q reads the signatures of pair
 // q and decides E2; the correspondence takes the pairs one by one with the
 // whole warp, as warp_correspond does, the next pair's polygons (the larger
 // clip's, and the first eight of the smaller one) loading while one is tested.
@@ -595,10 +595,11 @@ __global__ void __launch_bounds__(256, 4) edge_pair_check_kernel(pcl_params prm,
     const int4 none = make_int4(0, 0, 0, 0);
     const int tol = prm.edge_tol_dbu, M = prm.marker_dbu;
     unsigned long long kept = 0;
-    for (uint32_t t0 = w0 * 32; t0 < n; t0 += nw * 32) {  // warp-uniform
+    const uint32_t per = min(32u, (n + nw - 1) / nw);  // a short list is spread over all warps
+    for (uint32_t t0 = w0 * per; t0 < n; t0 += nw * per) {  // warp-uniform
         uint2 mine = make_uint2(0u, 0u);
         int offu = 0, nu = 0, offv = 0, nv = 0, tx = 0, ty = 0;
-        bool take = t0 + lane < n;
+        bool take = (uint32_t)lane < per && t0 + lane < n;
         if (take) {
             mine = w.list[t0 + lane];
             const int4 *eu = reinterpret_cast<const int4 *>(cs.esig + (size_t)mine.x * 8);

@@ -36,7 +36,7 @@ bool band_mma_covers(const Geo &, uint32_t);
 size_t band_mma_workspace(const Geo &, uint32_t);
 cudaError_t launch_band_mma(const pcl_params &, const pcl_clipset &, const uint32_t *, const uint32_t *,
                             const uint32_t *, void *, pcl_pair *, uint64_t, unsigned long long *,
-                            unsigned long long *, const unsigned int **, int, int *, unsigned long long, cudaStream_t);
+                            unsigned long long *, const unsigned int **, int, unsigned long long, cudaStream_t);
 
 namespace {
 
@@ -358,7 +358,7 @@ uint64_t shard_pairs(uint64_t n, uint32_t s, uint32_t S) {
 cudaError_t launch_band_join(const pcl_params &prm, const pcl_clipset &cs, void *ws, size_t ws_bytes,
                              pcl_pair *out, uint64_t cap, unsigned long long *count,
                              unsigned long long *gates, int num_sms, cudaStream_t st, uint32_t shard,
-                             uint32_t n_shards, int *d_err, unsigned long long wait_ns) {
+                             uint32_t n_shards, unsigned long long wait_ns) {
     if (n_shards == 0 || shard >= n_shards) return cudaErrorInvalidValue;
     const Geo g = make_geo(prm);
     const uint32_t n = cs.n_clips;
@@ -394,8 +394,8 @@ cudaError_t launch_band_join(const pcl_params &prm, const pcl_clipset &cs, void 
     // product; the band join then runs only if that gave up
     const unsigned int *only_if = nullptr;
     const size_t own = (band_join_workspace(g, n, topo) + 255) & ~(size_t)255;
-    if (!topo && n_shards == 1 && band_mma_covers(g, n) && d_err && ws_bytes >= own + band_mma_workspace(g, n)) {
-        e = launch_band_mma(prm, cs, order, spop, cum, w + own, out, cap, count, local, &only_if, num_sms, d_err,
+    if (!topo && n_shards == 1 && band_mma_covers(g, n) && ws_bytes >= own + band_mma_workspace(g, n)) {
+        e = launch_band_mma(prm, cs, order, spop, cum, w + own, out, cap, count, local, &only_if, num_sms,
                             wait_ns, st);
         if (e != cudaSuccess) return e;
     }

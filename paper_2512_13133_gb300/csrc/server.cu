@@ -56,7 +56,12 @@ cudaError_t launch_edge_match(const pcl_params &, const pcl_clipset &, const pcl
                               const unsigned long long *, pcl_record *, int, cudaStream_t);
 cudaError_t launch_cross_join(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const uint32_t *,
                               const uint32_t *, const uint32_t *, void *, size_t, pcl_pair *, uint64_t,
-                              unsigned long long *, unsigned long long *, int, cudaStream_t);
+                              unsigned long long *, unsigned long long *, int, cudaStream_t, void *,
+                              unsigned long long);
+size_t band_lib_bytes(const Geo &, uint32_t);
+size_t band_cross_workspace(const Geo &, uint32_t, uint32_t);
+cudaError_t launch_band_lib(const pcl_params &, const pcl_clipset &, const uint32_t *, const uint32_t *, void *,
+                            cudaStream_t);
 cudaError_t launch_exact_pairs(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const pcl_pair *,
                                uint64_t, const unsigned long long *, pcl_record *, int, unsigned long long *,
                                cudaStream_t);
@@ -152,6 +157,7 @@ struct ServerClass {
     pcl_clipset lib{};
     int engine = 0;  // kEdge, kFft, kTc or kExact
     uint32_t *lib_cum = nullptr, *lib_fill = nullptr, *lib_order = nullptr, *lib_spop = nullptr;
+    void *lib_vectors = nullptr;  // the density gate's vectors of the library clips (cosine; null: not used)
 };
 
 struct pcl_server {
@@ -171,16 +177,19 @@ constexpr int kEdge = 0, kFft = 1, kTc = 2, kExact = 3;
 
 // workspace of a cosine request: the band join's, then (same stream, after
 // it) the tensor-core engine's grouping buffers in the same bytes
-size_t request_ws(const pcl::Geo &g, int engine, uint32_t nq, uint32_t n_lib, uint64_t cap) {
+// (product: with room for the density gate as a matrix product)
+size_t request_ws(const pcl::Geo &g, int engine, uint32_t nq, uint32_t n_lib, uint64_t cap, bool product) {
     if (engine == kEdge) return 0;
-    const size_t cj = pcl::cross_join_workspace(g, nq, n_lib);
+    size_t cj = pcl::cross_join_workspace(g, nq, n_lib);
+    if (product) cj = align256(cj) + pcl::band_cross_workspace(g, nq, n_lib);
     if (engine == kFft || engine == kExact) return cj;
     const size_t tc = pcl::tc_workspace(cap);
     return cj > tc ? cj : tc;
 }
 
 // device bytes of one request of nq clips and R rectangles with candidate capacity cap
-size_t footprint(const pcl::Geo &g, uint32_t nq, uint64_t R, uint64_t cap, int engine, uint32_t n_lib) {
+size_t footprint(const pcl::Geo &g, uint32_t nq, uint64_t R, uint64_t cap, int engine, uint32_t n_lib,
+                 bool product) {
     size_t b = 0;
     b += align256(4ull * (nq + 1));                 // rect_off
     b += align256(16ull * (R ? R : 1));             // rects
@@ -196,12 +205,12 @@ size_t footprint(const pcl::Geo &g, uint32_t nq, uint64_t R, uint64_t cap, int e
     b += align256(8ull * cap) * 2;                  // cand, pass
     b += align256(40ull * cap);                     // records
     b += align256(64);                              // counts
-    b += align256(request_ws(g, engine, nq, n_lib, cap));     // band join / tensor-core workspace (cosine only)
+    b += align256(request_ws(g, engine, nq, n_lib, cap, product));  // band join / tensor-core workspace (cosine only)
     return b;
 }
 
 void carve(Slot &s, const pcl::Geo &g, char *base, uint32_t nq, uint64_t R, uint64_t cap, int engine,
-           uint32_t n_lib) {
+           uint32_t n_lib, bool product) {
     char *p = base;
     auto take = [&](size_t n) {
         char *r = p;
@@ -224,7 +233,7 @@ void carve(Slot &s, const pcl::Geo &g, char *base, uint32_t nq, uint64_t R, uint
     s.pass = reinterpret_cast<pcl_pair *>(take(8ull * cap));
     s.rec = reinterpret_cast<pcl_record *>(take(40ull * cap));
     s.counts = reinterpret_cast<unsigned long long *>(take(64));
-    s.ws_bytes = request_ws(g, engine, nq, n_lib, cap);
+    s.ws_bytes = request_ws(g, engine, nq, n_lib, cap, product);
     s.ws = s.ws_bytes ? take(s.ws_bytes) : nullptr;
 }
 
@@ -326,6 +335,16 @@ pcl_status pcl_server_create_classes(pcl_ctx *ctx, const pcl_params *params, con
         if (e == cudaSuccess)
             e = pcl::launch_area_sort(k.lib.pop, nl, V, k.lib_cum, k.lib_fill, k.lib_order, k.lib_spop,
                                       ctx->num_sms, 0);
+        // the library's side of the density gate as a matrix product, where it fits
+        const size_t vec = pcl::band_lib_bytes(k.g, nl);
+        if (e == cudaSuccess && vec) {
+            if (cudaMalloc(&k.lib_vectors, vec) == cudaSuccess) {
+                e = pcl::launch_band_lib(k.P, k.lib, k.lib_order, k.lib_spop, k.lib_vectors, 0);
+            } else {
+                cudaGetLastError();
+                k.lib_vectors = nullptr;
+            }
+        }
         if (e != cudaSuccess) break;
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -373,9 +392,16 @@ pcl_status pcl_server_submit_class(pcl_server *s, uint32_t cls, const uint32_t *
         }
     if (!sl) return fail(ctx, PCL_ERR_BUSY, "pcl_server_submit: no free slot");
     const uint64_t cap = (uint64_t)s->cfg.cand_per_query * n_clips + 64;
-    const size_t bytes = footprint(k.g, n_clips, R, cap, k.engine, k.lib.n_clips);
+    bool product = k.lib_vectors != nullptr;
+    size_t bytes = footprint(k.g, n_clips, R, cap, k.engine, k.lib.n_clips, product);
     size_t off = 0;
-    if (!s->arena.alloc(bytes, &off)) return fail(ctx, PCL_ERR_BUSY, "pcl_server_submit: memory budget full");
+    bool room = s->arena.alloc(bytes, &off);
+    if (!room && product) {  // the request runs without the matrix product's buffers as well
+        product = false;
+        bytes = footprint(k.g, n_clips, R, cap, k.engine, k.lib.n_clips, product);
+        room = s->arena.alloc(bytes, &off);
+    }
+    if (!room) return fail(ctx, PCL_ERR_BUSY, "pcl_server_submit: memory budget full");
     cudaError_t e = cudaSetDevice(ctx->device);
     sl->busy = true;
     sl->done = false;
@@ -389,7 +415,7 @@ pcl_status pcl_server_submit_class(pcl_server *s, uint32_t cls, const uint32_t *
     sl->rec_overflow.clear();
     sl->t_done = 0;
     sl->t_submit = now_ns();
-    carve(*sl, k.g, s->arena.base + off, n_clips, R, cap, k.engine, k.lib.n_clips);
+    carve(*sl, k.g, s->arena.base + off, n_clips, R, cap, k.engine, k.lib.n_clips, product);
     std::memcpy(sl->h_off, h_rect_off, 4ull * (n_clips + 1));
     const uint32_t base = h_rect_off[0];
     if (R) std::memcpy(sl->h_rects, h_rects + 4ull * base, 16ull * R);
@@ -414,7 +440,8 @@ pcl_status pcl_server_submit_class(pcl_server *s, uint32_t cls, const uint32_t *
     } else {
         if (e == cudaSuccess)
             e = pcl::launch_cross_join(k.P, sl->q, k.lib, k.lib_order, k.lib_spop, k.lib_cum, sl->ws, sl->ws_bytes,
-                                       sl->cand, cap, sl->counts + 0, nullptr, ctx->num_sms, st);
+                                       sl->cand, cap, sl->counts + 0, nullptr, ctx->num_sms, st,
+                                       product ? k.lib_vectors : nullptr, ctx->wait_ns);
         if (k.engine == kTc) {
             // candidates grouped by query clip through the direct correlation;
             // a bounded wait that runs out sets the request's own error word
@@ -549,6 +576,7 @@ void pcl_server_destroy(pcl_server *s) {
         cudaFree(k.lib_fill);
         cudaFree(k.lib_order);
         cudaFree(k.lib_spop);
+        cudaFree(k.lib_vectors);
     }
     cudaFree(s->arena_mem);
     delete s;

@@ -63,3 +63,38 @@ def test_overflow_takes_the_band_join(ctx):
     clips = [one if k % 10 else wl.clip(k).tolist() for k in range(n)]
     kept, _ = _check(ctx, synth.from_lists(clips, 1024, 4, 64), 95)
     assert kept > 2_000_000  # far more than the 65,536 listed pairs
+
+
+@pytest.mark.parametrize("nq,nl,px,num", [(1, 2048, 256, 95), (129, 2300, 256, 80), (700, 5000, 256, 90),
+                                          (300, 2100, 512, 80)])
+def test_two_sets_equal_pairs_of_the_union(ctx, nq, nl, px, num):
+    """queries x library through the product equal the cross pairs of the union's shards"""
+    import paper_2512_13133_gb300 as pcl
+    W, n = 4 * px, nq + nl
+    wl = synth.generate(n + num, n_clips=n, n_seeds=n // 20, n_copies=int(0.7 * n), window_dbu=W, margin_dbu=W // 16,
+                        min_rects=2, max_rects=30, edge_jitter=4, shift_max=W // 32)
+    clips = [[] if k % 301 == 0 else wl.clip(k).tolist() for k in range(n)]
+    wl = synth.from_lists(clips, W, 4, W // 16)
+    P = pcl.params(W, 4, W // 16, cos_num=num)
+    cs = pcl.alloc_clipset(P, wl.rect_off, wl.rects, with_spec=False)
+    pcl.pcl_rasterize(ctx, P, cs)
+    got, gates = pcl.candidates(ctx, P, pcl.MODE_COSINE, cs.view(P, 0, nq), b=cs.view(P, nq, n))
+    got = got.cpu().numpy().astype(np.int64)
+    want = np.concatenate([pcl.candidates(ctx, P, pcl.MODE_COSINE, cs, shard=s, n_shards=2)[0].cpu().numpy()
+                           for s in range(2)]).astype(np.int64)
+    want = want[(want[:, 0] < nq) & (want[:, 1] >= nq)]
+    np.testing.assert_array_equal(np.sort(got[:, 0] * n + got[:, 1] + nq), np.sort(want[:, 0] * n + want[:, 1]))
+    assert gates.sum() == nq * nl and gates[0] == len(got)
+
+
+def test_wait_limit_takes_the_band_join(ctx):
+    """a wait that runs out gives the product up; the result stays exact and no error is left"""
+    import paper_2512_13133_gb300 as pcl
+    wl = synth.generate(9, n_clips=3000, n_seeds=150, n_copies=2100, window_dbu=1024, margin_dbu=64, min_rects=3,
+                        max_rects=20, edge_jitter=2)
+    pcl.pcl_set_wait_limit(ctx, 1)
+    try:
+        _check(ctx, wl, 90)
+    finally:
+        pcl.pcl_set_wait_limit(ctx, 0)
+    _check(ctx, wl, 90)
