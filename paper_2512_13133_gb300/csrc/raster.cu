@@ -1,28 +1,13 @@
 // a1: rasterisation of Manhattan clips and the per-clip signatures read by the
 // lossless gates (Sec. 2.2.1 step 1; signatures for the pre-screening of
 // Sec. 3.1 stage 1).
-//
-// One CTA per clip, one thread per raster row (blockDim = N <= 512).  The
-// clip's rectangles are staged in shared memory in chunks; each thread ORs
-// the pixel-centre runs of the rectangles that cover its row centre into its
-// row words (registers), then the CTA derives the popcount, row/column
-// profiles and the 16x16 block counts from the row words in shared memory.
+#include <climits>
+
 #include "common.cuh"
 
 namespace pcl {
 
 namespace {
-
-constexpr int kRectChunk = 256;
-
-// Storage position of 16x16 block (by, bx) among the nb x nb blocks (nb a
-// multiple of 4): blocks are grouped by (by mod 4, bx mod 4), groups in
-// row-major order of that pair, blocks within a group row-major; at nb = 16
-// the first 64 positions are the block rows 0, 4, 8 and 12.
-__device__ __forceinline__ int blk_pos(int by, int bx, int nb) {
-    const int q = nb >> 2;
-    return (((by & 3) << 2) | (bx & 3)) * q * q + (by >> 2) * q + (bx >> 2);
-}
 
 // grid cell of coordinate v (floor division, clamped to the 64 cells)
 __device__ __forceinline__ int cell_of(int v, int csz) {
@@ -39,140 +24,160 @@ __device__ __forceinline__ int pix_from(int v, long long p, int N) {
     return (int)(q < 0 ? 0 : (q > N ? N : q));
 }
 
-// 32 x 32 bit transpose across a warp: on entry lane l holds row l (bit b =
-// column b), on return lane l holds column l (bit b = row b).  Five rounds of
-// exchanging the off-diagonal halves of 2s x 2s blocks with lane l ^ s.
-__device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, int lane) {
-#pragma unroll
-    for (int s = 16; s >= 1; s >>= 1) {
-        const uint32_t m = s == 16 ? 0x0000FFFFu : s == 8 ? 0x00FF00FFu : s == 4 ? 0x0F0F0F0Fu
-                         : s == 2 ? 0x33333333u : 0x55555555u;  // bit positions b with (b & s) == 0
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
-        x = (lane & s) ? ((x & ~m) | ((y & ~m) >> s)) : ((x & m) | ((y & m) << s));
-    }
-    return x;
+// log2 of v when it is a power of two, else -1
+__device__ __forceinline__ int log2_exact(int v) { return (v & (v - 1)) == 0 ? 31 - __clz(v) : -1; }
+
+// pix_from with psh >= 0: the pitch is 1 << psh
+__device__ __forceinline__ int pix_at(int v, int p, int psh, int N) {
+    if (psh < 0) return pix_from(v, p, N);
+    const long long q = (2LL * v + p - 1) >> (psh + 1);  // ceil((2 v - p) / (2 p))
+    return (int)(q < 0 ? 0 : (q > N ? N : q));
+}
+// cell_of with csh >= 0: the cell side is 1 << csh
+__device__ __forceinline__ int cell_at(int v, int csz, int csh) {
+    return csh >= 0 ? min(max(v >> csh, 0), 63) : cell_of(v, csz);
 }
 
 template <int NW>
-__global__ void __launch_bounds__(512) raster_kernel(pcl_params prm, pcl_clipset cs) {
-    constexpr int NR = 64 * NW;  // rows (N = 64 NW: 64^2 .. 512^2)
+struct RasterCta {
+    static constexpr int threads = NW == 8 ? 256 : 128;
+    static constexpr int chunk = 128;  // rectangles staged at a time
+    static constexpr int ctas = NW == 8 ? 4 : 12;  // resident per SM: registers and shared memory allow as many
+};
+
+// One CTA per clip.  The rectangles (a chunk at a time) become pixel
+// ranges in shared memory; then each warp has one job with a lane per
+// rectangle: setting the rows' bits, adding the pixels of its 16x16 blocks and
+// the ends of its column run to a difference array, marking the occupancy
+// grid, ordering by area and the edge signature.  If the pixels of all ranges
+// add up to the raster's ones, no two rectangles share a pixel and those sums
+// are the block counts and (after a prefix sum) the column counts; otherwise
+// both are counted from the rows.  Bound by issue slots and the latency of each
+// warp's job; the output is written once, 16 bytes a thread.  100,000 clips of
+// 256x256 px: 413 us (2.7 TB/s) against 1,265 us with a thread per row testing
+// every rectangle and column counts by bit transposes; 12 CTAs per SM (40
+// registers) against 10: 413 and 446 us.
+template <int NW>
+__global__ void __launch_bounds__(RasterCta<NW>::threads, RasterCta<NW>::ctas) raster_kernel(pcl_params prm, pcl_clipset cs) {
+    constexpr int N = 64 * NW, W32 = 2 * NW, NB = 4 * NW, NB2 = NB * NB;
+    constexpr int T = RasterCta<NW>::threads, CHUNK = RasterCta<NW>::chunk;
+    constexpr int SR = W32 + 1;  // row stride in shared memory (odd: the lanes of a rectangle's rows spread over the banks)
+    constexpr int FILL = T / 32 - 3;  // warps setting bits
     const Geo g = make_geo(prm);
-    const int c = blockIdx.x;
-    const int j = threadIdx.x;  // row (y index)
-    const int N = g.N;
-    __shared__ int4 rs[kRectChunk];          // pixel ranges {i0, i1, j0, j1} of staged rectangles
-    __shared__ uint64_t rows[NR * NW];
-    __shared__ uint8_t colpart[NR / 32][NR];  // column counts over each warp's 32 rows
-    __shared__ uint32_t red[32];
-
-    const uint32_t r0 = cs.rect_off[c], r1 = cs.rect_off[c + 1];
-    const long long p = g.p;
-    uint64_t w[NW];
-#pragma unroll
-    for (int k = 0; k < NW; ++k) w[k] = 0ull;
-
-    for (uint32_t base = r0; base < r1; base += kRectChunk) {
-        const uint32_t cnt = min((uint32_t)kRectChunk, r1 - base);
+    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ int4 rs[CHUNK];          // pixel ranges {i0, i1, j0, j1} of staged rectangles
+    __shared__ int4 rq[CHUNK];          // the rectangles
+    __shared__ long long areas[CHUNK];       // of the staged rectangles
+    // zeroed together: the rows, ones entering (leaving) at each column, block
+    // counts, and the occupancy grid's 64 rows (low and high word)
+    constexpr int Z = (N * SR + (N + 4) + NB2 + 128 + 3) / 4;
+    __shared__ uint4 zeroed[Z];
+    uint32_t *rows = reinterpret_cast<uint32_t *>(zeroed);
+    int *diff = reinterpret_cast<int *>(rows + N * SR);
+    uint32_t *cnt_s = rows + N * SR + N + 4, *occ_s = cnt_s + NB2;
+    __shared__ uint32_t red[T / 32];
+    __shared__ unsigned long long area_sum;  // pixels of all ranges
+    const uint32_t r0 = cs.rect_off[c], r1 = cs.rect_off[c + 1], nr = r1 - r0;
+    const int4 *r4 = reinterpret_cast<const int4 *>(cs.rects) + r0;
+    const int psh = log2_exact(g.p), csz = g.W / 64, csh = log2_exact(csz);
+    for (int t = tid; t < Z; t += T) zeroed[t] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) area_sum = 0ull;
+    // edge signature (warp 0): bbox over edges that are not on the window border
+    int hasx = 0, hasy = 0, border = 0;
+    int lox = INT_MAX, hix = INT_MIN, loy = INT_MAX, hiy = INT_MIN;
+    for (uint32_t base = 0; base < nr; base += CHUNK) {
+        const uint32_t cnt = min((uint32_t)CHUNK, nr - base);
         __syncthreads();
         // pixel (i, j) is set when x0 <= p i + p/2 < x1 and y0 <= p j + p/2 < y1
         // (doubled: 2 x0 <= 2 p i + p < 2 x1): columns [i0, i1), rows [j0, j1)
-        for (uint32_t t = threadIdx.x; t < cnt; t += blockDim.x) {
-            const int4 q = reinterpret_cast<const int4 *>(cs.rects)[base + t];
-            rs[t] = make_int4(pix_from(q.x, p, N), pix_from(q.z, p, N), pix_from(q.y, p, N), pix_from(q.w, p, N));
+        for (uint32_t t = tid; t < cnt; t += T) {
+            const int4 q = __ldg(r4 + base + t);
+            rq[t] = q;
+            areas[t] = (long long)(q.z - q.x) * (long long)(q.w - q.y);
+            rs[t] = make_int4(pix_at(q.x, g.p, psh, N), pix_at(q.z, g.p, psh, N), pix_at(q.y, g.p, psh, N),
+                              pix_at(q.w, g.p, psh, N));
         }
         __syncthreads();
-        if (j < N) {
-            for (uint32_t t = 0; t < cnt; ++t) {
+        if (warp >= 3) {
+            // bits: lane = rectangle; the warps share its rows
+            for (uint32_t t = lane; t < cnt; t += 32) {
                 const int4 q = rs[t];
-                if (!(q.z <= j && j < q.w)) continue;
-                const int i0 = q.x, i1 = q.y;
-#pragma unroll
-                for (int k = 0; k < NW; ++k) {
-                    const int lo = max(i0, 64 * k), hi = min(i1, 64 * k + 64);
-                    if (lo < hi) {
-                        const int len = hi - lo;
-                        const uint64_t m = (len == 64) ? ~0ull : (((1ull << len) - 1ull) << (lo - 64 * k));
-                        w[k] |= m;
+                if (q.x >= q.y) continue;
+                const int w0 = q.x >> 5, w1 = (q.y - 1) >> 5;
+                const uint32_t first = 0xffffffffu << (q.x & 31), last = 0xffffffffu >> (31 - ((q.y - 1) & 31));
+                for (int j = q.z + (warp - 3); j < q.w; j += FILL) {
+                    uint32_t *row = rows + j * SR;
+                    if (w0 == w1) {
+                        atomicOr(row + w0, first & last);
+                    } else {
+                        atomicOr(row + w0, first);
+                        for (int w = w0 + 1; w < w1; ++w) atomicOr(row + w, 0xffffffffu);
+                        atomicOr(row + w1, last);
                     }
                 }
             }
-        }
-    }
-    uint32_t rowpop = 0;
-    if (j < N) {
-        uint64_t *dst = cs.bits + ((size_t)c * N + j) * NW;
-#pragma unroll
-        for (int k = 0; k < NW; ++k) {
-            dst[k] = w[k];
-            rows[j * NW + k] = w[k];
-            rowpop += (uint32_t)__popcll(w[k]);
-        }
-        cs.prof[(size_t)c * 2 * N + j] = (uint16_t)rowpop;
-    }
-    // total popcount
-    uint32_t tot = __reduce_add_sync(0xffffffffu, rowpop);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = tot;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t s = 0;
-        for (int k = 0; k < (int)(blockDim.x + 31) / 32; ++k) s += red[k];
-        cs.pop[c] = s;
-    }
-    // column counts: each warp transposes its 32 rows in 32-column chunks
-    // (lane l then holds column l of the chunk) and counts them; the warps'
-    // partial counts are summed per column (blockDim = N, a multiple of 32)
-    {
-        const int lane = threadIdx.x & 31, wr = threadIdx.x >> 5;
-#pragma unroll
-        for (int h = 0; h < 2 * NW; ++h) {
-            const uint32_t x = (h & 1) ? (uint32_t)(w[h >> 1] >> 32) : (uint32_t)w[h >> 1];
-            colpart[wr][32 * h + lane] = (uint8_t)__popc(warp_transpose32(x, lane));
-        }
-    }
-    __syncthreads();
-    if (j < N) {
-        uint32_t q = 0;
-        for (int wr = 0; wr < N / 32; ++wr) q += colpart[wr][j];
-        cs.prof[(size_t)c * 2 * N + N + j] = (uint16_t)q;
-    }
-    // 16x16 block counts, then neighbourhood sums, each stored in the order of
-    // blk_pos: blocks spread over the whole clip come first, so the gates'
-    // chunked density bound sees every part of the clip in its first chunk
-    const int nb = g.nb, nb2 = nb * nb;
-    uint16_t *blk = cs.blk + (size_t)c * 2 * nb2;
-    __shared__ uint16_t cnt_s[32 * 32];
-    for (int t = threadIdx.x; t < nb2; t += blockDim.x) {
-        const int by = t / nb, bx = t % nb;
-        const int k = bx >> 2, sh = (bx & 3) * 16;
-        uint32_t s = 0;
-        for (int jj = 0; jj < 16; ++jj) s += (uint32_t)__popcll((rows[(by * 16 + jj) * NW + k] >> sh) & 0xffffull);
-        cnt_s[t] = (uint16_t)s;
-        blk[blk_pos(by, bx, nb)] = (uint16_t)s;
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nb2; t += blockDim.x) {
-        const int by = t / nb, bx = t % nb;
-        uint32_t s = 0;
-        for (int oy = -g.rb; oy <= g.rb; ++oy)
-            for (int ox = -g.rb; ox <= g.rb; ++ox) {
-                const int yy = by + oy, xx = bx + ox;
-                if (yy >= 0 && yy < nb && xx >= 0 && xx < nb) s += cnt_s[yy * nb + xx];
+        } else if (warp == 2) {
+            // block counts and column differences
+            unsigned long long area = 0;
+            for (uint32_t t = lane; t < cnt; t += 32) {
+                const int4 q = rs[t];
+                const int h = q.w - q.z;
+                if (q.x >= q.y || h <= 0) continue;
+                area += (unsigned long long)(q.y - q.x) * (unsigned)h;
+                atomicAdd(diff + q.x, h);
+                atomicAdd(diff + q.y, -h);
+                for (int by = q.z >> 4; by <= (q.w - 1) >> 4; ++by) {
+                    const int hh = min(q.w, 16 * by + 16) - max(q.z, 16 * by);
+                    for (int bx = q.x >> 4; bx <= (q.y - 1) >> 4; ++bx)
+                        atomicAdd(cnt_s + by * NB + bx, (uint32_t)(hh * (min(q.y, 16 * bx + 16) - max(q.x, 16 * bx))));
+                }
             }
-        blk[nb2 + blk_pos(by, bx, nb)] = (uint16_t)min(s, 65535u);
-    }
-    // edge signature (warp 0): bbox over edges that are not on the window border
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        const int W = g.W;
-        int hasx = 0, hasy = 0, border = 0;
-        int lox = INT_MAX, hix = INT_MIN, loy = INT_MAX, hiy = INT_MIN;
-        for (uint32_t t = r0 + lane; t < r1; t += 32) {
-            const int4 q = reinterpret_cast<const int4 *>(cs.rects)[t];
-            if (q.x != 0) { hasx = 1; lox = min(lox, q.x); hix = max(hix, q.x); } else border = 1;
-            if (q.z != W) { hasx = 1; lox = min(lox, q.z); hix = max(hix, q.z); } else border = 1;
-            if (q.y != 0) { hasy = 1; loy = min(loy, q.y); hiy = max(hiy, q.y); } else border = 1;
-            if (q.w != W) { hasy = 1; loy = min(loy, q.w); hiy = max(hiy, q.w); } else border = 1;
+            for (int o = 16; o; o >>= 1) area += __shfl_xor_sync(0xffffffffu, area, o);
+            if (lane == 0) area_sum += area;
+        } else if (warp == 1) {
+            // 64 x 64 occupancy grid (cell side W/64): a cell is marked when it holds an
+            // integer point of some rectangle's interior, so two rectangles that
+            // overlap with positive area always share a marked cell
+            for (uint32_t t = lane; t < cnt; t += 32) {
+                const int4 q = rq[t];
+                if (q.z <= q.x || q.w <= q.y) continue;
+                const int y0 = cell_at(q.y, csz, csh), y1 = cell_at(q.w - 1, csz, csh);
+                const int x0 = cell_at(q.x, csz, csh), x1 = cell_at(q.z - 1, csz, csh);
+                const unsigned long long m = (~0ull >> (63 - (x1 - x0))) << x0;
+                const uint32_t lo = (uint32_t)m, hi = (uint32_t)(m >> 32);
+                for (int cy = y0; cy <= y1; ++cy) {
+                    if (lo) atomicOr(occ_s + 2 * cy, lo);
+                    if (hi) atomicOr(occ_s + 2 * cy + 1, hi);
+                }
+            }
+        } else {
+            const int W = g.W;
+            for (uint32_t t = lane; t < cnt; t += 32) {
+                const int4 q = rq[t];
+                if (q.x != 0) { hasx = 1; lox = min(lox, q.x); hix = max(hix, q.x); } else border = 1;
+                if (q.z != W) { hasx = 1; lox = min(lox, q.z); hix = max(hix, q.z); } else border = 1;
+                if (q.y != 0) { hasy = 1; loy = min(loy, q.y); hiy = max(hiy, q.y); } else border = 1;
+                if (q.w != W) { hasy = 1; loy = min(loy, q.w); hiy = max(hiy, q.w); } else border = 1;
+            }
+            // rectangles by ascending area (ties by index): rank by counting
+            for (uint32_t t = lane; t < cnt; t += 32) {
+                const long long at = areas[t];  // before t: smaller areas, and equal ones of smaller index
+                uint32_t rank = 0;
+                if (nr <= CHUNK) {
+#pragma unroll 4
+                    for (uint32_t m = 0; m < nr; ++m) rank += areas[m] < at + (m < t ? 1 : 0) ? 1u : 0u;
+                } else {
+                    for (uint32_t m = 0; m < nr; ++m) {
+                        const int4 u = __ldg(r4 + m);
+                        const long long am = (long long)(u.z - u.x) * (long long)(u.w - u.y);
+                        rank += am < at + (m < base + t ? 1 : 0) ? 1u : 0u;
+                    }
+                }
+                cs.rorder[r0 + rank] = (uint16_t)(base + t);
+            }
         }
+    }
+    if (warp == 0) {
         hasx = __reduce_or_sync(0xffffffffu, hasx);
         hasy = __reduce_or_sync(0xffffffffu, hasy);
         border = __reduce_or_sync(0xffffffffu, border);
@@ -181,50 +186,115 @@ __global__ void __launch_bounds__(512) raster_kernel(pcl_params prm, pcl_clipset
         loy = __reduce_min_sync(0xffffffffu, loy);
         hiy = __reduce_max_sync(0xffffffffu, hiy);
         if (lane == 0) {
-            int32_t *e = cs.esig + (size_t)c * 8;
-            e[ES_N] = (int32_t)(r1 - r0);
-            e[ES_HASX] = hasx;
-            e[ES_LOX] = hasx ? lox : 0;
-            e[ES_HIX] = hasx ? hix : 0;
-            e[ES_HASY] = hasy;
-            e[ES_LOY] = hasy ? loy : 0;
-            e[ES_HIY] = hasy ? hiy : 0;
-            e[ES_BORDER] = border;
+            int4 *e = reinterpret_cast<int4 *>(cs.esig + (size_t)c * 8);
+            e[0] = make_int4((int)nr, hasx, hasx ? lox : 0, hasx ? hix : 0);  // ES_N, ES_HASX, ES_LOX, ES_HIX
+            e[1] = make_int4(hasy, hasy ? loy : 0, hasy ? hiy : 0, border);   // ES_HASY, ES_LOY, ES_HIY, ES_BORDER
+            if (cs.spec_state) cs.spec_state[c] = 0;
         }
     }
-    // 64 x 64 occupancy grid (cell side W/64): a cell is marked when it holds an
-    // integer point of some rectangle's interior, so two rectangles that
-    // overlap with positive area always share a marked cell
-    // (one thread per rectangle ORs its cells into the grid rows it spans)
-    const int csz = g.W / 64;
-    const int4 *r4 = reinterpret_cast<const int4 *>(cs.rects);
-    __shared__ unsigned long long occ_s[64];
-    for (int cy = threadIdx.x; cy < 64; cy += blockDim.x) occ_s[cy] = 0ull;
     __syncthreads();
-    for (uint32_t t = r0 + threadIdx.x; t < r1; t += blockDim.x) {
-        const int4 q = r4[t];
-        if (q.z <= q.x || q.w <= q.y) continue;
-        const int y0 = cell_of(q.y, csz), y1 = cell_of(q.w - 1, csz);
-        const int x0 = cell_of(q.x, csz), x1 = cell_of(q.z - 1, csz);
-        const unsigned long long m = (~0ull >> (63 - (x1 - x0))) << x0;
-        for (int cy = y0; cy <= y1; ++cy) atomicOr(&occ_s[cy], m);
+    // rows out (16 bytes a thread), row counts and the total
+    uint32_t tot = 0;
+    for (int j = tid; j < N; j += T) {
+        uint32_t n = 0;
+#pragma unroll
+        for (int w = 0; w < W32; ++w) n += (uint32_t)__popc(rows[j * SR + w]);
+        cs.prof[(size_t)c * 2 * N + j] = (uint16_t)n;
+        tot += n;
     }
-    __syncthreads();
-    for (int cy = threadIdx.x; cy < 64; cy += blockDim.x) cs.occ[(size_t)c * 64 + cy] = occ_s[cy];
-    // rectangles by ascending area (ties by index): rank by counting
-    const uint32_t nr = r1 - r0;
-    for (uint32_t t = threadIdx.x; t < nr; t += blockDim.x) {
-        const int4 q = r4[r0 + t];
-        const long long at = (long long)(q.z - q.x) * (long long)(q.w - q.y);
-        uint32_t rank = 0;
-        for (uint32_t m = 0; m < nr; ++m) {
-            const int4 u = r4[r0 + m];
-            const long long am = (long long)(u.z - u.x) * (long long)(u.w - u.y);
-            rank += (am < at || (am == at && m < t)) ? 1u : 0u;
+    tot = __reduce_add_sync(0xffffffffu, tot);
+    if (lane == 0) red[warp] = tot;
+    if constexpr (NW >= 2) {
+        uint4 *dst = reinterpret_cast<uint4 *>(cs.bits + (size_t)c * N * NW);
+        for (int t = tid; t < N * W32 / 4; t += T) {
+            const uint32_t *w = rows + (t / (W32 / 4)) * SR + 4 * (t % (W32 / 4));
+            dst[t] = make_uint4(w[0], w[1], w[2], w[3]);
         }
-        cs.rorder[r0 + rank] = (uint16_t)t;
+    } else {
+        uint2 *dst = reinterpret_cast<uint2 *>(cs.bits + (size_t)c * N * NW);
+        for (int t = tid; t < N; t += T) dst[t] = make_uint2(rows[t * SR], rows[t * SR + 1]);
     }
-    if (threadIdx.x == 0 && cs.spec_state) cs.spec_state[c] = 0;
+    for (int t = tid; t < 64; t += T)
+        cs.occ[(size_t)c * 64 + t] = (uint64_t)occ_s[2 * t] | ((uint64_t)occ_s[2 * t + 1] << 32);
+    __syncthreads();
+    tot = 0;
+#pragma unroll
+    for (int k = 0; k < T / 32; ++k) tot += red[k];
+    if (tid == 0) cs.pop[c] = tot;
+    uint16_t *cols = cs.prof + (size_t)c * 2 * N + N;
+    if (tot == area_sum) {
+        // no shared pixel: column counts by a prefix sum (lane l: N / 32 columns)
+        if (warp == 0) {
+            constexpr int K = N / 32;
+            int v[K], s = 0;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                s += diff[K * lane + k];
+                v[k] = s;
+            }
+            int x = s;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            x -= s;
+            __syncwarp();  // all differences are read: the counts take their place
+#pragma unroll
+            for (int k = 0; k < K; ++k) reinterpret_cast<uint16_t *>(diff)[K * lane + k] = (uint16_t)(x + v[k]);
+            __syncwarp();
+            for (int t = lane; t < N; t += 32) cols[t] = reinterpret_cast<const uint16_t *>(diff)[t];
+        }
+    } else {
+        // counted from the rows: each column's ones, each block's
+        for (int i = tid; i < N; i += T) {
+            uint32_t n = 0;
+            for (int j = 0; j < N; ++j) n += (rows[j * SR + (i >> 5)] >> (i & 31)) & 1u;
+            cols[i] = (uint16_t)n;
+        }
+        for (int t = tid; t < NB2; t += T) {
+            const int by = t / NB, bx = t % NB;
+            uint32_t n = 0;
+            for (int j = 0; j < 16; ++j)
+                n += (uint32_t)__popc((rows[(16 * by + j) * SR + (bx >> 1)] >> (16 * (bx & 1))) & 0xffffu);
+            cnt_s[t] = n;
+        }
+        __syncthreads();
+    }
+    // 16x16 block counts, then neighbourhood sums, each stored in the order of
+    // blk_pos: blocks spread over the whole clip come first, so the gates'
+    // chunked density bound sees every part of the clip in its first chunk;
+    // the sums by rows, then by columns (nbh: over the rows [by - rb, by + rb])
+    uint32_t *nbh = rows;  // the rows are written
+    static_assert(N * SR >= NB2, "room for the row sums");
+    __syncthreads();
+    const int rb = g.rb;
+    for (int t = tid; t < NB2; t += T) {
+        const int by = t / NB;
+        uint32_t s = cnt_s[t];
+        if (rb == 1) {
+            s += (by > 0 ? cnt_s[t - NB] : 0u) + (by < NB - 1 ? cnt_s[t + NB] : 0u);
+        } else {
+            for (int d = 1; d <= rb; ++d)
+                s += (by >= d ? cnt_s[t - d * NB] : 0u) + (by + d < NB ? cnt_s[t + d * NB] : 0u);
+        }
+        nbh[t] = s;
+    }
+    __syncthreads();
+    uint16_t *blk = cs.blk + (size_t)c * 2 * NB2;
+    constexpr int Q = NB / 4, QQ = Q * Q;
+    for (int t = tid; t < NB2; t += T) {  // t: position of a block in the stored order
+        const int grp = t / QQ, by = ((t % QQ) / Q) * 4 + (grp >> 2), bx = (t % Q) * 4 + (grp & 3);
+        const uint32_t *at = nbh + by * NB + bx;
+        uint32_t s = at[0];
+        if (rb == 1) {
+            s += (bx > 0 ? at[-1] : 0u) + (bx < NB - 1 ? at[1] : 0u);
+        } else {
+            for (int d = 1; d <= rb; ++d) s += (bx >= d ? at[-d] : 0u) + (bx + d < NB ? at[d] : 0u);
+        }
+        blk[t] = (uint16_t)cnt_s[by * NB + bx];
+        blk[NB2 + t] = (uint16_t)min(s, 65535u);
+    }
 }
 
 }  // namespace
@@ -232,12 +302,12 @@ __global__ void __launch_bounds__(512) raster_kernel(pcl_params prm, pcl_clipset
 cudaError_t launch_raster(const pcl_params &prm, const pcl_clipset &cs, cudaStream_t st) {
     const Geo g = make_geo(prm);
     if (cs.n_clips == 0) return cudaSuccess;
-    dim3 grid(cs.n_clips), block(g.N);
+    const unsigned grid = cs.n_clips;
     switch (g.nw) {
-        case 1: raster_kernel<1><<<grid, block, 0, st>>>(prm, cs); break;
-        case 2: raster_kernel<2><<<grid, block, 0, st>>>(prm, cs); break;
-        case 4: raster_kernel<4><<<grid, block, 0, st>>>(prm, cs); break;
-        case 8: raster_kernel<8><<<grid, block, 0, st>>>(prm, cs); break;
+        case 1: raster_kernel<1><<<grid, RasterCta<1>::threads, 0, st>>>(prm, cs); break;
+        case 2: raster_kernel<2><<<grid, RasterCta<2>::threads, 0, st>>>(prm, cs); break;
+        case 4: raster_kernel<4><<<grid, RasterCta<4>::threads, 0, st>>>(prm, cs); break;
+        case 8: raster_kernel<8><<<grid, RasterCta<8>::threads, 0, st>>>(prm, cs); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
