@@ -16,12 +16,63 @@ __device__ __forceinline__ int vslot(int item, int r, int k) {
     return (item * 9 + r) * (P + 1) + k;
 }
 
-__device__ __forceinline__ void build_twiddles(float2 *tw, int L, int sign) {
-    for (int k = threadIdx.x; k < L; k += blockDim.x) {
-        double s, c;
-        sincospi(2.0 * (double)k / (double)L, &s, &c);
-        tw[k] = make_float2((float)c, (float)(sign * s));
+// exp(2 pi i k / L) for the three FFT sides, k = 0 .. L - 1, rounded from double
+// (the values (float)cospi(2k/L), (float)sinpi(2k/L); computing them with double
+// sincospi in every CTA took a tenth of a spectrum's time and more of a pair's,
+// FP64 being slow on this part)
+struct Twiddle {
+    float c, s;
+};
+// cos and sin of 2 pi k / L from the Taylor series on [0, pi/4]
+constexpr Twiddle twiddle_of(int k, int L) {
+    const int k8 = 8 * k % (8 * L);       // angle in units of 2 pi / (8 L)
+    const int oct = k8 / L;               // octant 0..7
+    const int r = k8 - oct * L;           // within it, 0 <= r < L (units of pi / 4 / L)
+    const int a = (oct & 1) ? L - r : r;  // distance from the nearer axis of the octant's pair
+    const double x = 0.78539816339744830961566 * a / L;
+    double sn = x, cs = 1.0, ts = x, tc = 1.0;
+    for (int i = 1; i < 14; ++i) {
+        tc *= -x * x / ((2 * i - 1) * (2 * i));
+        ts *= -x * x / ((2 * i) * (2 * i + 1));
+        cs += tc;
+        sn += ts;
     }
+    // octants 1, 2, 5, 6 swap the two; signs by quadrant
+    const bool swap = ((oct + 1) & 2) != 0;
+    const double c0 = swap ? sn : cs, s0 = swap ? cs : sn;
+    const double c = (oct >= 2 && oct < 6 && c0 != 0.0) ? -c0 : c0, t = (oct >= 4 && s0 != 0.0) ? -s0 : s0;
+    return Twiddle{(float)c, (float)t};
+}
+template <int L>
+struct TwiddleTable {
+    Twiddle w[L];
+    constexpr TwiddleTable() : w() {
+        for (int k = 0; k < L; ++k) w[k] = twiddle_of(k, L);
+    }
+};
+template <int L>
+__device__ const TwiddleTable<L> kTwiddles{};
+
+// pass-1 twiddles of output row o = dy + P/2 at step k2, exp(2 pi i k2 dy / L),
+// in constant memory: every lane of a warp reads the same one
+template <int P>
+struct RowTwiddles {
+    Twiddle w[9][P + 1];
+    constexpr RowTwiddles() : w() {
+        for (int k2 = 0; k2 < 9; ++k2)
+            for (int o = 0; o <= P; ++o) {
+                const int dy = o - P / 2;
+                w[k2][o] = twiddle_of(k2 * (dy >= 0 ? dy : 9 * P + dy) % (9 * P), 9 * P);
+            }
+    }
+};
+template <int P>
+__constant__ const RowTwiddles<P> kRowTwiddles{};
+
+template <int L>
+__device__ __forceinline__ void load_twiddles(float2 *tw, int sign) {
+    for (int k = threadIdx.x; k < L; k += blockDim.x)
+        tw[k] = make_float2(kTwiddles<L>.w[k].c, (float)sign * kTwiddles<L>.w[k].s);
 }
 
 __device__ __forceinline__ float bitf(const uint64_t *rows, int nw, int y, int x) {
@@ -50,8 +101,7 @@ struct PairSmem {
     static constexpr size_t out1 = tw + sizeof(float2) * L;                  // [2][NO][LH] float2
     static constexpr size_t v2 = out1 + sizeof(float2) * 2 * NO * LH;        // [NO][9][P+1] float2
     static constexpr size_t misc = v2 + sizeof(float2) * NO * 9 * (P + 1);   // keys [2][32] u64, flags [8]
-    static constexpr size_t two = misc + 2 * 32 * 8 + 8 * 4;                 // [9][NO] float2: pass-1 twiddles
-    static constexpr size_t bytes = two + sizeof(float2) * 9 * NO;
+    static constexpr size_t bytes = misc + 2 * 32 * 8 + 8 * 4;
     // pass 1's second half accumulates in v2 ([2][NO][LH] float2 fits its
     // NO * 9 * (P + 1) entries: 2 LH = 9P + 2); surfaces reuse out1 once
     // pass 2 has read it: [2][NO][NO] float
@@ -116,16 +166,8 @@ __device__ __forceinline__ void pair_body(const pcl_params &prm, const pcl_clips
             return;
         }
     }
-    build_twiddles(tw, L, +1);
+    load_twiddles<L>(tw, +1);
     __syncthreads();
-    // pass-1 twiddles of output row o = dy + HW at step k2: w^(k2 n), n = dy mod L
-    float2 *two = reinterpret_cast<float2 *>(smem + SM::two);  // [9][NO]
-    for (int t = threadIdx.x; t < 9 * NO; t += blockDim.x) {
-        const int k2 = t / NO, dy = t % NO - HW;
-        two[t] = tw[(k2 * (dy >= 0 ? dy : L + dy)) % L];
-    }
-    __syncthreads();
-
     const float2 *fa = reinterpret_cast<const float2 *>(A.spec) + (size_t)pr.a * L * LS;
     const float2 *fb = reinterpret_cast<const float2 *>(B.spec) + (size_t)pr.b * L * LS;
     const float thr = kPcmEps * (float)pa * (float)pb;
@@ -163,7 +205,6 @@ __device__ __forceinline__ void pair_body(const pcl_params &prm, const pcl_clips
 #pragma unroll
                     for (int k1 = 0; k1 < P; ++k1) c[k1] = cmulc(ra[k1], rb[k1]);
                 }
-                const float2 *w2 = two + k2 * NO;
 #pragma unroll
                 for (int sig = 0; sig < 2; ++sig) {  // 0: phase correlation R, 1: correlation C
                     if (sig == 0 && !want_pcm) continue;
@@ -179,13 +220,28 @@ __device__ __forceinline__ void pair_body(const pcl_params &prm, const pcl_clips
                     }
                     dft_p<P, +1, RADIX>(v);
                     if (valid) {
+                        // the running sums of a batch of outputs are loaded together:
+                        // one at a time, each load would wait for the store before it
                         float2 *d = dst + (size_t)sig * NO * LH;
+                        constexpr int OB = NO > 17 ? 3 : NO;  // (11 outputs at a time spill registers: 9.1 ms for 40,000 pairs, 8.7 with 3)
+                        static_assert(NO % OB == 0, "whole batches");
 #pragma unroll
-                        for (int o = 0; o < NO; ++o) {
-                            const int dy = o - HW;
-                            const int n1 = dy >= 0 ? dy : P + dy;
-                            const float2 t = cmul(v[n1], w2[o]);
-                            d[(size_t)o * LH] = k2 == kb ? t : cadd(d[(size_t)o * LH], t);
+                        for (int o0 = 0; o0 < NO; o0 += OB) {
+                            float2 a[OB];
+                            if (k2 != kb) {
+#pragma unroll
+                                for (int q = 0; q < OB; ++q) a[q] = d[(size_t)(o0 + q) * LH];
+                            }
+#pragma unroll
+                            for (int q = 0; q < OB; ++q) {
+                                const int dy = o0 + q - HW;
+                                const int n1 = dy >= 0 ? dy : P + dy;
+                                const Twiddle w = kRowTwiddles<P>.w[k2][o0 + q];
+                                const float2 t = cmul(v[n1], make_float2(w.c, w.s));
+                                a[q] = k2 == kb ? t : cadd(a[q], t);
+                            }
+#pragma unroll
+                            for (int q = 0; q < OB; ++q) d[(size_t)(o0 + q) * LH] = a[q];
                         }
                     }
                 }
