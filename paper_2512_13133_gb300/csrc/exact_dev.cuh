@@ -21,9 +21,83 @@ namespace exact_dev {
 // the same for the 8 shifts of a task because the chunk starts at a multiple
 // of 8.  No phase-correlation surface is formed (pcm fields 0).  The caller has
 // checked the indices, emptiness and gates.
+// Only different row pairs are counted: a raster of rectangles has runs of
+// equal rows (at 512^2 about 45 of them per clip), so for one dy the pairs
+// (A row y, B row y - dy) fall into segments of equal pairs, at most one per run
+// of either clip; a segment is counted once, times its length, and segments
+// where either row is empty are left out.  12,001 same-seed pairs of 512^2 px:
+// 5.3 ms against 24.9-26.4 counting every row.
+
+// bit y % 32 of word y / 32: row y of the N staged rows differs from row y - 1
+// (row 0: set); rows of NV 16-byte vectors at stride SV
+__device__ __forceinline__ void row_starts(const uint4 *rows, int n_rows, int NV, int SV, uint32_t *starts) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    for (int w = warp; w < (n_rows + 31) / 32; w += nwarps) {
+        const int y = 32 * w + lane;
+        bool diff = y == 0;
+        if (y > 0 && y < n_rows)
+            for (int v = 0; v < NV && !diff; ++v) {
+                const uint4 a = rows[y * SV + v], b = rows[(y - 1) * SV + v];
+                diff = ((a.x ^ b.x) | (a.y ^ b.y) | (a.z ^ b.z) | (a.w ^ b.w)) != 0u;
+            }
+        const uint32_t m = __ballot_sync(0xffffffffu, diff);
+        if (lane == 0) starts[w] = m;
+    }
+}
+
+// The segments of equal row pairs (A row j, B row j + off), j in [j0, j1), whose
+// rows both hold ones: first rows in seg[0 .. count), lengths in len[..]; seg
+// has N + 1 entries.  sa, sb: row starts (row_starts; sb of nb rows); count_a,
+// count_b: ones per row.  One warp; the result is warp-uniform.
+template <int N, typename CA, typename CB>
+__device__ __forceinline__ int row_segments(const uint32_t *sa, const uint32_t *sb, int nb, int off, int j0, int j1,
+                                            const CA *count_a, const CB *count_b, uint16_t *seg, uint16_t *len,
+                                            int lane) {
+    constexpr int K = N / 32;  // rows per lane
+    static_assert(K <= 16, "a lane's rows fit a word");
+    const int y = K * lane;
+    uint32_t m = sa[y >> 5] >> (y & 31);
+    const int b = y + off, wi = b >= 0 ? b >> 5 : -((31 - b) >> 5), nw = (nb + 31) >> 5;
+    const uint32_t lo = wi >= 0 && wi < nw ? sb[wi] : 0u, hi = wi + 1 >= 0 && wi + 1 < nw ? sb[wi + 1] : 0u;
+    m |= __funnelshift_r(lo, hi, b & 31);
+    // rows [j0, j1) only; j0 starts a segment
+    const int l = j0 - y, h = j1 - y;
+    if (l >= 0 && l < K) m |= 1u << l;
+    m &= l <= 0 ? 0xffffffffu : l >= 32 ? 0u : 0xffffffffu << l;
+    m &= h >= 32 ? 0xffffffffu : h <= 0 ? 0u : (1u << h) - 1u;
+    m &= (1u << K) - 1u;
+    const int n = __popc(m);
+    int x = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += t;
+    }
+    const int total = __shfl_sync(0xffffffffu, x, 31);
+    __syncwarp();  // the previous task's segments are no longer read
+    for (int at = x - n; m; ++at, m &= m - 1u) seg[at] = (uint16_t)(y + __ffs(m) - 1);
+    if (lane == 0) seg[total] = (uint16_t)j1;
+    __syncwarp();
+    int kept = 0;
+    for (int i0 = 0; i0 < total; i0 += 32) {  // in place: kept <= i0
+        const int i = i0 + lane;
+        const int s = i < total ? seg[i] : 0, e = i < total ? seg[i + 1] : 0;
+        const bool keep = i < total && count_a[s] != 0 && count_b[s + off] != 0;
+        const unsigned k = __ballot_sync(0xffffffffu, keep);  // also orders the reads before the writes
+        const int at = kept + __popc(k & ((1u << lane) - 1u));
+        if (keep) {
+            seg[at] = (uint16_t)s;
+            len[at] = (uint16_t)(e - s);
+        }
+        kept += __popc(k);
+        __syncwarp();
+    }
+    return kept;
+}
+
 template <int NW32, int Q>
 __device__ __forceinline__ void exact_row_counts(const uint32_t (&a)[NW32], const uint32_t (&bp)[NW32 + 3], int rb,
-                                                 uint32_t (&cnt)[8]) {
+                                                 uint32_t times, uint32_t (&cnt)[8]) {
     // bp[i] = B's word i - 2 (zero outside the row); B moved by 32 Q + r has
     // word w = funnel(b[w - Q - 1], b[w - Q], r) = funnel(bp[w + 1 - Q], bp[w + 2 - Q], r)
 #pragma unroll
@@ -32,7 +106,7 @@ __device__ __forceinline__ void exact_row_counts(const uint32_t (&a)[NW32], cons
         uint32_t x[NW32];
 #pragma unroll
         for (int w = 0; w < NW32; ++w) x[w] = a[w] & __funnelshift_l(bp[w + 1 - Q], bp[w + 2 - Q], r);
-        cnt[u] += popc_sum<NW32>(x);
+        cnt[u] += times * popc_sum<NW32>(x);
     }
 }
 
@@ -57,6 +131,8 @@ __device__ __forceinline__ void exact_body(const pcl_params &prm, const pcl_clip
     uint32_t *lbest = cbound + 2 * SMAX + 1;  // [0]: L, [1]: tasks evaluated
     uint32_t *order = lbest + 4;                                                      // [1024] sort keys
     uint16_t *prof = reinterpret_cast<uint16_t *>(order + 1024);                      // [2][2N]: A's, B's
+    uint32_t *starts = reinterpret_cast<uint32_t *>(prof + 4 * N);                    // [2][N / 32]: A's, B's row starts
+    uint16_t *seg = reinterpret_cast<uint16_t *>(starts + 2 * (N / 32)) + warp * (2 * N + 2), *len = seg + N + 1;
     const uint4 *ga = reinterpret_cast<const uint4 *>(A.bits + (size_t)pr.a * N * NW);
     const uint4 *gb = reinterpret_cast<const uint4 *>(B.bits + (size_t)pr.b * N * NW);
     __syncthreads();  // the shared memory may still be read by the previous item
@@ -71,6 +147,8 @@ __device__ __forceinline__ void exact_body(const pcl_params &prm, const pcl_clip
     }
     if (threadIdx.x == 0) lbest[0] = lbest[1] = 0u;
     __syncthreads();
+    row_starts(sa, N, NV, SV, starts);
+    row_starts(sb, N, NV, SV, starts + N / 32);
     const int K = 2 * S + 1;
     // Upper bounds from the projection profiles (the bound of gate G2): rows y
     // of A and y - dy of B overlap in at most min(r_A(y), r_B(y - dy)) pixels,
@@ -110,7 +188,10 @@ __device__ __forceinline__ void exact_body(const pcl_params &prm, const pcl_clip
 #pragma unroll
         for (int u = 0; u < 8; ++u) cnt[u] = 0;
         const int j0 = dy > 0 ? dy : 0, j1 = dy < 0 ? N + dy : N;
-        for (int j = j0 + lane; j < j1; j += 32) {
+        const int n = row_segments<N>(starts, starts + N / 32, N, -dy, j0, j1, prof, prof + 2 * N, seg, len, lane);
+        for (int i = lane; i < n; i += 32) {
+            const int j = seg[i];
+            const uint32_t times = len[i];
             uint32_t a[NW32], bp[NW32 + 3];
             bp[0] = bp[1] = bp[NW32 + 2] = 0u;
 #pragma unroll
@@ -119,9 +200,9 @@ __device__ __forceinline__ void exact_body(const pcl_params &prm, const pcl_clip
                 a[4 * v] = x.x, a[4 * v + 1] = x.y, a[4 * v + 2] = x.z, a[4 * v + 3] = x.w;
                 bp[4 * v + 2] = y.x, bp[4 * v + 3] = y.y, bp[4 * v + 4] = y.z, bp[4 * v + 5] = y.w;
             }
-            if (q < 0) exact_row_counts<NW32, -1>(a, bp, rb, cnt);
-            else if (q == 0) exact_row_counts<NW32, 0>(a, bp, rb, cnt);
-            else exact_row_counts<NW32, 1>(a, bp, rb, cnt);
+            if (q < 0) exact_row_counts<NW32, -1>(a, bp, rb, times, cnt);
+            else if (q == 0) exact_row_counts<NW32, 0>(a, bp, rb, times, cnt);
+            else exact_row_counts<NW32, 1>(a, bp, rb, times, cnt);
         }
         uint32_t cmax = 0;
 #pragma unroll
@@ -212,8 +293,9 @@ __device__ __forceinline__ void exact_body(const pcl_params &prm, const pcl_clip
 template <int NW>
 constexpr size_t exact_smem() {
     // rasters (odd row stride), keys[32], R and C bounds (2 x 65), L and the task count (+ 2 pad),
-    // 1024 sort keys, profiles [2][2N] u16
-    return 2 * 16 * 64 * NW * ((NW / 2) | 1) + 32 * 8 + 4 * (2 * 65 + 4) + 4 * 1024 + 2 * 2 * 2 * 64 * NW;
+    // 1024 sort keys, profiles [2][2N] u16, row starts, each warp's segments (10 warps)
+    return 2 * 16 * 64 * NW * ((NW / 2) | 1) + 32 * 8 + 4 * (2 * 65 + 4) + 4 * 1024 + 2 * 2 * 2 * 64 * NW +
+           4 * 2 * 2 * NW + 10 * 2 * (2 * 64 * NW + 2);
 }
 
 }  // namespace exact_dev
