@@ -458,9 +458,8 @@ typedef struct pcl_work {
 
 /* Launch parameters picked by the autotuner: fft_radix 2 or 4 (register DFT
    of the FFT engine), ctas_per_sm (persistent CTAs per SM, 0 = as many as
-   fit), items_per_warp (cosine items each warp claims and gates per round,
-   1..64, 0 = 16: a CTA's round aligns the survivors of its 10 warps' claims,
-   so this sets the pairs per CTA per round). */
+   fit), items_per_warp (cosine items each gating warp claims at a time,
+   1..64, 0 = 16). */
 typedef struct pcl_tuning {
     uint32_t fft_radix;
     uint32_t ctas_per_sm;
@@ -469,14 +468,16 @@ typedef struct pcl_tuning {
 
 /* One record per work item, in list order, for n_classes (1..4) size classes
    (params[c], sets[c]; a class's set serves as both sides of its pairs).
-   Spectra of referenced clips are computed first when missing; then a single
-   persistent kernel gates the cosine items a warp at a time, aligns the
-   survivors with the FFT engine of their class, and evaluates the edge items
-   one per thread.  Cosine items of a 512^2 class (S <= 32) take the exact
+   Spectra of referenced clips are computed first when missing; then a fixed
+   sequence of persistent kernels evaluates the edge items, gates the cosine
+   items and aligns the survivors of each class with the FFT engine of its
+   size (a CUDA graph can hold the sequence).  Between the gates and the
+   alignment a surviving item's record is incomplete.  Cosine items of a
+   512^2 class (S <= 32) take the exact
    window scan of pcl_match_pairs instead of the FFT, so such a class needs
    no spec buffers (spec and spec_state may be NULL); with a shift_rule other
    than EXACT_ARGMAX, and in any other class with N > 256 or S > N/16, cosine
-   items get flags = PCL_GATE_UNSUPPORTED.  Uses 8 bytes of the context workspace.
+   items get flags = PCL_GATE_UNSUPPORTED.  Uses 40 bytes of the context workspace.
    Errors: PCL_ERR_INVALID, PCL_ERR_OOM, PCL_ERR_CUDA. */
 pcl_status pcl_match_mixed(pcl_ctx *ctx, const pcl_params *params, pcl_clipset *sets, uint32_t n_classes,
                            const pcl_work *d_work, uint64_t n_cosine, uint64_t n, pcl_record *d_out,

@@ -477,52 +477,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(BandWs w, unsi
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmem));
 }
 
-// G2 as a decision (warp_g2_rejects) with the shifts in groups of nine: a
-// group is bounded by the sum against B's profile dilated by 4,
-//   sum_y min(r_A(y), r_B(y - c - e)) <= sum_y min(r_A(y), max_|e|<=4 r_B(y - c - e)),
-// and only a group whose bound is above um has its shifts summed: at 256x256 px
-// 4 group sums and 2.5 shifts instead of 33.  scratch: 2 (N + 2 S + 32) u16 per warp.
-template <int NPL>
-__device__ __forceinline__ bool warp_g2_rejects_groups(const uint16_t *__restrict__ pa,
-                                                       const uint16_t *__restrict__ pb, int S, int64_t um, int lane,
-                                                       uint16_t *scratch) {
-    constexpr int N = 32 * NPL;
-    const int pad = S + 16, len = N + 2 * pad;  // index y + pad, -pad <= y < N + pad
-    uint16_t *B = scratch, *D = scratch + len;
-#pragma unroll 1
-    for (int ax = 0; ax < 2; ++ax) {
-        uint32_t av[NPL];
-#pragma unroll
-        for (int u = 0; u < NPL; ++u) av[u] = __ldg(pa + ax * N + lane + 32 * u);
-        __syncwarp();  // earlier reads of the scratch are done
-        for (int k = lane; k < len; k += 32) {
-            const int y = k - pad;
-            B[k] = y >= 0 && y < N ? __ldg(pb + ax * N + y) : (uint16_t)0;
-        }
-        __syncwarp();
-        for (int k = lane; k < len; k += 32) {  // max over k - 4 .. k + 4
-            uint32_t m = 0;
-#pragma unroll
-            for (int e = -4; e <= 4; ++e) m = max(m, (uint32_t)B[min(max(k + e, 0), len - 1)]);
-            D[k] = (uint16_t)m;
-        }
-        __syncwarp();
-        auto sum = [&](const uint16_t *V, int d) {
-            uint32_t t = 0;
-#pragma unroll
-            for (int u = 0; u < NPL; ++u) t += min(av[u], (uint32_t)V[lane + 32 * u - d + pad]);
-            return (int64_t)__reduce_add_sync(0xffffffffu, t);
-        };
-        bool above = false;
-        for (int c = 4 - S; c - 4 <= S && !above; c += 9) {
-            if (sum(D, c) <= um) continue;
-            for (int d = c - 4; d <= c + 4 && d <= S && !above; ++d) above = sum(B, d) > um;
-        }
-        if (!above) return true;
-    }
-    return false;
-}
-
 // The listed pairs: exact G3, then G2, a warp per pair; and the pairs of empty
 // clips.  A warp takes up to 32 pairs at a time: lane q reads pair q's clips and
 // finds its threshold, then the pairs go one by one, the next pair's first 64

@@ -102,43 +102,54 @@ static __device__ __noinline__ bool warp_g2_rejects_n(const uint16_t *pa, const 
     }
 }
 
-// G2 as a decision with B's two profiles staged by the warp in shared memory
-// (scratch: 2 (N + 2S) u16, zero padded by S on both sides, so no bounds
-// checks), A's profile in registers; otherwise as warp_g2_rejects.
+// G2 as a decision (warp_g2_rejects) with the shifts in groups of nine: a
+// group is bounded by the sum against B's profile dilated by 4,
+//   sum_y min(r_A(y), r_B(y - c - e)) <= sum_y min(r_A(y), max_|e|<=4 r_B(y - c - e)),
+// and only a group whose bound is above um has its shifts summed: at 256x256 px
+// 4 group sums and 2.5 shifts instead of 33.  scratch: 2 (N + 2 S + 32) u16 per warp.
 template <int NPL>
-__device__ __forceinline__ bool warp_g2_rejects_smem(const uint16_t *__restrict__ pa,
-                                                     const uint16_t *__restrict__ pb, int S, int64_t um, int lane,
-                                                     uint16_t *scratch) {
+__device__ __forceinline__ bool warp_g2_rejects_groups(const uint16_t *__restrict__ pa,
+                                                       const uint16_t *__restrict__ pb, int S, int64_t um, int lane,
+                                                       uint16_t *scratch) {
     constexpr int N = 32 * NPL;
-    const int L = N + 2 * S;
-    __syncwarp();  // the previous pair's reads of scratch are done
-    for (int k = lane; k < 2 * L; k += 32) {
-        const int ax = k >= L, i = k - ax * L - S;
-        scratch[k] = (i >= 0 && i < N) ? __ldg(pb + ax * N + i) : (uint16_t)0;
-    }
-    __syncwarp();
+    const int pad = S + 16, len = N + 2 * pad;  // index y + pad, -pad <= y < N + pad
+    uint16_t *B = scratch, *D = scratch + len;
 #pragma unroll 1
     for (int ax = 0; ax < 2; ++ax) {
-        const uint16_t *A = pa + ax * N;
-        const uint16_t *Bs = scratch + ax * L + S;  // Bs[k] = prof_B(k) for -S <= k < N + S
         uint32_t av[NPL];
 #pragma unroll
-        for (int u = 0; u < NPL; ++u) av[u] = __ldg(A + lane + 32 * u);
-        bool above = false;
-        for (int i = 0; i <= 2 * S && !above; ++i) {
-            const int d = (i & 1) ? (i + 1) >> 1 : -(i >> 1);
+        for (int u = 0; u < NPL; ++u) av[u] = __ldg(pa + ax * N + lane + 32 * u);
+        __syncwarp();  // earlier reads of the scratch are done
+        for (int k = lane; k < len; k += 32) {
+            const int y = k - pad;
+            B[k] = y >= 0 && y < N ? __ldg(pb + ax * N + y) : (uint16_t)0;
+        }
+        __syncwarp();
+        for (int k = lane; k < len; k += 32) {  // max over k - 4 .. k + 4
+            uint32_t m = 0;
+#pragma unroll
+            for (int e = -4; e <= 4; ++e) m = max(m, (uint32_t)B[min(max(k + e, 0), len - 1)]);
+            D[k] = (uint16_t)m;
+        }
+        __syncwarp();
+        auto sum = [&](const uint16_t *V, int d) {
             uint32_t t = 0;
 #pragma unroll
-            for (int u = 0; u < NPL; ++u) t += min(av[u], (uint32_t)Bs[lane + 32 * u - d]);
-            above = (int64_t)__reduce_add_sync(0xffffffffu, t) > um;
+            for (int u = 0; u < NPL; ++u) t += min(av[u], (uint32_t)V[lane + 32 * u - d + pad]);
+            return (int64_t)__reduce_add_sync(0xffffffffu, t);
+        };
+        bool above = false;
+        for (int c = 4 - S; c - 4 <= S && !above; c += 9) {
+            if (sum(D, c) <= um) continue;
+            for (int d = c - 4; d <= c + 4 && d <= S && !above; ++d) above = sum(B, d) > um;
         }
         if (!above) return true;
     }
     return false;
 }
 
-// shared-memory G2 scratch per warp (u16 elements) for rasters up to N = 512
-constexpr int kG2Scratch = 2 * (512 + 2 * 64);
+// shared-memory G2 scratch per warp (u16 elements) for rasters up to N = 512 with S <= N / 16
+constexpr int kG2Scratch = 2 * (512 + 2 * 32 + 32);
 
 // G2 for a band walk over small rasters (N <= 128, where the density bound of
 // 16-px blocks dilated by a block is loose and G2 decides most band pairs).
@@ -381,10 +392,10 @@ __device__ __forceinline__ int warp_cosine_gate(const pcl_clipset &A, uint32_t a
     bool g2;
     if (scratch) {
         switch (g.N) {
-            case 64: g2 = warp_g2_rejects_smem<2>(pra, prb, g.S, um, lane, scratch); break;
-            case 128: g2 = warp_g2_rejects_smem<4>(pra, prb, g.S, um, lane, scratch); break;
-            case 256: g2 = warp_g2_rejects_smem<8>(pra, prb, g.S, um, lane, scratch); break;
-            default: g2 = warp_g2_rejects_smem<16>(pra, prb, g.S, um, lane, scratch); break;
+            case 64: g2 = warp_g2_rejects_groups<2>(pra, prb, g.S, um, lane, scratch); break;
+            case 128: g2 = warp_g2_rejects_groups<4>(pra, prb, g.S, um, lane, scratch); break;
+            case 256: g2 = warp_g2_rejects_groups<8>(pra, prb, g.S, um, lane, scratch); break;
+            default: g2 = warp_g2_rejects_groups<16>(pra, prb, g.S, um, lane, scratch); break;
         }
     } else {
         g2 = warp_g2_rejects_n(pra, prb, g.N, g.S, um, lane);

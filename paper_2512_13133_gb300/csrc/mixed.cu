@@ -1,17 +1,18 @@
-// a9: one persistent launch over a mixed batch -- pairs of several raster
-// size classes, cosine (FFT phase correlation) and edge (Min-Max) modes
-// together, with uneven candidate lists.
+// a9: a mixed batch -- pairs of several raster size classes, cosine (FFT phase
+// correlation) and edge (Min-Max) modes together, with uneven candidate lists.
 //
-// The work list holds the cosine items first, then the edge items.  Each CTA
-// (320 threads, shared memory sized for the largest FFT) works in rounds:
-// every warp claims a run of consecutive cosine items and checks their
-// indices, emptiness and lossless gates one after the other; the round's
-// survivors are then aligned one after the other by the whole CTA with the
-// FFT body of their size class (512² rasters, beyond the FFT body's shared
-// memory, take the exact window scan of exact_body instead).  When the cosine
-// items are exhausted, every warp takes edge items 32 at a time: the lanes
-// run their items' gates, and the whole warp evaluates the survivors.  The register DFT radix (2 or 4) and the number
-// of CTAs per SM are tuning parameters (chosen by the autotuner).
+// The work list holds the cosine items first, then the edge items.  Every
+// kernel is persistent (a grid sized to the GPU) and finds its items in the
+// list itself, so the whole batch is a fixed sequence of launches that a CUDA
+// graph can replay: the edge items (lanes run the gates, the whole warp
+// evaluates the survivors); the cosine gates, at full occupancy (the alignment
+// bodies' registers and shared memory would leave ten warps per SM); then per
+// size class the alignment of the items the gates left, marked in their
+// records, by the FFT body of that size (512x512 px, beyond its shared memory:
+// the exact window scan).  The register DFT radix (2 or 4), the CTAs per SM and
+// the items a gating warp claims are tuning parameters (chosen by the
+// autotuner).  5.2 M items over 4 x 5,000 clips of 64-512 px: 2.8 ms against
+// 7.7 with gates, alignment and edge items in one kernel of 320-thread CTAs.
 #include "edge_dev.cuh"
 #include "exact_dev.cuh"
 #include "fft_dev.cuh"
@@ -25,9 +26,8 @@ using namespace exact_dev;
 using namespace edge_dev;
 
 constexpr int kMaxClasses = 4;
-constexpr int kThreads = 320;  // ten warps: the pass-1 tasks of P = 32
-constexpr int kWarps = kThreads / 32;
-constexpr int kClaimMax = 64;  // cosine items a warp claims per round, at most (a tuning parameter)
+constexpr int kClaimMax = 64;         // cosine items a warp claims at a time, at most (a tuning parameter)
+constexpr uint16_t kPending = 0xffff;  // flags of a record whose item still needs its alignment
 
 struct MixedArgs {
     pcl_params prm[kMaxClasses];
@@ -47,86 +47,124 @@ __global__ void mark_mixed_kernel(MixedArgs args, const pcl_work *work, uint64_t
     }
 }
 
-template <int RADIX>
-__global__ void __launch_bounds__(kThreads, 1)
-    mixed_kernel(MixedArgs args, const pcl_work *work, uint64_t n_cos, uint64_t n, pcl_record *out,
-                 unsigned long long *cursor, int claim) {
-    __shared__ uint64_t surv[kWarps * kClaimMax];
-    __shared__ int n_surv, exhausted;
+// Cosine items, `claim` consecutive ones per warp at a time.  A lane takes an
+// item's indices, emptiness and areas (G1, which ends most items of unrelated
+// clips); the warp then takes G3 and G2 of the rest one after the other.  An
+// item that ends here gets its record, the others a record with flags = kPending.
+__global__ void __launch_bounds__(256) mixed_gate_kernel(MixedArgs args, const pcl_work *work, uint64_t n_cos,
+                                                         pcl_record *out, unsigned long long *cursor, int claim) {
+    __shared__ uint16_t g2_scratch[8 * kG2Scratch];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // while gating, the alignment bodies' shared memory is free: each warp
-    // takes a slice of it for the G2 profiles
-    extern __shared__ __align__(16) unsigned char mixed_sm[];
-    uint16_t *g2_scratch = reinterpret_cast<uint16_t *>(mixed_sm);
-    // ---- cosine items, in rounds: every warp claims `claim` consecutive items
-    // and gates them one after the other (the gate cost varies a lot between
-    // items, so a round evens it out over `claim` items); the survivors of the
-    // round are then aligned one after the other by the whole CTA
     for (;;) {
-        if (threadIdx.x == 0) {
-            n_surv = 0;
-            exhausted = 0;
-        }
-        __syncthreads();
         uint64_t t0 = 0;
         if (lane == 0) t0 = atomicAdd(cursor, (unsigned long long)claim);
         t0 = __shfl_sync(0xffffffffu, t0, 0);
-        if (t0 >= n_cos && lane == 0) exhausted = 1;
-        for (uint64_t t = t0; t < t0 + (uint64_t)claim && t < n_cos; ++t) {
-            const pcl_work w = work[t];
-            pcl_record rec{};
-            rec.a = w.a;
-            rec.b = w.b;
-            rec.mode = PCL_MODE_COSINE;
-            bool done = true;
-            if (w.cls >= args.n_classes || w.a >= args.cs[w.cls].n_clips || w.b >= args.cs[w.cls].n_clips) {
-                rec.flags = PCL_GATE_BAD_INDEX;
-            } else {
-                const pcl_params &prm = args.prm[w.cls];
-                const pcl_clipset &cs = args.cs[w.cls];
-                const Geo g = make_geo(prm);
-                const uint64_t pa = cs.pop[w.a], pb = cs.pop[w.b];
-                if ((g.P > 32 && (g.P != 64 || prm.shift_rule != PCL_SHIFT_EXACT_ARGMAX)) || g.S > g.N / 16) {
-                    rec.flags = PCL_GATE_UNSUPPORTED;
-                } else if (pa == 0 && pb == 0) {
-                    rec.flags = PCL_F_EMPTY;
-                    rec.sim = 1.0f;
-                    rec.pass = 1;
+        if (t0 >= n_cos) break;
+        const uint64_t t1 = min(n_cos, t0 + (uint64_t)claim);
+        for (uint64_t b = t0; b < t1; b += 32) {
+            const uint64_t t = b + lane;
+            pcl_work w{};
+            bool open = false;
+            if (t < t1) {
+                w = work[t];
+                pcl_record rec{};
+                rec.a = w.a;
+                rec.b = w.b;
+                rec.mode = PCL_MODE_COSINE;
+                if (w.cls >= args.n_classes || w.a >= args.cs[w.cls].n_clips || w.b >= args.cs[w.cls].n_clips) {
+                    rec.flags = PCL_GATE_BAD_INDEX;
                 } else {
-                    int gate = 0;
-                    if (!(prm.flags & PCL_P_NO_GATES))
-                        gate = warp_cosine_gate(cs, w.a, cs, w.b, g, prm.cos_num, prm.cos_den, lane,
-                                                g2_scratch + warp * kG2Scratch);
-                    if (gate) rec.flags = (uint16_t)gate;
-                    else done = false;
+                    const pcl_params &prm = args.prm[w.cls];
+                    const pcl_clipset &cs = args.cs[w.cls];
+                    const Geo g = make_geo(prm);
+                    const uint64_t pa = cs.pop[w.a], pb = cs.pop[w.b];
+                    const uint64_t mn = pa < pb ? pa : pb, mx = pa < pb ? pb : pa;
+                    if ((g.P > 32 && (g.P != 64 || prm.shift_rule != PCL_SHIFT_EXACT_ARGMAX)) || g.S > g.N / 16) {
+                        rec.flags = PCL_GATE_UNSUPPORTED;
+                    } else if (mx == 0) {
+                        rec.flags = PCL_F_EMPTY;
+                        rec.sim = 1.0f;
+                        rec.pass = 1;
+                    } else if (prm.flags & PCL_P_NO_GATES) {
+                        rec.flags = kPending;
+                    } else if (!((uint64_t)prm.cos_den * prm.cos_den * mn > (uint64_t)prm.cos_num * prm.cos_num * mx)) {
+                        rec.flags = PCL_GATE_G1_AREA;
+                    } else {
+                        open = true;
+                    }
                 }
+                if (!open) out[t] = rec;
             }
-            if (lane == 0) {
-                if (done) out[t] = rec;
-                else surv[atomicAdd(&n_surv, 1)] = t;
+            unsigned m = __ballot_sync(0xffffffffu, open);
+            while (m) {
+                const int src = __ffs(m) - 1;
+                m &= m - 1u;
+                const uint32_t c = __shfl_sync(0xffffffffu, (uint32_t)w.cls, src);
+                pcl_record rec{};
+                rec.a = __shfl_sync(0xffffffffu, w.a, src);
+                rec.b = __shfl_sync(0xffffffffu, w.b, src);
+                rec.mode = PCL_MODE_COSINE;
+                const pcl_params &prm = args.prm[c];
+                const int gate = warp_cosine_gate(args.cs[c], rec.a, args.cs[c], rec.b, make_geo(prm), prm.cos_num,
+                                                  prm.cos_den, lane, g2_scratch + warp * kG2Scratch);
+                rec.flags = gate ? (uint16_t)gate : kPending;
+                if (lane == 0) out[b + src] = rec;
             }
+        }
+    }
+}
+
+// The pending items of class c, aligned one at a time by a whole CTA with the
+// engine of the class's size (P = N / 8; 64: the exact scan of 512^2 px).  A
+// CTA claims kScan consecutive items and collects the pending ones of its class.
+constexpr int kScan = 512;
+
+template <int P>
+struct AlignCta {
+    static constexpr int threads = P == 64 ? 320 : 32 * 2 * ((9 * P / 2 + 1 + 31) / 32);
+    static constexpr int ctas = P == 64 || P == 16 ? 2 : P == 32 ? 1 : 4;  // resident per SM
+    static constexpr size_t smem() {
+        if constexpr (P == 64) return exact_smem<8>();
+        else return PairSmem<P>::bytes;
+    }
+};
+
+template <int P, int RADIX>
+__global__ void __launch_bounds__(AlignCta<P>::threads, AlignCta<P>::ctas)
+    mixed_align_kernel(pcl_params prm, pcl_clipset cs, uint32_t c, const pcl_work *work, uint64_t n_cos,
+                       pcl_record *out, unsigned long long *cursor) {
+    __shared__ uint16_t list[kScan];
+    __shared__ int count;
+    __shared__ unsigned long long at;
+    for (;;) {
+        __syncthreads();  // the previous list is no longer read
+        if (threadIdx.x == 0) {
+            count = 0;
+            at = atomicAdd(cursor, (unsigned long long)kScan);
         }
         __syncthreads();
-        const int ns = n_surv;
-        for (int k = 0; k < ns; ++k) {
-            const uint64_t ti = surv[k];
-            const pcl_work w = work[ti];
-            const pcl_params &prm = args.prm[w.cls];
-            const pcl_clipset &cs = args.cs[w.cls];
-            switch (make_geo(prm).P) {
-                case 8: pair_body<8, RADIX>(prm, cs, cs, pcl_pair{w.a, w.b}, out + ti, true); break;
-                case 16: pair_body<16, RADIX>(prm, cs, cs, pcl_pair{w.a, w.b}, out + ti, true); break;
-                case 64: exact_body<8, 32>(prm, cs, cs, pcl_pair{w.a, w.b}, out + ti); break;  // 512²
-                default: pair_body<32, RADIX>(prm, cs, cs, pcl_pair{w.a, w.b}, out + ti, true); break;
-            }
+        const uint64_t t0 = at;
+        if (t0 >= n_cos) break;
+        for (int k = threadIdx.x; k < kScan && t0 + k < n_cos; k += blockDim.x)
+            if (out[t0 + k].flags == kPending && work[t0 + k].cls == c) list[atomicAdd(&count, 1)] = (uint16_t)k;
+        __syncthreads();
+        const int n = count;
+        for (int k = 0; k < n; ++k) {
+            const uint64_t t = t0 + list[k];
+            const pcl_pair pr{work[t].a, work[t].b};
+            if constexpr (P == 64) exact_body<8, 32>(prm, cs, cs, pr, out + t);
+            else pair_body<P, RADIX>(prm, cs, cs, pr, out + t, true);
             __syncthreads();
         }
-        if (exhausted) break;  // some warp found no items left: this round was the last
-        __syncthreads();       // exhausted and n_surv are reset only after every warp read them
     }
-    // ---- edge items: each lane takes one item and runs its gates (most items
-    // end there); the whole warp then evaluates the survivors one at a time
-    // (warp_edge_record).  Warps stride the list 32 items at a time.
+}
+
+// Edge items: each lane takes one item and runs its gates (most items end
+// there); the whole warp then evaluates the survivors one at a time
+// (warp_edge_record).  Warps stride the list 32 items at a time.
+__global__ void __launch_bounds__(256) mixed_edge_kernel(MixedArgs args, const pcl_work *work, uint64_t n_cos,
+                                                         uint64_t n, pcl_record *out) {
+    const int lane = threadIdx.x & 31;
     const uint64_t gw = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t base = n_cos + 32 * gw; base < n; base += 32 * nw) {
@@ -158,10 +196,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-size_t mixed_smem() {
-    size_t b = PairSmem<32>::bytes > exact_smem<8>() ? PairSmem<32>::bytes : exact_smem<8>();
-    const size_t g2 = sizeof(uint16_t) * kWarps * kG2Scratch;  // gating scratch, same memory
-    return b > g2 ? b : g2;
+template <int P, int RADIX>
+cudaError_t align_t(const pcl_params &prm, const pcl_clipset &cs, uint32_t c, const pcl_work *work, uint64_t n_cos,
+                    pcl_record *out, unsigned long long *cursor, uint32_t ctas_per_sm, int num_sms, cudaStream_t st) {
+    const size_t sm = AlignCta<P>::smem();
+    auto *kern = mixed_align_kernel<P, RADIX>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    int per_sm = 0;
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, AlignCta<P>::threads, sm);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) per_sm = 1;
+    if (ctas_per_sm != 0 && (int)ctas_per_sm < per_sm) per_sm = (int)ctas_per_sm;
+    kern<<<(unsigned)(num_sms * per_sm), AlignCta<P>::threads, sm, st>>>(prm, cs, c, work, n_cos, out, cursor);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -180,7 +228,7 @@ cudaError_t launch_mixed(const pcl_params *prm, const pcl_clipset *sets, uint32_
         args.prm[c] = prm[c];
         args.cs[c] = sets[c];
     }
-    cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), st);
+    cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long) * (1 + kMaxClasses), st);
     if (e != cudaSuccess) return e;
     if (n_cos) {
         mark_mixed_kernel<<<1024, 256, 0, st>>>(args, work, n_cos);
@@ -189,22 +237,25 @@ cudaError_t launch_mixed(const pcl_params *prm, const pcl_clipset *sets, uint32_
             if ((e = launch_spectra(prm[c], sets[c], nullptr, 0, true, st)) != cudaSuccess) return e;
         }
     }
-    const size_t sm = mixed_smem();
-    int per_sm = 0;
-    if (radix == 4) {
-        e = cudaFuncSetAttribute(mixed_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mixed_kernel<4>, kThreads, sm);
-    } else {
-        e = cudaFuncSetAttribute(mixed_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mixed_kernel<2>, kThreads, sm);
-    }
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
-    const int ctas = (ctas_per_sm == 0 || (int)ctas_per_sm > per_sm) ? per_sm : (int)ctas_per_sm;
-    const unsigned grid = (unsigned)(num_sms * ctas);
     if (n == 0) return cudaSuccess;
-    if (radix == 4) mixed_kernel<4><<<grid, kThreads, sm, st>>>(args, work, n_cos, n, out, cursor, claim);
-    else mixed_kernel<2><<<grid, kThreads, sm, st>>>(args, work, n_cos, n, out, cursor, claim);
+    if (n > n_cos) mixed_edge_kernel<<<num_sms * 8, 256, 0, st>>>(args, work, n_cos, n, out);
+    if (n_cos) {
+        mixed_gate_kernel<<<num_sms * 8, 256, 0, st>>>(args, work, n_cos, out, cursor, claim);
+        for (uint32_t c = 0; c < n_classes; ++c) {
+            const Geo g = make_geo(prm[c]);
+            unsigned long long *cur = cursor + 1 + c;
+            switch (g.P * 2 + (radix == 4 ? 1 : 0)) {
+                case 16: e = align_t<8, 2>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
+                case 17: e = align_t<8, 4>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
+                case 32: e = align_t<16, 2>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
+                case 33: e = align_t<16, 4>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
+                case 64: e = align_t<32, 2>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
+                case 65: e = align_t<32, 4>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
+                default: e = align_t<64, 2>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
+            }
+            if (e != cudaSuccess) return e;
+        }
+    }
     return cudaGetLastError();
 }
 
