@@ -49,7 +49,7 @@ cudaError_t launch_compact(const pcl_record *, uint64_t, const unsigned long lon
 bool tc_supported(const Geo &);
 cudaError_t launch_exact_pairs(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const pcl_pair *,
                                uint64_t, const unsigned long long *, pcl_record *, int, unsigned long long *,
-                               cudaStream_t);
+                               cudaStream_t, const uint32_t *list = nullptr, const uint32_t *n_list = nullptr);
 size_t tc_workspace(uint64_t);
 cudaError_t launch_tc(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const pcl_pair *, uint64_t,
                       const unsigned long long *, pcl_record *, void *, size_t, int, int *, unsigned long long,

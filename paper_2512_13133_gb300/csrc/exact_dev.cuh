@@ -110,6 +110,62 @@ __device__ __forceinline__ void exact_row_counts(const uint32_t (&a)[NW32], cons
     }
 }
 
+// Order of the ntask tasks by bound, largest bucket first, into order[]: a
+// counting sort into 256 buckets of equal width (hist: 256 u32 of shared memory,
+// zeroed).  bound(t, k) is task t's bound as a float (the thread's k-th task), top at least the largest;
+// order[] gets key(t).  Inside a bucket the order is arbitrary.  (A bitonic
+// sort took 36 to 55 barriers, this takes three.)  Returns with a barrier.
+constexpr int kBuckets = 256;
+__device__ __forceinline__ int bucket_of(float bound, float top) {
+    return top > 0.0f ? min(kBuckets - 1, (int)((top - bound) * ((float)kBuckets / top))) : 0;
+}
+template <int MAXT, typename Bound, typename Key, typename Out>
+__device__ __forceinline__ void bucket_order(int ntask, float top, uint32_t *hist, Bound bound, Key key, Out *order) {
+    const int lane = threadIdx.x & 31;
+    int bk[MAXT], rank[MAXT];
+#pragma unroll
+    for (int k = 0; k < MAXT; ++k) {
+        const int t = threadIdx.x + k * blockDim.x;
+        if (t < ntask) {
+            bk[k] = bucket_of(bound(t, k), top);
+            rank[k] = (int)atomicAdd(hist + bk[k], 1u);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {  // exclusive scan, eight buckets a lane
+        constexpr int R = kBuckets / 32;
+        uint32_t v[R], sum = 0;
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            v[k] = sum;
+            sum += hist[R * lane + k];
+        }
+        uint32_t x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) hist[R * lane + k] = x - sum + v[k];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < MAXT; ++k) {
+        const int t = threadIdx.x + k * blockDim.x;
+        if (t < ntask) order[hist[bk[k]] + rank[k]] = key(t);
+    }
+    __syncthreads();
+}
+
+// threads of a CTA that runs exact_body: at 512^2 two CTAs of ten warps fill
+// the SM's shared memory, at the smaller sizes CTAs of four warps leave room
+// for six and more, and their barriers cost less
+template <int NW>
+constexpr int exact_threads() {
+    return NW == 8 ? 320 : 128;
+}
+
 template <int NW, int SMAX>
 __device__ __forceinline__ void exact_body(const pcl_params &prm, const pcl_clipset &A, const pcl_clipset &B,
                                            const pcl_pair pr, pcl_record *dst,
@@ -129,8 +185,10 @@ __device__ __forceinline__ void exact_body(const pcl_params &prm, const pcl_clip
     uint32_t *rbound = reinterpret_cast<uint32_t *>(keys + 32);                      // [2 SMAX + 1]: R(dy)
     uint32_t *cbound = rbound + 2 * SMAX + 1;                                         // [2 SMAX + 1]: C(dx)
     uint32_t *lbest = cbound + 2 * SMAX + 1;  // [0]: L, [1]: tasks evaluated
-    uint32_t *order = lbest + 4;                                                      // [1024] sort keys
-    uint16_t *prof = reinterpret_cast<uint16_t *>(order + 1024);                      // [2][2N]: A's, B's
+    constexpr int MAXTASK = (2 * SMAX + 1) * (2 * ((SMAX + 7) / 8) + 1);             // tasks at S = SMAX
+    uint32_t *order = lbest + 4;                                                      // [MAXTASK] keys in order
+    uint32_t *hist = order + MAXTASK;                                                 // [256]
+    uint16_t *prof = reinterpret_cast<uint16_t *>(hist + kBuckets + (MAXTASK & 1));   // [2][2N]: A's, B's
     uint32_t *starts = reinterpret_cast<uint32_t *>(prof + 4 * N);                    // [2][N / 32]: A's, B's row starts
     uint16_t *seg = reinterpret_cast<uint16_t *>(starts + 2 * (N / 32)) + warp * (2 * N + 2), *len = seg + N + 1;
     const uint4 *ga = reinterpret_cast<const uint4 *>(A.bits + (size_t)pr.a * N * NW);
@@ -145,6 +203,7 @@ __device__ __forceinline__ void exact_body(const pcl_params &prm, const pcl_clip
         prof[t] = __ldg(A.prof + (size_t)pr.a * 2 * N + t);
         prof[2 * N + t] = __ldg(B.prof + (size_t)pr.b * 2 * N + t);
     }
+    for (int t = threadIdx.x; t < kBuckets; t += blockDim.x) hist[t] = 0u;
     if (threadIdx.x == 0) lbest[0] = lbest[1] = 0u;
     __syncthreads();
     row_starts(sa, N, NV, SV, starts);
@@ -217,39 +276,35 @@ __device__ __forceinline__ void exact_body(const pcl_params &prm, const pcl_clip
         }
         return cmax;
     };
-    // Best first: the tasks sorted by bound, descending (bitonic sort of
-    // keys bound << 12 | 4095 - task in shared memory; ties by task index);
-    // warp w takes sorted positions w, w + nwarps, ...  The first round (the
-    // nwarps largest bounds) sets L, the largest overlap counted so far, and
-    // every counted task raises it (shared atomic max).  A warp stops at its
-    // first position whose bound is below L: the positions after it have
-    // bounds no larger, and a task below L holds no shift whose overlap
-    // reaches the best, so the argmax and its ties are the full scan's.
-    const int ntask = K * nch;  // <= 65 x 9 = 585
-    int nsort = 32;
-    while (nsort < ntask) nsort <<= 1;
-    for (int t = threadIdx.x; t < nsort; t += blockDim.x)
-        order[t] = t < ntask ? (task_bound(t) << 12) | (uint32_t)(4095 - t) : 0u;
-    __syncthreads();
-    for (int k = 2; k <= nsort; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < nsort; i += blockDim.x) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const uint32_t x = order[i], y = order[l];
-                    if (((i & k) == 0) ? (x < y) : (x > y)) {  // descending runs first
-                        order[i] = y;
-                        order[l] = x;
-                    }
-                }
-            }
-            __syncthreads();
+    // Best first: the tasks by bound, descending by bucket (keys bound << 12 |
+    // task); warp w takes positions w, w + nwarps, ...  The first round (the
+    // largest bounds) sets L, the largest overlap counted so far, and every
+    // counted task raises it (shared atomic max).  A task whose bound is below L
+    // is skipped: it holds no shift whose overlap reaches the best, so the
+    // argmax and its ties are the full scan's.  A warp stops at its first
+    // position in a bucket that lies below L's: all bounds after it are below L.
+    const int ntask = K * nch;  // <= MAXTASK
+    float top;
+    {
+        uint32_t mr = 0, mc = 0;
+        for (int k = lane; k < K; k += 32) {
+            mr = max(mr, rbound[k]);
+            mc = max(mc, cbound[k]);
         }
+        top = (float)min(__reduce_max_sync(0xffffffffu, mr), __reduce_max_sync(0xffffffffu, mc));
+    }
+    constexpr int PER = (MAXTASK + exact_threads<NW>() - 1) / exact_threads<NW>();
+    bucket_order<PER>(
+        ntask, top, hist, [&](int t, int) { return (float)task_bound(t); },
+        [&](int t) { return (task_bound(t) << 12) | (uint32_t)t; }, order);
     for (int p = warp; p < ntask; p += nwarps) {
         const uint32_t key = order[p];
         const uint32_t lnow = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(lbest), 0);
-        if ((key >> 12) < lnow) break;  // warp-uniform
-        const uint32_t cm = eval_task(4095 - (int)(key & 4095u));
+        if ((key >> 12) < lnow) {  // warp-uniform
+            if (bucket_of((float)(key >> 12), top) > bucket_of((float)lnow, top)) break;
+            continue;
+        }
+        const uint32_t cm = eval_task((int)(key & 4095u));
         if (lane == 0) {
             atomicMax(lbest, cm);
             atomicAdd(lbest + 1, 1u);
@@ -290,12 +345,13 @@ __device__ __forceinline__ void exact_body(const pcl_params &prm, const pcl_clip
 }
 
 // shared memory of exact_body
-template <int NW>
+template <int NW, int SMAX>
 constexpr size_t exact_smem() {
-    // rasters (odd row stride), keys[32], R and C bounds (2 x 65), L and the task count (+ 2 pad),
-    // 1024 sort keys, profiles [2][2N] u16, row starts, each warp's segments (10 warps)
-    return 2 * 16 * 64 * NW * ((NW / 2) | 1) + 32 * 8 + 4 * (2 * 65 + 4) + 4 * 1024 + 2 * 2 * 2 * 64 * NW +
-           4 * 2 * 2 * NW + 10 * 2 * (2 * 64 * NW + 2);
+    // rasters (odd row stride), keys[32], R and C bounds (2 x (2 SMAX + 1)), L and the task count (+ 2 pad), the
+    // order and its buckets, profiles [2][2N] u16, row starts, each warp's segments
+    constexpr size_t tasks = (2 * SMAX + 1) * (2 * ((SMAX + 7) / 8) + 1), N = 64 * NW;
+    return 2 * 16 * N * ((NW / 2) | 1) + 32 * 8 + 4 * (2 * (2 * SMAX + 1) + 4) + 4 * (tasks + 1 + kBuckets) + 2 * 4 * N +
+           4 * 2 * (N / 32) + exact_threads<NW>() / 32 * 2 * (2 * N + 2);
 }
 
 }  // namespace exact_dev

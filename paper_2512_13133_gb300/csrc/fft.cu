@@ -202,12 +202,17 @@ __global__ void __launch_bounds__(32 * 2 * ((9 * P / 2 + 1 + 31) / 32), P == 32 
 // emptiness and lossless gates as in pair_body and the survivors take the
 // bound-pruned scan (exact_body<NW, SMAX>, N = 64 NW, S <= SMAX = N/16).  One
 // pair per CTA iteration, persistent grid.
-constexpr int kExactThreads = 320;
-
+// list (with its length n_list on the device): the listed pairs only, their gates done.
 template <int NW, int SMAX>
-__global__ void __launch_bounds__(kExactThreads, 2)
+__global__ void __launch_bounds__(exact_threads<NW>(), NW == 8 ? 2 : 6)
     exact_pair_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B, const pcl_pair *pairs, uint64_t npairs,
-                      const unsigned long long *d_n, pcl_record *out, unsigned long long *stats) {
+                      const unsigned long long *d_n, pcl_record *out, unsigned long long *stats,
+                      const uint32_t *list, const uint32_t *n_list) {
+    if (list) {
+        for (uint64_t k = blockIdx.x; k < *n_list; k += gridDim.x)
+            exact_body<NW, SMAX>(prm, A, B, pairs[list[k]], out + list[k], stats);
+        return;
+    }
     if (d_n && *d_n < npairs) npairs = *d_n;
     __shared__ int gate_s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -305,8 +310,9 @@ cudaError_t launch_mark(const pcl_pair *pairs, uint64_t n, const unsigned long l
 template <int NW, int SMAX>
 cudaError_t exact_t(const pcl_params &prm, const pcl_clipset &a, const pcl_clipset &b, const pcl_pair *pairs,
                     uint64_t n, const unsigned long long *d_n, pcl_record *out, int num_sms,
-                    unsigned long long *stats, cudaStream_t st) {
-    const size_t sm = exact_smem<NW>();
+                    unsigned long long *stats, const uint32_t *list, const uint32_t *n_list, cudaStream_t st) {
+    const size_t sm = exact_smem<NW, SMAX>();
+    constexpr int kExactThreads = exact_threads<NW>();
     auto *kern = exact_pair_kernel<NW, SMAX>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess || n == 0) return e;
@@ -315,19 +321,20 @@ cudaError_t exact_t(const pcl_params &prm, const pcl_clipset &a, const pcl_clips
     if (e != cudaSuccess) return e;
     const uint64_t cap = (uint64_t)num_sms * (uint64_t)(per_sm > 0 ? per_sm : 1);
     const unsigned grid = (unsigned)(n < cap ? n : cap);
-    kern<<<grid, kExactThreads, sm, st>>>(prm, a, b, pairs, n, d_n, out, stats);
+    kern<<<grid, kExactThreads, sm, st>>>(prm, a, b, pairs, n, d_n, out, stats, list, n_list);
     return cudaGetLastError();
 }
 
 cudaError_t launch_exact_pairs(const pcl_params &prm, const pcl_clipset &a, const pcl_clipset &b,
                                const pcl_pair *pairs, uint64_t n, const unsigned long long *d_n, pcl_record *out,
-                               int num_sms, unsigned long long *stats, cudaStream_t st) {
+                               int num_sms, unsigned long long *stats, cudaStream_t st, const uint32_t *list,
+                               const uint32_t *n_list) {
     const Geo g = make_geo(prm);
     if (g.S > g.N / 16) return cudaErrorNotSupported;
     switch (g.N) {
-        case 128: return exact_t<2, 8>(prm, a, b, pairs, n, d_n, out, num_sms, stats, st);
-        case 256: return exact_t<4, 16>(prm, a, b, pairs, n, d_n, out, num_sms, stats, st);
-        case 512: return exact_t<8, 32>(prm, a, b, pairs, n, d_n, out, num_sms, stats, st);
+        case 128: return exact_t<2, 8>(prm, a, b, pairs, n, d_n, out, num_sms, stats, list, n_list, st);
+        case 256: return exact_t<4, 16>(prm, a, b, pairs, n, d_n, out, num_sms, stats, list, n_list, st);
+        case 512: return exact_t<8, 32>(prm, a, b, pairs, n, d_n, out, num_sms, stats, list, n_list, st);
         default: return cudaErrorNotSupported;
     }
 }

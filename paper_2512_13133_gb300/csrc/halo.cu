@@ -211,12 +211,13 @@ __global__ void __launch_bounds__(kThreads, NW >= 8 ? 2 : 4) halo_pair_kernel(pc
     uint64_t *sh = sa + (size_t)N * SA;                         // [NH][SH]
     uint32_t *sn = reinterpret_cast<uint32_t *>(sh + (size_t)NH * SH);  // [K*K]
     Best *wb = reinterpret_cast<Best *>(sn + ((KK + 3) & ~3));  // [warps]
-    unsigned long long *order = reinterpret_cast<unsigned long long *>(wb + kThreads / 32);  // [1024] sort keys
-    unsigned long long *bestcn = order + 1024;                  // best (c << 32 | n) so far
+    uint32_t *order = reinterpret_cast<uint32_t *>(wb + kThreads / 32);  // [1024] tasks, best first
+    uint32_t *hist = order + 1024;                              // [256]
+    unsigned long long *bestcn = reinterpret_cast<unsigned long long *>(hist + pcl::exact_dev::kBuckets);  // best (c << 32 | n) so far
     uint32_t *hbd = reinterpret_cast<uint32_t *>(bestcn + 1);   // [2 NH]: hrow, hcol of B
     uint32_t *rhb = hbd + 2 * NH, *chb = rhb + K;               // [K] Rh(dy), [K] Ch(dx)
-    uint32_t *ntasks_done = chb + K;                            // [1]
-    uint16_t *prA = reinterpret_cast<uint16_t *>(ntasks_done + 1);  // [2N]: A's row, column counts
+    uint32_t *ntasks_done = chb + K, *maxkey = ntasks_done + 1;  // [1] each
+    uint16_t *prA = reinterpret_cast<uint16_t *>(ntasks_done + 2);  // [2N]: A's row, column counts
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     // row starts of A's window and of the halo raster, and each warp's segments
     // of equal row pairs (the exact scan's: exact_dev.cuh)
@@ -248,7 +249,9 @@ __global__ void __launch_bounds__(kThreads, NW >= 8 ? 2 : 4) halo_pair_kernel(pc
         for (int t = threadIdx.x; t < KK; t += blockDim.x) sn[t] = __ldg(gn + t);
         for (int t = threadIdx.x; t < 2 * NH; t += blockDim.x) hbd[t] = __ldg(gn + KK + t);
         for (int t = threadIdx.x; t < 2 * N; t += blockDim.x) prA[t] = __ldg(A.prof + (size_t)pr.a * 2 * N + t);
+        for (int t = threadIdx.x; t < pcl::exact_dev::kBuckets; t += blockDim.x) hist[t] = 0u;
         if (threadIdx.x == 0) {
+            *maxkey = 0u;
             *bestcn = 0ull;
             *ntasks_done = 0u;
         }
@@ -337,57 +340,62 @@ __global__ void __launch_bounds__(kThreads, NW >= 8 ? 2 : 4) halo_pair_kernel(pc
                 }
             }
         };
-        // best first: tasks sorted by their largest bound of U^2 / n_B (float
-        // keys, descending; ties by task index), bitonic sort in shared memory;
-        // the keys only order the work, the skip test above is exact
-        int nsort = 32;
-        while (nsort < ntask) nsort <<= 1;
-        for (int t = threadIdx.x; t < nsort; t += blockDim.x) {
-            unsigned long long key = 0ull;
-            if (t < ntask) {
-                const int dy = t / nch - S, sd0 = (t % nch) * 8;
-                float kb = 0.0f;
-                for (int u = 0; u < 8 && sd0 + u <= 2 * S; ++u) {
-                    const int dx = S - (sd0 + u);
-                    const uint32_t n = sn[(dy + S) * K + dx + S];
-                    const float U = (float)min(rhb[dy + S], chb[dx + S]);
-                    if (n) kb = fmaxf(kb, U * U / (float)n);
-                }
-                key = ((unsigned long long)__float_as_uint(kb) << 32) | (0xffffffffu - (uint32_t)t);
+        // best first: tasks in buckets of their largest bound of U^2 / n_B (floats,
+        // descending); they only order the work, the skip test above is exact
+        auto task_key = [&](int t) -> float {
+            const int dy = t / nch - S, sd0 = (t % nch) * 8;
+            float kb = 0.0f;
+            for (int u = 0; u < 8 && sd0 + u <= 2 * S; ++u) {
+                const int dx = S - (sd0 + u);
+                const uint32_t n = sn[(dy + S) * K + dx + S];
+                const float U = (float)min(rhb[dy + S], chb[dx + S]);
+                if (n) kb = fmaxf(kb, U * U / (float)n);
             }
-            order[t] = key;
+            return kb;
+        };
+        {
+            constexpr int PER = (65 * 9 + kThreads - 1) / kThreads;  // S <= 32: at most 65 x 9 tasks
+            float kb[PER], top = 0.0f;
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                const int t = threadIdx.x + k * kThreads;
+                kb[k] = t < ntask ? task_key(t) : 0.0f;
+                top = fmaxf(top, kb[k]);
+            }
+            const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(top));  // not negative: ordered as integers
+            if (lane == 0) atomicMax(maxkey, m);
+            __syncthreads();
+            pcl::exact_dev::bucket_order<PER>(
+                ntask, __uint_as_float(*maxkey), hist, [&](int, int k) { return kb[k]; },
+                [&](int t) { return (uint32_t)t; }, order);
         }
-        __syncthreads();
-        for (int k = 2; k <= nsort; k <<= 1)
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = threadIdx.x; i < nsort; i += blockDim.x) {
-                    const int l = i ^ j;
-                    if (l > i) {
-                        const unsigned long long x = order[i], y = order[l];
-                        if (((i & k) == 0) ? (x < y) : (x > y)) {
-                            order[i] = y;
-                            order[l] = x;
-                        }
+        // warp w takes positions w, w + nwarps, ..: each lane tests one of its
+        // next 32, the first that is left is counted, and the rest tested again
+        // against the best known then
+        for (int q0 = warp; q0 < ntask; q0 += 32 * nwarps) {
+            const int q = q0 + lane * nwarps;
+            const int task_l = q < ntask ? (int)order[q] : 0;
+            bool open = q < ntask;
+            for (;;) {
+                const unsigned long long bc =
+                    __shfl_sync(0xffffffffu, *reinterpret_cast<volatile unsigned long long *>(bestcn), 0);
+                open = open && !prunable(task_l, (uint32_t)(bc >> 32), (uint32_t)bc);
+                const unsigned m = __ballot_sync(0xffffffffu, open);
+                if (!m) break;
+                const int src = __ffs(m) - 1;
+                if (lane == src) open = false;
+                eval_task(__shfl_sync(0xffffffffu, task_l, src));
+                if (lane == 0) {
+                    atomicAdd(ntasks_done, 1u);
+                    if (best.valid && best.c > 0 && best.n > 0) {  // raise the shared best to this warp's
+                        unsigned long long old = *reinterpret_cast<volatile unsigned long long *>(bestcn), seen;
+                        do {
+                            seen = old;
+                            const uint32_t c0 = (uint32_t)(seen >> 32), n0 = (uint32_t)seen;
+                            if (c0 && (uint64_t)best.c * best.c * n0 <= (uint64_t)c0 * c0 * best.n) break;
+                            old = atomicCAS(bestcn, seen, ((unsigned long long)best.c << 32) | best.n);
+                        } while (old != seen);
                     }
-                }
-                __syncthreads();
-            }
-        for (int q = warp; q < ntask; q += nwarps) {
-            const int task = (int)(0xffffffffu - (uint32_t)order[q]);
-            const unsigned long long bc =
-                __shfl_sync(0xffffffffu, *reinterpret_cast<volatile unsigned long long *>(bestcn), 0);
-            if (prunable(task, (uint32_t)(bc >> 32), (uint32_t)bc)) continue;  // warp-uniform
-            eval_task(task);
-            if (lane == 0) {
-                atomicAdd(ntasks_done, 1u);
-                if (best.valid && best.c > 0 && best.n > 0) {  // raise the shared best to this warp's
-                    unsigned long long old = *reinterpret_cast<volatile unsigned long long *>(bestcn), seen;
-                    do {
-                        seen = old;
-                        const uint32_t c0 = (uint32_t)(seen >> 32), n0 = (uint32_t)seen;
-                        if (c0 && (uint64_t)best.c * best.c * n0 <= (uint64_t)c0 * c0 * best.n) break;
-                        old = atomicCAS(bestcn, seen, ((unsigned long long)best.c << 32) | best.n);
-                    } while (old != seen);
                 }
             }
         }
@@ -435,7 +443,7 @@ size_t raster_smem(const Geo &g) {
 size_t pair_smem(const Geo &g) {
     const int NH = halo_side(g.N, g.S), NWH = halo_words(g.N, g.S), K = 2 * g.S + 1;
     return 8ull * g.N * a_stride(g.nw) + 8ull * NH * h_stride(NWH) + 4ull * (((size_t)K * K + 3) & ~size_t(3)) +
-           sizeof(Best) * (kThreads / 32) + 8ull * 1024 + 8 + 4ull * (2 * NH + 2 * K + 1) + 2ull * 2 * g.N +
+           sizeof(Best) * (kThreads / 32) + 4ull * (1024 + pcl::exact_dev::kBuckets) + 8 + 4ull * (2 * NH + 2 * K + 2) + 2ull * 2 * g.N +
            4ull * (g.N / 32 + (NH + 31) / 32) + (kThreads / 32) * 2ull * (2 * g.N + 2) + 16;
 }
 

@@ -121,10 +121,10 @@ constexpr int kScan = 512;
 
 template <int P>
 struct AlignCta {
-    static constexpr int threads = P == 64 ? 320 : 32 * 2 * ((9 * P / 2 + 1 + 31) / 32);
+    static constexpr int threads = P == 64 ? exact_threads<8>() : 32 * 2 * ((9 * P / 2 + 1 + 31) / 32);
     static constexpr int ctas = P == 64 || P == 16 ? 2 : P == 32 ? 1 : 4;  // resident per SM
     static constexpr size_t smem() {
-        if constexpr (P == 64) return exact_smem<8>();
+        if constexpr (P == 64) return exact_smem<8, 32>();
         else return PairSmem<P>::bytes;
     }
 };

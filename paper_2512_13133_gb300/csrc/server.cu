@@ -64,7 +64,7 @@ cudaError_t launch_band_lib(const pcl_params &, const pcl_clipset &, const uint3
                             cudaStream_t);
 cudaError_t launch_exact_pairs(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const pcl_pair *,
                                uint64_t, const unsigned long long *, pcl_record *, int, unsigned long long *,
-                               cudaStream_t);
+                               cudaStream_t, const uint32_t *list = nullptr, const uint32_t *n_list = nullptr);
 }  // namespace pcl
 
 namespace {

@@ -59,6 +59,10 @@
 
 namespace pcl {
 
+cudaError_t launch_exact_pairs(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const pcl_pair *,
+                               uint64_t, const unsigned long long *, pcl_record *, int, unsigned long long *,
+                               cudaStream_t, const uint32_t *, const uint32_t *);
+
 namespace {
 using namespace tc_dev;
 
@@ -773,20 +777,27 @@ __global__ void tc_seg_kernel(const pcl_pair *pairs, const uint32_t *surv, const
 }
 
 // one item per (segment, batch of NB): written after a scan of segment heads;
-// seg_end[k] found as the next head
-__global__ void tc_items_kernel(const uint32_t *head, const uint32_t *hpos, const uint32_t *n_surv, int NB,
-                                TcItem *items, unsigned int *n_items, uint32_t cap) {
+// seg_end[k] found as the next head.  Batches of fewer than `few` members go to
+// the list of pairs for the exact scan instead (scan, its length in n_scan).
+__global__ void tc_items_kernel(const uint32_t *head, const uint32_t *surv, const uint32_t *n_surv, int NB, int few,
+                                TcItem *items, unsigned int *n_items, uint32_t cap, uint32_t *scan,
+                                uint32_t *n_scan) {
     const uint32_t ns = *n_surv;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < ns; i += gridDim.x * blockDim.x) {
         if (!head[i]) continue;
         uint32_t e = i + 1;
         while (e < ns && !head[e]) ++e;
         for (uint32_t f = i; f < e; f += (uint32_t)NB) {
+            const uint32_t m = min((uint32_t)NB, e - f);
+            if ((int)m < few) {
+                const uint32_t at = atomicAdd(n_scan, m);
+                for (uint32_t q = 0; q < m; ++q) scan[at + q] = surv[f + q];
+                continue;
+            }
             const unsigned int k = atomicAdd(n_items, 1u);
-            if (k < cap) items[k] = TcItem{f, min((uint32_t)NB, e - f)};
+            if (k < cap) items[k] = TcItem{f, m};
         }
     }
-    (void)hpos;
 }
 
 }  // namespace
@@ -795,7 +806,7 @@ __global__ void tc_items_kernel(const uint32_t *head, const uint32_t *hpos, cons
 // (window S = N/16) keeps the shifts of the smaller window
 bool tc_supported(const Geo &g) { return (g.N == 64 || g.N == 128 || g.N == 256) && g.S >= 0 && g.S <= g.N / 16; }
 
-size_t tc_workspace(uint64_t n) { return 4 * (3 * (size_t)n + 8) + sizeof(TcItem) * (size_t)(n + 1) + 256; }
+size_t tc_workspace(uint64_t n) { return 4 * (4 * (size_t)n + 8) + sizeof(TcItem) * (size_t)(n + 1) + 256; }
 
 namespace {
 
@@ -836,6 +847,18 @@ cudaError_t launch_tc(const pcl_params &prm, const pcl_clipset &a, const pcl_cli
                       int num_sms, int *d_err, unsigned long long wait_ns, cudaStream_t st) {
     const Geo g = make_geo(prm);
     if (!tc_supported(g)) return cudaErrorNotSupported;
+    // An item costs the tensor cores the same whatever its members, so few of
+    // them leave the M and N of its MMAs mostly empty: the exact window scan
+    // (exact_dev.cuh) then gives the same records sooner.  Measured on 60,000
+    // pairs of m members per representative, M pairs/s at 256x256 px: FP16 1.2
+    // (m = 1), 2.2 (6), 4.2 (12), 5.2 (16), E4M3 2.3, 4.1, 7.3, 8.4, the scan 4.1 for
+    // unrelated clips and 11 for same-seed ones whatever m; at 128x128 px FP16
+    // 4.1, 8.0, 15.3, E4M3 8.0, 15.4, 27.9, the scan 14.1 and 24.  So the line lies
+    // where the scan of unrelated clips, its worst case, is the slower one.  A
+    // context with a wait limit of its own keeps every item on the tensor
+    // cores: the limit says when to give them up.
+    const bool e4m3 = prm.cos_engine == PCL_ENGINE_TC_DIRECT_FP8;
+    const int few = g.N < 128 || wait_ns != 0 ? 0 : e4m3 ? 6 : 11;
     if (wait_ns == 0) wait_ns = kWaitNs;
     if (n == 0) return cudaSuccess;
     if (ws_bytes < tc_workspace(n) || n > 0xffffffffull) return cudaErrorInvalidValue;
@@ -847,7 +870,8 @@ cudaError_t launch_tc(const pcl_params &prm, const pcl_clipset &a, const pcl_cli
     uint32_t *keep = reinterpret_cast<uint32_t *>(w);
     uint32_t *pos = keep + n;           // n + 1
     uint32_t *surv = pos + n + 1;       // n
-    uint32_t *misc = surv + n;          // [0] n_items
+    uint32_t *scan = surv + n;          // n
+    uint32_t *misc = scan + n;          // [0] n_items, [1] pairs for the exact scan
     TcItem *items = reinterpret_cast<TcItem *>(((uintptr_t)(misc + 8) + 15) & ~uintptr_t(15));
     unsigned int *n_items = misc;
     cudaError_t e = cudaMemsetAsync(keep, 0, 4 * (size_t)n, st);
@@ -858,8 +882,12 @@ cudaError_t launch_tc(const pcl_params &prm, const pcl_clipset &a, const pcl_cli
     tc_compact_kernel<<<num_sms * 4, 256, 0, st>>>(keep, pos, n, d_n, surv);
     // segment heads over the survivors (keep reused as head flags)
     tc_seg_kernel<<<num_sms * 4, 256, 0, st>>>(pairs, surv, pos + n, keep);
-    tc_items_kernel<<<num_sms * 4, 256, 0, st>>>(keep, nullptr, pos + n, NB, items, n_items, (uint32_t)n + 1);
+    tc_items_kernel<<<num_sms * 4, 256, 0, st>>>(keep, surv, pos + n, NB, few, items, n_items, (uint32_t)n + 1, scan,
+                                                 misc + 1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (few && (e = launch_exact_pairs(prm, a, b, pairs, n, nullptr, out, num_sms, nullptr, st, scan, misc + 1)) !=
+                   cudaSuccess)
+        return e;
     switch (g.N) {
         case 64: return launch_corr_op<4, 1>(op, prm, a, b, pairs, surv, items, n_items, out, num_sms, d_err, wait_ns, st);
         case 128: return launch_corr_op<8, 2>(op, prm, a, b, pairs, surv, items, n_items, out, num_sms, d_err, wait_ns, st);
