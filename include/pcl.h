@@ -334,7 +334,9 @@ pcl_status pcl_candidates_cosine_noalloc(pcl_ctx *ctx, const pcl_params *P, cons
    and its ties are those of the full scan; pcl_stats_get reports how much of
    the window was counted.  cos_engine = PCL_ENGINE_EXACT_SCAN takes the same
    scan at 128^2 and 256^2 (S <= N/16; no spectra: spec/spec_state may be
-   NULL, EXACT_ARGMAX only).
+   NULL, EXACT_ARGMAX only).  Pairs of non-empty clips of at most 64
+   rectangles each, no two of a clip sharing a pixel, are not scanned: their
+   overlaps at every shift are summed from the rectangles (the same integers).
    With cos_engine = PCL_ENGINE_TC_DIRECT (FP16 operands),
    PCL_ENGINE_TC_DIRECT_BF16 (BF16 operands) or PCL_ENGINE_TC_DIRECT_FP8
    (E4M3 operands) the overlaps of every shift come
@@ -346,7 +348,10 @@ pcl_status pcl_candidates_cosine_noalloc(pcl_ctx *ctx, const pcl_params *P, cons
    S <= N/16 (the kernel of each size correlates the window S = N/16 and the
    argmax keeps the marker's shifts) and shift_rule = EXACT_ARGMAX (else
    PCL_ERR_UNSUPPORTED).  A
-   device-side wait that runs out is reported by pcl_device_error.
+   device-side wait that runs out is reported by pcl_device_error.  Unless the
+   context has a wait limit of its own, pairs that can take their overlaps
+   from the rectangles do so here as well, and representatives with few other
+   members take the window scan; the records are the same.
    With cos_engine = PCL_ENGINE_XYSEP the shift is not searched but
    synthesised by the XY-separation interval competition of Sec. 3.2.1 (2):
    polygon pairs from the pre-alignment of EDGE mode (each polygon of the
@@ -390,7 +395,8 @@ pcl_status pcl_set_wait_limit(pcl_ctx *ctx, uint64_t ns);
    out[1] = the groups in the windows of the pairs it aligned
    (pcl_match_pairs and serving; not the mixed batch); out[2], out[3] = the
    same for the re-extraction pair kernel (pcl_match_halo).  out[0] / out[1]
-   is the fraction of the definition's work the bounds left.  reset != 0
+   is the fraction of the definition's work the bounds left.  A pair whose
+   overlaps come from the rectangles counts as one group.  reset != 0
    zeroes the counters after reading them.  out: host array of 4.  Errors:
    PCL_ERR_INVALID (NULL ctx or out), PCL_ERR_CUDA. */
 pcl_status pcl_stats_get(pcl_ctx *ctx, uint64_t *out, int reset);
@@ -422,7 +428,9 @@ pcl_status pcl_stats_get(pcl_ctx *ctx, uint64_t *out, int reset);
    order: dx/dy the best shift (dbu), score c(s*), sim (FP32, FP64 inside
    the near band), pass, reserved = n_B(s*), flags ALIGNED (| EMPTY); no
    gates run (the lossless bounds assume fixed norms) and pcm fields are 0.
-   One CTA per pair with both rasters in shared memory; groups of shifts
+   Pairs that can (as in the exact scan, the representative not empty) take
+   their overlaps from the rectangles; for the others one CTA per pair with
+   both rasters in shared memory: groups of shifts
    are counted best first and skipped when min(row bound, column bound)^2
    n_best < c_best^2 n_B(s) for each of their shifts (a's profiles against
    b's bounds above), which leaves the chosen shift unchanged

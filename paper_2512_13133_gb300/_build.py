@@ -20,7 +20,7 @@ LIB = os.path.join(OUTDIR, "libpcl.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVFLAGS = ["-O3", "-lineinfo", "-std=c++20", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC",
            "-I", INCLUDE, "-I", CSRC]
-CUDA_SOURCES = ["api.cu", "raster.cu", "gates.cu", "band_mma.cu", "edge.cu", "edge_join.cu", "fft.cu", "noalloc.cu", "cross.cu", "server.cu", "mixed.cu", "tc.cu", "xysep.cu", "surprisal.cu", "halo.cu"]
+CUDA_SOURCES = ["api.cu", "raster.cu", "gates.cu", "band_mma.cu", "edge.cu", "edge_join.cu", "fft.cu", "noalloc.cu", "cross.cu", "server.cu", "mixed.cu", "rect_corr.cu", "tc.cu", "xysep.cu", "surprisal.cu", "halo.cu"]
 CXX_SOURCES = ["host_scp.cpp"]
 
 

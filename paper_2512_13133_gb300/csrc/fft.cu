@@ -27,9 +27,14 @@
 #include <climits>
 
 #include "exact_dev.cuh"
+#include "rect_corr.cuh"
 #include "fft_dev.cuh"
 
 namespace pcl {
+
+cudaError_t launch_rect_pairs(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const pcl_pair *, uint64_t,
+                              const unsigned long long *, pcl_record *, uint32_t *, int, unsigned long long *,
+                              cudaStream_t);
 
 namespace {
 
@@ -198,11 +203,12 @@ __global__ void __launch_bounds__(32 * 2 * ((9 * P / 2 + 1 + 31) / 32), P == 32 
 }
 
 // The exact window scan: at 512² the FFT body's buffers exceed shared memory,
-// and at 128² / 256² it is the exact-scan engine.  A pair passes the indices,
-// emptiness and lossless gates as in pair_body and the survivors take the
-// bound-pruned scan (exact_body<NW, SMAX>, N = 64 NW, S <= SMAX = N/16).  One
-// pair per CTA iteration, persistent grid.
-// list (with its length n_list on the device): the listed pairs only, their gates done.
+// and at 128² / 256² it is the exact-scan engine.  rect_pair_kernel comes first
+// (indices, emptiness, gates, and the record from the rectangles where it can);
+// the pairs it leaves pending take the bound-pruned scan of the rasters
+// (exact_body<NW, SMAX>, N = 64 NW, S <= SMAX = N/16), one pair per CTA
+// iteration: a CTA collects the pending ones of as many consecutive pairs as
+// it has threads.  list (with its length n_list on the device): those pairs instead.
 template <int NW, int SMAX>
 __global__ void __launch_bounds__(exact_threads<NW>(), NW == 8 ? 2 : 6)
     exact_pair_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B, const pcl_pair *pairs, uint64_t npairs,
@@ -213,40 +219,19 @@ __global__ void __launch_bounds__(exact_threads<NW>(), NW == 8 ? 2 : 6)
             exact_body<NW, SMAX>(prm, A, B, pairs[list[k]], out + list[k], stats);
         return;
     }
+    constexpr int T = exact_threads<NW>();
+    __shared__ uint16_t open_s[T];
+    __shared__ int count;
     if (d_n && *d_n < npairs) npairs = *d_n;
-    __shared__ int gate_s;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const Geo g = make_geo(prm);
-    for (uint64_t pid = blockIdx.x; pid < npairs; pid += gridDim.x) {
-        const pcl_pair pr = pairs[pid];
-        pcl_record rec{};
-        rec.a = pr.a;
-        rec.b = pr.b;
-        rec.mode = PCL_MODE_COSINE;
-        bool done = true;  // the same in every thread
-        if (pr.a >= A.n_clips || pr.b >= B.n_clips) {
-            rec.flags = PCL_GATE_BAD_INDEX;
-        } else if (A.pop[pr.a] == 0 && B.pop[pr.b] == 0) {
-            rec.flags = PCL_F_EMPTY;
-            rec.sim = 1.0f;
-            rec.pass = 1;
-        } else if (!(prm.flags & PCL_P_NO_GATES)) {
-            __syncthreads();
-            if (warp == 0) {
-                const int gt = warp_cosine_gate(A, pr.a, B, pr.b, g, prm.cos_num, prm.cos_den, lane);
-                if (lane == 0) gate_s = gt;
-            }
-            __syncthreads();
-            rec.flags = (uint16_t)gate_s;
-            done = gate_s != 0;
-        } else {
-            done = false;
-        }
-        if (done) {
-            if (threadIdx.x == 0) out[pid] = rec;
-            continue;
-        }
-        exact_body<NW, SMAX>(prm, A, B, pr, out + pid, stats);
+    for (uint64_t t0 = (uint64_t)blockIdx.x * T; t0 < npairs; t0 += (uint64_t)gridDim.x * T) {
+        __syncthreads();  // the previous list is no longer read
+        if (threadIdx.x == 0) count = 0;
+        __syncthreads();
+        const uint64_t t = t0 + threadIdx.x;
+        if (t < npairs && out[t].flags == rect_corr::kRectPending) open_s[atomicAdd(&count, 1)] = (uint16_t)threadIdx.x;
+        __syncthreads();
+        const int n = count;
+        for (int k = 0; k < n; ++k) exact_body<NW, SMAX>(prm, A, B, pairs[t0 + open_s[k]], out + t0 + open_s[k], stats);
     }
 }
 
@@ -331,6 +316,10 @@ cudaError_t launch_exact_pairs(const pcl_params &prm, const pcl_clipset &a, cons
                                const uint32_t *n_list) {
     const Geo g = make_geo(prm);
     if (g.S > g.N / 16) return cudaErrorNotSupported;
+    if (!list) {
+        const cudaError_t e = launch_rect_pairs(prm, a, b, pairs, n, d_n, out, nullptr, num_sms, stats, st);
+        if (e != cudaSuccess) return e;
+    }
     switch (g.N) {
         case 128: return exact_t<2, 8>(prm, a, b, pairs, n, d_n, out, num_sms, stats, list, n_list, st);
         case 256: return exact_t<4, 16>(prm, a, b, pairs, n, d_n, out, num_sms, stats, list, n_list, st);

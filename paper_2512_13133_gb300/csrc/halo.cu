@@ -22,6 +22,7 @@
 // norms.
 #include "ctx.h"
 #include "exact_dev.cuh"
+#include "rect_corr.cuh"
 
 using pcl::cos_exceeds;
 using pcl::Geo;
@@ -194,7 +195,111 @@ __device__ __forceinline__ bool before(const Best &b1, const Best &b2, uint64_t 
     return b1.dx < b2.dx;
 }
 
-// one CTA per pair (CTAs stride the list)
+// the record of the pair's best shift
+__device__ __forceinline__ pcl_record halo_record(const pcl_params &prm, const Geo &g, const pcl_pair pr, uint64_t pa,
+                                                  const Best &b) {
+    pcl_record rec{};
+    rec.a = pr.a;
+    rec.b = pr.b;
+    rec.mode = PCL_MODE_COSINE;
+    rec.dx_dbu = b.dx * g.p;
+    rec.dy_dbu = b.dy * g.p;
+    rec.score = b.c;
+    rec.reserved = b.n;
+    uint16_t fl = PCL_F_ALIGNED;
+    float sim = 0.0f;
+    if (pa == 0 && b.n == 0) {
+        sim = 1.0f;
+        rec.pass = 1;
+        fl |= PCL_F_EMPTY;
+    } else if (pa && b.n) {
+        sim = (float)b.c / sqrtf((float)pa * (float)b.n);
+        const float T = (float)prm.cos_num / (float)prm.cos_den;
+        if (fabsf(sim - T) < prm.near_band) {
+            fl |= PCL_F_NEAR_BAND;
+            sim = (float)((double)b.c / sqrt((double)pa * (double)b.n));
+        }
+        rec.pass = cos_exceeds(b.c, pa, b.n, prm.cos_num, prm.cos_den) ? 1 : 0;
+    }
+    rec.sim = sim;
+    rec.flags = fl;
+    return rec;
+}
+
+// One warp per pair: the record from the rectangles (rect_corr.cuh; A's cut to
+// its window, B's to the halo) for clips of few enough rectangles that share no
+// pixel, every shift's overlap against the tabulated n_B(s).  The other pairs
+// get a record with flags = kRectPending, for halo_pair_kernel.  A pair decided
+// here counts as one group of shifts in stats.
+constexpr int kRectWarps = 4;
+
+__global__ void __launch_bounds__(32 * kRectWarps) halo_rect_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B,
+                                                                    const uint32_t *__restrict__ norms,
+                                                                    const pcl_pair *pairs, uint64_t npairs,
+                                                                    const unsigned long long *d_n, pcl_record *out,
+                                                                    unsigned long long *stats) {
+    namespace rc = pcl::rect_corr;
+    if (d_n && *d_n < npairs) npairs = *d_n;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const Geo g = make_geo(prm);
+    const int N = g.N, S = g.S, K = 2 * S + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int psh = (g.p & (g.p - 1)) == 0 ? 31 - __clz(g.p) : -1;
+    const rc::Scratch s = rc::scratch_at(smem + warp * rc::scratch_bytes(S), S);
+    const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const bool rects = rc::has_rects(A) && rc::has_rects(B);
+    unsigned long long done_here = 0;
+    for (uint64_t t = w0; t < npairs; t += nw) {  // warp-uniform
+        const pcl_pair pr = pairs[t];
+        pcl_record rec{};
+        rec.a = pr.a;
+        rec.b = pr.b;
+        rec.mode = PCL_MODE_COSINE;
+        if (pr.a >= A.n_clips || pr.b >= B.n_clips) {
+            rec.flags = PCL_GATE_BAD_INDEX;
+            if (lane == 0) out[t] = rec;
+            continue;
+        }
+        const uint64_t pa = A.pop[pr.a];
+        const uint32_t oa = rects ? __ldg(A.rect_off + pr.a) : 0u, ob = rects ? __ldg(B.rect_off + pr.b) : 0u;
+        const int na = rects ? (int)(__ldg(A.rect_off + pr.a + 1) - oa) : 0;
+        const int nb = rects ? (int)(__ldg(B.rect_off + pr.b + 1) - ob) : 0;
+        bool ok = rects && pa != 0 && na <= rc::kRectMax && nb <= rc::kRectMax;
+        if (ok) {
+            __syncwarp();  // the scratch's previous contents are no longer read
+            const uint32_t aa = rc::stage_rects(reinterpret_cast<const int4 *>(A.rects) + oa, na, g.p, psh, 0, N, s.ra, lane);
+            rc::stage_rects(reinterpret_cast<const int4 *>(B.rects) + ob, nb, g.p, psh, -S, N + S, s.rb, lane);
+            __syncwarp();
+            ok = aa == pa && rc::ranges_disjoint(s.rb, nb, lane);
+        }
+        if (!ok) {
+            rec.flags = rc::kRectPending;
+            if (lane == 0) out[t] = rec;
+            continue;
+        }
+        const uint32_t *gn = norms + (size_t)pr.b * norms_stride(N, S);
+        Best best{0, 0, 0, 0, false};
+        rc::rect_surface(s, na, nb, S, lane, [&](uint32_t c, int dx, int dy) {
+            const Best cand{c, __ldg(gn + (dy + S) * K + dx + S), dx, dy, true};
+            if (before(cand, best, pa)) best = cand;
+        });
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            const Best other{__shfl_xor_sync(0xffffffffu, best.c, o), __shfl_xor_sync(0xffffffffu, best.n, o),
+                             __shfl_xor_sync(0xffffffffu, best.dx, o), __shfl_xor_sync(0xffffffffu, best.dy, o),
+                             __shfl_xor_sync(0xffffffffu, (int)best.valid, o) != 0};
+            if (before(other, best, pa)) best = other;
+        }
+        if (lane == 0) out[t] = halo_record(prm, g, pr, pa, best);
+        ++done_here;
+    }
+    if (lane == 0 && stats && done_here) {
+        atomicAdd(stats + 2, done_here);
+        atomicAdd(stats + 3, done_here * (unsigned long long)(K * (2 * S / 8 + 1)));
+    }
+}
+
+// One CTA per pending pair (a CTA collects those of kThreads consecutive pairs)
 template <int NW>
 __global__ void __launch_bounds__(kThreads, NW >= 8 ? 2 : 4) halo_pair_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B,
                                                              const uint64_t *__restrict__ hbits,
@@ -224,19 +329,19 @@ __global__ void __launch_bounds__(kThreads, NW >= 8 ? 2 : 4) halo_pair_kernel(pc
     uint32_t *starts = reinterpret_cast<uint32_t *>(prA + 2 * N), *starts_h = starts + N / 32;
     uint16_t *seg = reinterpret_cast<uint16_t *>(starts_h + (NH + 31) / 32) + warp * (2 * N + 2), *len = seg + N + 1;
     if (d_n && *d_n < npairs) npairs = *d_n;
-    for (uint64_t pid = blockIdx.x; pid < npairs; pid += gridDim.x) {
+    __shared__ uint16_t open_s[kThreads];
+    __shared__ int count;
+    for (uint64_t t0 = (uint64_t)blockIdx.x * kThreads; t0 < npairs; t0 += (uint64_t)gridDim.x * kThreads) {
+      __syncthreads();  // the previous list is no longer read
+      if (threadIdx.x == 0) count = 0;
+      __syncthreads();
+      if (t0 + threadIdx.x < npairs && out[t0 + threadIdx.x].flags == pcl::rect_corr::kRectPending)
+          open_s[atomicAdd(&count, 1)] = (uint16_t)threadIdx.x;
+      __syncthreads();
+      const int n_open = count;
+      for (int k_open = 0; k_open < n_open; ++k_open) {
+        const uint64_t pid = t0 + open_s[k_open];
         const pcl_pair pr = pairs[pid];
-        pcl_record rec{};
-        rec.a = pr.a;
-        rec.b = pr.b;
-        rec.mode = PCL_MODE_COSINE;
-        if (pr.a >= A.n_clips || pr.b >= B.n_clips) {
-            if (threadIdx.x == 0) {
-                rec.flags = PCL_GATE_BAD_INDEX;
-                out[pid] = rec;
-            }
-            continue;
-        }
         __syncthreads();  // the previous pair's buffers are no longer read
         const uint64_t *ga = A.bits + (size_t)pr.a * N * NW;
         const uint64_t *gh = hbits + (size_t)pr.b * NH * NWH;
@@ -409,29 +514,9 @@ __global__ void __launch_bounds__(kThreads, NW >= 8 ? 2 : 4) halo_pair_kernel(pc
             Best b = wb[0];
             for (int w = 1; w < nwarps; ++w)
                 if (before(wb[w], b, pa)) b = wb[w];
-            rec.dx_dbu = b.dx * g.p;
-            rec.dy_dbu = b.dy * g.p;
-            rec.score = b.c;
-            rec.reserved = b.n;
-            uint16_t fl = PCL_F_ALIGNED;
-            float sim = 0.0f;
-            if (pa == 0 && b.n == 0) {
-                sim = 1.0f;
-                rec.pass = 1;
-                fl |= PCL_F_EMPTY;
-            } else if (pa && b.n) {
-                sim = (float)b.c / sqrtf((float)pa * (float)b.n);
-                const float T = (float)prm.cos_num / (float)prm.cos_den;
-                if (fabsf(sim - T) < prm.near_band) {
-                    fl |= PCL_F_NEAR_BAND;
-                    sim = (float)((double)b.c / sqrt((double)pa * (double)b.n));
-                }
-                rec.pass = cos_exceeds(b.c, pa, b.n, prm.cos_num, prm.cos_den) ? 1 : 0;
-            }
-            rec.sim = sim;
-            rec.flags = fl;
-            out[pid] = rec;
+            out[pid] = halo_record(prm, g, pr, pa, b);
         }
+      }
     }
 }
 
@@ -459,6 +544,18 @@ cudaError_t launch_pair(const pcl_params &prm, const Geo &g, const pcl_clipset &
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, halo_pair_kernel<NW>, kThreads, sm);
     if (e != cudaSuccess) return e;
     const uint64_t cap = (uint64_t)num_sms * (uint64_t)(per_sm > 0 ? per_sm : 1);
+    {
+        const size_t rs = kRectWarps * pcl::rect_corr::scratch_bytes(g.S);
+        e = cudaFuncSetAttribute(halo_rect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+        int rect_sm = 0;
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rect_sm, halo_rect_kernel, 32 * kRectWarps, rs);
+        if (e != cudaSuccess) return e;
+        const uint64_t most = (uint64_t)num_sms * (uint64_t)(rect_sm > 0 ? rect_sm : 1);
+        const uint64_t need = (n + kRectWarps - 1) / kRectWarps;
+        halo_rect_kernel<<<(unsigned)(need < most ? need : most), 32 * kRectWarps, rs, st>>>(prm, a, b, nb, pairs, n, d_n,
+                                                                                            out, stats);
+    }
     halo_pair_kernel<NW><<<(unsigned)(n < cap ? n : cap), kThreads, sm, st>>>(prm, a, b, hb, nb, pairs, n, d_n, out,
                                                                              stats);
     return cudaGetLastError();

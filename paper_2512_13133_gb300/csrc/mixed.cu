@@ -16,6 +16,7 @@
 #include "edge_dev.cuh"
 #include "exact_dev.cuh"
 #include "fft_dev.cuh"
+#include "rect_corr.cuh"
 
 namespace pcl {
 
@@ -27,7 +28,7 @@ using namespace edge_dev;
 
 constexpr int kMaxClasses = 4;
 constexpr int kClaimMax = 64;         // cosine items a warp claims at a time, at most (a tuning parameter)
-constexpr uint16_t kPending = 0xffff;  // flags of a record whose item still needs its alignment
+constexpr uint16_t kPending = rect_corr::kRectPending;  // flags of a record whose item still needs its alignment
 
 struct MixedArgs {
     pcl_params prm[kMaxClasses];
@@ -110,6 +111,33 @@ __global__ void __launch_bounds__(256) mixed_gate_kernel(MixedArgs args, const p
                 rec.flags = gate ? (uint16_t)gate : kPending;
                 if (lane == 0) out[b + src] = rec;
             }
+        }
+    }
+}
+
+// The pending items of a 512x512 px class c from their rectangles
+// (rect_corr.cuh), a warp per item; those it cannot take stay pending.
+constexpr int kRectWarps = 4;
+
+__global__ void __launch_bounds__(32 * kRectWarps) mixed_rect_kernel(pcl_params prm, pcl_clipset cs, uint32_t c,
+                                                                     const pcl_work *work, uint64_t n_cos,
+                                                                     pcl_record *out) {
+    extern __shared__ __align__(16) unsigned char mixed_sm[];
+    const Geo g = make_geo(prm);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int psh = (g.p & (g.p - 1)) == 0 ? 31 - __clz(g.p) : -1;
+    const rect_corr::Scratch s = rect_corr::scratch_at(mixed_sm + warp * rect_corr::scratch_bytes(g.S), g.S);
+    const uint64_t gw = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    for (uint64_t base = 32 * gw; base < n_cos; base += 32 * nw) {
+        const uint64_t t = base + lane;
+        unsigned m = __ballot_sync(0xffffffffu, t < n_cos && out[t].flags == kPending && work[t].cls == c);
+        while (m) {
+            const int src = __ffs(m) - 1;
+            m &= m - 1u;
+            const pcl_pair pr{work[base + src].a, work[base + src].b};
+            if (cs.pop[pr.a] != 0 && cs.pop[pr.b] != 0)
+                rect_corr::rect_record(prm, g, psh, cs, cs, pr, s, out + base + src, lane);
         }
     }
 }
@@ -251,7 +279,15 @@ cudaError_t launch_mixed(const pcl_params *prm, const pcl_clipset *sets, uint32_
                 case 33: e = align_t<16, 4>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
                 case 64: e = align_t<32, 2>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
                 case 65: e = align_t<32, 4>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
-                default: e = align_t<64, 2>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
+                default: {
+                    const size_t rs = kRectWarps * rect_corr::scratch_bytes(g.S);
+                    e = cudaFuncSetAttribute(mixed_rect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+                    if (e != cudaSuccess) return e;
+                    if (g.S <= g.N / 16)
+                        mixed_rect_kernel<<<num_sms * 3, 32 * kRectWarps, rs, st>>>(prm[c], sets[c], c, work, n_cos, out);
+                    e = align_t<64, 2>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st);
+                    break;
+                }
             }
             if (e != cudaSuccess) return e;
         }
