@@ -255,10 +255,12 @@ pcl_status pcl_spectra(pcl_ctx *ctx, const pcl_params *P, pcl_clipset *cs, const
    sizes 1 KB per clip more and |b| / 96 + 512 bytes per clip of a).  EDGE uses it for the list of pairs
    left for the exact check (pairs past the list are checked inside the
    screen): the self-join 8 bytes per entry, 2^19 to 2^23 entries, beside 2 MB
-   of tables per 256 clips (at most 134 MB) and 172 bytes per clip; two sets
+   of tables per 256 clips (at most 134 MB) and 172 bytes per clip; two sets,
+   and the self-join where that does not fit,
    16 bytes per entry, one entry per 256 pairs screened, at least 65,536 and
    at most 2^24 entries.  Calls that use the context workspace run
-   in stream order on one stream at a time.
+   in stream order on one stream at a time; in a stream capture a call takes
+   what the workspace has room for.
    With P->flags & PCL_P_TOPO_HASH (self-join only) a lossy topological
    pre-screen runs first (Sec. 3.1 stage 1 filters with topological hashing
    before the exact tests): a pair is kept only if both clips have the same
@@ -509,7 +511,10 @@ pcl_status pcl_match_mixed(pcl_ctx *ctx, const pcl_params *params, pcl_clipset *
    2,000,000 library clips fit in ~21 GB).  An EDGE library needs its rasters
    and edge signatures only (esig, occ, rorder).  The server then allocates
    max_inflight request slots (one stream each, pinned staging) and one
-   device arena of mem_budget bytes, shared by all classes.
+   device arena of mem_budget bytes, shared by all classes (and, beside the
+   vectors of the density gate, its buffers for the requests in flight, at most
+   a sixteenth of mem_budget more; a request that finds no room there takes the
+   band join).
    pcl_server_submit_class admits a request of n_clips query clips of size
    class `cls` (host rectangles h_rects indexed by h_rect_off, clip i owning
    rectangles h_rect_off[i] .. h_rect_off[i+1]; copied before return) when

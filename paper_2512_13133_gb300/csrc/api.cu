@@ -30,7 +30,7 @@ cudaError_t launch_area_sort(const uint32_t *, uint32_t, uint32_t, uint32_t *, u
 size_t cross_join_workspace(const Geo &, uint32_t, uint32_t);
 cudaError_t launch_cross_join(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const uint32_t *,
                               const uint32_t *, const uint32_t *, void *, size_t, pcl_pair *, uint64_t,
-                              unsigned long long *, unsigned long long *, int, cudaStream_t, void *,
+                              unsigned long long *, unsigned long long *, int, cudaStream_t, void *, void *,
                               unsigned long long);
 size_t band_lib_bytes(const Geo &, uint32_t);
 size_t band_cross_workspace(const Geo &, uint32_t, uint32_t);
@@ -104,6 +104,25 @@ pcl_status ensure_ws(pcl_ctx *ctx, size_t bytes) {
     }
     ctx->ws_bytes = want;
     return PCL_OK;
+}
+
+// A larger workspace for a faster path, if it can be had: not while st is being
+// captured (an allocation would end the capture; a smaller one may be there
+// from an earlier call), and a size that did not fit is not tried again, as each try gives
+// the present workspace back first.
+bool ensure_ws_optional(pcl_ctx *ctx, size_t bytes, cudaStream_t st) {
+    if (bytes <= ctx->ws_bytes) return true;
+    if (ctx->ws_refused && bytes >= ctx->ws_refused) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return false;
+    if (ensure_ws(ctx, bytes) == PCL_OK) return true;
+    ctx->ws_refused = bytes;
+    ctx->err.clear();
+    return false;
 }
 
 bool pow2_raster(int N) { return N == 64 || N == 128 || N == 256 || N == 512; }
@@ -279,20 +298,20 @@ pcl_status pcl_candidates(pcl_ctx *ctx, const pcl_params *P, uint32_t mode, cons
     // cross join's own part
     const uint32_t V = (uint32_t)g.N * g.N + 2, nb = b->n_clips;
     const size_t sort_bytes = ((4 * (2 * (size_t)V + 2 * (size_t)nb)) + 255) & ~(size_t)255;
-    const size_t join_bytes = cross_join_workspace(g, a->n_clips, nb) + 256;
+    const size_t join_bytes = (cross_join_workspace(g, a->n_clips, nb) + 255) & ~(size_t)255;
     size_t lib_bytes = a->n_clips ? band_lib_bytes(g, nb) : 0;
     const size_t more = lib_bytes ? band_cross_workspace(g, a->n_clips, nb) : 0;
-    if (lib_bytes && ensure_ws(ctx, sort_bytes + lib_bytes + join_bytes + more)) lib_bytes = 0;
+    if (lib_bytes && !ensure_ws_optional(ctx, sort_bytes + lib_bytes + join_bytes + more, st)) lib_bytes = 0;
     if (!lib_bytes && (s = ensure_ws(ctx, sort_bytes + join_bytes))) return s;
-    ctx->err.clear();
     uint32_t *cum = static_cast<uint32_t *>(ctx->ws), *fill = cum + V, *order = fill + V, *spop = order + nb;
     char *lib = lib_bytes ? static_cast<char *>(ctx->ws) + sort_bytes : nullptr;
     e = launch_area_sort(b->pop, nb, V, cum, fill, order, spop, ctx->num_sms, st);
     if (e == cudaSuccess && lib) e = launch_band_lib(*P, *b, order, spop, lib, st);
     const size_t at = sort_bytes + lib_bytes;
+    char *product = lib ? static_cast<char *>(ctx->ws) + at + join_bytes : nullptr;
     if (e == cudaSuccess)
         e = launch_cross_join(*P, *a, *b, order, spop, cum, static_cast<char *>(ctx->ws) + at, ctx->ws_bytes - at,
-                              d_out, cap, cnt, gates, ctx->num_sms, st, lib, ctx->wait_ns);
+                              d_out, cap, cnt, gates, ctx->num_sms, st, lib, product, ctx->wait_ns);
     return e == cudaSuccess ? PCL_OK : cuda_fail(ctx, e, "band join (two sets)");
 }
 
@@ -319,14 +338,14 @@ pcl_status pcl_candidates_shard(pcl_ctx *ctx, const pcl_params *P, uint32_t mode
         const size_t need = band_join_workspace(g, cs->n_clips, topo);
         const size_t more = topo || n_shards != 1 ? 0 : band_mma_workspace(g, cs->n_clips);
         // without memory for the matrix product's vectors the band join alone does it
-        if ((!more || ensure_ws(ctx, need + 256 + more)) && (s = ensure_ws(ctx, need))) return s;
-        ctx->err.clear();
+        if ((!more || !ensure_ws_optional(ctx, need + 256 + more, st)) && (s = ensure_ws(ctx, need))) return s;
         e = launch_band_join(*P, *cs, ctx->ws, ctx->ws_bytes, d_out, cap, cnt, gates, ctx->num_sms, st, shard,
                              n_shards, ctx->wait_ns);
         return e == cudaSuccess ? PCL_OK : cuda_fail(ctx, e, "band join");
     }
-    if (mode == PCL_MODE_EDGE && n_shards == 1 && !topo) {
-        if ((s = ensure_ws(ctx, edge_join_workspace(cs->n_clips)))) return s;
+    // without memory for the bit tables the tiled screen does it
+    if (mode == PCL_MODE_EDGE && n_shards == 1 && !topo &&
+        ensure_ws_optional(ctx, edge_join_workspace(cs->n_clips), st)) {
         e = launch_edge_join(*P, *cs, ctx->ws, ctx->ws_bytes, d_out, cap, cnt, gates, ctx->num_sms, st);
         return e == cudaSuccess ? PCL_OK : cuda_fail(ctx, e, "edge join");
     }

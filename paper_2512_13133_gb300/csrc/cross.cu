@@ -286,7 +286,7 @@ cudaError_t launch_cross_join(const pcl_params &prm, const pcl_clipset &Q, const
                               const uint32_t *lib_order, const uint32_t *lib_spop, const uint32_t *lib_cum,
                               void *ws, size_t ws_bytes, pcl_pair *out, uint64_t cap, unsigned long long *count,
                               unsigned long long *gates, int num_sms, cudaStream_t st, void *lib_vectors,
-                              unsigned long long wait_ns) {
+                              void *product_ws, unsigned long long wait_ns) {
     const Geo g = make_geo(prm);
     const uint32_t nq = Q.n_clips, n_ch = lib_chunks(L.n_clips);
     if (ws_bytes < cross_join_workspace(g, nq, L.n_clips)) return cudaErrorInvalidValue;
@@ -308,9 +308,8 @@ cudaError_t launch_cross_join(const pcl_params &prm, const pcl_clipset &Q, const
         // with the library's vectors and workspace G3 is a matrix product, and
         // the join of the chunks runs only if that gave up
         const unsigned int *only_if = nullptr;
-        const size_t own = (cross_join_workspace(g, nq, L.n_clips) + 255) & ~(size_t)255;
-        if (lib_vectors && ws_bytes >= own + band_cross_workspace(g, nq, L.n_clips)) {
-            e = launch_band_cross(prm, Q, L, lib_order, lib_spop, lib_vectors, qorder, qspop, beg, endp, w + own, out,
+        if (lib_vectors && product_ws) {
+            e = launch_band_cross(prm, Q, L, lib_order, lib_spop, lib_vectors, qorder, qspop, beg, endp, product_ws, out,
                                   cap, count, local, &only_if, num_sms, wait_ns, st);
             if (e != cudaSuccess) return e;
         }

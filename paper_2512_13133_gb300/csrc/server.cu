@@ -21,6 +21,7 @@
 // list; a host callback on the stream stamps the completion time.  With the
 // tensor-core engine the spectra and phase-correlation steps are replaced by
 // the grouped direct correlation of the candidates (exact argmax).
+#include <algorithm>
 #include <chrono>
 #include <cstring>
 #include <map>
@@ -56,7 +57,7 @@ cudaError_t launch_edge_match(const pcl_params &, const pcl_clipset &, const pcl
                               const unsigned long long *, pcl_record *, int, cudaStream_t);
 cudaError_t launch_cross_join(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const uint32_t *,
                               const uint32_t *, const uint32_t *, void *, size_t, pcl_pair *, uint64_t,
-                              unsigned long long *, unsigned long long *, int, cudaStream_t, void *,
+                              unsigned long long *, unsigned long long *, int, cudaStream_t, void *, void *,
                               unsigned long long);
 size_t band_lib_bytes(const Geo &, uint32_t);
 size_t band_cross_workspace(const Geo &, uint32_t, uint32_t);
@@ -125,6 +126,7 @@ struct Slot {
     cudaStream_t st = nullptr;
     cudaEvent_t ev = nullptr;
     size_t off = 0, bytes = 0;
+    size_t product_off = 0, product_bytes = 0;  // in the server's product arena (0 bytes: none)
     uint32_t nq = 0;
     uint64_t cap = 0;
     pcl_clipset q{};
@@ -166,6 +168,9 @@ struct pcl_server {
     std::vector<ServerClass> cls;
     char *arena_mem = nullptr;
     Arena arena;
+    // the density gate's product: buffers beside mem_budget, so that they take no room from admission
+    char *product_mem = nullptr;
+    Arena product_arena;
     std::vector<Slot> slots;
     std::mutex mu;
 };
@@ -177,19 +182,16 @@ constexpr int kEdge = 0, kFft = 1, kTc = 2, kExact = 3;
 
 // workspace of a cosine request: the band join's, then (same stream, after
 // it) the tensor-core engine's grouping buffers in the same bytes
-// (product: with room for the density gate as a matrix product)
-size_t request_ws(const pcl::Geo &g, int engine, uint32_t nq, uint32_t n_lib, uint64_t cap, bool product) {
+size_t request_ws(const pcl::Geo &g, int engine, uint32_t nq, uint32_t n_lib, uint64_t cap) {
     if (engine == kEdge) return 0;
-    size_t cj = pcl::cross_join_workspace(g, nq, n_lib);
-    if (product) cj = align256(cj) + pcl::band_cross_workspace(g, nq, n_lib);
+    const size_t cj = pcl::cross_join_workspace(g, nq, n_lib);
     if (engine == kFft || engine == kExact) return cj;
     const size_t tc = pcl::tc_workspace(cap);
     return cj > tc ? cj : tc;
 }
 
 // device bytes of one request of nq clips and R rectangles with candidate capacity cap
-size_t footprint(const pcl::Geo &g, uint32_t nq, uint64_t R, uint64_t cap, int engine, uint32_t n_lib,
-                 bool product) {
+size_t footprint(const pcl::Geo &g, uint32_t nq, uint64_t R, uint64_t cap, int engine, uint32_t n_lib) {
     size_t b = 0;
     b += align256(4ull * (nq + 1));                 // rect_off
     b += align256(16ull * (R ? R : 1));             // rects
@@ -205,12 +207,12 @@ size_t footprint(const pcl::Geo &g, uint32_t nq, uint64_t R, uint64_t cap, int e
     b += align256(8ull * cap) * 2;                  // cand, pass
     b += align256(40ull * cap);                     // records
     b += align256(64);                              // counts
-    b += align256(request_ws(g, engine, nq, n_lib, cap, product));  // band join / tensor-core workspace (cosine only)
+    b += align256(request_ws(g, engine, nq, n_lib, cap));     // band join / tensor-core workspace (cosine only)
     return b;
 }
 
 void carve(Slot &s, const pcl::Geo &g, char *base, uint32_t nq, uint64_t R, uint64_t cap, int engine,
-           uint32_t n_lib, bool product) {
+           uint32_t n_lib) {
     char *p = base;
     auto take = [&](size_t n) {
         char *r = p;
@@ -233,7 +235,7 @@ void carve(Slot &s, const pcl::Geo &g, char *base, uint32_t nq, uint64_t R, uint
     s.pass = reinterpret_cast<pcl_pair *>(take(8ull * cap));
     s.rec = reinterpret_cast<pcl_record *>(take(40ull * cap));
     s.counts = reinterpret_cast<unsigned long long *>(take(64));
-    s.ws_bytes = request_ws(g, engine, nq, n_lib, cap, product);
+    s.ws_bytes = request_ws(g, engine, nq, n_lib, cap);
     s.ws = s.ws_bytes ? take(s.ws_bytes) : nullptr;
 }
 
@@ -347,6 +349,22 @@ pcl_status pcl_server_create_classes(pcl_ctx *ctx, const pcl_params *params, con
         }
         if (e != cudaSuccess) break;
     }
+    // the products' buffers: every slot's largest request, at most a sixteenth of the budget
+    size_t product = 0;
+    for (const auto &k : s->cls) {
+        const size_t b =
+            k.lib_vectors ? align256(pcl::band_cross_workspace(k.g, cfg->max_query_clips, k.lib.n_clips)) : 0;
+        product = b > product ? b : product;
+    }
+    product = std::min<size_t>(product * cfg->max_inflight, cfg->mem_budget / 16) & ~(size_t)255;
+    if (e == cudaSuccess && product) {
+        if (cudaMalloc(&s->product_mem, product) == cudaSuccess) {
+            s->product_arena.init(s->product_mem, product);
+        } else {
+            cudaGetLastError();
+            s->product_mem = nullptr;
+        }
+    }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cleanup(PCL_ERR_CUDA, std::string("library preparation: ") + cudaGetErrorString(e));
     s->slots.resize(cfg->max_inflight);
@@ -392,16 +410,9 @@ pcl_status pcl_server_submit_class(pcl_server *s, uint32_t cls, const uint32_t *
         }
     if (!sl) return fail(ctx, PCL_ERR_BUSY, "pcl_server_submit: no free slot");
     const uint64_t cap = (uint64_t)s->cfg.cand_per_query * n_clips + 64;
-    bool product = k.lib_vectors != nullptr;
-    size_t bytes = footprint(k.g, n_clips, R, cap, k.engine, k.lib.n_clips, product);
+    const size_t bytes = footprint(k.g, n_clips, R, cap, k.engine, k.lib.n_clips);
     size_t off = 0;
-    bool room = s->arena.alloc(bytes, &off);
-    if (!room && product) {  // the request runs without the matrix product's buffers as well
-        product = false;
-        bytes = footprint(k.g, n_clips, R, cap, k.engine, k.lib.n_clips, product);
-        room = s->arena.alloc(bytes, &off);
-    }
-    if (!room) return fail(ctx, PCL_ERR_BUSY, "pcl_server_submit: memory budget full");
+    if (!s->arena.alloc(bytes, &off)) return fail(ctx, PCL_ERR_BUSY, "pcl_server_submit: memory budget full");
     cudaError_t e = cudaSetDevice(ctx->device);
     sl->busy = true;
     sl->done = false;
@@ -409,13 +420,16 @@ pcl_status pcl_server_submit_class(pcl_server *s, uint32_t cls, const uint32_t *
     sl->cls = cls;
     sl->off = off;
     sl->bytes = bytes;
+    // without room for the matrix product's buffers the request takes the band join
+    sl->product_bytes = k.lib_vectors ? pcl::band_cross_workspace(k.g, n_clips, k.lib.n_clips) : 0;
+    if (sl->product_bytes && !s->product_arena.alloc(sl->product_bytes, &sl->product_off)) sl->product_bytes = 0;
     sl->nq = n_clips;
     sl->cap = cap;
     sl->overflow.clear();
     sl->rec_overflow.clear();
     sl->t_done = 0;
     sl->t_submit = now_ns();
-    carve(*sl, k.g, s->arena.base + off, n_clips, R, cap, k.engine, k.lib.n_clips, product);
+    carve(*sl, k.g, s->arena.base + off, n_clips, R, cap, k.engine, k.lib.n_clips);
     std::memcpy(sl->h_off, h_rect_off, 4ull * (n_clips + 1));
     const uint32_t base = h_rect_off[0];
     if (R) std::memcpy(sl->h_rects, h_rects + 4ull * base, 16ull * R);
@@ -441,7 +455,8 @@ pcl_status pcl_server_submit_class(pcl_server *s, uint32_t cls, const uint32_t *
         if (e == cudaSuccess)
             e = pcl::launch_cross_join(k.P, sl->q, k.lib, k.lib_order, k.lib_spop, k.lib_cum, sl->ws, sl->ws_bytes,
                                        sl->cand, cap, sl->counts + 0, nullptr, ctx->num_sms, st,
-                                       product ? k.lib_vectors : nullptr, ctx->wait_ns);
+                                       k.lib_vectors,
+                                       sl->product_bytes ? s->product_mem + sl->product_off : nullptr, ctx->wait_ns);
         if (k.engine == kTc) {
             // candidates grouped by query clip through the direct correlation;
             // a bounded wait that runs out sets the request's own error word
@@ -472,6 +487,7 @@ pcl_status pcl_server_submit_class(pcl_server *s, uint32_t cls, const uint32_t *
         // the slot keeps its memory until its stream is idle
         cudaStreamSynchronize(st);
         s->arena.release(sl->off, sl->bytes);
+        if (sl->product_bytes) s->product_arena.release(sl->product_off, sl->product_bytes);
         sl->busy = false;
         return fail(ctx, PCL_ERR_CUDA, std::string("pcl_server_submit: ") + cudaGetErrorString(e));
     }
@@ -538,6 +554,7 @@ pcl_status pcl_server_release(pcl_server *s, uint64_t request_id) {
     for (auto &sl : s->slots) {
         if (sl.busy && sl.done && sl.id == request_id) {
             s->arena.release(sl.off, sl.bytes);
+            if (sl.product_bytes) s->product_arena.release(sl.product_off, sl.product_bytes);
             sl.busy = false;
             sl.done = false;
             return PCL_OK;
@@ -579,6 +596,7 @@ void pcl_server_destroy(pcl_server *s) {
         cudaFree(k.lib_vectors);
     }
     cudaFree(s->arena_mem);
+    cudaFree(s->product_mem);
     delete s;
 }
 
