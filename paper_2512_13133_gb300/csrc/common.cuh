@@ -391,4 +391,16 @@ __device__ __forceinline__ uint32_t cta_scan(const uint32_t *in, uint32_t *out, 
     return carry;
 }
 
+// 32 x 32 bit transpose across a warp: lane l holds row l on entry, column l on return
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
+#pragma unroll
+    for (int s = 16; s >= 1; s >>= 1) {
+        const uint32_t m = s == 16 ? 0x0000FFFFu : s == 8 ? 0x00FF00FFu : s == 4 ? 0x0F0F0F0Fu
+                         : s == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
+        x = (lane & s) ? ((x & ~m) | ((y & ~m) >> s)) : ((x & m) | ((y & m) << s));
+    }
+    return x;
+}
+
 }  // namespace pcl

@@ -228,18 +228,6 @@ __global__ void __launch_bounds__(256) join_e2_kernel(JoinWs w, int tol, pcl_pai
     if (kept) atomicAdd(w.local, kept);
 }
 
-// 32 x 32 bit transpose across a warp: lane l holds row l on entry, column l on return
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
-#pragma unroll
-    for (int s = 16; s >= 1; s >>= 1) {
-        const uint32_t m = s == 16 ? 0x0000FFFFu : s == 8 ? 0x00FF00FFu : s == 4 ? 0x0F0F0F0Fu
-                         : s == 2 ? 0x33333333u : 0x55555555u;
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
-        x = (lane & s) ? ((x & ~m) | ((y & ~m) >> s)) : ((x & m) | ((y & m) << s));
-    }
-    return x;
-}
-
 // The bit tables of one batch: CTA (g, quarter) sorts the group's members and
 // writes the table entries of cell rows [16 quarter, 16 quarter + 16) from the
 // grids' rows [16 quarter, +24) transposed into shared memory.

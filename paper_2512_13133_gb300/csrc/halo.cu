@@ -44,88 +44,133 @@ __host__ __device__ inline int norms_stride(int N, int S) { return (2 * S + 1) *
 __host__ __device__ inline int a_stride(int NW) { return NW | 1; }
 __host__ __device__ inline int h_stride(int NWH) { return (NWH + 1) | 1; }
 
-__device__ __forceinline__ int floor_div(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
-__device__ __forceinline__ int ceil_div(int a, int b) { return -floor_div(-a, b); }
+// One CTA per clip: halo raster rows, the window sums n_B(s), and the pair
+// kernel's bounds.  Bound by issue slots.  The rows' bits are set with a lane per rectangle.
+// A window that moves by one takes one row (column) of ones in and leaves one
+// out, so nothing is summed again for another shift: a thread slides along a row for its counts at
+// every dx, a warp along 32 columns (transposed 32 rows at a time) for the
+// column bound, and the sums over the rows at dy = -S are followed by prefix sums
+// of what enters and leaves up to dy = S.  12,200 clips of 256x256 px and S = 16:
+// about 200 us against 1,346 with every row testing every rectangle and each shift
+// summed for itself.
+constexpr int kRasterThreads = 288;  // nine warps: the rows and the column words of 256x256 px with S = 16
+constexpr int kRectChunk = 128;      // rectangles staged at a time
 
-// one CTA per clip: halo raster rows, then the window sums n_B(s)
-__global__ void __launch_bounds__(kThreads) halo_raster_kernel(pcl_params prm, pcl_clipset cs, uint64_t *hbits,
-                                                               uint32_t *norms) {
+__host__ __device__ inline int row_stride(int NWH) { return (2 * NWH) | 1; }  // 32-bit words of a row, odd
+__host__ __device__ inline int cnt_stride(int NH) { return (NH + 1) & ~1; }
+
+__global__ void __launch_bounds__(kRasterThreads) halo_raster_kernel(pcl_params prm, pcl_clipset cs, uint64_t *hbits,
+                                                                     uint32_t *norms) {
     const Geo g = make_geo(prm);
-    const int N = g.N, S = g.S, p = g.p, NH = halo_side(N, S), NWH = halo_words(N, S), K = 2 * S + 1;
+    const int N = g.N, S = g.S, NH = halo_side(N, S), NWH = halo_words(N, S), K = 2 * S + 1;
+    const int RS = row_stride(NWH), CS = cnt_stride(NH);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int T = kRasterThreads, W = T / 32;
     extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t *rows = reinterpret_cast<uint64_t *>(smem);                     // [NH][NWH]
-    uint16_t *cnt = reinterpret_cast<uint16_t *>(rows + (size_t)NH * NWH);   // [NH][K]
+    uint32_t *rows = reinterpret_cast<uint32_t *>(smem);              // [NH][RS]
+    uint32_t *nb_s = rows + (size_t)NH * RS;                          // [K][K] n_B, dy by dy
+    uint16_t *cnt = reinterpret_cast<uint16_t *>(nb_s + (size_t)K * K);  // [K][CS] ones of each row in the window at dx
+    __shared__ short4 rs[kRectChunk];  // pixel ranges {x0, x1, y0, y1} in the halo raster
     const uint32_t c = blockIdx.x;
+    const int psh = (g.p & (g.p - 1)) == 0 ? 31 - __clz(g.p) : -1;
     const int32_t *r = cs.rects + 4 * (size_t)cs.rect_off[c];
     const int nr = (int)(cs.rect_off[c + 1] - cs.rect_off[c]);
-    // row t = j + S has its pixel centres at y = p j + p/2 (doubled: 2 p j + p)
-    for (int t = threadIdx.x; t < NH; t += blockDim.x) {
-        uint64_t w[9];
-        for (int k = 0; k < NWH; ++k) w[k] = 0ull;
-        const int Y2 = 2 * p * (t - S) + p;
-        for (int q = 0; q < nr; ++q) {
-            const int x0 = r[4 * q], y0 = r[4 * q + 1], x1 = r[4 * q + 2], y1 = r[4 * q + 3];
-            if (!(2 * y0 <= Y2 && Y2 < 2 * y1)) continue;
-            // columns i with 2 x0 <= 2 p i + p < 2 x1, as halo bits i + S
-            int b0 = ceil_div(2 * x0 - p, 2 * p) + S, b1 = ceil_div(2 * x1 - p, 2 * p) + S;
-            b0 = b0 < 0 ? 0 : b0;
-            b1 = b1 > NH ? NH : b1;
-            for (int k = 0; k < NWH; ++k) {
-                const int lo = max(b0, 64 * k), hi = min(b1, 64 * k + 64);
-                if (lo >= hi) continue;
-                const int n = hi - lo, o = lo - 64 * k;
-                w[k] |= (n == 64 ? ~0ull : ((1ull << n) - 1ull)) << o;
+    for (int t = tid; t < NH * RS; t += T) rows[t] = 0u;
+    for (int base = 0; base < nr; base += kRectChunk) {
+        const int n = min(kRectChunk, nr - base);
+        __syncthreads();
+        if (tid < n) {
+            const int32_t *q = r + 4 * (size_t)(base + tid);
+            auto at = [&](int v) { return (short)(pcl::rect_corr::pix_index(v, g.p, psh, -S, N + S) + S); };
+            rs[tid] = make_short4(at(q[0]), at(q[2]), at(q[1]), at(q[3]));
+        }
+        __syncthreads();
+        for (int t = lane; t < n; t += 32) {
+            const short4 q = rs[t];
+            if (q.x >= q.y) continue;
+            const int w0 = q.x >> 5, w1 = (q.y - 1) >> 5;
+            const uint32_t first = 0xffffffffu << (q.x & 31), last = 0xffffffffu >> (31 - ((q.y - 1) & 31));
+            for (int j = q.z + warp; j < q.w; j += W) {
+                uint32_t *row = rows + (size_t)j * RS;
+                if (w0 == w1) {
+                    atomicOr(row + w0, first & last);
+                } else {
+                    atomicOr(row + w0, first);
+                    for (int w = w0 + 1; w < w1; ++w) atomicOr(row + w, 0xffffffffu);
+                    atomicOr(row + w1, last);
+                }
             }
         }
-        for (int k = 0; k < NWH; ++k) {
-            rows[(size_t)t * NWH + k] = w[k];
-            hbits[((size_t)c * NH + t) * NWH + k] = w[k];
-        }
     }
     __syncthreads();
-    // cnt[t][dx + S]: bits of halo row t at positions [S - dx, S - dx + N)
-    for (int task = threadIdx.x; task < NH * K; task += blockDim.x) {
-        const int t = task / K, dx = task % K - S;
-        const int lo = S - dx, hi = lo + N;
-        uint32_t n = 0;
-        for (int k = lo >> 6; k <= (hi - 1) >> 6; ++k) {
-            uint64_t m = ~0ull;
-            if (64 * k < lo) m &= ~0ull << (lo - 64 * k);
-            if (64 * k + 64 > hi) m &= (hi - 64 * k) >= 64 ? ~0ull : ((1ull << (hi - 64 * k)) - 1ull);
-            n += (uint32_t)__popcll(rows[(size_t)t * NWH + k] & m);
-        }
-        cnt[(size_t)t * K + dx + S] = (uint16_t)n;
-    }
-    __syncthreads();
-    // n_B(dx, dy) = sum over window rows y of cnt[y - dy + S][dx]
     uint32_t *nrm = norms + (size_t)c * norms_stride(N, S);
-    for (int task = threadIdx.x; task < K * K; task += blockDim.x) {
-        const int dy = task / K - S, kx = task % K;
-        uint32_t s = 0;
-        for (int y = 0; y < N; ++y) s += cnt[(size_t)(y - dy + S) * K + kx];
-        nrm[task] = s;
+    for (int t = tid; t < NH * NWH; t += T) {
+        const uint32_t *w = rows + (size_t)(t / NWH) * RS + 2 * (t % NWH);
+        hbits[(size_t)c * NH * NWH + t] = (uint64_t)w[0] | ((uint64_t)w[1] << 32);
     }
-    // bounds for the pair kernel: hrow[t] = the most ones halo row t has in
-    // the N columns of a moved window (max over dx), hcol[x] = the most ones
-    // halo column x has in the N rows of a moved window (max over dy: rows
-    // [t0, t0 + N), t0 = S - dy = 0 .. 2S, a sliding sum)
-    for (int t = threadIdx.x; t < NH; t += blockDim.x) {
-        uint32_t m = 0;
-        for (int k = 0; k < K; ++k) m = max(m, (uint32_t)cnt[(size_t)t * K + k]);
-        nrm[K * K + t] = m;
-    }
-    for (int x = threadIdx.x; x < NH; x += blockDim.x) {
-        const int w = x >> 6, b = x & 63;
-        uint32_t win = 0;
-        for (int t = 0; t < N; ++t) win += (uint32_t)((rows[(size_t)t * NWH + w] >> b) & 1ull);
-        uint32_t m = win;
-        for (int t0 = 1; t0 <= 2 * S; ++t0) {
-            win += (uint32_t)((rows[(size_t)(t0 + N - 1) * NWH + w] >> b) & 1ull);
-            win -= (uint32_t)((rows[(size_t)(t0 - 1) * NWH + w] >> b) & 1ull);
-            m = max(m, win);
+    // rows: cnt[dx + S][t], the bits of halo row t at [S - dx, S - dx + N), and
+    // their largest over dx.  From dx - 1 to dx bit S - dx enters, bit S - dx + N leaves.
+    for (int t = tid; t < NH; t += T) {
+        const uint32_t *w = rows + (size_t)t * RS;
+        int n = 0;
+        for (int k = 0; k < 2 * NWH; ++k) n += __popc(w[k]);
+        uint64_t lo = 0, hi = 0;  // bits [0, 2S) and [N, N + 2S)
+        if (S > 0) {
+            lo = ((uint64_t)w[0] | ((uint64_t)w[1] << 32)) & (~0ull >> (64 - 2 * S));
+            hi = (uint64_t)w[2 * g.nw] | ((uint64_t)w[2 * g.nw + 1] << 32);
         }
-        nrm[K * K + NH + x] = m;
+        n -= __popcll(lo);
+        int m = n;
+        cnt[t] = (uint16_t)n;
+        for (int k = 1; k < K; ++k) {
+            const int j = 2 * S - k;
+            n += (int)((lo >> j) & 1u) - (int)((hi >> j) & 1u);
+            m = max(m, n);
+            cnt[(size_t)k * CS + t] = (uint16_t)n;
+        }
+        nrm[K * K + t] = (uint32_t)m;
     }
+    // columns, 32 per warp: the most ones halo column x has in N rows [t0, t0 + N), t0 = 0 .. 2S
+    for (int w = warp; w < 2 * NWH; w += W) {
+        int n = 0;
+        uint64_t lo = 0, hi = 0;  // this lane's column: rows [0, 64) and [N, N + 64)
+        for (int b = 0; 32 * b < NH; ++b) {
+            const int t = 32 * b + lane;
+            const uint32_t col = pcl::transpose32(t < NH ? rows[(size_t)t * RS + w] : 0u, lane);
+            if (b < 2) lo |= (uint64_t)col << (32 * b);
+            if (32 * b < N) n += __popc(col);
+            else hi |= (uint64_t)col << (32 * b - N);
+        }
+        int m = n;
+        for (int j = 0; j < 2 * S; ++j) {
+            n += (int)((hi >> j) & 1u) - (int)((lo >> j) & 1u);
+            m = max(m, n);
+        }
+        if (32 * w + lane < NH) nrm[K * K + NH + 32 * w + lane] = (uint32_t)m;
+    }
+    __syncthreads();
+    // n_B(dx, dy) = sum over the rows t in [S - dy, S - dy + N) of cnt, a warp per dx:
+    // from dy - 1 to dy row S - dy enters, row S - dy + N leaves
+    for (int k = warp; k < K; k += W) {
+        const uint16_t *ck = cnt + (size_t)k * CS;
+        int sum = 0;
+        for (int t = lane; t < N; t += 32) sum += ck[2 * S + t];
+        sum = __reduce_add_sync(0xffffffffu, sum);  // dy = -S
+        if (lane == 0) nb_s[k] = (uint32_t)sum;
+        for (int i0 = 0; i0 < 2 * S; i0 += 32) {
+            const int t = 2 * S - 1 - (i0 + lane);
+            int v = t >= 0 ? (int)ck[t] - (int)ck[t + N] : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += u;
+            }
+            if (t >= 0) nb_s[(size_t)(i0 + lane + 1) * K + k] = (uint32_t)(sum + v);
+            sum += __shfl_sync(0xffffffffu, v, 31);
+        }
+    }
+    __syncthreads();
+    for (int t = tid; t < K * K; t += T) nrm[t] = nb_s[t];
 }
 
 // c for 8 shifts of one row pair: A's 32-bit word w against halo bits
@@ -522,7 +567,7 @@ __global__ void __launch_bounds__(kThreads, NW >= 8 ? 2 : 4) halo_pair_kernel(pc
 
 size_t raster_smem(const Geo &g) {
     const int NH = halo_side(g.N, g.S), NWH = halo_words(g.N, g.S), K = 2 * g.S + 1;
-    return 8ull * NH * NWH + 2ull * NH * K;
+    return 4ull * NH * row_stride(NWH) + 4ull * K * K + 2ull * K * cnt_stride(NH);
 }
 
 size_t pair_smem(const Geo &g) {
@@ -601,7 +646,7 @@ pcl_status pcl_rasterize_halo(pcl_ctx *ctx, const pcl_params *P, const pcl_clips
     const size_t sm = raster_smem(g);
     e = cudaFuncSetAttribute(halo_raster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e == cudaSuccess) {
-        halo_raster_kernel<<<cs->n_clips, kThreads, sm, (cudaStream_t)stream>>>(*P, *cs, d_hbits, d_norms);
+        halo_raster_kernel<<<cs->n_clips, kRasterThreads, sm, (cudaStream_t)stream>>>(*P, *cs, d_hbits, d_norms);
         e = cudaGetLastError();
     }
     return e == cudaSuccess ? PCL_OK : cuda_fail(ctx, e, "halo raster kernel");
