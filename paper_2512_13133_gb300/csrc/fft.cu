@@ -190,12 +190,22 @@ __global__ void mark_kernel(const pcl_pair *pairs, uint64_t n, const unsigned lo
     }
 }
 
-// persistent: each CTA walks the pair list with a grid stride
+// persistent: each CTA walks the pair list with a grid stride.  One CTA of ten
+// warps per SM at P = 32 (registers and shared memory allow no second), so it is
+// bound by latency: issue slots were half busy, a third of pass 1 was the wait
+// for a step's 2 P loads and another third the sums in shared memory.  40,000 pairs of
+// 256x256 px 8.73 -> 7.30 ms: the sums' next batch loading during an addition
+// and the tables once per CTA 0.8 ms, the next step's rows and the rasters of
+// the final check fetched into L2 0.6 ms, the order of the units over the schedulers
+// 0.1 ms.  Measured on the way: pass 1's twiddles in shared memory instead of
+// constant memory 10.0 ms, the leftover columns' halves sharing a warp 8.9 ms, the
+// next pair's first rows fetched as well 8.1 ms.
 template <int P>
 __global__ void __launch_bounds__(32 * 2 * ((9 * P / 2 + 1 + 31) / 32), P == 32 ? 1 : P == 16 ? 2 : 4)
     pair_fft_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B, const pcl_pair *pairs, uint64_t npairs,
                     const unsigned long long *d_n, pcl_record *out) {
     if (d_n && *d_n < npairs) npairs = *d_n;
+    load_pair_table<P>();
     for (uint64_t pid = blockIdx.x; pid < npairs; pid += gridDim.x) {
         __syncthreads();
         pair_body<P>(prm, A, B, pairs[pid], out + pid);

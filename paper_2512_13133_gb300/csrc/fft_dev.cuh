@@ -103,9 +103,36 @@ struct PairSmem {
     static constexpr size_t misc = v2 + sizeof(float2) * NO * 9 * (P + 1);   // keys [2][32] u64, flags [8]
     static constexpr size_t bytes = misc + 2 * 32 * 8 + 8 * 4;
     // pass 1's second half accumulates in v2 ([2][NO][LH] float2 fits its
-    // NO * 9 * (P + 1) entries: 2 LH = 9P + 2); surfaces reuse out1 once
-    // pass 2 has read it: [2][NO][NO] float
+    // NO * 9 * (P + 1) entries: 2 LH = 9P + 2)
 };
+
+// The table of pair_body, exp(2 pi i k / L), once per CTA before its first pair
+template <int P>
+__device__ __forceinline__ void load_pair_table() {
+    extern __shared__ __align__(16) unsigned char smem[];
+    load_twiddles<PairSmem<P>::L>(reinterpret_cast<float2 *>(smem + PairSmem<P>::tw), +1);
+}
+
+// 1/sqrt of a normal number: rsqrtf without its scaling of subnormal ones
+__device__ __forceinline__ float rsqrt_normal(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// the columns [kx0, kx0 + 32) of the spectrum rows ky = 9 k1 + k2 of a pass 1 step into
+// L2: lane k1 takes a row (256 bytes, over up to three lines)
+template <int P>
+__device__ __forceinline__ void prefetch_step(const float2 *f, int k2, int kx0, int lane) {
+    constexpr int LS = (9 * P / 2 + 1 + 3) & ~3;
+    if (lane >= P) return;
+    const float2 *row = f + (size_t)(9 * lane + k2) * LS + kx0;
+    const int last = min(31, LS - 1 - kx0);
+#pragma unroll
+    for (int o = 0; o < 48; o += 16) prefetch_l2(row + min(o, last));
+}
 
 // One pair on the whole CTA.  gates_done: the caller has already checked the
 // pair's indices, emptiness and gates (the mixed-batch kernel gates a warp's
@@ -122,12 +149,11 @@ __device__ __forceinline__ void pair_body(const pcl_params &prm, const pcl_clips
     const int S = g.S;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     extern __shared__ __align__(16) unsigned char smem[];
-    float2 *tw = reinterpret_cast<float2 *>(smem + SM::tw);
+    const float2 *tw = reinterpret_cast<const float2 *>(smem + SM::tw);  // load_pair_table
     float2 *out1 = reinterpret_cast<float2 *>(smem + SM::out1);
     float2 *v2 = reinterpret_cast<float2 *>(smem + SM::v2);
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(smem + SM::misc);  // [2][32]
     int *flags = reinterpret_cast<int *>(smem + SM::misc + 2 * 32 * 8);                 // [8]
-    float *surf = reinterpret_cast<float *>(smem + SM::out1);                           // [2][NO][NO]
 
     if (threadIdx.x < 8) flags[threadIdx.x] = 0;
     pcl_record rec{};
@@ -166,14 +192,16 @@ __device__ __forceinline__ void pair_body(const pcl_params &prm, const pcl_clips
             return;
         }
     }
-    load_twiddles<L>(tw, +1);
-    __syncthreads();
     const float2 *fa = reinterpret_cast<const float2 *>(A.spec) + (size_t)pr.a * L * LS;
     const float2 *fb = reinterpret_cast<const float2 *>(B.spec) + (size_t)pr.b * L * LS;
     const float thr = kPcmEps * (float)pa * (float)pb;
     const float thr2 = thr * thr;
     const bool want_pcm = !(prm.flags & PCL_P_NO_PCM);
 
+    // the rasters of the popcount check after the transforms (P = 32, as in pass 1)
+    if constexpr (P == 32)
+      for (int t = threadIdx.x; t < 2 * (N * NW / 16); t += blockDim.x)
+          prefetch_l2((t & 1 ? B.bits + (size_t)pr.b * N * NW : A.bits + (size_t)pr.a * N * NW) + (t >> 1) * 16);
     // ---- pass 1: along ky, pruned to |dy| <= HW.  Warp task = (column
     // chunk, half of the k2 steps): the task loads both spectra of its 32
     // columns once per step, forms C = F_A conj(F_B) and from it the phase-
@@ -185,8 +213,11 @@ __device__ __forceinline__ void pair_body(const pcl_params &prm, const pcl_clips
         float2 *part = v2;  // [2][NO][LH] partial sums of the second half
         constexpr int K2H = 5;  // first half: k2 = 0..4, second half: 5..8
         for (int task = warp; task < 2 * CHUNKS; task += nwarps) {
-            const int half = task / CHUNKS;
-            const int kx = (task % CHUNKS) * 32 + lane;
+            // P = 32: warps w, w + 4 and w + 8 share a scheduler; the units of five steps
+            // go to warps 2, 6, 3, 7 and 0, so that none has more than 13 steps of 45
+            const int unit = P == 32 ? (int)((0x9831752064ull >> (4 * task)) & 15) : task;
+            const int half = unit / CHUNKS;
+            const int kx = (unit % CHUNKS) * 32 + lane;
             const bool valid = kx < LH;
             float2 *dst = (half ? part : out1) + kx;  // signal s, output o at dst[(s NO + o) LH]
             const int kb = half ? K2H : 0, ke = half ? 9 : K2H;
@@ -202,6 +233,11 @@ __device__ __forceinline__ void pair_body(const pcl_params &prm, const pcl_clips
                         ra[k1] = valid ? __ldg(fa + (size_t)ky * LS + kx) : make_float2(0.f, 0.f);
                         rb[k1] = valid ? __ldg(fb + (size_t)ky * LS + kx) : make_float2(0.f, 0.f);
                     }
+                    // the next step's rows (smaller spectra mostly are in L2: there it cost 4 %)
+                    if (P == 32 && k2 + 1 < ke) {
+                        prefetch_step<P>(fa, k2 + 1, kx - lane, lane);
+                        prefetch_step<P>(fb, k2 + 1, kx - lane, lane);
+                    }
 #pragma unroll
                     for (int k1 = 0; k1 < P; ++k1) c[k1] = cmulc(ra[k1], rb[k1]);
                 }
@@ -214,34 +250,36 @@ __device__ __forceinline__ void pair_body(const pcl_params &prm, const pcl_clips
                         float2 x = c[k1];
                         if (sig == 0) {
                             const float m2 = fmaf(x.x, x.x, x.y * x.y);
-                            x = (m2 > thr2) ? cscale(x, rsqrtf(m2)) : make_float2(0.f, 0.f);
+                            x = (m2 > thr2) ? cscale(x, rsqrt_normal(m2)) : make_float2(0.f, 0.f);
                         }
                         v[k1] = x;
                     }
                     dft_p<P, +1, RADIX>(v);
                     if (valid) {
-                        // the running sums of a batch of outputs are loaded together:
-                        // one at a time, each load would wait for the store before it
+                        // outputs in batches, the running sums of the next batch loading
+                        // while one is added: each load would else wait for the stores
+                        // before it (more at a time spill registers)
                         float2 *d = dst + (size_t)sig * NO * LH;
-                        constexpr int OB = NO > 17 ? 3 : NO;  // (11 outputs at a time spill registers: 9.1 ms for 40,000 pairs, 8.7 with 3)
-                        static_assert(NO % OB == 0, "whole batches");
+                        constexpr int OB = NO > 17 ? 2 : NO;
+                        float2 a[2][OB];
+                        auto fetch = [&](int o0, float2 (&x)[OB]) {
+#pragma unroll
+                            for (int q = 0; q < OB && o0 + q < NO; ++q)
+                                x[q] = k2 != kb ? d[(size_t)(o0 + q) * LH] : make_float2(0.f, 0.f);
+                        };
+                        fetch(0, a[0]);
 #pragma unroll
                         for (int o0 = 0; o0 < NO; o0 += OB) {
-                            float2 a[OB];
-                            if (k2 != kb) {
+                            const int cur = (o0 / OB) & 1;
+                            if (o0 + OB < NO) fetch(o0 + OB, a[cur ^ 1]);
 #pragma unroll
-                                for (int q = 0; q < OB; ++q) a[q] = d[(size_t)(o0 + q) * LH];
-                            }
-#pragma unroll
-                            for (int q = 0; q < OB; ++q) {
+                            for (int q = 0; q < OB && o0 + q < NO; ++q) {
                                 const int dy = o0 + q - HW;
                                 const int n1 = dy >= 0 ? dy : P + dy;
                                 const Twiddle w = kRowTwiddles<P>.w[k2][o0 + q];
                                 const float2 t = cmul(v[n1], make_float2(w.c, w.s));
-                                a[q] = k2 == kb ? t : cadd(a[q], t);
+                                d[(size_t)(o0 + q) * LH] = k2 == kb ? t : cadd(a[cur][q], t);
                             }
-#pragma unroll
-                            for (int q = 0; q < OB; ++q) d[(size_t)(o0 + q) * LH] = a[q];
                         }
                     }
                 }
@@ -273,35 +311,28 @@ __device__ __forceinline__ void pair_body(const pcl_params &prm, const pcl_clips
         for (int n1 = 0; n1 < P; ++n1) v2[vslot<P>(oy, k2, n1)] = v[n1];
     }
     __syncthreads();
-    // ---- pass 2 step 2: outputs (dy, dx) in the computed window
+    // ---- pass 2 step 2: outputs (dy, dx) in the computed window, r_pcm (real part)
+    // and c~; exact argmax (rounded correlation) and phase-correlation peak
     const float inv = 1.0f / ((float)L * (float)L);
-    for (int task = threadIdx.x; task < NO * NO; task += blockDim.x) {
-        const int oy = task / NO, ox = task % NO;
-        const int dx = ox - HW;
-        const int n = dx >= 0 ? dx : L + dx;
-        const int n1 = dx >= 0 ? dx : P + dx;
-        float2 z = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int k2 = 0; k2 < 9; ++k2) z = cadd(z, cmul(v2[vslot<P>(oy, k2, n1)], tw[(k2 * n) % L]));
-        surf[oy * NO + ox] = z.x * inv;             // r_pcm
-        surf[NO * NO + oy * NO + ox] = z.y * inv;   // c~
-    }
-    __syncthreads();
-    // ---- exact argmax (rounded correlation) and phase-correlation peak
     unsigned long long kc = 0, kp = 0;
     int guard = 0;
     for (int task = threadIdx.x; task < NO * NO; task += blockDim.x) {
         const int oy = task / NO, ox = task % NO;
         const int dx = ox - HW, dy = oy - HW;
         if (dx < -S || dx > S || dy < -S || dy > S) continue;
-        const float cf = surf[NO * NO + task];
+        const int n = dx >= 0 ? dx : L + dx;
+        const int n1 = dx >= 0 ? dx : P + dx;
+        float2 z = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k2 = 0; k2 < 9; ++k2) z = cadd(z, cmul(v2[vslot<P>(oy, k2, n1)], tw[(k2 * n) % L]));
+        const float cf = z.y * inv;
         const float ci = rintf(cf);
         if (fabsf(cf - ci) > 0.25f || ci < 0.f) guard = 1;
         const uint32_t cu = ci < 0.f ? 0u : (uint32_t)ci;
         const unsigned long long k1 = shift_key(cu, dx, dy, S);
         kc = k1 > kc ? k1 : kc;
         const unsigned long long lo = k1 & 0xffffffffull;
-        const unsigned long long k2 = ((unsigned long long)float_order(surf[task]) << 32) | lo;
+        const unsigned long long k2 = ((unsigned long long)float_order(z.x * inv) << 32) | lo;
         kp = k2 > kp ? k2 : kp;
     }
     kc = warp_max_u64(kc);
@@ -333,18 +364,14 @@ __device__ __forceinline__ void pair_body(const pcl_params &prm, const pcl_clips
     // popcount check of the chosen shift (rows spread over the whole CTA),
     // fall back on mismatch
     if (!gflag) {
-        if (threadIdx.x == 0) flags[4] = 0;
-        __syncthreads();
         const uint32_t part = __reduce_add_sync(
             0xffffffffu, corr_rows_partial(ba, bbits, N, NW, sdx, sdy, (int)threadIdx.x, (int)blockDim.x));
         if (lane == 0) atomicAdd(flags + 4, (int)part);
         __syncthreads();
-        if (threadIdx.x == 0 && (uint32_t)flags[4] != cbest) flags[2] = 1;
-        __syncthreads();
-        gflag = flags[2];
+        gflag = (uint32_t)flags[4] != cbest;
     }
-    __syncthreads();
     if (gflag) {
+        __syncthreads();  // every warp has read the keys
         // exact popcount scan of the whole window, one shift per warp
         const int K = 2 * S + 1;
         unsigned long long kk = 0;

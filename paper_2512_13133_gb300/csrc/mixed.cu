@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(AlignCta<P>::threads, AlignCta<P>::ctas)
     __shared__ uint16_t list[kScan];
     __shared__ int count;
     __shared__ unsigned long long at;
+    if constexpr (P != 64) load_pair_table<P>();
     for (;;) {
         __syncthreads();  // the previous list is no longer read
         if (threadIdx.x == 0) {
