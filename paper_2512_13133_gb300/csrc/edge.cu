@@ -329,199 +329,26 @@ __global__ void __launch_bounds__(256, 4) edge_screen_kernel(pcl_params prm, pcl
     }
 }
 
-// warp_edge_record as {dx, dy, E, flags | pass << 16}; out of line: clips of more
-// than 64 polygons are rare and would cost the loop below registers
-__device__ __noinline__ uint4 wide_record(const pcl_params &prm, const pcl_clipset &A, const pcl_clipset &B,
-                                          pcl_pair pr, int lane) {
-    const pcl_record r = warp_edge_record(prm, A, B, pr, lane);
-    return make_uint4((uint32_t)r.dx_dbu, (uint32_t)r.dy_dbu, r.score, r.flags | (uint32_t)r.pass << 16);
-}
-
-// Min-Max records, up to 32 pairs per warp at a time: lane q reads pair q's
-// signatures, decides indices, emptiness and E2, and keeps its record; the
-// pairs left go one by one with the whole warp, lane m holding polygons m and
-// m + 32 of the larger clip and the smaller clip's polygons staged in shared
-// memory, the next pair's polygons loading meanwhile.  A lane whose polygon is
-// hit keeps the small polygon that hit it, so that the correspondence (each
-// small polygon hits one lane, no lane is hit twice), the displacements and
-// the re-check at T need no search.  The grid test that the screen runs before
-// the correspondence is left out: it can only reject what the correspondence
-// rejects with the same record.  Clips of more than 64 polygons take
-// warp_edge_record.  Bound by issue slots; 1,000,000 screened pairs of 256x256
-// px: 636 us (4 CTAs per SM spill: 731) against 1,130 with each pair's signatures read and its record
-// written by one warp at a time.
-__global__ void __launch_bounds__(256, 3) edge_match_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B,
-                                                            const pcl_pair *pairs, uint64_t n,
-                                                            const unsigned long long *d_n, pcl_record *out) {
-    if (d_n && *d_n < n) n = *d_n;
-    const unsigned full = 0xffffffffu;
-    __shared__ int4 small_s[8][64];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int4 *small = small_s[warp];
-    const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const uint64_t per64 = (n + nw - 1) / nw;
-    const uint32_t per = per64 < 32 ? (uint32_t)per64 : 32u;  // a short list is spread over all warps
-    const int W = prm.window_dbu, M = prm.marker_dbu, tol = prm.edge_tol_dbu;
-    const bool gates = !(prm.flags & PCL_P_NO_GATES);
-    const int4 *ra = reinterpret_cast<const int4 *>(A.rects), *rb = reinterpret_cast<const int4 *>(B.rects);
-    const int4 none = make_int4(0, 0, 0, 0);
-    for (uint64_t t0 = w0 * per; t0 < n; t0 += nw * per) {  // warp-uniform
-        const bool mine = (uint32_t)lane < per && t0 + lane < n;
-        // this lane's record: shift, E, flags | pass << 16
-        int dx = 0, dy = 0, E = 0;
-        uint32_t fp = 0;
-        int offa = 0, na = 0, offb = 0, nb = 0, s0x = 0, s0y = 0;
-        bool open = false;
-        if (mine) {
-            const pcl_pair pr = pairs[t0 + lane];
-            if (pr.a >= A.n_clips || pr.b >= B.n_clips) {
-                fp = PCL_GATE_BAD_INDEX;
-            } else {
-                const int4 *e4a = reinterpret_cast<const int4 *>(A.esig + (size_t)pr.a * 8);
-                const int4 *e4b = reinterpret_cast<const int4 *>(B.esig + (size_t)pr.b * 8);
-                const int4 alo = __ldg(e4a), ahi = __ldg(e4a + 1), blo = __ldg(e4b), bhi = __ldg(e4b + 1);
-                // {n, hasx, lox, hix}, {hasy, loy, hiy, border}
-                offa = (int)__ldg(A.rect_off + pr.a);
-                offb = (int)__ldg(B.rect_off + pr.b);
-                na = alo.x;
-                nb = blo.x;
-                if (na == 0 && nb == 0) {
-                    fp = PCL_F_EMPTY | 1u << 16;
-                } else if (na == 0 || nb == 0) {
-                    fp = PCL_GATE_E1_MATCH;
-                } else if (gates && na == nb && !ahi.w && !bhi.w &&
-                           (abs((alo.w - alo.z) - (blo.w - blo.z)) > 2 * tol ||
-                            abs((ahi.z - ahi.y) - (bhi.z - bhi.y)) > 2 * tol)) {
-                    fp = PCL_GATE_E2_BBOX;
-                } else {
-                    s0x = (alo.y && blo.y) ? clampi(((alo.z + alo.w) - (blo.z + blo.w)) / 2, -M, M) : 0;
-                    s0y = (ahi.x && bhi.x) ? clampi(((ahi.y + ahi.z) - (bhi.y + bhi.z)) / 2, -M, M) : 0;
-                    open = true;
-                }
-            }
-        }
-        unsigned todo = __ballot_sync(full, open);
-        int4 l0n = none, l1n = none, s0n = none, s1n = none;  // the next pair's polygons
-        auto fetch = [&](int q) {
-            const int ca = __shfl_sync(full, na, q), cb = __shfl_sync(full, nb, q);
-            const int oa = __shfl_sync(full, offa, q), ob = __shfl_sync(full, offb, q);
-            const bool sa = ca <= cb;
-            const int4 *sr = sa ? ra + oa : rb + ob, *lr = sa ? rb + ob : ra + oa;
-            const int ns = sa ? ca : cb, nl = sa ? cb : ca;
-            s0n = lane < ns ? __ldg(sr + lane) : none;
-            s1n = lane + 32 < ns ? __ldg(sr + lane + 32) : none;
-            l0n = lane < nl ? __ldg(lr + lane) : none;
-            l1n = lane + 32 < nl ? __ldg(lr + lane + 32) : none;
-        };
-        if (todo) fetch(__ffs(todo) - 1);
-        while (todo) {
-            const int q = __ffs(todo) - 1;
-            todo &= todo - 1u;
-            const int ca = __shfl_sync(full, na, q), cb = __shfl_sync(full, nb, q);
-            const bool sa = ca <= cb;  // the small clip is A
-            const int ns = sa ? ca : cb, nl = sa ? cb : ca;
-            const int px = __shfl_sync(full, s0x, q), py = __shfl_sync(full, s0y, q);
-            const int4 l0 = l0n, l1 = l1n;
-            __syncwarp();  // the previous pair's polygons are no longer read
-            small[lane] = s0n;
-            if (ns > 32) small[lane + 32] = s1n;
-            __syncwarp();
-            if (todo) fetch(__ffs(todo) - 1);
-            if (nl > 64) {
-                const uint4 w = wide_record(prm, A, B, pairs[t0 + q], lane);
-                if (lane == q) dx = (int)w.x, dy = (int)w.y, E = (int)w.z, fp = w.w;
-                continue;
-            }
-            // an overlap of A's polygon with B's moved by t is the plain overlap
-            // of the small polygon with the large one moved by t (small on side A) or -t
-            const int ux = sa ? px : -px, uy = sa ? py : -py;
-            const bool v0 = lane < nl, v1 = lane + 32 < nl;
-            int c0 = 0, c1 = 0, k0 = -1, k1 = -1;  // hits of this lane's polygons, and by which
-            bool good = true;
-            for (int k = 0; k < ns; ++k) {
-                const int4 s = small[k];
-                const bool h0 = v0 && s.x < l0.z + ux && l0.x + ux < s.z && s.y < l0.w + uy && l0.y + uy < s.w;
-                unsigned b0 = __ballot_sync(full, h0);
-                if (nl > 32) {
-                    const bool h1 = v1 && s.x < l1.z + ux && l1.x + ux < s.z && s.y < l1.w + uy && l1.y + uy < s.w;
-                    const unsigned b1 = __ballot_sync(full, h1);
-                    good = __popc(b0) + __popc(b1) == 1;
-                    c1 += h1 ? 1 : 0;
-                    k1 = h1 ? k : k1;
-                } else {
-                    good = b0 != 0u && !(b0 & (b0 - 1u));
-                }
-                if (!good) break;
-                c0 += h0 ? 1 : 0;
-                k0 = h0 ? k : k0;
-            }
-            good = good && !__any_sync(full, c0 > 1 || c1 > 1);
-            if (!good) {
-                if (lane == q) dx = px, dy = py, fp = PCL_GATE_E1_MATCH;
-                continue;
-            }
-            // displacements d = e_A - e_B of matched edges off the window border
-            int dminx = INT_MAX, dmaxx = INT_MIN, dminy = INT_MAX, dmaxy = INT_MIN;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k = h ? k1 : k0;
-                if (k < 0) continue;
-                const int4 sp = small[k], lp = h ? l1 : l0;
-                const int4 pa = sa ? sp : lp, pb = sa ? lp : sp;
-                if (pa.x != 0 && pb.x != 0) { const int d = pa.x - pb.x; dminx = min(dminx, d); dmaxx = max(dmaxx, d); }
-                if (pa.z != W && pb.z != W) { const int d = pa.z - pb.z; dminx = min(dminx, d); dmaxx = max(dmaxx, d); }
-                if (pa.y != 0 && pb.y != 0) { const int d = pa.y - pb.y; dminy = min(dminy, d); dmaxy = max(dmaxy, d); }
-                if (pa.w != W && pb.w != W) { const int d = pa.w - pb.w; dminy = min(dminy, d); dmaxy = max(dmaxy, d); }
-            }
-            dminx = __reduce_min_sync(full, dminx);
-            dmaxx = __reduce_max_sync(full, dmaxx);
-            dminy = __reduce_min_sync(full, dminy);
-            dmaxy = __reduce_max_sync(full, dmaxy);
-            // Eq. 6 per separable axis: midpoint (trunc toward zero), clamped
-            const bool cx = dminx <= dmaxx, cy = dminy <= dmaxy;
-            const int Tx = cx ? clampi((dminx + dmaxx) / 2, -M, M) : px;
-            const int Ty = cy ? clampi((dminy + dmaxy) / 2, -M, M) : py;
-            const int Ex = cx ? max(Tx - dminx, dmaxx - Tx) : 0;
-            const int Ey = cy ? max(Ty - dminy, dmaxy - Ty) : 0;
-            // the correspondence must hold at T with the same partners: every
-            // lane is hit there by what hit it at the pre-alignment, and by nothing else
-            bool moved = false;
-            if (Tx != px || Ty != py) {
-                const int vx = sa ? Tx : -Tx, vy = sa ? Ty : -Ty;
-                for (int k = 0; k < ns; ++k) {
-                    const int4 s = small[k];
-                    const bool h0 = v0 && s.x < l0.z + vx && l0.x + vx < s.z && s.y < l0.w + vy && l0.y + vy < s.w;
-                    moved = moved || h0 != (k == k0);
-                    if (nl > 32) {
-                        const bool h1 = v1 && s.x < l1.z + vx && l1.x + vx < s.z && s.y < l1.w + vy && l1.y + vy < s.w;
-                        moved = moved || h1 != (k == k1);
-                    }
-                }
-                moved = __any_sync(full, moved);
-            }
-            if (lane == q) {
-                dx = Tx;
-                dy = Ty;
-                E = max(Ex, Ey);
-                fp = PCL_F_ALIGNED | (moved ? PCL_F_EDGE_VERIFY_FAIL : 0u) | (!moved && E <= tol ? 1u << 16 : 0u);
-            }
-        }
-        if (mine) {
-            const pcl_pair pr = pairs[t0 + lane];
-            pcl_record r{};
-            r.a = pr.a;
-            r.b = pr.b;
-            r.mode = PCL_MODE_EDGE;
-            r.dx_dbu = dx;
-            r.dy_dbu = dy;
-            r.score = (uint32_t)E;
-            r.sim = (float)E;
-            r.flags = (uint16_t)fp;
-            r.pass = (uint8_t)(fp >> 16);
-            out[t0 + lane] = r;
-        }
+// Min-Max records of the listed pairs (edge_records)
+struct PairList {
+    static constexpr bool one_class = true;
+    pcl_params prm;
+    pcl_clipset a, b;
+    const pcl_pair *pairs;
+    __device__ __forceinline__ bool item(uint64_t t, pcl_pair &pr, uint32_t &cls) const {
+        pr = pairs[t];
+        cls = 0;
+        return pr.a < a.n_clips && pr.b < b.n_clips;
     }
+    __device__ __forceinline__ const pcl_params &params(uint32_t) const { return prm; }
+    __device__ __forceinline__ const pcl_clipset &A(uint32_t) const { return a; }
+    __device__ __forceinline__ const pcl_clipset &B(uint32_t) const { return b; }
+};
+
+__global__ void __launch_bounds__(256, 3) edge_match_kernel(PairList list, uint64_t n, const unsigned long long *d_n,
+                                                            pcl_record *out) {
+    if (d_n && *d_n < n) n = *d_n;
+    edge_records(list, n, out);
 }
 
 // The exact correspondence (Sec. 2.2.2 condition 1) of the pairs the screen
@@ -669,7 +496,7 @@ cudaError_t launch_edge_match(const pcl_params &prm, const pcl_clipset &a, const
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_match_kernel, 256, 0);
     if (e != cudaSuccess) return e;
     const uint64_t cap = (uint64_t)num_sms * (uint64_t)(per_sm > 0 ? per_sm : 1);  // resident blocks
-    edge_match_kernel<<<(unsigned)(need < cap ? need : cap), 256, 0, st>>>(prm, a, b, pairs, n, d_n, out);
+    edge_match_kernel<<<(unsigned)(need < cap ? need : cap), 256, 0, st>>>(PairList{prm, a, b, pairs}, n, d_n, out);
     return cudaGetLastError();
 }
 

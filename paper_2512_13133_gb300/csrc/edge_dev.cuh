@@ -414,69 +414,6 @@ __device__ inline EdgeOut warp_edge_eval(const ClipView &A, const ClipView &B, i
     return o;
 }
 
-// The gates of the edge-mode record for one pair in one thread (empty clips,
-// E2, the occupancy pre-check of E1): true when the pair passes them and needs
-// the rest of the procedure (then *rec is not set); otherwise *rec is the
-// record warp_edge_record would write.
-__device__ inline bool edge_gate_record(const pcl_params &prm, const pcl_clipset &A, const pcl_clipset &B,
-                                        pcl_pair pr, pcl_record *rec) {
-    pcl_record r{};
-    r.a = pr.a;
-    r.b = pr.b;
-    r.mode = PCL_MODE_EDGE;
-    if (pr.a >= A.n_clips || pr.b >= B.n_clips) {
-        r.flags = PCL_GATE_BAD_INDEX;
-        *rec = r;
-        return false;
-    }
-    const int4 *e4a = reinterpret_cast<const int4 *>(A.esig + (size_t)pr.a * 8);
-    const int4 *e4b = reinterpret_cast<const int4 *>(B.esig + (size_t)pr.b * 8);
-    const int4 alo = __ldg(e4a), ahi = __ldg(e4a + 1), blo = __ldg(e4b), bhi = __ldg(e4b + 1);
-    // {n, hasx, lox, hix}, {hasy, loy, hiy, border}
-    const int na = alo.x, nb = blo.x;
-    if (na == 0 && nb == 0) {
-        r.flags = PCL_F_EMPTY;
-        r.pass = 1;
-        *rec = r;
-        return false;
-    }
-    if (na == 0 || nb == 0) {
-        r.flags = PCL_GATE_E1_MATCH;
-        *rec = r;
-        return false;
-    }
-    if (prm.flags & PCL_P_NO_GATES) return true;
-    const int W = prm.window_dbu, M = prm.marker_dbu, tol = prm.edge_tol_dbu;
-    if (na == nb && !ahi.w && !bhi.w &&
-        (abs((alo.w - alo.z) - (blo.w - blo.z)) > 2 * tol || abs((ahi.z - ahi.y) - (bhi.z - bhi.y)) > 2 * tol)) {
-        r.flags = PCL_GATE_E2_BBOX;
-        *rec = r;
-        return false;
-    }
-    const int s0x = (alo.y && blo.y) ? clampi(((alo.z + alo.w) - (blo.z + blo.w)) / 2, -M, M) : 0;
-    const int s0y = (ahi.x && bhi.x) ? clampi(((ahi.y + ahi.z) - (bhi.y + bhi.z)) / 2, -M, M) : 0;
-    const bool small_is_a = na <= nb;
-    const uint32_t oa = __ldg(A.rect_off + pr.a), ob = __ldg(B.rect_off + pr.b);
-    const int4 *rs = reinterpret_cast<const int4 *>(small_is_a ? A.rects : B.rects) + (small_is_a ? oa : ob);
-    const uint16_t *ro = (small_is_a ? A.rorder : B.rorder) + (small_is_a ? oa : ob);
-    const uint64_t *occ_l = small_is_a ? B.occ + (size_t)pr.b * 64 : A.occ + (size_t)pr.a * 64;
-    const int ns = small_is_a ? na : nb;
-    const int csz = W / 64;
-    const int csh = (csz & (csz - 1)) == 0 ? __ffs(csz) - 1 : -1;
-    const int sx = small_is_a ? -s0x : s0x, sy = small_is_a ? -s0y : s0y;
-    for (int k = 0; k < ns; ++k) {
-        const int4 q = __ldg(rs + __ldg(ro + k));
-        if (!grid_hit(occ_l, q.x + sx, q.y + sy, q.z + sx, q.w + sy, csz, csh)) {
-            r.flags = PCL_GATE_E1_MATCH;
-            r.dx_dbu = s0x;
-            r.dy_dbu = s0y;
-            *rec = r;
-            return false;
-        }
-    }
-    return true;
-}
-
 // One edge-mode record for pair pr (bounds-checked), computed by a whole warp
 // (every lane gets the record)
 __device__ __forceinline__ pcl_record warp_edge_record(const pcl_params &prm, const pcl_clipset &A,
@@ -514,6 +451,214 @@ __device__ __forceinline__ pcl_record warp_edge_record(const pcl_params &prm, co
         r.pass = o.pass ? 1 : 0;
     }
     return r;
+}
+
+// warp_edge_record as {dx, dy, E, flags | pass << 16}; out of line: clips of more
+// than 64 polygons are rare and would cost the loop below registers
+static __device__ __noinline__ uint4 wide_record(const pcl_params &prm, const pcl_clipset &A, const pcl_clipset &B,
+                                          pcl_pair pr, int lane) {
+    const pcl_record r = warp_edge_record(prm, A, B, pr, lane);
+    return make_uint4((uint32_t)r.dx_dbu, (uint32_t)r.dy_dbu, r.score, r.flags | (uint32_t)r.pass << 16);
+}
+
+// Min-Max records, up to 32 pairs per warp at a time: lane q reads pair q's
+// signatures, decides indices, emptiness and E2, and keeps its record; the
+// pairs left go one by one with the whole warp, lane m holding polygons m and
+// m + 32 of the larger clip and the smaller clip's polygons staged in shared
+// memory, the next pair's polygons loading meanwhile.  A lane whose polygon is
+// hit keeps the small polygon that hit it, so that the correspondence (each
+// small polygon hits one lane, no lane is hit twice), the displacements and
+// the re-check at T need no search.  The grid test that the screen runs before
+// the correspondence is left out: it can only reject what the correspondence
+// rejects with the same record.  Clips of more than 64 polygons take
+// warp_edge_record.  Bound by issue slots; 1,000,000 screened pairs of 256x256
+// px: 636 us at 3 CTAs per SM (4 spill: 731) against 1,130 with each pair's signatures read and its
+// record written by one warp at a time; the mixed batch's 2.6 M edge items, half of them of unrelated
+// clips, 886 us against 1,080 with a lane per item testing the grid and a warp per item left.
+// List: item t's clips and class (false: no such clips), and each class's
+// parameters and clip sets.  Blocks of 256 threads.
+template <class List>
+__device__ __forceinline__ void edge_records(const List &list, uint64_t n, pcl_record *out) {
+    const unsigned full = 0xffffffffu;
+    __shared__ int4 small_s[8][64];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int4 *small = small_s[warp];
+    const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const uint64_t per64 = (n + nw - 1) / nw;
+    const uint32_t per = per64 < 32 ? (uint32_t)per64 : 32u;  // a short list is spread over all warps
+    const int4 none = make_int4(0, 0, 0, 0);
+    for (uint64_t t0 = w0 * per; t0 < n; t0 += nw * per) {  // warp-uniform
+        const bool mine = (uint32_t)lane < per && t0 + lane < n;
+        // this lane's record: shift, E, flags | pass << 16
+        int dx = 0, dy = 0, E = 0;
+        uint32_t fp = 0;
+        int offa = 0, na = 0, offb = 0, nb = 0, s0x = 0, s0y = 0;
+        bool open = false;
+        uint32_t cls = 0;
+        if (mine) {
+            pcl_pair pr;
+            if (!list.item(t0 + lane, pr, cls)) {
+                fp = PCL_GATE_BAD_INDEX;
+            } else {
+                const pcl_params &prm = list.params(cls);
+                const pcl_clipset &A = list.A(cls), &B = list.B(cls);
+                const int M = prm.marker_dbu, tol = prm.edge_tol_dbu;
+                const bool gates = !(prm.flags & PCL_P_NO_GATES);
+                const int4 *e4a = reinterpret_cast<const int4 *>(A.esig + (size_t)pr.a * 8);
+                const int4 *e4b = reinterpret_cast<const int4 *>(B.esig + (size_t)pr.b * 8);
+                const int4 alo = __ldg(e4a), ahi = __ldg(e4a + 1), blo = __ldg(e4b), bhi = __ldg(e4b + 1);
+                // {n, hasx, lox, hix}, {hasy, loy, hiy, border}
+                offa = (int)__ldg(A.rect_off + pr.a);
+                offb = (int)__ldg(B.rect_off + pr.b);
+                na = alo.x;
+                nb = blo.x;
+                if (na == 0 && nb == 0) {
+                    fp = PCL_F_EMPTY | 1u << 16;
+                } else if (na == 0 || nb == 0) {
+                    fp = PCL_GATE_E1_MATCH;
+                } else if (gates && na == nb && !ahi.w && !bhi.w &&
+                           (abs((alo.w - alo.z) - (blo.w - blo.z)) > 2 * tol ||
+                            abs((ahi.z - ahi.y) - (bhi.z - bhi.y)) > 2 * tol)) {
+                    fp = PCL_GATE_E2_BBOX;
+                } else {
+                    s0x = (alo.y && blo.y) ? clampi(((alo.z + alo.w) - (blo.z + blo.w)) / 2, -M, M) : 0;
+                    s0y = (ahi.x && bhi.x) ? clampi(((ahi.y + ahi.z) - (bhi.y + bhi.z)) / 2, -M, M) : 0;
+                    open = true;
+                }
+            }
+        }
+        unsigned todo = __ballot_sync(full, open);
+        int4 l0n = none, l1n = none, s0n = none, s1n = none;  // the next pair's polygons
+        auto class_of = [&](int q) { return List::one_class ? 0u : __shfl_sync(full, cls, q); };
+        auto fetch = [&](int q) {
+            const uint32_t c = class_of(q);
+            const int4 *ra = reinterpret_cast<const int4 *>(list.A(c).rects);
+            const int4 *rb = reinterpret_cast<const int4 *>(list.B(c).rects);
+            const int ca = __shfl_sync(full, na, q), cb = __shfl_sync(full, nb, q);
+            const int oa = __shfl_sync(full, offa, q), ob = __shfl_sync(full, offb, q);
+            const bool sa = ca <= cb;
+            const int4 *sr = sa ? ra + oa : rb + ob, *lr = sa ? rb + ob : ra + oa;
+            const int ns = sa ? ca : cb, nl = sa ? cb : ca;
+            s0n = lane < ns ? __ldg(sr + lane) : none;
+            s1n = lane + 32 < ns ? __ldg(sr + lane + 32) : none;
+            l0n = lane < nl ? __ldg(lr + lane) : none;
+            l1n = lane + 32 < nl ? __ldg(lr + lane + 32) : none;
+        };
+        if (todo) fetch(__ffs(todo) - 1);
+        while (todo) {
+            const int q = __ffs(todo) - 1;
+            todo &= todo - 1u;
+            const int ca = __shfl_sync(full, na, q), cb = __shfl_sync(full, nb, q);
+            const bool sa = ca <= cb;  // the small clip is A
+            const int ns = sa ? ca : cb, nl = sa ? cb : ca;
+            const int px = __shfl_sync(full, s0x, q), py = __shfl_sync(full, s0y, q);
+            const int4 l0 = l0n, l1 = l1n;
+            const uint32_t c = class_of(q);
+            const int W = list.params(c).window_dbu, M = list.params(c).marker_dbu, tol = list.params(c).edge_tol_dbu;
+            __syncwarp();  // the previous pair's polygons are no longer read
+            small[lane] = s0n;
+            if (ns > 32) small[lane + 32] = s1n;
+            __syncwarp();
+            if (todo) fetch(__ffs(todo) - 1);
+            if (nl > 64) {
+                pcl_pair pr;
+                uint32_t same;
+                list.item(t0 + q, pr, same);
+                const uint4 w = wide_record(list.params(c), list.A(c), list.B(c), pr, lane);
+                if (lane == q) dx = (int)w.x, dy = (int)w.y, E = (int)w.z, fp = w.w;
+                continue;
+            }
+            // an overlap of A's polygon with B's moved by t is the plain overlap
+            // of the small polygon with the large one moved by t (small on side A) or -t
+            const int ux = sa ? px : -px, uy = sa ? py : -py;
+            const bool v0 = lane < nl, v1 = lane + 32 < nl;
+            int c0 = 0, c1 = 0, k0 = -1, k1 = -1;  // hits of this lane's polygons, and by which
+            bool good = true;
+            for (int k = 0; k < ns; ++k) {
+                const int4 s = small[k];
+                const bool h0 = v0 && s.x < l0.z + ux && l0.x + ux < s.z && s.y < l0.w + uy && l0.y + uy < s.w;
+                unsigned b0 = __ballot_sync(full, h0);
+                if (nl > 32) {
+                    const bool h1 = v1 && s.x < l1.z + ux && l1.x + ux < s.z && s.y < l1.w + uy && l1.y + uy < s.w;
+                    const unsigned b1 = __ballot_sync(full, h1);
+                    good = __popc(b0) + __popc(b1) == 1;
+                    c1 += h1 ? 1 : 0;
+                    k1 = h1 ? k : k1;
+                } else {
+                    good = b0 != 0u && !(b0 & (b0 - 1u));
+                }
+                if (!good) break;
+                c0 += h0 ? 1 : 0;
+                k0 = h0 ? k : k0;
+            }
+            good = good && !__any_sync(full, c0 > 1 || c1 > 1);
+            if (!good) {
+                if (lane == q) dx = px, dy = py, fp = PCL_GATE_E1_MATCH;
+                continue;
+            }
+            // displacements d = e_A - e_B of matched edges off the window border
+            int dminx = INT_MAX, dmaxx = INT_MIN, dminy = INT_MAX, dmaxy = INT_MIN;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = h ? k1 : k0;
+                if (k < 0) continue;
+                const int4 sp = small[k], lp = h ? l1 : l0;
+                const int4 pa = sa ? sp : lp, pb = sa ? lp : sp;
+                if (pa.x != 0 && pb.x != 0) { const int d = pa.x - pb.x; dminx = min(dminx, d); dmaxx = max(dmaxx, d); }
+                if (pa.z != W && pb.z != W) { const int d = pa.z - pb.z; dminx = min(dminx, d); dmaxx = max(dmaxx, d); }
+                if (pa.y != 0 && pb.y != 0) { const int d = pa.y - pb.y; dminy = min(dminy, d); dmaxy = max(dmaxy, d); }
+                if (pa.w != W && pb.w != W) { const int d = pa.w - pb.w; dminy = min(dminy, d); dmaxy = max(dmaxy, d); }
+            }
+            dminx = __reduce_min_sync(full, dminx);
+            dmaxx = __reduce_max_sync(full, dmaxx);
+            dminy = __reduce_min_sync(full, dminy);
+            dmaxy = __reduce_max_sync(full, dmaxy);
+            // Eq. 6 per separable axis: midpoint (trunc toward zero), clamped
+            const bool cx = dminx <= dmaxx, cy = dminy <= dmaxy;
+            const int Tx = cx ? clampi((dminx + dmaxx) / 2, -M, M) : px;
+            const int Ty = cy ? clampi((dminy + dmaxy) / 2, -M, M) : py;
+            const int Ex = cx ? max(Tx - dminx, dmaxx - Tx) : 0;
+            const int Ey = cy ? max(Ty - dminy, dmaxy - Ty) : 0;
+            // the correspondence must hold at T with the same partners: every
+            // lane is hit there by what hit it at the pre-alignment, and by nothing else
+            bool moved = false;
+            if (Tx != px || Ty != py) {
+                const int vx = sa ? Tx : -Tx, vy = sa ? Ty : -Ty;
+                for (int k = 0; k < ns; ++k) {
+                    const int4 s = small[k];
+                    const bool h0 = v0 && s.x < l0.z + vx && l0.x + vx < s.z && s.y < l0.w + vy && l0.y + vy < s.w;
+                    moved = moved || h0 != (k == k0);
+                    if (nl > 32) {
+                        const bool h1 = v1 && s.x < l1.z + vx && l1.x + vx < s.z && s.y < l1.w + vy && l1.y + vy < s.w;
+                        moved = moved || h1 != (k == k1);
+                    }
+                }
+                moved = __any_sync(full, moved);
+            }
+            if (lane == q) {
+                dx = Tx;
+                dy = Ty;
+                E = max(Ex, Ey);
+                fp = PCL_F_ALIGNED | (moved ? PCL_F_EDGE_VERIFY_FAIL : 0u) | (!moved && E <= tol ? 1u << 16 : 0u);
+            }
+        }
+        if (mine) {
+            pcl_pair pr;
+            list.item(t0 + lane, pr, cls);
+            pcl_record r{};
+            r.a = pr.a;
+            r.b = pr.b;
+            r.mode = PCL_MODE_EDGE;
+            r.dx_dbu = dx;
+            r.dy_dbu = dy;
+            r.score = (uint32_t)E;
+            r.sim = (float)E;
+            r.flags = (uint16_t)fp;
+            r.pass = (uint8_t)(fp >> 16);
+            out[t0 + lane] = r;
+        }
+    }
 }
 
 }  // namespace edge_dev

@@ -4,14 +4,13 @@
 // The work list holds the cosine items first, then the edge items.  Every
 // kernel is persistent (a grid sized to the GPU) and finds its items in the
 // list itself, so the whole batch is a fixed sequence of launches that a CUDA
-// graph can replay: the edge items (lanes run the gates, the whole warp
-// evaluates the survivors); the cosine gates, at full occupancy (the alignment
+// graph can replay: the edge items (edge_records, as for a pair list); the cosine gates, at full occupancy (the alignment
 // bodies' registers and shared memory would leave ten warps per SM); then per
 // size class the alignment of the items the gates left, marked in their
 // records, by the FFT body of that size (512x512 px, beyond its shared memory:
 // the exact window scan).  The register DFT radix (2 or 4), the CTAs per SM and
 // the items a gating warp claims are tuning parameters (chosen by the
-// autotuner).  5.2 M items over 4 x 5,000 clips of 64-512 px: 2.8 ms against
+// autotuner).  5.2 M items over 4 x 5,000 clips of 64-512 px: 2.34 ms against
 // 7.7 with gates, alignment and edge items in one kernel of 320-thread CTAs.
 #include "edge_dev.cuh"
 #include "exact_dev.cuh"
@@ -50,25 +49,34 @@ __global__ void mark_mixed_kernel(MixedArgs args, const pcl_work *work, uint64_t
 
 // Cosine items, `claim` consecutive ones per warp at a time.  A lane takes an
 // item's indices, emptiness and areas (G1, which ends most items of unrelated
-// clips); the warp then takes G3 and G2 of the rest one after the other.  An
-// item that ends here gets its record, the others a record with flags = kPending.
+// clips) and the largest overlap that fails Eq. 2; the warp then takes G3 and G2 of the rest
+// one after the other, the next item's first 64 blocks loading while one is
+// tested.  An item that ends here gets its record, the others a record with
+// flags = kPending.  Bound by issue slots: 2.6 M items, 1,090 us against 1,400 with the
+// class's geometry, the overlap bound and the areas found by the whole warp for each item.
 __global__ void __launch_bounds__(256) mixed_gate_kernel(MixedArgs args, const pcl_work *work, uint64_t n_cos,
                                                          pcl_record *out, unsigned long long *cursor, int claim) {
+    const unsigned full = 0xffffffffu;
     __shared__ uint16_t g2_scratch[8 * kG2Scratch];
+    __shared__ Geo geo[kMaxClasses];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint16_t *scratch = g2_scratch + warp * kG2Scratch;
+    if (threadIdx.x < args.n_classes) geo[threadIdx.x] = make_geo(args.prm[threadIdx.x]);
+    __syncthreads();
     for (;;) {
         uint64_t t0 = 0;
         if (lane == 0) t0 = atomicAdd(cursor, (unsigned long long)claim);
-        t0 = __shfl_sync(0xffffffffu, t0, 0);
+        t0 = __shfl_sync(full, t0, 0);
         if (t0 >= n_cos) break;
         const uint64_t t1 = min(n_cos, t0 + (uint64_t)claim);
         for (uint64_t b = t0; b < t1; b += 32) {
             const uint64_t t = b + lane;
             pcl_work w{};
+            int um = 0, area_a = 0, area_b = 0;
             bool open = false;
+            pcl_record rec{};
             if (t < t1) {
                 w = work[t];
-                pcl_record rec{};
                 rec.a = w.a;
                 rec.b = w.b;
                 rec.mode = PCL_MODE_COSINE;
@@ -77,7 +85,7 @@ __global__ void __launch_bounds__(256) mixed_gate_kernel(MixedArgs args, const p
                 } else {
                     const pcl_params &prm = args.prm[w.cls];
                     const pcl_clipset &cs = args.cs[w.cls];
-                    const Geo g = make_geo(prm);
+                    const Geo &g = geo[w.cls];
                     const uint64_t pa = cs.pop[w.a], pb = cs.pop[w.b];
                     const uint64_t mn = pa < pb ? pa : pb, mx = pa < pb ? pb : pa;
                     if ((g.P > 32 && (g.P != 64 || prm.shift_rule != PCL_SHIFT_EXACT_ARGMAX)) || g.S > g.N / 16) {
@@ -92,25 +100,69 @@ __global__ void __launch_bounds__(256) mixed_gate_kernel(MixedArgs args, const p
                         rec.flags = PCL_GATE_G1_AREA;
                     } else {
                         open = true;
+                        area_a = (int)pa;
+                        area_b = (int)pb;
+                        um = (int)cos_umax(pa, pb, prm.cos_num, prm.cos_den);
                     }
                 }
-                if (!open) out[t] = rec;
             }
-            unsigned m = __ballot_sync(0xffffffffu, open);
+            unsigned m = __ballot_sync(full, open);
+            uint32_t ca = 0, da = 0, cb = 0, db = 0;  // the next item's first chunk: counts and neighbourhood sums
+            auto fetch = [&](int q) {
+                const uint32_t c = __shfl_sync(full, (uint32_t)w.cls, q);
+                const uint32_t qa = __shfl_sync(full, w.a, q), qb = __shfl_sync(full, w.b, q);
+                const int nb2 = geo[c].nb * geo[c].nb, words = nb2 / 2;
+                const uint32_t *x = reinterpret_cast<const uint32_t *>(args.cs[c].blk) + (size_t)qa * nb2;
+                const uint32_t *y = reinterpret_cast<const uint32_t *>(args.cs[c].blk) + (size_t)qb * nb2;
+                const bool v = lane < words;
+                ca = v ? __ldg(x + lane) : 0u;
+                da = v ? __ldg(x + words + lane) : 0u;
+                cb = v ? __ldg(y + lane) : 0u;
+                db = v ? __ldg(y + words + lane) : 0u;
+            };
+            if (m) fetch(__ffs(m) - 1);
             while (m) {
-                const int src = __ffs(m) - 1;
+                const int q = __ffs(m) - 1;
                 m &= m - 1u;
-                const uint32_t c = __shfl_sync(0xffffffffu, (uint32_t)w.cls, src);
-                pcl_record rec{};
-                rec.a = __shfl_sync(0xffffffffu, w.a, src);
-                rec.b = __shfl_sync(0xffffffffu, w.b, src);
-                rec.mode = PCL_MODE_COSINE;
-                const pcl_params &prm = args.prm[c];
-                const int gate = warp_cosine_gate(args.cs[c], rec.a, args.cs[c], rec.b, make_geo(prm), prm.cos_num,
-                                                  prm.cos_den, lane, g2_scratch + warp * kG2Scratch);
-                rec.flags = gate ? (uint16_t)gate : kPending;
-                if (lane == 0) out[b + src] = rec;
+                const uint32_t c = __shfl_sync(full, (uint32_t)w.cls, q);
+                const uint32_t qa = __shfl_sync(full, w.a, q), qb = __shfl_sync(full, w.b, q);
+                const int u = __shfl_sync(full, um, q);
+                const int tA = __shfl_sync(full, area_a, q) - u, tB = __shfl_sync(full, area_b, q) - u;
+                // G3 (warp_g3_rejects), 64 blocks at a time
+                uint32_t sa = __reduce_add_sync(full, ca - __vminu2(ca, db));
+                uint32_t sb = __reduce_add_sync(full, cb - __vminu2(cb, da));
+                if (m) fetch(__ffs(m) - 1);
+                int DA = (int)((sa & 0xffffu) + (sa >> 16)), DB = (int)((sb & 0xffffu) + (sb >> 16));
+                bool rej = DA >= tA || DB >= tB;
+                const Geo &g = geo[c];
+                const pcl_clipset &cs = args.cs[c];
+                const int nb2 = g.nb * g.nb, words = nb2 / 2;
+                const uint32_t *x = reinterpret_cast<const uint32_t *>(cs.blk) + (size_t)qa * nb2;
+                const uint32_t *y = reinterpret_cast<const uint32_t *>(cs.blk) + (size_t)qb * nb2;
+                for (int k = 32 + lane; !rej && k < words; k += 32) {  // past 32 words there are a multiple of 32
+                    const uint32_t c0 = __ldg(x + k), d0 = __ldg(x + words + k), c1 = __ldg(y + k),
+                                   d1 = __ldg(y + words + k);
+                    sa = __reduce_add_sync(full, c0 - __vminu2(c0, d1));
+                    sb = __reduce_add_sync(full, c1 - __vminu2(c1, d0));
+                    DA += (int)((sa & 0xffffu) + (sa >> 16));
+                    DB += (int)((sb & 0xffffu) + (sb >> 16));
+                    rej = DA >= tA || DB >= tB;
+                }
+                uint16_t flags = PCL_GATE_G3_DENSITY;
+                if (!rej) {
+                    const uint16_t *pa = cs.prof + (size_t)qa * 2 * g.N, *pb = cs.prof + (size_t)qb * 2 * g.N;
+                    bool g2;
+                    switch (g.N) {
+                        case 64: g2 = warp_g2_rejects_groups<2>(pa, pb, g.S, u, lane, scratch); break;
+                        case 128: g2 = warp_g2_rejects_groups<4>(pa, pb, g.S, u, lane, scratch); break;
+                        case 256: g2 = warp_g2_rejects_groups<8>(pa, pb, g.S, u, lane, scratch); break;
+                        default: g2 = warp_g2_rejects_groups<16>(pa, pb, g.S, u, lane, scratch); break;
+                    }
+                    flags = g2 ? PCL_GATE_G2_PROFILE : kPending;
+                }
+                if (lane == q) rec.flags = flags;
             }
+            if (t < t1) out[t] = rec;
         }
     }
 }
@@ -188,41 +240,24 @@ __global__ void __launch_bounds__(AlignCta<P>::threads, AlignCta<P>::ctas)
     }
 }
 
-// Edge items: each lane takes one item and runs its gates (most items end
-// there); the whole warp then evaluates the survivors one at a time
-// (warp_edge_record).  Warps stride the list 32 items at a time.
-__global__ void __launch_bounds__(256) mixed_edge_kernel(MixedArgs args, const pcl_work *work, uint64_t n_cos,
-                                                         uint64_t n, pcl_record *out) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t gw = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t base = n_cos + 32 * gw; base < n; base += 32 * nw) {
-        const uint64_t t = base + lane;
-        bool surv_e = false;
-        pcl_work w{};
-        if (t < n) {
-            w = work[t];
-            pcl_record r{};
-            if (w.cls >= args.n_classes) {
-                r.a = w.a;
-                r.b = w.b;
-                r.mode = PCL_MODE_EDGE;
-                r.flags = PCL_GATE_BAD_INDEX;
-            } else {
-                surv_e = edge_gate_record(args.prm[w.cls], args.cs[w.cls], args.cs[w.cls], pcl_pair{w.a, w.b}, &r);
-            }
-            if (!surv_e) out[t] = r;
-        }
-        unsigned m = __ballot_sync(0xffffffffu, surv_e);
-        while (m) {
-            const int src = __ffs(m) - 1;
-            m &= m - 1;
-            const uint32_t cls = __shfl_sync(0xffffffffu, (uint32_t)w.cls, src);
-            const uint32_t a = __shfl_sync(0xffffffffu, w.a, src), b = __shfl_sync(0xffffffffu, w.b, src);
-            const pcl_record r = warp_edge_record(args.prm[cls], args.cs[cls], args.cs[cls], pcl_pair{a, b}, lane);
-            if (lane == 0) out[base + src] = r;
-        }
+// Edge items (edge_records)
+struct EdgeItems {
+    static constexpr bool one_class = false;
+    MixedArgs args;
+    const pcl_work *work;
+    __device__ __forceinline__ bool item(uint64_t t, pcl_pair &pr, uint32_t &cls) const {
+        const pcl_work w = work[t];
+        pr = pcl_pair{w.a, w.b};
+        cls = w.cls < args.n_classes ? w.cls : 0u;
+        return w.cls < args.n_classes && w.a < args.cs[cls].n_clips && w.b < args.cs[cls].n_clips;
     }
+    __device__ __forceinline__ const pcl_params &params(uint32_t c) const { return args.prm[c]; }
+    __device__ __forceinline__ const pcl_clipset &A(uint32_t c) const { return args.cs[c]; }
+    __device__ __forceinline__ const pcl_clipset &B(uint32_t c) const { return args.cs[c]; }
+};
+
+__global__ void __launch_bounds__(256, 3) mixed_edge_kernel(EdgeItems items, uint64_t n, pcl_record *out) {
+    edge_records(items, n, out);
 }
 
 template <int P, int RADIX>
@@ -267,7 +302,7 @@ cudaError_t launch_mixed(const pcl_params *prm, const pcl_clipset *sets, uint32_
         }
     }
     if (n == 0) return cudaSuccess;
-    if (n > n_cos) mixed_edge_kernel<<<num_sms * 8, 256, 0, st>>>(args, work, n_cos, n, out);
+    if (n > n_cos) mixed_edge_kernel<<<num_sms * 3, 256, 0, st>>>(EdgeItems{args, work + n_cos}, n - n_cos, out + n_cos);
     if (n_cos) {
         mixed_gate_kernel<<<num_sms * 8, 256, 0, st>>>(args, work, n_cos, out, cursor, claim);
         for (uint32_t c = 0; c < n_classes; ++c) {
