@@ -34,16 +34,19 @@
 // pairs: E2's rejections are counted among the clips of equal polygon count
 // without border edges, and E1 is all pairs minus the survivors minus E2.
 //
-// Bound: issue slots (65 % busy) and table reads (L1 70 %, mostly from L2).
-// 100,000 clips of 256x256 px (5.0e9 pairs), one GB300: 10.2 ms a call - the
-// screen 6.1 ms, the exact check of 15 M pairs 3.1 ms, the tables (0.8 GB
+// Bound: issue slots, table reads (mostly from L2) and their latency together.
+// 100,000 clips of 256x256 px (5.0e9 pairs), one GB300: 10.0 ms a call - the
+// screen 5.7 ms, the exact check of 15 M pairs 3.1 ms, the tables (0.8 GB
 // written, 134 MB held) 0.26 ms, the sort and E2 0.2 ms - against 78.6 ms for
 // the screen of pairs one by one in tiles (edge.cu), which stays for shards of
 // the pair space, two clip sets and the topological pre-screen.  At 1,000
 // clips the two take the same 0.1 ms.  Measured on the way: a table per group
 // instead of per four interleaved groups 7.6 ms for the screen (more L1 tags
-// per read), one polygon at a time 11.0 ms (latency), 5 or 8 CTAs per SM 6.4
-// and 6.5 ms; the check without the next pair's loads in flight 3.7 ms.
+// per read), one polygon at a time 11.0 ms and two 6.1 (latency), 5 or 8 CTAs
+// per SM 6.4 and 6.5 ms with two, entries for every width of 1 to 8 cells (half the
+// reads, twice the tables) 6.4 ms with two and 6.0 with four, eight groups per warp
+// with the lower words read only where they have members 6.4 ms; the check
+// without the next pair's loads in flight 3.7 ms.
 #include <type_traits>
 
 #include "edge_dev.cuh"
@@ -517,17 +520,22 @@ __global__ void __launch_bounds__(256, 6) join_screen_kernel(pcl_params prm, pcl
             }
             const bool wide = __any_sync(0xffffffffu, place.y & kWide);
             bool any = true;
-            // two polygons at a time: eight independent loads
-            for (int k = 0; k < 8 && k0 + k < nu; k += 2) {
-                const int src = (lane & 24) | k;
-                const uint32_t x0 = __shfl_sync(0xffffffffu, place.x, src), y0 = __shfl_sync(0xffffffffu, place.y, src);
-                const uint32_t x1 = __shfl_sync(0xffffffffu, place.x, src + 1);
-                const uint32_t y1 = __shfl_sync(0xffffffffu, place.y, src + 1);
+            // four polygons at a time: sixteen independent loads (past the last polygon: the entry of ones)
+            for (int k = 0; k < 8 && k0 + k < nu; k += 4) {
+                uint32_t x[4], y[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    x[j] = __shfl_sync(0xffffffffu, place.x, (lane & 24) | (k + j));
+                    y[j] = __shfl_sync(0xffffffffu, place.y, (lane & 24) | (k + j));
+                }
                 if (!wide) {
-                    if (m) m &= covered(x0, y0) & covered(x1, y1);
+                    if (m) m &= (covered(x[0], y[0]) & covered(x[1], y[1])) & (covered(x[2], y[2]) & covered(x[3], y[3]));
                 } else {
-                    const uint32_t b0 = __shfl_sync(0xffffffffu, box, src), b1 = __shfl_sync(0xffffffffu, box, src + 1);
-                    if (m) m &= covered_wide(x0, y0, b0) & covered_wide(x1, y1, b1);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const uint32_t bj = __shfl_sync(0xffffffffu, box, (lane & 24) | (k + j));
+                        if (m) m &= covered_wide(x[j], y[j], bj);
+                    }
                 }
                 any = __any_sync(0xffffffffu, m != 0u);
                 if (!any) break;
