@@ -88,30 +88,32 @@ def peaks():
 
 
 # DRAM bytes (read + write) per launch of the kernels on the default scale
-# workload, from single-pass ncu captures (dram__bytes_read.sum +
-# dram__bytes_write.sum) of `bench.py --only edge|band` at 100,000 clips
+# workload, from ncu captures (dram__bytes_read.sum +
+# dram__bytes_write.sum) of the step at 100,000 clips
 # and of `bench.py --only fft --clips 10000` (the FFT figure is per pair:
 # every pair reads its member's spectrum, so a launch's traffic grows with
 # its pairs).  A
 # figure counts only while the kernel's sources hash as they did when it was
 # taken; otherwise the bench reports null.
 TRAFFIC = {
-    "cand_edge": {"sources": {"paper_2512_13133_gb300/csrc/edge.cu":
-                              "7349ebd251d836e7fc04690f8b35fdd30c83e684cafe58233c1fb6738c3a06b4",
+    "cand_edge": {"sources": {"paper_2512_13133_gb300/csrc/edge_join.cu":
+                              "a98420467a82b2cd50f154de3548627a18ed09acd0a9bcf5627b862a081e4995",
                               "paper_2512_13133_gb300/csrc/edge_dev.cuh":
-                              "91b43fe9f14b6cc097d8b42b10055358e7d3ba02c7518a45ff01bacbb54247c7"},
-                  # the screen (1.63 GB + 201.62 MB) and its list's check (257.92 + 16.15 MB)
-                  "bytes": 1.63e9 + 201.62e6 + 257.92e6 + 16.15e6},
-    "cand_cos": {"sources": {"paper_2512_13133_gb300/csrc/gates.cu":
-                             "5935883332fb8b84d06ddb62a40a0e119ddaeb97da669f62ebc438834c34e99b",
-                             "paper_2512_13133_gb300/csrc/gates.cuh":
-                             "7383112e07955c850196dd11d6cdf0d93e2e08c1eab2c834c73868a92928f7d0"},
-                 "bytes": 185.34e6 + 4.26e6},
+                              "4f1e36548acb751b0875d56619a4f35f69b46bd22ae3b093f125dd69dad76d12"},
+                  # the screen (1.74 GB + 668 MB), its tables (60 + 478 MB), the check of its list
+                  # (241 MB) and the sort (47 MB)
+                  "bytes": 1.737e9 + 668.1e6 + 59.7e6 + 477.8e6 + 241.0e6 + 46.9e6},
+    "cand_cos": {"sources": {"paper_2512_13133_gb300/csrc/band_mma.cu":
+                              "6fab5e9b089beff9dd83d8c414d24764305e07e216e42720901b078919709024",
+                              "paper_2512_13133_gb300/csrc/gates.cuh":
+                              "92d997f60ce4817716d6079168f3f8c8143326c9a15e4d69bfd84c6e4a0c5d98"},
+                 # the list's check (188 MB), the product (215 MB), the vectors (249 MB), the sort
+                 "bytes": 188.1e6 + 214.7e6 + 249.3e6 + 1.5e6},
     "fft_pair": {"sources": {"paper_2512_13133_gb300/csrc/fft.cu":
-                             "177f4ab710f11721ca4eafa1eb5504eab2340ddff890639dd517e226bbcea14a",
-                             "paper_2512_13133_gb300/csrc/fft_dev.cuh":
-                             "4d9f3af534542246324fde57ec52870a89fd65b7e26992bfb3de8f32547de133"},
-                 "bytes_per_pair": (21.04e9 + 6.18e6) / 56470},
+                              "87068e32a9adbbc12751aebb076eb2d08762b38077946e59b51789a3ab87d8d2",
+                              "paper_2512_13133_gb300/csrc/fft_dev.cuh":
+                              "06abd6fe56cba25f508b157a7acc2c72976652ee0c65bf2a3b4fed1e2c102011"},
+                 "bytes_per_pair": (23.65e9 + 5.82e6) / 56470},
 }
 
 
@@ -129,6 +131,11 @@ def captured_traffic(stage: str, default_workload: bool, pairs: int = 0):
         except OSError:
             return None
     return t["bytes_per_pair"] * pairs if "bytes_per_pair" in t else t["bytes"]
+
+
+def product_join(N: int, n: int) -> bool:
+    """whether the cosine self-join takes G3 as a matrix product"""
+    return N in (256, 512) and n >= 2048
 
 
 def alu_peak_tops(sm_mhz: float) -> float:
@@ -1004,25 +1011,32 @@ def run_ours(args, rank, world, local_rank):
             for name, lst in (("same_seed", fp), ("dense32", dense)):
                 tl = torch.from_numpy(np.ascontiguousarray(lst)).to(dev)
                 rl = torch.empty((len(lst), 40), dtype=torch.uint8, device=dev)
-                pcl.pcl_match_pairs(ctx, Pt, pcl.MODE_COSINE, cs, cs, tl, rl)
-                torch.cuda.synchronize()
-                t_ms = []
-                for _ in range(max(args.steps, 1)):
-                    flush.zero_()
-                    a0 = torch.cuda.Event(enable_timing=True)
-                    a1 = torch.cuda.Event(enable_timing=True)
-                    a0.record()
+                # as a user calls it (pairs that can take their overlaps from the rectangles),
+                # and with a wait limit of the context's own, which keeps every pair on the
+                # tensor cores: only that is set against their peak
+                means = []
+                for limit in (1_000_000_000, 0):
+                    pcl.pcl_set_wait_limit(ctx, limit)
                     pcl.pcl_match_pairs(ctx, Pt, pcl.MODE_COSINE, cs, cs, tl, rl)
-                    a1.record()
                     torch.cuda.synchronize()
-                    t_ms.append(a0.elapsed_time(a1))
-                ms = float(np.mean(t_ms))
+                    t_ms = []
+                    for _ in range(max(args.steps, 1)):
+                        flush.zero_()
+                        a0 = torch.cuda.Event(enable_timing=True)
+                        a1 = torch.cuda.Event(enable_timing=True)
+                        a0.record()
+                        pcl.pcl_match_pairs(ctx, Pt, pcl.MODE_COSINE, cs, cs, tl, rl)
+                        a1.record()
+                        torch.cuda.synchronize()
+                        t_ms.append(a0.elapsed_time(a1))
+                    means.append(float(np.mean(t_ms)))
+                tensor_ms, ms = means
                 flop = 2.0 * (2 * cs.S + 1) ** 2 * cs.N * cs.N * len(lst)
                 key = f"{eng_name}_{name}"
                 tc[key] = {"pairs": int(len(lst)), "ms": ms, "pairs_per_s": len(lst) / (ms / 1e3),
-                           "tflops_useful": flop / (ms / 1e3) / 1e12,
+                           "tensor_ms": tensor_ms, "tflops_useful": flop / (tensor_ms / 1e3) / 1e12,
                            "peak_tflops": pk["bf16_tflops"] * peak_mult,
-                           "frac_of_peak": flop / (ms / 1e3) / 1e12 / (pk["bf16_tflops"] * peak_mult)}
+                           "frac_of_peak": flop / (tensor_ms / 1e3) / 1e12 / (pk["bf16_tflops"] * peak_mult)}
                 if name == "dense32":
                     rt = pcl.records_to_numpy(rl)
                     tc[key]["agrees_with_fft"] = bool((rt["score"] == dense_fft["score"]).all() and
@@ -1226,18 +1240,20 @@ def run_ours(args, rank, world, local_rank):
         ach = ops / (per_stage[dom] / 1e3) / 1e12
         roof = {"bound": "alu", "achieved": ach, "peak": alu_peak_tops(2070.0), "unit": "Tops/s"}
     elif dom == "cand_edge":
-        # algorithmic work: the plain E1 procedure's overlap tests (8 integer
-        # ops each: four compares, three ANDs, one count) plus 20 ops of
-        # pre-alignment per pair; the kernel reaches the same decisions with
-        # an occupancy-grid pre-check, so this is an effective rate
+        # the self-join tests 32 pairs per operation, so there is no count of
+        # operations per pair to set against the ALU peak; beside the rate,
+        # what the plain E1 procedure's overlap tests (8 integer ops each: four
+        # compares, three ANDs, one count) plus 20 ops of pre-alignment per
+        # pair would amount to
         tpp = plain_e1_tests_per_pair(wl)
-        ops = total_pairs * (20 + 8 * tpp)
-        ach = ops / (per_stage[dom] / 1e3) / 1e12
-        roof = {"bound": "alu", "achieved": ach, "peak": alu_peak_tops(2070.0), "unit": "Tops/s",
-                "work": f"{20 + 8 * tpp:.0f} int ops/pair (plain E1: {tpp:.1f} overlap tests/pair)"}
+        sec = per_stage[dom] / 1e3
+        roof = {"bound": "issue slots, table reads and their latency", "achieved": total_pairs / sec / 1e9,
+                "peak": None, "unit": "Gpairs/s", "work": "pairs screened",
+                "plain_procedure": {"int_ops_per_pair": 20 + 8 * tpp, "overlap_tests_per_pair": tpp,
+                                    "effective_tops": total_pairs * (20 + 8 * tpp) / sec / 1e12}}
     else:
         roof = {"bound": "alu", "achieved": None, "peak": alu_peak_tops(2070.0), "unit": "Tops/s"}
-    roof["frac"] = (roof["achieved"] / roof["peak"]) if roof.get("achieved") else None
+    roof["frac"] = (roof["achieved"] / roof["peak"]) if roof.get("achieved") and roof["peak"] else None
     roof["traffic"] = captured_traffic(dom, args.config == "scale" and not args.clips)
     roof["kernel"] = dom
     roof["peak_source"] = pk_kind
@@ -1255,10 +1271,17 @@ def run_ours(args, rank, world, local_rank):
                                 "peak": pk["hbm_gbs"], "unit": "GB/s",
                                 "work": "N^2/8 + 4N + 4 nb^2 + 36 B written per clip + rectangles read"})
     band = int(g[0][0] + g[0][2] + g[0][3])
-    rooflines["cand_cos"] = frac({"bound": "alu", "achieved": band * 4 * nb * nb / (per_stage["cand_cos"] / 1e3) / 1e12,
-                                  "peak": alu_peak_tops(2070.0), "unit": "Tops/s",
-                                  "work": f"{band} band pairs (G1 survivors) x 4 nb^2 integer ops (G3 both ways)",
-                                  "traffic": captured_traffic("cand_cos", args.config == "scale" and not args.clips)})
+    traffic_cos = captured_traffic("cand_cos", args.config == "scale" and not args.clips)
+    if product_join(N, n):
+        rooflines["cand_cos"] = frac({"bound": "tensor", "achieved": band * 2 * 1024 / (per_stage["cand_cos"] / 1e3) / 1e12,
+                                      "peak": 2 * pk["bf16_tflops"], "unit": "TFLOP/s",
+                                      "work": f"{band} band pairs (G1 survivors) x 2 x 1,024 FLOP (G3 as an E4M3 product; "
+                                              "peak: twice bf16), the whole stage's time", "traffic": traffic_cos})
+    else:
+        rooflines["cand_cos"] = frac({"bound": "alu", "achieved": band * 4 * nb * nb / (per_stage["cand_cos"] / 1e3) / 1e12,
+                                      "peak": alu_peak_tops(2070.0), "unit": "Tops/s",
+                                      "work": f"{band} band pairs (G1 survivors) x 4 nb^2 integer ops (G3 both ways)",
+                                      "traffic": traffic_cos})
     if dom == "cand_edge":
         rooflines["cand_edge"] = dict(roof)
     if fft:
@@ -1301,10 +1324,13 @@ def run_ours(args, rank, world, local_rank):
         "topo_prescreen": topo,
         "next": nxt,
     }
-    # kernels launched per step: raster 1, band join 5, edge screen 2 (the screen and the
-    # correspondence check of its list), cosine match 4 (mark, two spectra sweeps counted
-    # once for a self-join, pair) -> 3, edge match 1, compact 2
-    line["gpu_launches"] = args.steps * (1 + 5 + 2 + 3 + 1 + 2)
+    # kernels launched per step: raster 1, cosine candidates 10 with G3 as a product (sort 3,
+    # vectors, items, product, list, count, the join that stands by, gates) or 5, edge
+    # candidates (sort 5 or 1, E2, per 64 groups of 256 clips tables, screen and check,
+    # gates), cosine match 3 (mark, spectra, pair), edge match 1, compact 2
+    groups = (n + 255) // 256
+    line["gpu_launches"] = args.steps * (1 + (10 if product_join(N, n) else 5) + (5 if n > 8192 else 1) + 1 +
+                                         3 * ((groups + 63) // 64) + 1 + 3 + 1 + 2)
     if not args.no_cpu_baseline and world == 1:
         n_s = args.cpu_sample or default_sample(args.config)
         a, t, thr = oracle_sample(wl, n_s)
