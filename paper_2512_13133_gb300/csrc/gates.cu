@@ -80,6 +80,16 @@ __global__ void scatter_kernel(const uint32_t *pop, uint32_t n, const uint32_t *
     }
 }
 
+// A small set has fewer representatives than the GPU has warps, and one warp
+// per band makes its length the time of the call: such bands are shared by up to eight
+// warps, each taking every parts-th group of eight members.  1,000 clips of
+// 128x128 px: 65 us with a warp per band, 53 us with eight.
+constexpr uint32_t kBandStep = 8;
+static uint32_t band_parts(uint64_t reps, uint64_t warps) {
+    const uint64_t p = reps ? warps / reps : 1;
+    return p < 2 ? 1u : p > 8 ? 8u : (uint32_t)p;
+}
+
 // spop holds the sorted keys: the area, or with the topological pre-screen
 // class * V + area (V = N^2 + 2), so that a band never leaves its class
 // LP: the lane-per-member first chunk of G3 (WPL = 4, blk 16-byte aligned;
@@ -91,7 +101,8 @@ __global__ void __launch_bounds__(256, LP ? 6 : 8) band_join_kernel(pcl_params p
                                                         unsigned long long *count,
                                                         unsigned long long *local_gates,
                                                         unsigned int *next_pos, uint32_t shard,
-                                                        uint32_t n_shards, const unsigned int *only_if) {
+                                                        uint32_t n_shards, uint32_t parts,
+                                                        const unsigned int *only_if) {
     if (only_if && !*only_if) return;  // decided already
     const Geo g = make_geo(prm);
     const int lane = threadIdx.x & 31;
@@ -104,6 +115,9 @@ __global__ void __launch_bounds__(256, LP ? 6 : 8) band_join_kernel(pcl_params p
         uint32_t p = 0;
         if (lane == 0) p = atomicAdd(next_pos, 1u);
         p = __shfl_sync(0xffffffffu, p, 0);
+        // part s of the band: every parts-th group of `step` members (band_parts)
+        const uint32_t s = parts > 1 ? p % parts : 0u, step = parts > 1 ? kBandStep : 32u;
+        if (parts > 1) p /= parts;
         // the representative: the clip at sorted position p, or with shards
         // the clip of index shard + p S
         const uint64_t ai = sharded ? (uint64_t)shard + (uint64_t)p * n_shards : p;
@@ -146,7 +160,7 @@ __global__ void __launch_bounds__(256, LP ? 6 : 8) band_join_kernel(pcl_params p
             __syncwarp();
         }
         if (pa == 0) {  // the band holds the other empty clips only: similar by definition
-            for (uint32_t q0 = start; q0 < end; q0 += 32) {
+            for (uint32_t q0 = start + 32 * s; q0 < end; q0 += 32 * parts) {
                 const uint32_t bq = q0 + lane < end ? order[q0 + lane] : 0u;
                 const bool v = q0 + lane < end && (!sharded || bq > a);
                 const unsigned m = __ballot_sync(0xffffffffu, v);
@@ -183,20 +197,21 @@ __global__ void __launch_bounds__(256, LP ? 6 : 8) band_join_kernel(pcl_params p
         // band members 32 at a time: lane l sets up member q0 + l (index,
         // thresholds; members of a non-empty representative are non-empty),
         // then the warp tests them one after the other
-        for (uint32_t q0 = start; q0 < end; q0 += 32) {
+        for (uint32_t q0 = start + step * s; q0 < end; q0 += step * parts) {
             const uint32_t q = q0 + lane;
+            const bool in = q < end && (uint32_t)lane < step;
             uint32_t b = 0;
             int tA = 0, tB = 0;  // areas are below 2^31, so are the thresholds (clamped below)
-            if (q < end) {
+            if (in) {
                 b = order[q];
                 const uint64_t pb = spop[q] % V;
                 const int64_t um = cos_umax(pa, pb, prm.cos_num, prm.cos_den);
                 tA = (int)max((int64_t)pa - um, (int64_t)INT_MIN);
                 tB = (int)max((int64_t)pb - um, (int64_t)INT_MIN);
             }
-            int cnt = (int)min(32u, end - q0);
+            int cnt = (int)min(step, end - q0);
             if (sharded) {  // the members b > a only, moved to the low lanes in order
-                const unsigned mem = __ballot_sync(0xffffffffu, q < end && b > a);
+                const unsigned mem = __ballot_sync(0xffffffffu, in && b > a);
                 const int src = nth_set_bit(mem, lane);  // lane of this lane's member
                 const int from = src >= 0 ? src : lane;
                 b = __shfl_sync(0xffffffffu, b, from);
@@ -402,19 +417,21 @@ cudaError_t launch_band_join(const pcl_params &prm, const pcl_clipset &cs, void 
     // the lane-per-member first chunk at 256² (4 words per lane; at 512² the
     // first 64 of 1,024 blocks decide too few pairs to pay for the staging)
     const bool lp = (reinterpret_cast<uintptr_t>(cs.blk) & 15u) == 0;  // 16-byte copies of block rows
+    const uint32_t parts =
+        band_parts(((uint64_t)n + n_shards - 1) / n_shards, (uint64_t)num_sms * 8 * (g.N == 256 && lp ? 6 : 8));
     switch ((g.nb * g.nb / 2 + 31) / 32) {  // u32 words of block counts per lane
         case 1: band_join_kernel<1><<<num_sms * 8, 256, band_g2_smem(g.N, g.S), st>>>(prm, cs, order, spop, cum, V,
                                                                                        vall, out, cap, count,
-                                                                 local, next_pos, shard, n_shards, only_if); break;
+                                                                 local, next_pos, shard, n_shards, parts, only_if); break;
         case 4:
             if (lp) band_join_kernel<4, true><<<num_sms * 6, 256, band_lp_smem(), st>>>(prm, cs, order, spop, cum, V,
                                                                                      vall, out, cap, count, local,
-                                                                                     next_pos, shard, n_shards, only_if);
+                                                                                     next_pos, shard, n_shards, parts, only_if);
             else band_join_kernel<4><<<num_sms * 8, 256, 0, st>>>(prm, cs, order, spop, cum, V, vall, out, cap, count,
-                                                                  local, next_pos, shard, n_shards, only_if);
+                                                                  local, next_pos, shard, n_shards, parts, only_if);
             break;
         case 16: band_join_kernel<16><<<num_sms * 8, 256, 0, st>>>(prm, cs, order, spop, cum, V, vall, out, cap,
-                                                                   count, local, next_pos, shard, n_shards, only_if); break;
+                                                                   count, local, next_pos, shard, n_shards, parts, only_if); break;
         default: return cudaErrorInvalidValue;
     }
     const unsigned long long total = shard_pairs(n, shard, n_shards);
