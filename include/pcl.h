@@ -252,7 +252,8 @@ pcl_status pcl_spectra(pcl_ctx *ctx, const pcl_params *P, pcl_clipset *cs, const
    256x256 and 512x512 px from 2,048 clips 2 KB per clip more for the vectors of
    G3 as a matrix product, done without where they do not fit; two sets: about
    16 (N^2 + 2) + 16 |a| + 8 |b| bytes, with 2,048 or more clips in b at those
-   sizes 1 KB per clip more and |b| / 96 + 512 bytes per clip of a).  EDGE uses it for the list of pairs
+   sizes 1 KB per clip more and |b| / 32 + 512 bytes per clip of a, where that
+   is 64 MB or less).  EDGE uses it for the list of pairs
    left for the exact check (pairs past the list are checked inside the
    screen): the self-join 8 bytes per entry, 2^19 to 2^23 entries, beside 2 MB
    of tables per 256 clips (at most 134 MB) and 172 bytes per clip; two sets,

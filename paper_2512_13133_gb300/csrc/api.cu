@@ -301,6 +301,7 @@ pcl_status pcl_candidates(pcl_ctx *ctx, const pcl_params *P, uint32_t mode, cons
     const size_t join_bytes = (cross_join_workspace(g, a->n_clips, nb) + 255) & ~(size_t)255;
     size_t lib_bytes = a->n_clips ? band_lib_bytes(g, nb) : 0;
     const size_t more = lib_bytes ? band_cross_workspace(g, a->n_clips, nb) : 0;
+    if (!more) lib_bytes = 0;
     if (lib_bytes && !ensure_ws_optional(ctx, sort_bytes + lib_bytes + join_bytes + more, st)) lib_bytes = 0;
     if (!lib_bytes && (s = ensure_ws(ctx, sort_bytes + join_bytes))) return s;
     uint32_t *cum = static_cast<uint32_t *>(ctx->ws), *fill = cum + V, *order = fill + V, *spop = order + nb;

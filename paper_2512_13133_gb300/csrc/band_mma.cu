@@ -47,6 +47,7 @@ constexpr int kStage = 32768;              // bytes of one ring stage: 256 membe
 constexpr int kSeg = 16;                   // member blocks per item at most
 constexpr int kMmaThreads = 256;
 constexpr uint32_t kTmem = 512;
+constexpr uint64_t kMaxList = 1u << 23;   // listed pairs at most
 constexpr float kSlack = 1.0f - 1.0f / 1024.0f;  // on T sqrt(|A| |B|): float rounding, with room to spare
 
 // K bytes per clip: L thresholds of nb2 blocks, at most 1,024
@@ -83,7 +84,7 @@ size_t band_layout(const Geo &g, uint32_t rows, uint32_t cols, uint64_t list_cap
     w.panels = (rows + kPanel - 1) / kPanel;
     w.blocks = (cols + kBlock - 1) / kBlock;
     w.kb = kbytes_of(g.nb * g.nb);
-    w.list_cap = list_cap < (1u << 12) ? (1u << 12) : list_cap > (1u << 23) ? (1u << 23) : (uint32_t)list_cap;
+    w.list_cap = list_cap < (1u << 12) ? (1u << 12) : list_cap > kMaxList ? (uint32_t)kMaxList : (uint32_t)list_cap;
     size_t o = 0;
     auto part = [&](auto *&p, size_t bytes) {
         p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(ws + o);
@@ -109,9 +110,12 @@ size_t band_layout(const Geo &g, uint32_t rows, uint32_t cols, uint64_t list_cap
 }
 
 // listed pairs there is room for: the bound leaves 0.55 % of a band of about
-// an eighth of the members; nearly identical clips leave more, and overflow
+// an eighth of the members; nearly identical clips leave more, and overflow.  A
+// query's band also holds smaller members, of which the bound (its own counts against their
+// sums) leaves more: room for 3 % of it, as with 1 % every request against
+// 2,000,000 clips overflowed and took the band join after all.
 uint64_t list_room(uint64_t rows, uint64_t cols, bool self) {
-    const uint64_t c = self ? rows * cols / 512 : rows * (cols / 768 + 64);
+    const uint64_t c = self ? rows * cols / 512 : rows * (cols / 256 + 64);
     return self && c < (1u << 16) ? 1u << 16 : c;
 }
 
@@ -663,7 +667,12 @@ cudaError_t launch_band_lib(const pcl_params &prm, const pcl_clipset &L, const u
     return cudaGetLastError();
 }
 
+// the most queries whose list fits; more of them take the band join
+uint32_t band_cross_most(uint32_t n_lib) { return (uint32_t)(kMaxList / ((uint64_t)n_lib / 256 + 64)); }
+
+// 0: not covered
 size_t band_cross_workspace(const Geo &g, uint32_t nq, uint32_t n_lib) {
+    if (nq > band_cross_most(n_lib)) return 0;
     BandWs w;
     return band_layout(g, nq, n_lib, list_room(nq, n_lib, false), false, false, nullptr, w);
 }

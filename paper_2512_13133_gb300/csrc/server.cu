@@ -61,6 +61,7 @@ cudaError_t launch_cross_join(const pcl_params &, const pcl_clipset &, const pcl
                               unsigned long long);
 size_t band_lib_bytes(const Geo &, uint32_t);
 size_t band_cross_workspace(const Geo &, uint32_t, uint32_t);
+uint32_t band_cross_most(uint32_t);
 cudaError_t launch_band_lib(const pcl_params &, const pcl_clipset &, const uint32_t *, const uint32_t *, void *,
                             cudaStream_t);
 cudaError_t launch_exact_pairs(const pcl_params &, const pcl_clipset &, const pcl_clipset &, const pcl_pair *,
@@ -352,8 +353,8 @@ pcl_status pcl_server_create_classes(pcl_ctx *ctx, const pcl_params *params, con
     // the products' buffers: every slot's largest request, at most a sixteenth of the budget
     size_t product = 0;
     for (const auto &k : s->cls) {
-        const size_t b =
-            k.lib_vectors ? align256(pcl::band_cross_workspace(k.g, cfg->max_query_clips, k.lib.n_clips)) : 0;
+        const uint32_t nq = std::min(cfg->max_query_clips, pcl::band_cross_most(k.lib.n_clips));
+        const size_t b = k.lib_vectors ? align256(pcl::band_cross_workspace(k.g, nq, k.lib.n_clips)) : 0;
         product = b > product ? b : product;
     }
     product = std::min<size_t>(product * cfg->max_inflight, cfg->mem_budget / 16) & ~(size_t)255;
