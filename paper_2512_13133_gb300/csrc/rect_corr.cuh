@@ -17,9 +17,12 @@
 // scan of the rasters, 100,000 of 256x256 px 0.54 ms against 6.5 (scan) and 21 ms
 // (FP16 tensor cores, full items); re-extraction of 60,000 pairs 5.9 -> 0.6 ms.
 //
-// One warp per pair of clips.  Clips of more than kRectMax rectangles, or whose
-// rectangles share pixels (their areas do not add up to the raster's ones),
-// are left to the callers' other paths.
+// One warp per pair of clips.  Clips of more than kRectMax rectangles, whose
+// rectangles share pixels, or whose rectangles are not the raster's (a caller may
+// have written the buffer again: the rasters are what a record is about), are
+// left to the callers' other paths: the ranges must be disjoint, every pixel of
+// theirs set, and their areas add up to the raster's ones.  The look at the
+// raster takes a lane per row of a rectangle.
 #pragma once
 
 #include "common.cuh"
@@ -99,6 +102,27 @@ __device__ __forceinline__ bool ranges_disjoint(const short4 *r, int n, int lane
         }
     }
     return !__any_sync(0xffffffffu, shared_px);
+}
+
+// every pixel of the n staged ranges is set in the raster: rows of nw words, the
+// pixel (x, y) at bit x + o of row y + o
+__device__ __forceinline__ bool ranges_set(const short4 *r, int n, const uint64_t *__restrict__ bits, int nw, int o,
+                                           int lane) {
+    bool unset = false;
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+        const short4 q = r[i];
+        const int x0 = q.x + o, x1 = q.y + o - 1, w0 = x0 >> 6, w1 = x1 >> 6;
+        const uint64_t first = ~0ull << (x0 & 63), last = ~0ull >> (63 - (x1 & 63));
+        for (int y = q.z + lane; q.x < q.y && y < q.w; y += 32) {
+            const uint64_t *row = bits + (size_t)(y + o) * nw;
+            for (int w = w0; w <= w1; ++w) {
+                const uint64_t m = (w == w0 ? first : ~0ull) & (w == w1 ? last : ~0ull);
+                unset = unset || (__ldg(row + w) & m) != m;
+            }
+        }
+    }
+    return !__any_sync(0xffffffffu, unset);
 }
 
 // the entries of f's second difference on one axis: position in [0, 2S] and weight (0: none)
@@ -240,8 +264,16 @@ __device__ __forceinline__ void rect_surface(const Scratch &s, int na, int nb, i
     __syncwarp();  // the scratch is free again
 }
 
+// the n staged ranges are the window raster of clip c of set cs, whose pixels
+// they number `area`, and share none
+__device__ __forceinline__ bool ranges_are_raster(const short4 *r, int n, uint32_t area, const pcl_clipset &cs,
+                                                  uint32_t c, const Geo &g, int lane) {
+    return area == cs.pop[c] && ranges_disjoint(r, n, lane) &&
+           ranges_set(r, n, cs.bits + (size_t)c * g.N * g.nw, g.nw, 0, lane);
+}
+
 // Whether the pair takes this path: few enough rectangles, and (after staging)
-// areas that add up to the rasters' ones.  Stages both clips.
+// ranges that are the rasters.  Stages both clips.
 __device__ __forceinline__ bool stage_pair(const pcl_clipset &A, const pcl_clipset &B, const pcl_pair pr, const Geo &g,
                                            int psh, const Scratch &s, int &na, int &nb, int lane) {
     const uint32_t oa = __ldg(A.rect_off + pr.a), ob = __ldg(B.rect_off + pr.b);
@@ -251,7 +283,8 @@ __device__ __forceinline__ bool stage_pair(const pcl_clipset &A, const pcl_clips
     __syncwarp();  // the scratch's previous contents are no longer read
     const uint32_t aa = stage_rects(reinterpret_cast<const int4 *>(A.rects) + oa, na, g.p, psh, 0, g.N, s.ra, lane);
     const uint32_t ab = stage_rects(reinterpret_cast<const int4 *>(B.rects) + ob, nb, g.p, psh, 0, g.N, s.rb, lane);
-    return aa == A.pop[pr.a] && ab == B.pop[pr.b];
+    __syncwarp();
+    return ranges_are_raster(s.ra, na, aa, A, pr.a, g, lane) && ranges_are_raster(s.rb, nb, ab, B, pr.b, g, lane);
 }
 
 // The cosine record of one pair by the exact argmax (one warp; lane 0 writes
