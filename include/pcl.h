@@ -434,7 +434,9 @@ pcl_status pcl_stats_get(pcl_ctx *ctx, uint64_t *out, int reset);
    the near band), pass, reserved = n_B(s*), flags ALIGNED (| EMPTY); no
    gates run (the lossless bounds assume fixed norms) and pcm fields are 0.
    Pairs that can (as in the exact scan, the representative not empty) take
-   their overlaps from the rectangles; for the others one CTA per pair with
+   their overlaps from the rectangles: rect_off and rects of both sets are
+   read unless NULL, and rectangles that are not the ones of a's raster or of
+   b's halo raster are noticed; for the others one CTA per pair with
    both rasters in shared memory: groups of shifts
    are counted best first and skipped when min(row bound, column bound)^2
    n_best < c_best^2 n_B(s) for each of their shifts (a's profiles against

@@ -271,14 +271,41 @@ __device__ __forceinline__ pcl_record halo_record(const pcl_params &prm, const G
     return rec;
 }
 
+// The n staged ranges are clip b's halo raster (hb) and share no pixel: every
+// pixel of theirs is set, and the windows of the four corner shifts, which
+// together cover the halo (2 S <= N), hold as many of them as tabulated (gn).
+__device__ __forceinline__ bool ranges_are_halo(const short4 *r, int n, const uint64_t *__restrict__ hb,
+                                                const uint32_t *__restrict__ gn, const Geo &g, int lane) {
+    const int N = g.N, S = g.S, K = 2 * S + 1;
+    uint32_t c[4] = {0u, 0u, 0u, 0u};
+    for (int t = lane; t < n; t += 32) {
+        const short4 q = r[t];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int dx = k & 1 ? S : -S, dy = k & 2 ? S : -S;  // the window starts at (-dx, -dy)
+            const int w = min((int)q.y, N - dx) - max((int)q.x, -dx), h = min((int)q.w, N - dy) - max((int)q.z, -dy);
+            c[k] += w > 0 && h > 0 ? (uint32_t)w * (uint32_t)h : 0u;
+        }
+    }
+    bool same = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        same = same && __reduce_add_sync(0xffffffffu, c[k]) == __ldg(gn + (k & 2 ? 2 * S * K : 0) + (k & 1 ? 2 * S : 0));
+    return same && pcl::rect_corr::ranges_disjoint(r, n, lane) &&
+           pcl::rect_corr::ranges_set(r, n, hb, halo_words(N, S), S, lane);
+}
+
 // One warp per pair: the record from the rectangles (rect_corr.cuh; A's cut to
 // its window, B's to the halo) for clips of few enough rectangles that share no
-// pixel, every shift's overlap against the tabulated n_B(s).  The other pairs
+// pixel and are the rasters (the buffers may have been written again, and b may be
+// another set of clips than the halo rasters were made from), every shift's
+// overlap against the tabulated n_B(s).  The other pairs
 // get a record with flags = kRectPending, for halo_pair_kernel.  A pair decided
 // here counts as one group of shifts in stats.
 constexpr int kRectWarps = 4;
 
 __global__ void __launch_bounds__(32 * kRectWarps) halo_rect_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B,
+                                                                    const uint64_t *__restrict__ hbits,
                                                                     const uint32_t *__restrict__ norms,
                                                                     const pcl_pair *pairs, uint64_t npairs,
                                                                     const unsigned long long *d_n, pcl_record *out,
@@ -315,7 +342,9 @@ __global__ void __launch_bounds__(32 * kRectWarps) halo_rect_kernel(pcl_params p
             const uint32_t aa = rc::stage_rects(reinterpret_cast<const int4 *>(A.rects) + oa, na, g.p, psh, 0, N, s.ra, lane);
             rc::stage_rects(reinterpret_cast<const int4 *>(B.rects) + ob, nb, g.p, psh, -S, N + S, s.rb, lane);
             __syncwarp();
-            ok = aa == pa && rc::ranges_disjoint(s.rb, nb, lane);
+            ok = rc::ranges_are_raster(s.ra, na, aa, A, pr.a, g, lane) &&
+                 ranges_are_halo(s.rb, nb, hbits + (size_t)pr.b * halo_side(N, S) * halo_words(N, S),
+                                 norms + (size_t)pr.b * norms_stride(N, S), g, lane);
         }
         if (!ok) {
             rec.flags = rc::kRectPending;
@@ -598,8 +627,8 @@ cudaError_t launch_pair(const pcl_params &prm, const Geo &g, const pcl_clipset &
         if (e != cudaSuccess) return e;
         const uint64_t most = (uint64_t)num_sms * (uint64_t)(rect_sm > 0 ? rect_sm : 1);
         const uint64_t need = (n + kRectWarps - 1) / kRectWarps;
-        halo_rect_kernel<<<(unsigned)(need < most ? need : most), 32 * kRectWarps, rs, st>>>(prm, a, b, nb, pairs, n, d_n,
-                                                                                            out, stats);
+        halo_rect_kernel<<<(unsigned)(need < most ? need : most), 32 * kRectWarps, rs, st>>>(prm, a, b, hb, nb, pairs, n,
+                                                                                            d_n, out, stats);
     }
     halo_pair_kernel<NW><<<(unsigned)(n < cap ? n : cap), kThreads, sm, st>>>(prm, a, b, hb, nb, pairs, n, d_n, out,
                                                                              stats);
