@@ -512,8 +512,9 @@ pcl_status pcl_match_mixed(pcl_ctx *ctx, const pcl_params *params, pcl_clipset *
    as well, 1 KB per clip, where memory allows); with
    the FFT engine its spectra are computed too (spec/spec_state required),
    while the tensor-core engine and the exact scan read the rasters only
-   (spec may be NULL: ~10.6 KB per 256^2 clip instead of ~350 KB, so
-   2,000,000 library clips fit in ~21 GB).  An EDGE library needs its rasters
+   (spec may be NULL: ~10.6 KB per 256^2 clip, with the gate's vectors 11.6,
+   instead of ~350 KB, so 2,000,000 library clips fit in ~24 GB; rect_off and
+   rects are not read, so every aligned pair takes the engine itself).  An EDGE library needs its rasters
    and edge signatures only (esig, occ, rorder).  The server then allocates
    max_inflight request slots (one stream each, pinned staging) and one
    device arena of mem_budget bytes, shared by all classes (and, beside the

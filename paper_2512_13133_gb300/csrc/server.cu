@@ -305,6 +305,10 @@ pcl_status pcl_server_create_classes(pcl_ctx *ctx, const pcl_params *params, con
         classes[c].P = *P;
         classes[c].g = g;
         classes[c].lib = *library;
+        if (!edge) {  // a cosine library is its rasters: its rectangles may be gone by now
+            classes[c].lib.rect_off = nullptr;
+            classes[c].lib.rects = nullptr;
+        }
         classes[c].engine = engine;
     }
     cudaError_t e = cudaSetDevice(ctx->device);
