@@ -307,6 +307,9 @@ cudaError_t launch_mixed(const pcl_params *prm, const pcl_clipset *sets, uint32_
         mixed_gate_kernel<<<num_sms * 8, 256, 0, st>>>(args, work, n_cos, out, cursor, claim);
         for (uint32_t c = 0; c < n_classes; ++c) {
             const Geo g = make_geo(prm[c]);
+            // no item is pending past this marker (PCL_GATE_UNSUPPORTED), and at 512x512 px
+            // the tables of shifts would outgrow shared memory from S = 60 on
+            if (g.S > g.N / 16) continue;
             unsigned long long *cur = cursor + 1 + c;
             switch (g.P * 2 + (radix == 4 ? 1 : 0)) {
                 case 16: e = align_t<8, 2>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st); break;
@@ -319,8 +322,7 @@ cudaError_t launch_mixed(const pcl_params *prm, const pcl_clipset *sets, uint32_
                     const size_t rs = kRectWarps * rect_corr::scratch_bytes(g.S);
                     e = cudaFuncSetAttribute(mixed_rect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
                     if (e != cudaSuccess) return e;
-                    if (g.S <= g.N / 16)
-                        mixed_rect_kernel<<<num_sms * 3, 32 * kRectWarps, rs, st>>>(prm[c], sets[c], c, work, n_cos, out);
+                    mixed_rect_kernel<<<num_sms * 3, 32 * kRectWarps, rs, st>>>(prm[c], sets[c], c, work, n_cos, out);
                     e = align_t<64, 2>(prm[c], sets[c], c, work, n_cos, out, cur, ctas_per_sm, num_sms, st);
                     break;
                 }
