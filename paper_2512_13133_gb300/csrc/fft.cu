@@ -217,8 +217,11 @@ __global__ void __launch_bounds__(32 * 2 * ((9 * P / 2 + 1 + 31) / 32), P == 32 
 // (indices, emptiness, gates, and the record from the rectangles where it can);
 // the pairs it leaves pending take the bound-pruned scan of the rasters
 // (exact_body<NW, SMAX>, N = 64 NW, S <= SMAX = N/16), one pair per CTA
-// iteration: a CTA collects the pending ones of as many consecutive pairs as
-// it has threads.  list (with its length n_list on the device): those pairs instead.
+// iteration.  CTA b owns the pairs b, b + G, b + 2G, .. of a grid of G, looks at
+// as many of them as it has threads and scans the pending ones: neighbours in
+// a list mostly share a clip and are pending together, and consecutive
+// pairs per CTA left most of the GPU idle (1,000 pairs of clips of 100 rectangles:
+// 20.7 ms against 0.42 at 512x512 px, 2.65 against 0.09 at 256x256).  list (with its length n_list on the device): those pairs instead.
 template <int NW, int SMAX>
 __global__ void __launch_bounds__(exact_threads<NW>(), NW == 8 ? 2 : 6)
     exact_pair_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B, const pcl_pair *pairs, uint64_t npairs,
@@ -233,15 +236,18 @@ __global__ void __launch_bounds__(exact_threads<NW>(), NW == 8 ? 2 : 6)
     __shared__ uint16_t open_s[T];
     __shared__ int count;
     if (d_n && *d_n < npairs) npairs = *d_n;
-    for (uint64_t t0 = (uint64_t)blockIdx.x * T; t0 < npairs; t0 += (uint64_t)gridDim.x * T) {
+    for (uint64_t t0 = blockIdx.x; t0 < npairs; t0 += (uint64_t)gridDim.x * T) {
         __syncthreads();  // the previous list is no longer read
         if (threadIdx.x == 0) count = 0;
         __syncthreads();
-        const uint64_t t = t0 + threadIdx.x;
+        const uint64_t t = t0 + (uint64_t)threadIdx.x * gridDim.x;
         if (t < npairs && out[t].flags == rect_corr::kRectPending) open_s[atomicAdd(&count, 1)] = (uint16_t)threadIdx.x;
         __syncthreads();
         const int n = count;
-        for (int k = 0; k < n; ++k) exact_body<NW, SMAX>(prm, A, B, pairs[t0 + open_s[k]], out + t0 + open_s[k], stats);
+        for (int k = 0; k < n; ++k) {
+            const uint64_t p = t0 + (uint64_t)open_s[k] * gridDim.x;
+            exact_body<NW, SMAX>(prm, A, B, pairs[p], out + p, stats);
+        }
     }
 }
 
