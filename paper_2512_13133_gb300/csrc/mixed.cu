@@ -196,7 +196,11 @@ __global__ void __launch_bounds__(32 * kRectWarps) mixed_rect_kernel(pcl_params 
 
 // The pending items of class c, aligned one at a time by a whole CTA with the
 // engine of the class's size (P = N / 8; 64: the exact scan of 512^2 px).  A
-// CTA claims kScan consecutive items and collects the pending ones of its class.
+// CTA claims up to kScan items and collects the pending ones of its class.  Of a list
+// cut into C claims, claim c holds the groups of 32 consecutive items c, c + C, ..:
+// pending items lie side by side (one clip's, one class's), and a claim of 512
+// consecutive ones left them to a few CTAs (2,048 of 256x256 px side by side: 12.8 ms).  A claim is an eighth of a
+// CTA's share at most, so that short lists reach every CTA.
 constexpr int kScan = 512;
 
 template <int P>
@@ -217,21 +221,27 @@ __global__ void __launch_bounds__(AlignCta<P>::threads, AlignCta<P>::ctas)
     __shared__ int count;
     __shared__ unsigned long long at;
     if constexpr (P != 64) load_pair_table<P>();
+    const uint64_t groups = (n_cos + 31) / 32, share = groups / (8 * (uint64_t)gridDim.x);
+    const uint32_t per = share < 1 ? 1u : share < kScan / 32 ? (uint32_t)share : kScan / 32;  // groups a claim
+    const uint64_t claims = (groups + per - 1) / per;
+    auto item = [&](uint64_t c, uint32_t k) { return 32 * (c + (k >> 5) * claims) + (k & 31u); };
     for (;;) {
         __syncthreads();  // the previous list is no longer read
         if (threadIdx.x == 0) {
             count = 0;
-            at = atomicAdd(cursor, (unsigned long long)kScan);
+            at = atomicAdd(cursor, 1ull);
         }
         __syncthreads();
-        const uint64_t t0 = at;
-        if (t0 >= n_cos) break;
-        for (int k = threadIdx.x; k < kScan && t0 + k < n_cos; k += blockDim.x)
-            if (out[t0 + k].flags == kPending && work[t0 + k].cls == c) list[atomicAdd(&count, 1)] = (uint16_t)k;
+        const uint64_t claim = at;
+        if (claim >= claims) break;
+        for (uint32_t k = threadIdx.x; k < 32 * per; k += blockDim.x) {
+            const uint64_t t = item(claim, k);
+            if (t < n_cos && out[t].flags == kPending && work[t].cls == c) list[atomicAdd(&count, 1)] = (uint16_t)k;
+        }
         __syncthreads();
         const int n = count;
         for (int k = 0; k < n; ++k) {
-            const uint64_t t = t0 + list[k];
+            const uint64_t t = item(claim, list[k]);
             const pcl_pair pr{work[t].a, work[t].b};
             if constexpr (P == 64) exact_body<8, 32>(prm, cs, cs, pr, out + t);
             else pair_body<P, RADIX>(prm, cs, cs, pr, out + t, true);
