@@ -91,14 +91,16 @@ __device__ __forceinline__ uint32_t stage_rects(const int4 *rects, int n, int p,
     return __reduce_add_sync(0xffffffffu, area);
 }
 
-// no two of the n staged ranges share a pixel
+// no two of the n staged ranges share a pixel (an empty range has none, though the
+// zeros that stand for it lie inside a halo range over the origin)
 __device__ __forceinline__ bool ranges_disjoint(const short4 *r, int n, int lane) {
     bool shared_px = false;
+#pragma unroll 4
     for (int i = 0; i + 1 < n; ++i) {
         const short4 a = r[i];
         for (int j = i + 1 + lane; j < n; j += 32) {
             const short4 b = r[j];
-            shared_px = shared_px || (a.x < b.y && b.x < a.y && a.z < b.w && b.z < a.w);
+            shared_px |= (a.x < b.y) & (b.x < a.y) & (a.z < b.w) & (b.z < a.w) & (a.x < a.y) & (b.x < b.y);
         }
     }
     return !__any_sync(0xffffffffu, shared_px);
