@@ -291,8 +291,7 @@ __device__ __forceinline__ bool ranges_are_halo(const short4 *r, int n, const ui
 #pragma unroll
     for (int k = 0; k < 4; ++k)
         same = same && __reduce_add_sync(0xffffffffu, c[k]) == __ldg(gn + (k & 2 ? 2 * S * K : 0) + (k & 1 ? 2 * S : 0));
-    return same && pcl::rect_corr::ranges_disjoint(r, n, lane) &&
-           pcl::rect_corr::ranges_set(r, n, hb, halo_words(N, S), S, lane);
+    return same && pcl::rect_corr::ranges_in_raster(r, n, hb, halo_words(N, S), S, lane);
 }
 
 // One warp per pair: the record from the rectangles (rect_corr.cuh; A's cut to
@@ -304,7 +303,7 @@ __device__ __forceinline__ bool ranges_are_halo(const short4 *r, int n, const ui
 // here counts as one group of shifts in stats.
 constexpr int kRectWarps = 4;
 
-__global__ void __launch_bounds__(32 * kRectWarps) halo_rect_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B,
+__global__ void __launch_bounds__(32 * kRectWarps, 8) halo_rect_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B,
                                                                     const uint64_t *__restrict__ hbits,
                                                                     const uint32_t *__restrict__ norms,
                                                                     const pcl_pair *pairs, uint64_t npairs,

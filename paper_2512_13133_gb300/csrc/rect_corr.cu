@@ -15,11 +15,14 @@ constexpr int kWarps = 4;
 // from the rectangles.  A pair that does not take that path is left to the
 // caller's next kernel: keep[t] = 1 (else 0), or without keep a record with
 // flags = kRectPending.  stats: groups of shifts as pcl_stats_get counts them, a pair
-// decided here counting as one.
-__global__ void __launch_bounds__(32 * kWarps) rect_pair_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B,
-                                                                const pcl_pair *pairs, uint64_t n,
-                                                                const unsigned long long *d_n, pcl_record *out,
-                                                                uint32_t *keep, unsigned long long *stats) {
+// decided here counting as one.  CTAS: resident per SM, 8 (64 registers) where the
+// tables of shifts leave room for them (100,000 pairs of 256x256 px: 1.16 -> 1.03 ms a
+// call against 5), else 3 (12,001 of 512x512 px: 0.31 -> 0.26 ms against 8's registers).
+template <int CTAS>
+__global__ void __launch_bounds__(32 * kWarps, CTAS) rect_pair_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B,
+                                                                      const pcl_pair *pairs, uint64_t n,
+                                                                      const unsigned long long *d_n, pcl_record *out,
+                                                                      uint32_t *keep, unsigned long long *stats) {
     if (d_n && *d_n < n) n = *d_n;
     extern __shared__ __align__(16) unsigned char smem[];
     const Geo g = make_geo(prm);
@@ -77,14 +80,15 @@ cudaError_t launch_rect_pairs(const pcl_params &prm, const pcl_clipset &a, const
     if (n == 0) return cudaSuccess;
     const Geo g = make_geo(prm);
     const size_t sm = kWarps * scratch_bytes(g.S);
-    cudaError_t e = cudaFuncSetAttribute(rect_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    auto *kern = 8 * sm <= 200 * 1024 ? rect_pair_kernel<8> : rect_pair_kernel<3>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     int per_sm = 0;
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rect_pair_kernel, 32 * kWarps, sm);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kWarps, sm);
     if (e != cudaSuccess) return e;
     const uint64_t cap = (uint64_t)num_sms * (uint64_t)(per_sm > 0 ? per_sm : 1), need = (n + kWarps - 1) / kWarps;
-    rect_pair_kernel<<<(unsigned)(need < cap ? need : cap), 32 * kWarps, sm, st>>>(prm, a, b, pairs, n, d_n, out, keep,
-                                                                                  stats);
+    kern<<<(unsigned)(need < cap ? need : cap), 32 * kWarps, sm, st>>>(prm, a, b, pairs, n, d_n, out, keep,
+                                                                       stats);
     return cudaGetLastError();
 }
 

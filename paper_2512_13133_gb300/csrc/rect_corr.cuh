@@ -10,19 +10,21 @@
 // non-zero entries (the first two values and a +-1 at each breakpoint inside),
 // so a pair of rectangles adds at most 36 products to a K x K table (K = 2S + 1),
 // and two prefix sums along each axis turn the table into c(s) for every shift,
-// in integers (mod 2^32; c itself is below 2^18).  No raster is read: a pair of
+// in integers (mod 2^32; c itself is below 2^18).  A pair of
 // clips costs a few thousand warp instructions instead of a popcount per shift,
-// row and word.  Bound by issue slots.  One GB300, same-seed pairs of clips of 21
-// rectangles: 12,001 pairs of 512x512 px 0.16 ms against 4.2 ms for the window
-// scan of the rasters, 100,000 of 256x256 px 0.54 ms against 6.5 (scan) and 21 ms
-// (FP16 tensor cores, full items); re-extraction of 60,000 pairs 5.9 -> 0.6 ms.
+// row and word.  Bound by issue slots and, at about 16 warps an SM, latency.
 //
 // One warp per pair of clips.  Clips of more than kRectMax rectangles, whose
 // rectangles share pixels, or whose rectangles are not the raster's (a caller may
 // have written the buffer again: the rasters are what a record is about), are
 // left to the callers' other paths: the ranges must be disjoint, every pixel of
-// theirs set, and their areas add up to the raster's ones.  The look at the
-// raster takes a lane per row of a rectangle.
+// theirs set, and their areas add up to the raster's ones.  That look takes a
+// third of the instructions.
+//
+// One GB300, same-seed pairs of clips of 21 rectangles, a call: 12,001 pairs of
+// 512x512 px 0.26 ms (0.19 without the look at the rasters) against 4.2 ms for their window
+// scan, 100,000 of 256x256 px 1.03 ms (0.63) against 6.5 (scan) and 21 ms (FP16
+// tensor cores, full items).
 #pragma once
 
 #include "common.cuh"
@@ -91,40 +93,74 @@ __device__ __forceinline__ uint32_t stage_rects(const int4 *rects, int n, int p,
     return __reduce_add_sync(0xffffffffu, area);
 }
 
-// no two of the n staged ranges share a pixel (an empty range has none, though the
-// zeros that stand for it lie inside a halo range over the origin)
+// no two of the n staged ranges share a pixel (an empty range, (0, 0, 0, 0), has
+// none): lane i compares range i with the n / 2 ranges after it, past the last
+// one from the first on
 __device__ __forceinline__ bool ranges_disjoint(const short4 *r, int n, int lane) {
     bool shared_px = false;
+    for (int i = lane; i - lane < n; i += 32) {
+        const short4 a = i < n ? r[i] : make_short4(0, 0, 0, 0);
+        int j = i;
 #pragma unroll 4
-    for (int i = 0; i + 1 < n; ++i) {
-        const short4 a = r[i];
-        for (int j = i + 1 + lane; j < n; j += 32) {
+        for (int d = 0; d < n / 2; ++d) {
+            j = j + 1 < n ? j + 1 : 0;
             const short4 b = r[j];
-            shared_px |= (a.x < b.y) & (b.x < a.y) & (a.z < b.w) & (b.z < a.w) & (a.x < a.y) & (b.x < b.y);
+            shared_px |= (max(a.x, b.x) < min(a.y, b.y)) & (max(a.z, b.z) < min(a.w, b.w));
         }
     }
     return !__any_sync(0xffffffffu, shared_px);
 }
 
 // every pixel of the n staged ranges is set in the raster: rows of nw words, the
-// pixel (x, y) at bit x + o of row y + o
+// pixel (x, y) at bit x + o of row y + o.  Eight lanes per rectangle, four of its
+// rows per lane at a time, the first and the last word of each: eight loads in
+// flight.  With 32 lanes per rectangle, a word and a rectangle after the other, it
+// took longer than the tables: 12,000 pairs of 40 rectangles 401 us at 256x256 px and 988
+// at 512x512, now 240 and 619, without any look at the raster 167 and 282.
 __device__ __forceinline__ bool ranges_set(const short4 *r, int n, const uint64_t *__restrict__ bits, int nw, int o,
                                            int lane) {
-    bool unset = false;
-#pragma unroll 4
-    for (int i = 0; i < n; ++i) {
-        const short4 q = r[i];
+    uint64_t unset = 0ull;
+    bool wide = false;  // some rectangle covers a word between its first and its last
+#pragma unroll 1
+    for (int i0 = 0; i0 < n; i0 += 4) {
+        const int i = i0 + (lane >> 3), sub = lane & 7;
+        const short4 q = i < n ? r[i] : make_short4(0, 0, 0, 0);
         const int x0 = q.x + o, x1 = q.y + o - 1, w0 = x0 >> 6, w1 = x1 >> 6;
-        const uint64_t first = ~0ull << (x0 & 63), last = ~0ull >> (63 - (x1 & 63));
-        for (int y = q.z + lane; q.x < q.y && y < q.w; y += 32) {
-            const uint64_t *row = bits + (size_t)(y + o) * nw;
-            for (int w = w0; w <= w1; ++w) {
-                const uint64_t m = (w == w0 ? first : ~0ull) & (w == w1 ? last : ~0ull);
-                unset = unset || (__ldg(row + w) & m) != m;
+        uint64_t first = ~0ull << (x0 & 63), last = ~0ull >> (63 - (x1 & 63));
+        const bool two = w1 > w0;
+        if (!two) first &= last, last = 0ull;
+        wide |= w1 > w0 + 1;
+        const int rows = __reduce_max_sync(0xffffffffu, q.w - q.z), mine = q.w - q.z - sub;
+        const uint64_t *p = bits + (q.z + sub + o) * nw + w0;
+#pragma unroll 1
+        for (int y = 0; y < rows; y += 32, p += 32 * nw) {
+            uint64_t a[4], b[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const bool in = y + 8 * j < mine;
+                a[j] = in ? __ldg(p + 8 * j * nw) : ~0ull;
+                b[j] = in && two ? __ldg(p + 8 * j * nw + (w1 - w0)) : ~0ull;
             }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) unset |= (~a[j] & first) | (~b[j] & last);
         }
     }
-    return !__any_sync(0xffffffffu, unset);
+    if (__any_sync(0xffffffffu, wide)) {
+        for (int i = 0; i < n; ++i) {
+            const short4 q = r[i];
+            for (int y = q.z + lane; y < q.w; y += 32)
+                for (int w = ((q.x + o) >> 6) + 1; w < (q.y + o - 1) >> 6; ++w) unset |= ~__ldg(bits + (y + o) * nw + w);
+        }
+    }
+    return !__any_sync(0xffffffffu, unset != 0ull);
+}
+
+// the n staged ranges share no pixel, and all of theirs are set in the raster.  Out
+// of line: it is needed for both clips, and its code beside the tables' in a
+// kernel twice costs instruction fetches (a quarter of the stalls)
+static __device__ __noinline__ bool ranges_in_raster(const short4 *r, int n, const uint64_t *__restrict__ bits, int nw,
+                                                     int o, int lane) {
+    return ranges_disjoint(r, n, lane) && ranges_set(r, n, bits, nw, o, lane);
 }
 
 // the entries of f's second difference on one axis: position in [0, 2S] and weight (0: none)
@@ -270,8 +306,7 @@ __device__ __forceinline__ void rect_surface(const Scratch &s, int na, int nb, i
 // they number `area`, and share none
 __device__ __forceinline__ bool ranges_are_raster(const short4 *r, int n, uint32_t area, const pcl_clipset &cs,
                                                   uint32_t c, const Geo &g, int lane) {
-    return area == cs.pop[c] && ranges_disjoint(r, n, lane) &&
-           ranges_set(r, n, cs.bits + (size_t)c * g.N * g.nw, g.nw, 0, lane);
+    return area == cs.pop[c] && ranges_in_raster(r, n, cs.bits + (size_t)c * g.N * g.nw, g.nw, 0, lane);
 }
 
 // Whether the pair takes this path: few enough rectangles, and (after staging)
