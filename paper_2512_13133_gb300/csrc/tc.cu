@@ -809,7 +809,7 @@ __global__ void tc_items_kernel(const uint32_t *head, const uint32_t *surv, cons
 // (window S = N/16) keeps the shifts of the smaller window
 bool tc_supported(const Geo &g) { return (g.N == 64 || g.N == 128 || g.N == 256) && g.S >= 0 && g.S <= g.N / 16; }
 
-size_t tc_workspace(uint64_t n) { return 4 * (4 * (size_t)n + 8) + sizeof(TcItem) * (size_t)(n + 1) + 256; }
+size_t tc_workspace(uint64_t n) { return 4 * (3 * (size_t)n + 8) + sizeof(TcItem) * (size_t)(n + 1) + 256; }
 
 namespace {
 
@@ -874,9 +874,12 @@ cudaError_t launch_tc(const pcl_params &prm, const pcl_clipset &a, const pcl_cli
     uint32_t *keep = reinterpret_cast<uint32_t *>(w);
     uint32_t *pos = keep + n;           // n + 1
     uint32_t *surv = pos + n + 1;       // n
-    uint32_t *scan = surv + n;          // n
-    uint32_t *misc = scan + n;          // [0] n_items, [1] pairs for the exact scan
+    uint32_t *misc = surv + n;          // [0] n_items, [1] pairs for the exact scan
     TcItem *items = reinterpret_cast<TcItem *>(((uintptr_t)(misc + 8) + 15) & ~uintptr_t(15));
+    // the list for the scan (n at most) is the second half of the items' room: with it
+    // an item has `few` members or more, and n / few of them fit the first half
+    const uint32_t item_cap = few ? (uint32_t)(n / 2) + 1 : (uint32_t)n + 1;
+    uint32_t *scan = reinterpret_cast<uint32_t *>(items + item_cap);
     unsigned int *n_items = misc;
     cudaError_t e = cudaMemsetAsync(keep, 0, 4 * (size_t)n, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(misc, 0, 32, st);
@@ -890,7 +893,7 @@ cudaError_t launch_tc(const pcl_params &prm, const pcl_clipset &a, const pcl_cli
     tc_compact_kernel<<<num_sms * 4, 256, 0, st>>>(keep, pos, n, d_n, surv);
     // segment heads over the survivors (keep reused as head flags)
     tc_seg_kernel<<<num_sms * 4, 256, 0, st>>>(pairs, surv, pos + n, keep);
-    tc_items_kernel<<<num_sms * 4, 256, 0, st>>>(keep, surv, pos + n, NB, few, items, n_items, (uint32_t)n + 1, scan,
+    tc_items_kernel<<<num_sms * 4, 256, 0, st>>>(keep, surv, pos + n, NB, few, items, n_items, item_cap, scan,
                                                  misc + 1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (few && (e = launch_exact_pairs(prm, a, b, pairs, n, nullptr, out, num_sms, nullptr, st, scan, misc + 1)) !=
