@@ -61,6 +61,7 @@ cudaError_t launch_mixed(const pcl_params *, const pcl_clipset *, uint32_t, cons
 }  // namespace pcl
 
 #include "ctx.h"
+#include "workspace.h"
 
 using namespace pcl;
 
@@ -86,43 +87,6 @@ pcl_status enter(pcl_ctx *ctx) {
     const cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaSetDevice");
     return PCL_OK;
-}
-
-pcl_status ensure_ws(pcl_ctx *ctx, size_t bytes) {
-    if (bytes <= ctx->ws_bytes) return PCL_OK;
-    if (ctx->ws) {
-        cudaFree(ctx->ws);  // synchronises the device: no kernel still uses it
-        ctx->ws = nullptr;
-        ctx->ws_bytes = 0;
-    }
-    const size_t want = bytes + bytes / 4 + 4096;
-    const cudaError_t e = cudaMalloc(&ctx->ws, want);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        ctx->ws = nullptr;
-        return fail(ctx, PCL_ERR_OOM, "workspace allocation of %s%lld bytes failed", "", (long long)want);
-    }
-    ctx->ws_bytes = want;
-    return PCL_OK;
-}
-
-// A larger workspace for a faster path, if it can be had: not while st is being
-// captured (an allocation would end the capture; a smaller one may be there
-// from an earlier call), and a size that did not fit is not tried again, as each try gives
-// the present workspace back first.
-bool ensure_ws_optional(pcl_ctx *ctx, size_t bytes, cudaStream_t st) {
-    if (bytes <= ctx->ws_bytes) return true;
-    if (ctx->ws_refused && bytes >= ctx->ws_refused) return false;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    if (cap != cudaStreamCaptureStatusNone) return false;
-    if (ensure_ws(ctx, bytes) == PCL_OK) return true;
-    ctx->ws_refused = bytes;
-    ctx->err.clear();
-    return false;
 }
 
 bool pow2_raster(int N) { return N == 64 || N == 128 || N == 256 || N == 512; }

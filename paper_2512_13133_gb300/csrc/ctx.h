@@ -9,7 +9,7 @@ struct pcl_ctx {
     std::string err;
     void *ws = nullptr;
     size_t ws_bytes = 0;
-    size_t ws_refused = 0;  // the smallest optional workspace that did not fit (0: none yet)
+    size_t ws_refused = 0;  // an optional workspace that did not fit (0: none since one did)
     int *d_err = nullptr;  // device error word set by kernels whose bounded waits ran out
     unsigned long long wait_ns = 0;  // limit of each bounded device-side wait (0: one second)
     // device work counters: [0] window tasks the exact scan counted, [1] tasks in its windows,
