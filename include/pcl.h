@@ -309,7 +309,10 @@ pcl_status pcl_candidates_shard(pcl_ctx *ctx, const pcl_params *P, uint32_t mode
    mode = PCL_MODE_COSINE, but the scratch (area histogram, sorted order) is a
    fixed 8 MiB array in the library's device memory instead of the context
    workspace: 8 (N^2 + 2) + 8 n + 192 bytes must fit, otherwise
-   PCL_ERR_INVALID with the required size in pcl_last_error.  The first call
+   PCL_ERR_INVALID with the required size in pcl_last_error.  Where the array
+   also holds the vectors and the list of G3 as a matrix product (2,048 to 3,456
+   clips of 256x256 px, say), that is used, with the context's wait limit; otherwise the
+   band join does it all.  The first call
    on a device looks up the array's device address (cudaGetSymbolAddress);
    make that first call before any stream capture.  All calls share the one
    array: calls whose work overlaps on the GPU (other streams, other host

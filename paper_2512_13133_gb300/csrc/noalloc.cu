@@ -100,11 +100,14 @@ extern "C" pcl_status pcl_candidates_cosine_noalloc(pcl_ctx *ctx, const pcl_para
     cudaStream_t st = (cudaStream_t)stream;
     e = cudaMemsetAsync(d_count, 0, sizeof(uint64_t), st);
     // launch_band_join zeroes the counters, histogram and fill slots it uses
-    // before its kernels run; the sorted order is fully rewritten each call
+    // before its kernels run; the sorted order is fully rewritten each call; where
+    // the scratch has room for the product of G3 as well (2,048 to 3,456 clips of
+    // 256^2 px, say), it takes that
     if (e == cudaSuccess)
         e = pcl::launch_band_join(*P, *cs, ws, kScratchBytes, d_out, cap,
                                   reinterpret_cast<unsigned long long *>(d_count),
-                                  reinterpret_cast<unsigned long long *>(d_gate_counts), ctx->num_sms, st, 0, 1, 0);
+                                  reinterpret_cast<unsigned long long *>(d_gate_counts), ctx->num_sms, st, 0, 1,
+                                  ctx->wait_ns);
     if (e != cudaSuccess) {
         ctx->err = std::string("band join: ") + cudaGetErrorString(e);
         return PCL_ERR_CUDA;
