@@ -143,23 +143,19 @@ def alu_peak_tops(sm_mhz: float) -> float:
     return 152 * 128 * sm_mhz * 1e6 / 1e12
 
 
-def popc_peak_t(sm_mhz: float) -> float:
-    # 152 SMs x 16 population counts per SM per clock (a quarter of the
-    # 64-lane integer pipe)
-    return 152 * 16 * sm_mhz * 1e6 / 1e12
+# what the printed line holds of a run; everything else goes to DETAIL
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "roofline", "clocks", "e2e", "gpu_launches", "cpu_baseline")
+DETAIL = os.path.join(ROOT, "bench_detail.json")
 
 
-def popc_bound(pairs: int, ms: float, K: int, N: int, done: float = 1.0) -> dict:
-    """Popcount view of a window scan: by definition (2S+1)^2 N N/32 popcounts
-    of 32-bit words per pair, times the fraction of the window the scan
-    counted (done; the 512^2 scan skips groups of shifts by their profile
-    bounds); the carry-save sums issue 11 popcounts per 16 words, so this is
-    an effective rate of the popcount pipe."""
-    per = K * K * N * N / 32
-    ach = pairs * per * done / (ms / 1e3) / 1e12
-    return {"achieved": ach, "peak": popc_peak_t(2070.0), "unit": "T popc/s", "frac": ach / popc_peak_t(2070.0),
-            "work": f"{per:.3g} 32-bit popcounts per pair by definition x {done:.4f} of the window counted",
-            "peak_source": "derived: 152 SMs x 16 popcounts x 2.07 GHz"}
+def emit(line: dict, detail: str = DETAIL) -> None:
+    """Print the headline fields as one JSON line and write the whole record
+    (every stage's roofline, the engines, serving, mixed batches) to a file:
+    with all of it the line had grown past what is read back of a run's output."""
+    with open(detail, "w") as f:
+        json.dump(line, f, indent=1)
+    print(json.dumps({**{k: line[k] for k in HEADLINE if k in line}, "detail": os.path.basename(detail)}), flush=True)
 
 
 class Clocks:
@@ -615,7 +611,7 @@ def run_next(pcl, ctx, dev, wl, cs, P, steps: int, seed: int):
         return float(np.mean(ms))
 
     out = {}
-    # 512^2 rasters: the exact window scan (S = 32) on the same-seed pairs of
+    # 512^2 rasters: the exact engine (S = 32) on the same-seed pairs of
     # a 10,000-clip set of the scale recipe at that size, gates off
     w5 = exact512_workload(seed, 10_000)
     P5 = pcl.params(w5.window_dbu, w5.pitch_dbu, w5.marker_dbu, COS_NUM, COS_DEN, TOL, flags=pcl.P_NO_GATES)
@@ -626,19 +622,12 @@ def run_next(pcl, ctx, dev, wl, cs, P, steps: int, seed: int):
     pcl.pcl_stats_get(ctx, reset=True)
     e_ms = timed(lambda: pcl.pcl_match_pairs(ctx, P5, pcl.MODE_COSINE, cs5, cs5, p5, rec5), steps)
     ev5, tot5 = pcl.pcl_stats_get(ctx, reset=True)  # groups of shifts counted / in the windows
-    done5 = ev5 / tot5 if tot5 else 1.0
-    K5, NW5 = 2 * cs5.S + 1, cs5.N // 64
-    ops5 = 6.0 * K5 * K5 * cs5.N * NW5
-    ach5 = p5.shape[0] * ops5 * done5 / (e_ms / 1e3) / 1e12
+    groups5 = (2 * cs5.S + 1) * (cs5.S // 8 + (cs5.S + 7) // 8 + 1)  # in a pair's window
+    # 1: every pair was taken from its rectangles, which no popcount or ALU peak bounds
     out["exact_scan_512"] = {"clips": w5.n, "pairs": int(p5.shape[0]), "ms": e_ms,
                              "pairs_per_s": p5.shape[0] / (e_ms / 1e3),
                              "passes": int(pcl.records_to_numpy(rec5)["pass_"].sum()),
-                             "window_counted": done5,
-                             "roofline": {"bound": "alu", "achieved": ach5, "peak": alu_peak_tops(2070.0),
-                                          "unit": "Tops/s", "frac": ach5 / alu_peak_tops(2070.0),
-                                          "work": f"{ops5:.3g} int ops per pair (6 per shift, row and 64-bit word)"
-                                                  f" x {done5:.4f} of the window counted"},
-                             "popc_bound": popc_bound(int(p5.shape[0]), e_ms, K5, cs5.N, done5)}
+                             "groups_counted_per_pair": groups5 * ev5 / tot5 if tot5 else None}
     del cs5, p5, rec5
     # re-extraction
     hw = synth.preset("scale", seed=seed + 400, n_clips=wl.n, halo_dbu=wl.marker_dbu)
@@ -652,20 +641,12 @@ def run_next(pcl, ctx, dev, wl, cs, P, steps: int, seed: int):
     pcl.pcl_stats_get(ctx, reset=True, kernel="halo")
     m_ms = timed(lambda: pcl.pcl_match_halo(ctx, Ph, hcs, hcs, hb, nb, hp, hrec), steps)
     hev, htot = pcl.pcl_stats_get(ctx, reset=True, kernel="halo")
-    hdone = hev / htot if htot else 1.0
+    groups = (2 * hcs.S + 1) * (2 * hcs.S // 8 + 1)
     hr = pcl.records_to_numpy(hrec)
-    K, NW = 2 * hcs.S + 1, hcs.N // 64
-    ops = 6.0 * K * K * hcs.N * NW  # per pair: funnel shift, AND, popcount, add over every shift and word
     out["reextraction"] = {"clips": hw.n, "halo_dbu": hw.marker_dbu, "pairs": int(hp.shape[0]),
                            "halo_raster_ms": r_ms, "match_ms": m_ms,
                            "pairs_per_s": hp.shape[0] / (m_ms / 1e3), "passes": int(hr["pass_"].sum()),
-                           "window_counted": hdone,
-                           "roofline": {"bound": "alu", "achieved": hp.shape[0] * ops * hdone / (m_ms / 1e3) / 1e12,
-                                        "peak": alu_peak_tops(2070.0), "unit": "Tops/s",
-                                        "work": f"{ops:.3g} int ops per pair (6 per shift, row and word)"
-                                                f" x {hdone:.4f} of the window counted"}}
-    out["reextraction"]["roofline"]["frac"] = out["reextraction"]["roofline"]["achieved"] / alu_peak_tops(2070.0)
-    out["reextraction"]["popc_bound"] = popc_bound(int(hp.shape[0]), m_ms, K, hcs.N, hdone)
+                           "groups_counted_per_pair": groups * hev / htot if htot else None}
     del hcs, hb, nb, hp, hrec
     # surprisal of a pass graph: 1,000,000 nodes, 16,000,000 random edges
     rng = np.random.default_rng(seed)
@@ -1014,7 +995,8 @@ def run_ours(args, rank, world, local_rank):
                 # as a user calls it (pairs that can take their overlaps from the rectangles),
                 # and with a wait limit of the context's own, which keeps every pair on the
                 # tensor cores: only that is set against their peak
-                means = []
+                means, agree = [], []
+                ref = dense_fft if name == "dense32" else recs
                 for limit in (1_000_000_000, 0):
                     pcl.pcl_set_wait_limit(ctx, limit)
                     pcl.pcl_match_pairs(ctx, Pt, pcl.MODE_COSINE, cs, cs, tl, rl)
@@ -1030,6 +1012,10 @@ def run_ours(args, rank, world, local_rank):
                         torch.cuda.synchronize()
                         t_ms.append(a0.elapsed_time(a1))
                     means.append(float(np.mean(t_ms)))
+                    rt = pcl.records_to_numpy(rl)
+                    agree.append(bool(all((rt[f] == ref[f]).all() for f in ("score", "dx_dbu", "dy_dbu", "pass_"))))
+                    if name == "same_seed" and limit:  # the tensor cores' own records
+                        same_seed_recs[f"tc_{eng_name}"] = rt
                 tensor_ms, ms = means
                 flop = 2.0 * (2 * cs.S + 1) ** 2 * cs.N * cs.N * len(lst)
                 key = f"{eng_name}_{name}"
@@ -1037,21 +1023,8 @@ def run_ours(args, rank, world, local_rank):
                            "tensor_ms": tensor_ms, "tflops_useful": flop / (tensor_ms / 1e3) / 1e12,
                            "peak_tflops": pk["bf16_tflops"] * peak_mult,
                            "frac_of_peak": flop / (tensor_ms / 1e3) / 1e12 / (pk["bf16_tflops"] * peak_mult)}
-                if name == "dense32":
-                    rt = pcl.records_to_numpy(rl)
-                    tc[key]["agrees_with_fft"] = bool((rt["score"] == dense_fft["score"]).all() and
-                                                      (rt["dx_dbu"] == dense_fft["dx_dbu"]).all() and
-                                                      (rt["dy_dbu"] == dense_fft["dy_dbu"]).all() and
-                                                      (rt["pass_"] == dense_fft["pass_"]).all())
-                    tc[key]["speedup_vs_fft"] = fft["dense32"]["ms"] / ms
-                if name == "same_seed":
-                    tc[key]["speedup_vs_fft"] = fms / ms
-                    rt = pcl.records_to_numpy(rl)
-                    same_seed_recs[f"tc_{eng_name}"] = rt
-                    tc[key]["agrees_with_fft"] = bool((rt["score"] == recs["score"]).all() and
-                                                      (rt["dx_dbu"] == recs["dx_dbu"]).all() and
-                                                      (rt["dy_dbu"] == recs["dy_dbu"]).all() and
-                                                      (rt["pass_"] == recs["pass_"]).all())
+                tc[key]["tensor_agrees_with_fft"], tc[key]["agrees_with_fft"] = agree
+                tc[key]["speedup_vs_fft"] = (fft["dense32"]["ms"] if name == "dense32" else fms) / ms
         tc["device_error"] = pcl.pcl_device_error(ctx)
         fft["tc_engine"] = tc
         # the bound-pruned exact window scan as a cosine engine (no spectra):
@@ -1079,7 +1052,9 @@ def run_ours(args, rank, world, local_rank):
             ms = float(np.mean(x_ms))
             rt = pcl.records_to_numpy(rl)
             ex[name] = {"pairs": int(len(lst)), "ms": ms, "pairs_per_s": len(lst) / (ms / 1e3),
-                        "speedup_vs_fft": ref_ms / ms, "window_counted": ev / tot if tot else None,
+                        "speedup_vs_fft": ref_ms / ms,
+                        "groups_counted_per_pair": (2 * cs.S + 1) * (cs.S // 8 + (cs.S + 7) // 8 + 1) * ev / tot if tot
+                        else None,
                         "agrees_with_fft": bool((rt["score"] == ref["score"]).all() and
                                                 (rt["dx_dbu"] == ref["dx_dbu"]).all() and
                                                 (rt["dy_dbu"] == ref["dy_dbu"]).all() and
@@ -1343,7 +1318,7 @@ def run_ours(args, rank, world, local_rank):
                                 "single_thread": {"value": a1 / t1, "unit": UNIT, "cores": 1,
                                                   "sample": f"first {n_1} clips ({n_1*(n_1-1)//2} pairs screened "
                                                             f"both modes, {a1} aligned), {t1:.1f} s"}}
-    print(json.dumps(line), flush=True)
+    emit(line)
 
 
 def run_only(args):
