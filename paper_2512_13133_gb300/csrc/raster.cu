@@ -45,6 +45,32 @@ struct RasterCta {
     static constexpr int ctas = NW == 8 ? 4 : 12;  // resident per SM: registers and shared memory allow as many
 };
 
+// Indices of the nr rectangles by ascending area (ties by index) into order, by rank
+// counting with all T threads of the CTA, the areas staged CHUNK at a time (5,000
+// clips of 1,000 rectangles, 512x512 px: 10.1 ms by one warp from global memory, now
+// 1.7).  Clips of more than CHUNK rectangles are rare.
+template <int T, int CHUNK>
+__device__ __forceinline__ void order_many(const int4 *r4, uint32_t nr, long long *areas, uint16_t *order) {
+    auto area_of = [&](uint32_t m) {
+        const int4 q = __ldg(r4 + m);
+        return (long long)(q.z - q.x) * (long long)(q.w - q.y);
+    };
+    for (uint32_t t0 = 0; t0 < nr; t0 += T) {
+        const uint32_t t = t0 + threadIdx.x;
+        const long long at = t < nr ? area_of(t) : 0;
+        uint32_t rank = 0;
+        for (uint32_t base = 0; base < nr; base += CHUNK) {
+            const uint32_t cnt = min((uint32_t)CHUNK, nr - base);
+            __syncthreads();  // the areas staged before are no longer read
+            for (uint32_t m = threadIdx.x; m < cnt; m += T) areas[m] = area_of(base + m);
+            __syncthreads();
+#pragma unroll 4
+            for (uint32_t m = 0; m < cnt; ++m) rank += areas[m] < at + (base + m < t ? 1 : 0) ? 1u : 0u;
+        }
+        if (t < nr) order[rank] = (uint16_t)t;
+    }
+}
+
 // One CTA per clip.  The rectangles (a chunk at a time) become pixel
 // ranges in shared memory; then each warp has one job with a lane per
 // rectangle: setting the rows' bits, adding the pixels of its 16x16 blocks and
@@ -160,7 +186,8 @@ __global__ void __launch_bounds__(RasterCta<NW>::threads, RasterCta<NW>::ctas) r
                 if (q.w != W) { hasy = 1; loy = min(loy, q.w); hiy = max(hiy, q.w); } else border = 1;
             }
             // rectangles by ascending area (ties by index): rank by counting
-            for (uint32_t t = lane; nr <= CHUNK && t < cnt; t += 32) {
+            for (uint32_t t = lane; t < cnt; t += 32) {
+                if (nr > CHUNK) break;  // order_many
                 const long long at = areas[t];  // before t: smaller areas, and equal ones of smaller index
                 uint32_t rank = 0;
 #pragma unroll 4
@@ -169,26 +196,7 @@ __global__ void __launch_bounds__(RasterCta<NW>::threads, RasterCta<NW>::ctas) r
             }
         }
     }
-    // the same for more than a chunk of rectangles by all threads, the areas staged a
-    // chunk at a time (5,000 clips of 1,000 rectangles, 512x512 px: 10.1 ms by the one warp, now 1.7)
-    for (uint32_t t0 = 0; nr > CHUNK && t0 < nr; t0 += T) {
-        const uint32_t t = t0 + tid;
-        auto area_of = [&](uint32_t m) {
-            const int4 q = __ldg(r4 + m);
-            return (long long)(q.z - q.x) * (long long)(q.w - q.y);
-        };
-        const long long at = t < nr ? area_of(t) : 0;
-        uint32_t rank = 0;
-        for (uint32_t base = 0; base < nr; base += CHUNK) {
-            const uint32_t cnt = min((uint32_t)CHUNK, nr - base);
-            __syncthreads();  // the areas staged before are no longer read
-            for (uint32_t m = tid; m < cnt; m += T) areas[m] = area_of(base + m);
-            __syncthreads();
-#pragma unroll 4
-            for (uint32_t m = 0; m < cnt; ++m) rank += areas[m] < at + (base + m < t ? 1 : 0) ? 1u : 0u;
-        }
-        if (t < nr) cs.rorder[r0 + rank] = (uint16_t)t;
-    }
+    if (nr > CHUNK) order_many<T, CHUNK>(r4, nr, areas, cs.rorder + r0);
     if (warp == 0) {
         hasx = __reduce_or_sync(0xffffffffu, hasx);
         hasy = __reduce_or_sync(0xffffffffu, hasy);
