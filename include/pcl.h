@@ -344,7 +344,8 @@ pcl_status pcl_candidates_cosine_noalloc(pcl_ctx *ctx, const pcl_params *P, cons
    rectangles each, no two of a clip sharing a pixel, are not scanned: their
    overlaps at every shift are summed from the rectangles (the same integers;
    rectangles that are not the ones of the raster are noticed, and the pair is
-   scanned, but rect_off has to hold offsets into rects).
+   scanned, but rect_off has to hold offsets into rects; until the call's work
+   is done the records hold values of its own).
    With cos_engine = PCL_ENGINE_TC_DIRECT (FP16 operands),
    PCL_ENGINE_TC_DIRECT_BF16 (BF16 operands) or PCL_ENGINE_TC_DIRECT_FP8
    (E4M3 operands) the overlaps of every shift come

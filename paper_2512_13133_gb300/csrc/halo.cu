@@ -294,6 +294,42 @@ __device__ __forceinline__ bool ranges_are_halo(const short4 *r, int n, const ui
     return same && pcl::rect_corr::ranges_in_raster(r, n, hb, halo_words(N, S), S, lane);
 }
 
+// The clips' verdicts (rect_corr.cuh), a warp per clip: the representatives' against
+// their window rasters, then the members' against their halo rasters
+constexpr int kRectWarps = 4;
+
+__global__ void __launch_bounds__(32 * kRectWarps) halo_verdict_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B,
+                                                                      const uint64_t *__restrict__ hbits,
+                                                                      const uint32_t *__restrict__ norms, uint64_t n,
+                                                                      const unsigned long long *d_n, pcl_record *out) {
+    namespace rc = pcl::rect_corr;
+    const uint64_t clips = (uint64_t)A.n_clips + B.n_clips;
+    if (d_n && *d_n < n) n = *d_n;
+    if (!rc::verdicts_pay(n, clips)) return;
+    __shared__ short4 ranges[kRectWarps][rc::kRectMax];
+    const Geo g = make_geo(prm);
+    const int N = g.N, S = g.S, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int psh = (g.p & (g.p - 1)) == 0 ? 31 - __clz(g.p) : -1;
+    short4 *r = ranges[warp];
+    for (uint64_t k = (uint64_t)blockIdx.x * kRectWarps + warp; k < clips; k += (uint64_t)gridDim.x * kRectWarps) {
+        bool ok = false;
+        if (k < A.n_clips) {
+            ok = rc::window_verdict(A, (uint32_t)k, g, psh, r, lane);
+        } else {
+            const uint32_t c = (uint32_t)(k - A.n_clips), o = __ldg(B.rect_off + c);
+            const int m = (int)(__ldg(B.rect_off + c + 1) - o);
+            if (m >= 0 && m <= rc::kRectMax) {
+                __syncwarp();  // the previous clip's ranges are no longer read
+                rc::stage_rects(reinterpret_cast<const int4 *>(B.rects) + o, m, g.p, psh, -S, N + S, r, lane);
+                __syncwarp();
+                ok = ranges_are_halo(r, m, hbits + (size_t)c * halo_side(N, S) * halo_words(N, S),
+                                     norms + (size_t)c * norms_stride(N, S), g, lane);
+            }
+        }
+        if (lane == 0) *rc::verdict_at(out, k) = ok ? 1 : 0;
+    }
+}
+
 // One warp per pair: the record from the rectangles (rect_corr.cuh; A's cut to
 // its window, B's to the halo) for clips of few enough rectangles that share no
 // pixel and are the rasters (the buffers may have been written again, and b may be
@@ -301,16 +337,15 @@ __device__ __forceinline__ bool ranges_are_halo(const short4 *r, int n, const ui
 // overlap against the tabulated n_B(s).  The other pairs
 // get a record with flags = kRectPending, for halo_pair_kernel.  A pair decided
 // here counts as one group of shifts in stats.
-constexpr int kRectWarps = 4;
-
 __global__ void __launch_bounds__(32 * kRectWarps, 8) halo_rect_kernel(pcl_params prm, pcl_clipset A, pcl_clipset B,
                                                                     const uint64_t *__restrict__ hbits,
                                                                     const uint32_t *__restrict__ norms,
                                                                     const pcl_pair *pairs, uint64_t npairs,
                                                                     const unsigned long long *d_n, pcl_record *out,
-                                                                    unsigned long long *stats) {
+                                                                    unsigned long long *stats, bool verdicts) {
     namespace rc = pcl::rect_corr;
     if (d_n && *d_n < npairs) npairs = *d_n;
+    verdicts = verdicts && rc::verdicts_pay(npairs, (uint64_t)A.n_clips + B.n_clips);
     extern __shared__ __align__(16) unsigned char smem[];
     const Geo g = make_geo(prm);
     const int N = g.N, S = g.S, K = 2 * S + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -335,15 +370,16 @@ __global__ void __launch_bounds__(32 * kRectWarps, 8) halo_rect_kernel(pcl_param
         const uint32_t oa = rects ? __ldg(A.rect_off + pr.a) : 0u, ob = rects ? __ldg(B.rect_off + pr.b) : 0u;
         const int na = rects ? (int)(__ldg(A.rect_off + pr.a + 1) - oa) : 0;
         const int nb = rects ? (int)(__ldg(B.rect_off + pr.b + 1) - ob) : 0;
-        bool ok = rects && pa != 0 && na <= rc::kRectMax && nb <= rc::kRectMax;
+        bool ok = rects && pa != 0 && na >= 0 && nb >= 0 && na <= rc::kRectMax && nb <= rc::kRectMax;
+        if (verdicts) ok = ok && out[t].reserved != 0;
         if (ok) {
             __syncwarp();  // the scratch's previous contents are no longer read
             const uint32_t aa = rc::stage_rects(reinterpret_cast<const int4 *>(A.rects) + oa, na, g.p, psh, 0, N, s.ra, lane);
             rc::stage_rects(reinterpret_cast<const int4 *>(B.rects) + ob, nb, g.p, psh, -S, N + S, s.rb, lane);
             __syncwarp();
-            ok = rc::ranges_are_raster(s.ra, na, aa, A, pr.a, g, lane) &&
-                 ranges_are_halo(s.rb, nb, hbits + (size_t)pr.b * halo_side(N, S) * halo_words(N, S),
-                                 norms + (size_t)pr.b * norms_stride(N, S), g, lane);
+            ok = verdicts || (rc::ranges_are_raster(s.ra, na, aa, A, pr.a, g, lane) &&
+                              ranges_are_halo(s.rb, nb, hbits + (size_t)pr.b * halo_side(N, S) * halo_words(N, S),
+                                              norms + (size_t)pr.b * norms_stride(N, S), g, lane));
         }
         if (!ok) {
             rec.flags = rc::kRectPending;
@@ -630,8 +666,18 @@ cudaError_t launch_pair(const pcl_params &prm, const Geo &g, const pcl_clipset &
         if (e != cudaSuccess) return e;
         const uint64_t most = (uint64_t)num_sms * (uint64_t)(rect_sm > 0 ? rect_sm : 1);
         const uint64_t need = (n + kRectWarps - 1) / kRectWarps;
-        halo_rect_kernel<<<(unsigned)(need < most ? need : most), 32 * kRectWarps, rs, st>>>(prm, a, b, hb, nb, pairs, n,
-                                                                                            d_n, out, stats);
+        namespace rc = pcl::rect_corr;
+        const uint64_t clips = (uint64_t)a.n_clips + b.n_clips, grid = (clips + kRectWarps - 1) / kRectWarps;
+        const bool verdicts = clips && rc::has_rects(a) && rc::has_rects(b) && rc::verdicts_pay(n, clips);
+        if (verdicts) {
+            const uint64_t full = (uint64_t)num_sms * 16, blocks = (n + 255) / 256;
+            halo_verdict_kernel<<<(unsigned)(grid < full ? grid : full), 32 * kRectWarps, 0, st>>>(prm, a, b, hb, nb, n,
+                                                                                                  d_n, out);
+            rc::pair_verdict_kernel<<<(unsigned)(blocks < full ? blocks : full), 256, 0, st>>>(
+                a.n_clips, b.n_clips, a.n_clips, clips, pairs, n, d_n, out);
+        }
+        halo_rect_kernel<<<(unsigned)(need < most ? need : most), 32 * kRectWarps, rs, st>>>(
+            prm, a, b, hb, nb, pairs, n, d_n, out, stats, verdicts);
     }
     halo_pair_kernel<NW><<<(unsigned)(n < cap ? n : cap), kThreads, sm, st>>>(prm, a, b, hb, nb, pairs, n, d_n, out,
                                                                              stats);

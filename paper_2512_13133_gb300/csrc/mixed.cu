@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(32 * kRectWarps) mixed_rect_kernel(pcl_params 
             m &= m - 1u;
             const pcl_pair pr{work[base + src].a, work[base + src].b};
             if (cs.pop[pr.a] != 0 && cs.pop[pr.b] != 0)
-                rect_corr::rect_record(prm, g, psh, cs, cs, pr, s, out + base + src, lane);
+                rect_corr::rect_record(prm, g, psh, cs, cs, pr, s, -1, out + base + src, lane);
         }
     }
 }
